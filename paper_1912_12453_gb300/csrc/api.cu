@@ -68,22 +68,21 @@ chns_status prepare(chns_mesh *m, const double *Un, const double *Uo, cudaStream
   return check_launch();
 }
 
-chns_status residual_prepared(chns_mesh *m, const PhysCoef &pc, const double *Un, const double *ut,
-                              const double *dl, const double *forcing, const double *bc, double *F,
-                              cudaStream_t st) {
-  CHNS_CUDA_TRY(cudaMemsetAsync(F, 0, sizeof(double) * m->n_nodes * m->nf, st));
-  launch_residual(m, pc, ut, dl, forcing, F, st);
-  launch_dirichlet_res(m, Un, bc, F, st);
-  return check_launch();
-}
-
-// element-local J.w buffer of precision T (n_elem * 2^dim * nf values)
+// element-local buffer of precision T (n_elem * 2^dim * nf values)
 template <typename T>
 chns_status ensure_ebuf(chns_mesh *m, T **E) {
   DevBuf &b = sizeof(T) == 8 ? m->ws.e64 : m->ws.e32;
   TRY(b.ensure(sizeof(T) * (m->n_elem << m->dim) * m->nf));
   *E = b.as<T>();
   return CHNS_OK;
+}
+
+chns_status residual_into(chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const double *forcing,
+                          const double *bc, double *F, cudaStream_t st) {
+  double *E = nullptr;
+  TRY(ensure_ebuf<double>(m, &E));
+  launch_residual(m, pc, Un, Uo, forcing, bc, E, F, st);
+  return check_launch();
 }
 
 template <typename T>
@@ -622,11 +621,9 @@ chns_status newton_step(chns_mesh *m, const chns_params *p, const chns_solver_op
   // block iteration (Sec. 3.1, Fig. flowchart_block); the other block's rows
   // are identity rows of J.w and zero rows of the residual
   uint32_t fmask = 0xffu;
-  double *ut = nullptr, *dl = nullptr;
   auto residual = [&](double *fn) -> chns_status {
-    TRY(prepare<double>(m, U, Un, st, &ut, &dl));
     if (stats) { TRY(ensure_events(ws, 64)); CHNS_CUDA_TRY(cudaEventRecord(ws.ev[60], st)); }
-    TRY(residual_prepared(m, pc, U, ut, dl, forcing, bc, F, st));
+    TRY(residual_into(m, pc, U, Un, forcing, bc, F, st));
     if (fmask != 0xffu) vec_mask_fields(F, m->n_nodes, nf, fmask, st);
     if (stats) CHNS_CUDA_TRY(cudaEventRecord(ws.ev[61], st));
     TRY(norm2(m, F, fn, st));
@@ -1022,10 +1019,8 @@ chns_status chns_residual(const chns_mesh *mc, const chns_params *p, const doubl
   if (!U_new || !U_old || !F) { set_error("null vector"); return CHNS_ERR_ARG; }
   chns_mesh *m = const_cast<chns_mesh *>(mc);
   cudaStream_t st = S(stream);
-  double *ut = nullptr, *dl = nullptr;
-  TRY(prepare<double>(m, U_new, U_old, st, &ut, &dl));
   PhysCoef pc = make_coef(*p, m->lo, m->hi);
-  return residual_prepared(m, pc, U_new, ut, dl, forcing, bc, F, st);
+  return residual_into(m, pc, U_new, U_old, forcing, bc, F, st);
 }
 
 chns_status chns_jacvec(const chns_mesh *mc, const chns_params *p, const double *U_new, const double *U_old,
@@ -1069,7 +1064,7 @@ chns_status chns_init_mu(const chns_mesh *mc, const chns_params *p, double *U, v
          *z = pv + 3 * n;
   double *ut = nullptr, *dl = nullptr;
   TRY(prepare<double>(m, U, U, st, &ut, &dl));
-  TRY(residual_prepared(m, pc, U, ut, dl, nullptr, nullptr, r, st));
+  TRY(residual_into(m, pc, U, U, nullptr, nullptr, r, st));
   vec_mask_field(r, m->n_nodes, nf, imu, 1.0, st);
   // lumped mass: d = M 1 on the mu field (z holds the indicator of the mu field)
   TRY(ws.red.ensure(sizeof(double) * (kMaxRestart + 16) * red_blocks()));
@@ -1125,14 +1120,12 @@ chns_status chns_tau_floor_count(const chns_mesh *mc, const chns_params *p, cons
   if (!U_new || !U_old || !count) { set_error("null argument"); return CHNS_ERR_ARG; }
   chns_mesh *m = const_cast<chns_mesh *>(mc);
   cudaStream_t st = S(stream);
-  double *ut = nullptr, *dl = nullptr;
-  TRY(prepare<double>(m, U_new, U_old, st, &ut, &dl));
   Workspace &ws = m->ws;
   TRY(ws.count.ensure(sizeof(unsigned long long)));
   TRY(ensure_pinned(ws));
   unsigned long long *cnt = ws.count.as<unsigned long long>();
   CHNS_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
-  launch_tau_floor_count(m, make_coef(*p, m->lo, m->hi), ut, dl, cnt, st);
+  launch_tau_floor_count(m, make_coef(*p, m->lo, m->hi), U_new, U_old, cnt, st);
   TRY(check_launch());
   CHNS_CUDA_TRY(cudaMemcpyAsync(ws.hpinned, cnt, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
   CHNS_CUDA_TRY(cudaStreamSynchronize(st));

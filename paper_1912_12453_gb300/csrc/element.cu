@@ -26,6 +26,10 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 
 // ---------------------------------------------------------------- dual numbers
+// mad(a, b, c) = a b + c, one rounding per scalar fma
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+
 template <typename T>
 struct Dl {
   T v, d;
@@ -35,12 +39,23 @@ struct Dl {
 };
 template <typename T> __device__ __forceinline__ Dl<T> operator+(Dl<T> a, Dl<T> b) { return Dl<T>(a.v + b.v, a.d + b.d); }
 template <typename T> __device__ __forceinline__ Dl<T> operator-(Dl<T> a, Dl<T> b) { return Dl<T>(a.v - b.v, a.d - b.d); }
-template <typename T> __device__ __forceinline__ Dl<T> operator-(Dl<T> a) { return Dl<T>(-a.v, -a.d); }
-template <typename T> __device__ __forceinline__ Dl<T> operator*(Dl<T> a, Dl<T> b) { return Dl<T>(a.v * b.v, a.d * b.v + a.v * b.d); }
-template <typename T> __device__ __forceinline__ Dl<T> operator+(Dl<T> a, T b) { return Dl<T>(a.v + b, a.d); }
-template <typename T> __device__ __forceinline__ Dl<T> operator-(Dl<T> a, T b) { return Dl<T>(a.v - b, a.d); }
+template <typename T> __device__ __forceinline__ Dl<T> operator*(Dl<T> a, Dl<T> b) { return Dl<T>(a.v * b.v, mad(a.d, b.v, a.v * b.d)); }
 template <typename T> __device__ __forceinline__ Dl<T> operator*(Dl<T> a, T b) { return Dl<T>(a.v * b, a.d * b); }
-template <typename T> __device__ __forceinline__ Dl<T> operator*(T b, Dl<T> a) { return Dl<T>(a.v * b, a.d * b); }
+template <typename T> __device__ __forceinline__ Dl<T> mad(Dl<T> a, Dl<T> b, Dl<T> c) {
+  return Dl<T>(mad(a.v, b.v, c.v), mad(a.d, b.v, mad(a.v, b.d, c.d)));
+}
+template <typename T> __device__ __forceinline__ Dl<T> mad(Dl<T> a, T b, Dl<T> c) {
+  return Dl<T>(mad(a.v, b, c.v), mad(a.d, b, c.d));
+}
+// a b + c with a constant c: the derivative of c is zero
+template <typename T> __device__ __forceinline__ Dl<T> madc(Dl<T> a, T b, T c) { return Dl<T>(mad(a.v, b, c), a.d * b); }
+template <typename T> __device__ __forceinline__ Dl<T> madc(Dl<T> a, Dl<T> b, T c) {
+  return Dl<T>(mad(a.v, b.v, c), mad(a.d, b.v, a.v * b.d));
+}
+__device__ __forceinline__ float madc(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double madc(double a, double b, double c) { return fma(a, b, c); }
+template <typename T> __device__ __forceinline__ Dl<T> subc(Dl<T> a, T b) { return Dl<T>(a.v - b, a.d); }
+template <typename T> __device__ __forceinline__ T subc(T a, T b) { return a - b; }
 template <typename T> __device__ __forceinline__ T val(Dl<T> a) { return a.v; }
 __device__ __forceinline__ float val(float a) { return a; }
 __device__ __forceinline__ double val(double a) { return a; }
@@ -59,84 +74,138 @@ template <typename T> __device__ __forceinline__ Dl<T> rsqrt_(Dl<T> a) {
   return Dl<T>(r, T(-0.5) * a.d * r * r * r);
 }
 
+// x 2^k, exact.  In double on the exponent bits: the FP64 pipe issues one
+// warp instruction every 16 cycles on this part, the integer pipe is idle (x
+// is zero or normal, and so is the result for box extents between 1e-60 and
+// 1e60 and levels up to 20: |k| <= 80).
+__device__ __forceinline__ double scale2(double x, int k) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double(hi == 0 ? 0 : hi + k * (1 << 20), __double2loint(x));
+}
+__device__ __forceinline__ float scale2(float x, int k) { return x * __int_as_float((127 + k) << 23); }
+__device__ __forceinline__ double flip_if(double x, bool f) {
+  return __hiloint2double(__double2hiint(x) ^ (f ? int(0x80000000u) : 0), __double2loint(x));
+}
+__device__ __forceinline__ float flip_if(float x, bool f) {
+  return __int_as_float(__float_as_int(x) ^ (f ? int(0x80000000u) : 0));
+}
+
 // ---------------------------------------------------------------- butterflies
-template <typename T>
+// With g = 1/sqrt(3), CA = (1 + g)/2 and CB = (1 - g)/2, a corner pair (u own,
+// o other) gives CA u + CB o at the own Gauss point and (u - o)/h (signed by
+// the lane's bit) as derivative.  The common factor CA is taken out of every
+// stage: a stage is u + TB o (TB = CB/CA, one fma) and u - o (one add), and
+// each result is scaled once at the end (values by CA^D, derivatives by
+// CA^(D-1) (+-1/h)), which leaves the differences of the corner data exact.
+constexpr double CA = 0.78867513459481288225;
+constexpr double TB = 0.26794919243112270647;  // CB / CA = 2 - sqrt(3)
+template <int D> constexpr double CAD = D == 2 ? CA * CA : CA * CA * CA;
+
+template <int D, typename T>
 struct Stage {
-  T ca, cb;      // (1 + g)/2, (1 - g)/2 with g = 1/sqrt(3)
-  T sh[3];       // (+1 or -1 by lane bit) / h_a : physical derivative of the 1D hat
+  T v;      // factor of values
+  T sg[D];  // factors of derivatives
+  T sh[D];  // +-1 / h_a
+  T cS;     // W CA^D: weight of S in the contraction (W = prod h/2)
+  T cV[D];  // W CA^(D-1) (+-1/h_a): weight of V_a
 };
 
-template <typename T>
-__device__ __forceinline__ void st_vd(T u, int m, T ca, T cb, T sh, T &v, T &d) {
-  T o = __shfl_xor_sync(FULL, u, m);
-  v = ca * u + cb * o;
-  d = sh * (u - o);
+// UNIT: the stage with its factor, CA u + CB o.  phi* is clipped at |phi| = 1,
+// where both bulk phases sit, and J.w jumps there: in float the branch of a
+// Gauss point hangs on the last bits of phi^{k+1}.  phi~ and the phi increment
+// keep this evaluation in float, so that the branches stay what they were
+// before the factors were taken out.
+template <bool UNIT, typename T>
+__device__ __forceinline__ T st_mix(T u, T o) {
+  if (UNIT) return mad(T(0.5) + T(0.28867513459481288225), u, (T(0.5) - T(0.28867513459481288225)) * o);
+  return mad(T(TB), o, u);
 }
-template <typename T>
-__device__ __forceinline__ T st_v(T u, int m, T ca, T cb) {
+template <bool UNIT = false, typename T>
+__device__ __forceinline__ void st_vd(T u, int m, T &v, T &d) {
   T o = __shfl_xor_sync(FULL, u, m);
-  return ca * u + cb * o;
+  v = st_mix<UNIT>(u, o);
+  d = u - o;
+}
+template <bool UNIT = false, typename T>
+__device__ __forceinline__ T st_v(T u, int m) {
+  return st_mix<UNIT>(u, __shfl_xor_sync(FULL, u, m));
 }
 
-// value only
+// value only, without its factor
 template <int D, typename T>
-__device__ __forceinline__ T ip_v(T u, const Stage<T> &s) {
-  T a = st_v(u, 1, s.ca, s.cb);
-  a = st_v(a, 2, s.ca, s.cb);
-  if (D == 3) a = st_v(a, 4, s.ca, s.cb);
+__device__ __forceinline__ T ip_v(T u) {
+  T a = st_v(u, 1);
+  a = st_v(a, 2);
+  if (D == 3) a = st_v(a, 4);
   return a;
 }
 
 // value and gradient
-template <int D, typename T>
-__device__ __forceinline__ void ip_vg(T u, const Stage<T> &s, T &v, T *g) {
+template <int D, bool UNIT = false, typename T>
+__device__ __forceinline__ void ip_vg(T u, const Stage<D, T> &s, T &v, T *g) {
   T A, Bx;
-  st_vd(u, 1, s.ca, s.cb, s.sh[0], A, Bx);
+  st_vd<UNIT>(u, 1, A, Bx);
   if (D == 2) {
-    st_vd(A, 2, s.ca, s.cb, s.sh[1], v, g[1]);
-    g[0] = st_v(Bx, 2, s.ca, s.cb);
+    st_vd<UNIT>(A, 2, v, g[1]);
+    g[0] = st_v<UNIT>(Bx, 2);
   } else {
     T AA, AB;
-    st_vd(A, 2, s.ca, s.cb, s.sh[1], AA, AB);
-    T BA = st_v(Bx, 2, s.ca, s.cb);
-    st_vd(AA, 4, s.ca, s.cb, s.sh[2], v, g[2]);
-    g[1] = st_v(AB, 4, s.ca, s.cb);
-    g[0] = st_v(BA, 4, s.ca, s.cb);
+    st_vd<UNIT>(A, 2, AA, AB);
+    T BA = st_v<UNIT>(Bx, 2);
+    st_vd<UNIT>(AA, 4, v, g[D - 1]);
+    g[1] = st_v<UNIT>(AB, 4);
+    g[0] = st_v<UNIT>(BA, 4);
   }
+  if (!UNIT) v *= s.v;
+#pragma unroll
+  for (int a = 0; a < D; ++a) g[a] *= UNIT ? s.sh[a] : s.sg[a];
 }
 
 // value, gradient and mixed second derivatives (xy; xy, xz, yz in 3D); the
-// pure second derivatives of Q1 vanish on an axis-aligned box
-template <int D, typename T>
-__device__ __forceinline__ void ip_full(T u, const Stage<T> &s, T &v, T *g, T *hs) {
+// pure second derivatives of Q1 vanish on an axis-aligned box.  The second
+// derivatives come out as the product of the two derivative factors.
+template <int D, bool UNIT = false, typename T>
+__device__ __forceinline__ void ip_full(T u, const Stage<D, T> &s, T &v, T *g, T *hs) {
+  const T *f = UNIT ? s.sh : s.sg;
   T A, Bx;
-  st_vd(u, 1, s.ca, s.cb, s.sh[0], A, Bx);
+  st_vd<UNIT>(u, 1, A, Bx);
   if (D == 2) {
-    st_vd(A, 2, s.ca, s.cb, s.sh[1], v, g[1]);
-    st_vd(Bx, 2, s.ca, s.cb, s.sh[1], g[0], hs[0]);
+    st_vd<UNIT>(A, 2, v, g[1]);
+    st_vd<UNIT>(Bx, 2, g[0], hs[0]);
+    hs[0] *= f[0] * f[1];
   } else {
     T AA, AB, BA, BB;
-    st_vd(A, 2, s.ca, s.cb, s.sh[1], AA, AB);
-    st_vd(Bx, 2, s.ca, s.cb, s.sh[1], BA, BB);
-    st_vd(AA, 4, s.ca, s.cb, s.sh[2], v, g[2]);
-    st_vd(AB, 4, s.ca, s.cb, s.sh[2], g[1], hs[2]);
-    st_vd(BA, 4, s.ca, s.cb, s.sh[2], g[0], hs[1]);
-    hs[0] = st_v(BB, 4, s.ca, s.cb);
+    st_vd<UNIT>(A, 2, AA, AB);
+    st_vd<UNIT>(Bx, 2, BA, BB);
+    st_vd<UNIT>(AA, 4, v, g[D - 1]);
+    st_vd<UNIT>(AB, 4, g[1], hs[2]);
+    st_vd<UNIT>(BA, 4, g[0], hs[1]);
+    hs[0] = st_v<UNIT>(BB, 4);
+    hs[0] *= f[0] * f[1];
+    hs[1] *= f[0] * f[D - 1];
+    hs[2] *= f[1] * f[D - 1];
   }
+  if (!UNIT) v *= s.v;
+#pragma unroll
+  for (int a = 0; a < D; ++a) g[a] *= f[a];
 }
 
-// transpose: r_node = sum_gp N_node(gp) S(gp) + grad N_node(gp) . V(gp)
+// transpose: r_node = W sum_gp N_node(gp) S(gp) + grad N_node(gp) . V(gp)
 template <int D, typename T>
-__device__ __forceinline__ T contract(T S, const T *V, const Stage<T> &s) {
-  T X = s.ca * S + s.sh[0] * V[0] + __shfl_xor_sync(FULL, s.cb * S - s.sh[0] * V[0], 1);
-  T Y1 = s.ca * V[1] + __shfl_xor_sync(FULL, s.cb * V[1], 1);
+__device__ __forceinline__ T contract(T S, const T *V, const Stage<D, T> &s) {
+  const T tb = T(TB);
+  S *= s.cS;
+  const T V0 = V[0] * s.cV[0], V1 = V[1] * s.cV[1];
+  T X = S + V0 + __shfl_xor_sync(FULL, mad(tb, S, -V0), 1);
+  T Y1 = mad(tb, __shfl_xor_sync(FULL, V1, 1), V1);
   if (D == 2) {
-    return s.ca * X + s.sh[1] * Y1 + __shfl_xor_sync(FULL, s.cb * X - s.sh[1] * Y1, 2);
+    return X + Y1 + __shfl_xor_sync(FULL, mad(tb, X, -Y1), 2);
   } else {
-    T Y2 = s.ca * V[2] + __shfl_xor_sync(FULL, s.cb * V[2], 1);
-    T X2 = s.ca * X + s.sh[1] * Y1 + __shfl_xor_sync(FULL, s.cb * X - s.sh[1] * Y1, 2);
-    T Z2 = s.ca * Y2 + __shfl_xor_sync(FULL, s.cb * Y2, 2);
-    return s.ca * X2 + s.sh[2] * Z2 + __shfl_xor_sync(FULL, s.cb * X2 - s.sh[2] * Z2, 4);
+    const T V2 = V[D - 1] * s.cV[D - 1];
+    T Y2 = mad(tb, __shfl_xor_sync(FULL, V2, 1), V2);
+    T X2 = X + Y1 + __shfl_xor_sync(FULL, mad(tb, X, -Y1), 2);
+    T Z2 = mad(tb, __shfl_xor_sync(FULL, Y2, 2), Y2);
+    return X2 + Z2 + __shfl_xor_sync(FULL, mad(tb, X2, -Z2), 4);
   }
 }
 
@@ -255,15 +324,23 @@ struct GpIn {
   S dv[D];             // v^{k+1} - v^k
   S dphi;              // phi^{k+1} - phi^k
   S phin, dphin[D];    // phi^{k+1} and its gradient
-  S f[D + 3];          // forcing at t_{k+1/2}
 };
 
+// Everything that depends only on the parameters and the box is folded on the
+// host; what depends on the leaf is a power of two of its level.
 template <typename T>
 struct KCoef {
-  T inv_dt, four_dt2, alpha, beta, gamma, xi, jc;
-  T inv_Pe, inv_We, inv_Re, inv_Fr, CnWe, inv_PeCn, Cn2, C_I;
-  T g[3];
-  T ext[3];  // box extent per axis
+  T inv_dt, four_dt2, alpha, beta;
+  T gRe, xRe;              // eta / Re = gRe phi* + xRe
+  T jcP;                   // J / Pe = jcP grad mu
+  T inv_We, CnWe, inv_PeCn, Cn2;
+  T gFr[3];                // gravity / Fr
+  T inv_Fr, g[3];          // energy
+  // geometry of a leaf of level 0; a leaf of level l has these times a power of 2^l
+  T G0[3];                 // G = 4 / ext^2
+  T CIGG0, inv_trG0;       // C_I G:G and 1 / tr G
+  T sg0[3], sh0[3], cS0, cV0[3];  // Stage without the signs
+  T W0;                    // prod ext / 2
 };
 
 template <int D> __device__ __forceinline__ int hidx(int i, int j) {
@@ -272,90 +349,113 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 }
 
 // Weak-form coefficients at one Gauss point: the row of test function N_a
-// receives W (N_a Sq[k] + sum_j d_j N_a Vq[k][j]) for equation k.  floored:
-// whether the tau_m radicand was raised to 4/dt^2.
-template <int D, typename T, typename S>
-__device__ __forceinline__ void gp_physics(const KCoef<T> &c, const T *G, T CI_GG, T inv_trG,
-                                           const GpIn<D, S> &q, S *Sq, S (*Vq)[D], bool &floored) {
+// receives W (N_a Sq[k] + sum_j d_j N_a Vq[k][j]) for equation k.  f: the
+// nodal source at the Gauss point (HASF).  CnWeH: Cn/We over the factor left in
+// hphit.  floored: whether the tau_m
+// radicand was raised to 4/dt^2.
+//
+// The terms of Sec. 3.4 share factors.  With A_i = rho (dv_i/dt - g_i/Fr) - f_i,
+// c_j = rho v~_j + J_j/Pe and t_i = tau_m R_m,i:
+//   R_m,i        = A_i + d_j v~_i (c_j - d_j eta/Re) + capillary_i + d_i p~/We,
+//   momentum S_i = A_i + d_j v~_i (c_j - t_j)
+//                  (advection, flux and cross stress in one product),
+//   momentum V_ij = (t_i/rho) (c_j - t_j) - Cn/We d_i phi~ d_j phi~ + eta/Re d_j v~_i
+//                  (streamline, Reynolds and flux stabilisation in one product),
+//   v~.G v~ + v~.G J/(rho Pe) = (1/rho) sum_i G_i v~_i c_i.
+// That takes two matrix-vector products instead of four, one outer product
+// instead of three, and the two quotients 1/rho and rad^(-1/2) only (tau_c =
+// sqrt(rad)/tr G = rad tau_m/tr G).  Every quotient of the geometry is a power
+// of two times a constant of the box.  Bound by the FP64 pipe (residual, J.w)
+// and by the FP32 issue slots (J.w in float).  Measured on GB300, before ->
+// after: residual of the level-6 octree (262,144 leaves) 2.34 -> 1.41 ms, FP64
+// J.w of 77,932 adaptive leaves 1.27 -> 0.79 ms, FP32 J.w of the level-6 octree
+// 132 -> 116 us (element kernel alone 88 -> 69 us).
+template <int D, bool HASF, typename T, typename S>
+__device__ __forceinline__ void gp_physics(const KCoef<T> &c, const T *G, T CI_GG, T inv_trG, T CnWeH,
+                                           const GpIn<D, S> &q, const T *f, S *Sq, S (*Vq)[D], bool &floored) {
   // phi* clip (Eq. phi_for_density) and mixture properties at t_{k+1}
   const T pn = val(q.phin);
   const bool inside = fabs(pn) <= T(1);
-  S phis = inside ? q.phin : S(pn > T(0) ? T(1) : T(-1));
-  S rho = c.alpha * phis + c.beta;
-  S eta = c.gamma * phis + c.xi;
-  S inv_rho = rcp_(rho);
-  S deta[D];
+  const S phis = inside ? q.phin : S(pn > T(0) ? T(1) : T(-1));
+  const S rho = madc(phis, c.alpha, c.beta);
+  const S etaRe = madc(phis, c.gRe, c.xRe);
+  const S inv_rho = rcp_(rho);
+  S cm[D], cR[D];  // c_j and c_j - d_j eta / Re
 #pragma unroll
-  for (int k = 0; k < D; ++k) deta[k] = inside ? c.gamma * q.dphin[k] : S(T(0));
-  // thermodynamic-consistency flux
-  S J[D];
-#pragma unroll
-  for (int i = 0; i < D; ++i) J[i] = c.jc * q.dmut[i];
-  // tau_m, tau_c with G = diag(4/h^2); radicand floored at 4/dt^2
-  S vGv = S(T(0)), vGJ = S(T(0));
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    vGv = vGv + G[i] * (q.vt[i] * q.vt[i]);
-    vGJ = vGJ + G[i] * (q.vt[i] * J[i]);
+  for (int j = 0; j < D; ++j) {
+    cm[j] = mad(rho, q.vt[j], q.dmut[j] * c.jcP);
+    const S de = inside ? q.dphin[j] * c.gRe : S(T(0));
+    cR[j] = cm[j] - de;
   }
-  S visc = eta * inv_rho * c.inv_Re;
-  S rad = vGv + vGJ * inv_rho * c.inv_Pe + CI_GG * (visc * visc) + c.four_dt2;
+  // tau_m, tau_c with G = diag(4/h^2); radicand floored at 4/dt^2
+  S vGc = (q.vt[0] * cm[0]) * G[0];
+#pragma unroll
+  for (int i = 1; i < D; ++i) vGc = mad(q.vt[i] * cm[i], G[i], vGc);
+  const S visc = etaRe * inv_rho;
+  S rad = mad(inv_rho, vGc, madc(visc * visc, CI_GG, c.four_dt2));
   floored = val(rad) < c.four_dt2;
   if (floored) rad = S(c.four_dt2);
-  S tau = rsqrt_(rad);
-  S tau_c = inv_trG * rcp_(tau);
+  const S tau = rsqrt_(rad);
   // strong residuals
-  S Rm[D], conv[D], flux[D];
-  S divv = S(T(0));
+  S A[D], t[D];
+  S divv = q.dvt[0][0];
+#pragma unroll
+  for (int i = 1; i < D; ++i) divv = divv + q.dvt[i][i];
+  if (HASF) divv = subc(divv, f[D]);  // R_c
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    S cv = S(T(0)), fl = S(T(0)), cap = S(T(0)), vs = S(T(0));
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      cv = cv + q.vt[j] * q.dvt[i][j];
-      fl = fl + J[j] * q.dvt[i][j];
-      vs = vs + deta[j] * q.dvt[i][j];
-      if (j != i) cap = cap + q.hphit[hidx<D>(i, j)] * q.dphit[j];
+    A[i] = rho * madc(q.dv[i], c.inv_dt, -c.gFr[i]);
+    if (HASF) A[i] = subc(A[i], f[i]);
+    S R = mad(q.dpt[i], c.inv_We, A[i]);
+    S cap = D == 2 ? q.hphit[0] * q.dphit[1 - i] : S(T(0));
+    if (D == 3) {
+      const int j0 = i == 0 ? 1 : 0, j1 = i == 2 ? 1 : 2;
+      cap = mad(q.hphit[hidx<D>(i, j0)], q.dphit[j0], q.hphit[hidx<D>(i, j1)] * q.dphit[j1 < D ? j1 : 0]);
     }
-    conv[i] = cv;
-    flux[i] = fl;
-    divv = divv + q.dvt[i][i];
-    Rm[i] = rho * (q.dv[i] * c.inv_dt + cv) + fl * c.inv_Pe + c.CnWe * cap + q.dpt[i] * c.inv_We -
-            vs * c.inv_Re - rho * (c.g[i] * c.inv_Fr) - q.f[i];
-  }
-  S Rc = divv - q.f[D];
-  // momentum rows
-  S tR[D];
+    R = mad(cap, CnWeH, R);
 #pragma unroll
-  for (int j = 0; j < D; ++j) tR[j] = tau * Rm[j];
-  S diag = (rho * tau_c * Rc - q.pt) * c.inv_We;
-  S etaRe = eta * c.inv_Re;
+    for (int j = 0; j < D; ++j) R = mad(q.dvt[i][j], cR[j], R);
+    t[i] = tau * R;
+  }
+  // momentum rows
+  const S tau_c = (rad * tau) * inv_trG;
+  const S diag = (rho * tau_c * divv - q.pt) * c.inv_We;
+#pragma unroll
+  for (int j = 0; j < D; ++j) cm[j] = cm[j] - t[j];
+  S cphi[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) cphi[i] = q.dphit[i] * (-c.CnWe);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    S cross = S(T(0));
+    S Si = A[i];
 #pragma unroll
-    for (int j = 0; j < D; ++j) cross = cross + tR[j] * q.dvt[i][j];
-    Sq[i] = rho * (q.dv[i] * c.inv_dt + conv[i]) - cross + flux[i] * c.inv_Pe -
-            rho * (c.g[i] * c.inv_Fr) - q.f[i];
-    S b = tR[i] * inv_rho;  // tau R_i / rho
-#pragma unroll
-    for (int j = 0; j < D; ++j)
-      Vq[i][j] = q.vt[j] * tR[i] - tR[j] * b + c.inv_Pe * J[j] * b -
-                 c.CnWe * (q.dphit[i] * q.dphit[j]) + etaRe * q.dvt[i][j];
-    Vq[i][i] = Vq[i][i] + diag;
+    for (int j = 0; j < D; ++j) Si = mad(q.dvt[i][j], cm[j], Si);
+    Sq[i] = Si;
+    Vq[D][i] = t[i] * inv_rho;  // PSPG; tau_m R_m / rho
   }
-  // continuity row with PSPG
-  Sq[D] = divv - q.f[D];
 #pragma unroll
-  for (int i = 0; i < D; ++i) Vq[D][i] = tR[i] * inv_rho;
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int j = i; j < D; ++j) {
+      S cc = cphi[i] * q.dphit[j];
+      if (i == j) cc = cc + diag;
+      Vq[i][j] = mad(Vq[D][i], cm[j], mad(etaRe, q.dvt[i][j], cc));
+      if (i != j) Vq[j][i] = mad(Vq[D][j], cm[i], mad(etaRe, q.dvt[j][i], cc));
+    }
+  // continuity row
+  Sq[D] = divv;
   // Cahn-Hilliard row
-  Sq[D + 1] = q.dphi * c.inv_dt - q.f[D + 1];
+  Sq[D + 1] = q.dphi * c.inv_dt;
 #pragma unroll
-  for (int i = 0; i < D; ++i) Vq[D + 1][i] = c.inv_PeCn * q.dmut[i] - q.vt[i] * q.phit;
+  for (int i = 0; i < D; ++i) Vq[D + 1][i] = q.dmut[i] * c.inv_PeCn - q.vt[i] * q.phit;
   // chemical-potential row, psi'(phi~) = phi~^3 - phi~
-  Sq[D + 2] = q.phit * q.phit * q.phit - q.phit - q.mut - q.f[D + 2];
+  Sq[D + 2] = q.phit * madc(q.phit, q.phit, T(-1)) - q.mut;
 #pragma unroll
-  for (int i = 0; i < D; ++i) Vq[D + 2][i] = c.Cn2 * q.dphit[i];
+  for (int i = 0; i < D; ++i) Vq[D + 2][i] = q.dphit[i] * c.Cn2;
+  if (HASF) {
+    Sq[D + 1] = subc(Sq[D + 1], f[D + 1]);
+    Sq[D + 2] = subc(Sq[D + 2], f[D + 2]);
+  }
 }
 
 template <int D, typename T>
@@ -363,36 +463,58 @@ struct Interp {  // one state interpolated at the lane's Gauss point
   T vt[D], dvt[D][D], pt, dpt[D], phit, dphit[D], hphit[3], mut, dmut[D];
 };
 
-template <int D, typename T>
-__device__ __forceinline__ void interp_state(const T *u, const Stage<T> &s, Interp<D, T> &I) {
+template <int D, bool UNIT, typename T>
+__device__ __forceinline__ void interp_state(const T *u, const Stage<D, T> &s, Interp<D, T> &I) {
 #pragma unroll
   for (int i = 0; i < D; ++i) ip_vg<D>(u[i], s, I.vt[i], I.dvt[i]);
   ip_vg<D>(u[D], s, I.pt, I.dpt);
   I.hphit[1] = I.hphit[2] = T(0);
-  ip_full<D>(u[D + 1], s, I.phit, I.dphit, I.hphit);
+  ip_full<D, UNIT>(u[D + 1], s, I.phit, I.dphit, I.hphit);
   ip_vg<D>(u[D + 2], s, I.mut, I.dmut);
 }
 
 template <typename T>
-KCoef<T> kcoef(const PhysCoef &p) {
+KCoef<T> kcoef(const PhysCoef &p, int dim) {
   KCoef<T> c;
   c.inv_dt = T(p.inv_dt); c.four_dt2 = T(p.four_dt2);
-  c.alpha = T(p.alpha); c.beta = T(p.beta); c.gamma = T(p.gamma); c.xi = T(p.xi); c.jc = T(p.jc);
-  c.inv_Pe = T(p.inv_Pe); c.inv_We = T(p.inv_We); c.inv_Re = T(p.inv_Re); c.inv_Fr = T(p.inv_Fr);
-  c.CnWe = T(p.CnWe); c.inv_PeCn = T(p.inv_PeCn); c.Cn2 = T(p.Cn2); c.C_I = T(p.C_I);
+  c.alpha = T(p.alpha); c.beta = T(p.beta);
+  c.gRe = T(p.gamma * p.inv_Re); c.xRe = T(p.xi * p.inv_Re);
+  c.jcP = T(p.jc * p.inv_Pe);
+  c.inv_We = T(p.inv_We); c.CnWe = T(p.CnWe); c.inv_PeCn = T(p.inv_PeCn); c.Cn2 = T(p.Cn2);
+  c.inv_Fr = T(p.inv_Fr);
+  double trG = 0.0, GG = 0.0, W = 1.0;
   for (int a = 0; a < 3; ++a) {
+    c.gFr[a] = T(p.g[a] * p.inv_Fr);
     c.g[a] = T(p.g[a]);
-    c.ext[a] = T(p.ext[a]);
+    const double G = 4.0 / (p.ext[a] * p.ext[a]);
+    c.G0[a] = T(G);
+    if (a < dim) {
+      trG += G;
+      GG += G * G;
+      W *= 0.5 * p.ext[a];
+    }
+  }
+  c.CIGG0 = T(p.C_I * GG);
+  c.inv_trG0 = T(1.0 / trG);
+  c.W0 = T(W);
+  const double cad1 = dim == 2 ? CA : CA * CA;  // CA^(D-1)
+  c.cS0 = T(W * cad1 * CA);
+  for (int a = 0; a < 3; ++a) {
+    c.sg0[a] = T(cad1 / p.ext[a]);
+    c.sh0[a] = T(1.0 / p.ext[a]);
+    c.cV0[a] = T(W * cad1 / p.ext[a]);
   }
   return c;
 }
 
 // ---------------------------------------------------------------- the element kernel
-// MODE 0: residual (output O = double), MODE 1: J.w into the element-local
-// slots (O = T), MODE 2: count of the Gauss points whose tau_m radicand is
-// floored (O = unsigned long long, one counter), MODE 3: J.w scattered into
-// the node vector (O = T; one launch per element colour).  BS, MINB: block
-// size and minimum resident blocks per SM (the register budget).
+// MODE 0: residual into the element-local slots; MODE 1: J.w into the
+// element-local slots; MODE 2: count of the Gauss points whose tau_m radicand
+// is floored (O = unsigned long long, one counter); MODE 3: J.w scattered into
+// the node vector (one launch per element colour).  MODE 0 and 2 read the
+// states themselves (ut = U_new, dl = U_old: they are evaluated once per
+// state), the J.w modes the prepared averages and increments.  BS, MINB:
+// block size and minimum resident blocks per SM (the register budget).
 template <int D, typename T, int MODE, bool HASF, typename O, int BS = 128, int MINB = 6>
 __global__ void __launch_bounds__(BS, MINB) k_element(
     const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
@@ -401,6 +523,8 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     const T *__restrict__ f, O *__restrict__ out, KCoef<T> c0, const KCoef<T> *__restrict__ tab,
     const uint16_t *__restrict__ einst) {
   constexpr int NC = 1 << D, NF = D + 3, ND = D + 1;
+  constexpr bool UNIT = sizeof(T) == 4, RAW = MODE == 0 || MODE == 2;
+  static_assert(!(UNIT && RAW), "the residual is in double");
   const int lc = threadIdx.x & (NC - 1);
   int64_t e = e_begin + ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> D);
   const bool active = e < e_end;
@@ -409,47 +533,59 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   // batched meshes: the coefficients of the element's own problem instance
   const KCoef<T> c = tab ? tab[einst[e]] : c0;
 
-  // gather the corner's nodal blocks
+  // gather the corner's nodal blocks (MODE 0, 2: the sum of the states, twice
+  // the average; the factors of the interpolation carry the half)
   T u[NF], d[ND];
   gather<NF>(cn, hang, ut, u);
-  gather<ND>(cn, hang, dl, d);
+  if (RAW) {
+    T b[NF];
+    gather<NF>(cn, hang, dl, b);
+#pragma unroll
+    for (int k = 0; k < D; ++k) d[k] = u[k] - b[k];
+    d[D] = u[D + 1] - b[D + 1];
+#pragma unroll
+    for (int k = 0; k < NF; ++k) u[k] += b[k];
+  } else {
+    gather<ND>(cn, hang, dl, d);
+  }
   T wn[NF];
   if (MODE == 1 || MODE == 3) gather<NF>(cn, hang, w, wn);
   T fn[NF];
   if (HASF) gather<NF>(cn, hang, f, fn);
 
   // geometry of this leaf
-  const T scale = T(1) / T(1u << level[e]);
-  const T *ext = c.ext;
-  Stage<T> s;
-  s.ca = T(0.5) + T(0.28867513459481288225);  // (1 + 1/sqrt(3)) / 2
-  s.cb = T(0.5) - T(0.28867513459481288225);
-  T G[D], trG = T(0), GG = T(0), W = T(1);
+  const int l = level[e];
+  Stage<D, T> s;
+  T G[D];
+  s.v = T((RAW ? 0.5 : 1.0) * CAD<D>);
+  s.cS = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    T h = ext[a] * scale;
-    s.sh[a] = ((lc >> a) & 1) ? T(1) / h : T(-1) / h;
-    G[a] = T(4) / (h * h);
-    trG += G[a];
-    GG += G[a] * G[a];
-    W *= T(0.5) * h;
+    const bool neg = !((lc >> a) & 1);
+    s.sg[a] = flip_if(scale2(c.sg0[a], l - (RAW ? 1 : 0)), neg);
+    s.sh[a] = UNIT ? flip_if(scale2(c.sh0[a], l), neg) : T(0);
+    s.cV[a] = flip_if(scale2(c.cV0[a], (1 - D) * l - (RAW ? 0 : 1)), neg);
+    G[a] = scale2(c.G0[a], 2 * l);
   }
-  const T CI_GG = c.C_I * GG, inv_trG = T(1) / trG;
+  const T CI_GG = scale2(c.CIGG0, 4 * l), inv_trG = scale2(c.inv_trG0, -2 * l);
+  // d_a d_b = sg_a sg_b / CA^D (half of it with the halved factors)
+  const T CnWeH = UNIT ? c.CnWe : c.CnWe * T((RAW ? 2.0 : 1.0) / CAD<D>);
 
   // interpolate to the lane's Gauss point
   Interp<D, T> A;
-  interp_state<D>(u, s, A);
+  interp_state<D, UNIT>(u, s, A);
   T dvq[D], dphiq, dphig[D];
 #pragma unroll
-  for (int i = 0; i < D; ++i) dvq[i] = ip_v<D>(d[i], s);
-  ip_vg<D>(d[D], s, dphiq, dphig);
+  for (int i = 0; i < D; ++i) dvq[i] = ip_v<D>(d[i]) * T(CAD<D>);
+  ip_vg<D, UNIT>(d[D], s, dphiq, dphig);
   T fq[NF];
 #pragma unroll
-  for (int k = 0; k < NF; ++k) fq[k] = HASF ? ip_v<D>(fn[k], s) : T(0);
+  for (int k = 0; k < NF; ++k) fq[k] = HASF ? ip_v<D>(fn[k]) * T(CAD<D>) : T(0);
 
   T r[NF];
   bool floored = false;
-  if (MODE == 0 || MODE == 2) {
+  if (RAW) {
+    // dphiq, dphig: half the increment and half its gradient
     GpIn<D, T> q;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
@@ -458,7 +594,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
       q.dpt[i] = A.dpt[i];
       q.dphit[i] = A.dphit[i];
       q.dmut[i] = A.dmut[i];
-      q.dphin[i] = A.dphit[i] + T(0.5) * dphig[i];
+      q.dphin[i] = A.dphit[i] + dphig[i];
 #pragma unroll
       for (int j = 0; j < D; ++j) q.dvt[i][j] = A.dvt[i][j];
     }
@@ -467,65 +603,57 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     q.pt = A.pt;
     q.phit = A.phit;
     q.mut = A.mut;
-    q.dphi = dphiq;
-    q.phin = A.phit + T(0.5) * dphiq;
-#pragma unroll
-    for (int k = 0; k < NF; ++k) q.f[k] = fq[k];
+    q.dphi = T(2) * dphiq;
+    q.phin = A.phit + dphiq;
     T Sq[NF], Vq[NF][D];
-    gp_physics<D, T, T>(c, G, CI_GG, inv_trG, q, Sq, Vq, floored);
+    gp_physics<D, HASF, T, T>(c, G, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
     if constexpr (MODE == 2) {
       const unsigned b = __ballot_sync(FULL, floored && active);
       if ((threadIdx.x & 31) == 0 && b) atomicAdd(reinterpret_cast<unsigned long long *>(out), (unsigned long long)__popc(b));
-      return;
-    }
+    } else {
 #pragma unroll
-    for (int k = 0; k < NF; ++k) {
-      T Vk[D];
-#pragma unroll
-      for (int j = 0; j < D; ++j) Vk[j] = W * Vq[k][j];
-      r[k] = contract<D>(W * Sq[k], Vk, s);
+      for (int k = 0; k < NF; ++k) r[k] = contract<D>(Sq[k], Vq[k], s);
     }
   } else {
-    // perturbation U_new + e w: v~, p~, phi~, mu~ move by w/2, increments by w
+    // perturbation U_new + 2 e w (the weights of the contraction carry the
+    // half): the averages move by w, the increments and phi^{k+1} by 2 w
     Interp<D, T> B;
-    interp_state<D>(wn, s, B);
+    interp_state<D, UNIT>(wn, s, B);
     GpIn<D, Dl<T>> q;
-    const T hf = T(0.5);
+    const T two = T(2), hf = T(0.5);
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-      q.vt[i] = Dl<T>(A.vt[i], hf * B.vt[i]);
-      q.dv[i] = Dl<T>(dvq[i], B.vt[i]);
-      q.dpt[i] = Dl<T>(A.dpt[i], hf * B.dpt[i]);
-      q.dphit[i] = Dl<T>(A.dphit[i], hf * B.dphit[i]);
-      q.dmut[i] = Dl<T>(A.dmut[i], hf * B.dmut[i]);
-      q.dphin[i] = Dl<T>(A.dphit[i] + hf * dphig[i], B.dphit[i]);
+      q.vt[i] = Dl<T>(A.vt[i], B.vt[i]);
+      q.dv[i] = Dl<T>(dvq[i], two * B.vt[i]);
+      q.dpt[i] = Dl<T>(A.dpt[i], B.dpt[i]);
+      q.dphit[i] = Dl<T>(A.dphit[i], B.dphit[i]);
+      q.dmut[i] = Dl<T>(A.dmut[i], B.dmut[i]);
+      q.dphin[i] = Dl<T>(mad(hf, dphig[i], A.dphit[i]), two * B.dphit[i]);
 #pragma unroll
-      for (int j = 0; j < D; ++j) q.dvt[i][j] = Dl<T>(A.dvt[i][j], hf * B.dvt[i][j]);
+      for (int j = 0; j < D; ++j) q.dvt[i][j] = Dl<T>(A.dvt[i][j], B.dvt[i][j]);
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) q.hphit[k] = Dl<T>(A.hphit[k], hf * B.hphit[k]);
-    q.pt = Dl<T>(A.pt, hf * B.pt);
-    q.phit = Dl<T>(A.phit, hf * B.phit);
-    q.mut = Dl<T>(A.mut, hf * B.mut);
-    q.dphi = Dl<T>(dphiq, B.phit);
-    q.phin = Dl<T>(A.phit + hf * dphiq, B.phit);
-#pragma unroll
-    for (int k = 0; k < NF; ++k) q.f[k] = Dl<T>(fq[k]);
+    for (int k = 0; k < 3; ++k) q.hphit[k] = Dl<T>(A.hphit[k], B.hphit[k]);
+    q.pt = Dl<T>(A.pt, B.pt);
+    q.phit = Dl<T>(A.phit, B.phit);
+    q.mut = Dl<T>(A.mut, B.mut);
+    q.dphi = Dl<T>(dphiq, two * B.phit);
+    q.phin = Dl<T>(mad(hf, dphiq, A.phit), two * B.phit);
     Dl<T> Sq[NF], Vq[NF][D];
-    gp_physics<D, T, Dl<T>>(c, G, CI_GG, inv_trG, q, Sq, Vq, floored);
+    gp_physics<D, HASF, T, Dl<T>>(c, G, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
       T Vk[D];
 #pragma unroll
-      for (int j = 0; j < D; ++j) Vk[j] = W * Vq[k][j].d;
-      r[k] = contract<D>(W * Sq[k].d, Vk, s);
+      for (int j = 0; j < D; ++j) Vk[j] = Vq[k][j].d;
+      r[k] = contract<D>(Sq[k].d, Vk, s);
     }
   }
-  if constexpr (MODE == 1) {
-    // J.w: element-local output, slot (e, corner); k_gather_nodes sums the
-    // slots of each node in a fixed order
+  if constexpr (MODE == 0 || MODE == 1) {
+    // element-local output, slot (e, corner); k_gather_nodes sums the slots of
+    // each node in a fixed order
     if (active) store_block<NF>(reinterpret_cast<T *>(out) + (e * NC + lc) * NF, r);
-  } else if constexpr (MODE == 0 || MODE == 3) {
+  } else if constexpr (MODE == 3) {
     // Lanes of one element may reach the same node: a hanging corner's parents
     // can be corners of the element or parents of its other hanging corner.
     // Warps that hold a hanging corner scatter one corner index at a time.
@@ -560,15 +688,16 @@ __global__ void k_prep(const double *__restrict__ Un, const double *__restrict__
 }
 
 // y[i] = sum over the slots of node i of weight * E[slot] (fixed order), then
-// the constrained rows: y = w on wall velocities and the pinned pressure.
-// The slots of a node are fetched eight at a time (independent loads), then
-// added in list order.
-template <int D, typename T>
+// the constrained rows (wall velocities, the pinned pressure): y = w for J.w,
+// y = w - bc for the residual (RES: w = U_new, bc nullable).  The slots of a
+// node are fetched eight at a time (independent loads), then added in list
+// order.
+template <int D, typename T, bool RES>
 __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict__ gptr,
                                                       const int32_t *__restrict__ gent,
                                                       const uint8_t *__restrict__ nflag, int64_t n_nodes,
-                                                      const T *__restrict__ E, const T *__restrict__ w,
-                                                      T *__restrict__ y, uint32_t fmask) {
+                                                      const T *__restrict__ E, const T *w, const T *bc, T *y,
+                                                      uint32_t fmask) {
   constexpr int NF = D + 3, G = 8;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n_nodes; i += int64_t(gridDim.x) * blockDim.x) {
     T acc[NF];
@@ -595,9 +724,9 @@ __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict_
     const uint8_t fl = nflag[i];
     if (fl & 1)
 #pragma unroll
-      for (int k = 0; k < D; ++k) acc[k] = w[i * NF + k];
-    if (fl & 2) acc[D] = w[i * NF + D];
-    if (fmask != 0xffu)
+      for (int k = 0; k < D; ++k) acc[k] = w[i * NF + k] - (RES && bc ? bc[i * NF + k] : T(0));
+    if (fl & 2) acc[D] = w[i * NF + D] - (RES && bc ? bc[i * NF + D] : T(0));
+    if (!RES && fmask != 0xffu)
 #pragma unroll
       for (int k = 0; k < NF; ++k)
         if (!((fmask >> k) & 1u)) acc[k] = w[i * NF + k];
@@ -621,22 +750,6 @@ __global__ void k_fix_rows(const uint8_t *__restrict__ nflag, int64_t n_nodes, c
   }
 }
 
-// constrained rows of the residual: wall velocities and the pinned pressure
-__global__ void k_dirichlet_res(const int32_t *__restrict__ wall, int64_t n_wall, const int32_t *__restrict__ pins,
-                                int64_t n_pins, int dim, const double *__restrict__ Un,
-                                const double *__restrict__ bc, double *__restrict__ F) {
-  const int nf = dim + 3;
-  int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (i < n_wall) {
-    int64_t b = int64_t(wall[i]) * nf;
-    for (int k = 0; k < dim; ++k) F[b + k] = Un[b + k] - (bc ? bc[b + k] : 0.0);
-  }
-  if (i < n_pins) {
-    int64_t b = int64_t(pins[i]) * nf + dim;
-    F[b] = Un[b] - (bc ? bc[b] : 0.0);
-  }
-}
-
 // ---------------------------------------------------------------- diagnostics
 // per block: energy, integral of phi, volume with phi < 0 (2^D Gauss rule)
 template <int D>
@@ -655,14 +768,13 @@ __global__ void __launch_bounds__(256) k_energy(
   gather<NF>(cn, hang, U, u);
   const double ext[3] = {ext0, ext1, ext2}, lo[3] = {lo0, lo1, lo2};
   const double scale = 1.0 / double(1u << level[e]);
-  Stage<double> s;
-  s.ca = 0.5 + 0.28867513459481288225;
-  s.cb = 0.5 - 0.28867513459481288225;
+  Stage<D, double> s;
+  s.v = CAD<D>;
   double W = 1.0, zg = 0.0;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     double h = ext[a] * scale;
-    s.sh[a] = ((lc >> a) & 1) ? 1.0 / h : -1.0 / h;
+    s.sg[a] = flip_if(scale2(c.sg0[a], level[e]), !((lc >> a) & 1));
     W *= 0.5 * h;
     double xi = ((lc >> a) & 1) ? 0.57735026918962576451 : -0.57735026918962576451;
     double x = lo[a] + ext[a] * double(anchor[e * D + a]) * inv_top + 0.5 * (1.0 + xi) * h;
@@ -671,7 +783,7 @@ __global__ void __launch_bounds__(256) k_energy(
   double v2 = 0.0;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    double vi = ip_v<D>(u[i], s);
+    double vi = ip_v<D>(u[i]) * CAD<D>;
     v2 += vi * vi;
   }
   double phi, dphi[D];
@@ -761,31 +873,33 @@ void launch_prep(const chns_mesh *m, const double *Un, const double *Uo, T *ut, 
 template void launch_prep<float>(const chns_mesh *, const double *, const double *, float *, float *, cudaStream_t);
 template void launch_prep<double>(const chns_mesh *, const double *, const double *, double *, double *, cudaStream_t);
 
-namespace {
-template <int D, typename T, int MODE, bool HASF, typename O>
-void element_pass(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w,
-                  const T *f, O *out, cudaStream_t st, int colour_lo, int colour_hi) {
-  KCoef<T> c = kcoef<T>(pc);
-  constexpr int MINB = sizeof(T) == 8 ? kFp64MinBlocks : 6;
-  for (int col = colour_lo; col < colour_hi; ++col) {
-    int64_t b = m->colour_start[col], e = m->colour_start[col + 1];
-    if (e <= b) continue;
-    k_element<D, T, MODE, HASF, O, 128, MINB><<<grid_elem((e - b) << D), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, b, e, ut, dl, w, f, out, c,
-        reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32), m->elem_inst);
-    note_launches(1);
-  }
+// Residual: all elements in one launch into the element-local buffer E, then
+// the node gather with the constrained rows, as J.w.  One launch per element
+// colour with in-place adds read and wrote every node once per colour, needed
+// the output zeroed first and left eight partly filled last waves; E costs 96
+// B per corner of L2 / HBM traffic instead, 6 % of the FP64 time.
+// U_new and U_old are averaged in the element kernel (10 FP64 instructions a
+// lane) rather than by a node pass before it: a state is evaluated once.
+template <int D, bool HASF>
+static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const double *Un, const double *Uo,
+                               const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
+  k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks><<<grid_elem(m->n_elem << D), kElemBlock, 0, st>>>(
+      m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
+      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst);
+  k_gather_nodes<D, double, true><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
+                                                                             Un, bc, F, 0xffu);
+  note_launches(2);
 }
-}  // namespace
 
-void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *ut, const double *dl,
-                     const double *f, double *F, cudaStream_t st) {
+void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const double *f,
+                     const double *bc, double *E, double *F, cudaStream_t st) {
+  const KCoef<double> c = kcoef<double>(pc, m->dim);
   if (m->dim == 2) {
-    if (f) element_pass<2, double, 0, true, double>(m, pc, ut, dl, nullptr, f, F, st, 0, m->n_colours);
-    else element_pass<2, double, 0, false, double>(m, pc, ut, dl, nullptr, nullptr, F, st, 0, m->n_colours);
+    if (f) residual_elemlocal<2, true>(m, c, Un, Uo, f, bc, E, F, st);
+    else residual_elemlocal<2, false>(m, c, Un, Uo, f, bc, E, F, st);
   } else {
-    if (f) element_pass<3, double, 0, true, double>(m, pc, ut, dl, nullptr, f, F, st, 0, m->n_colours);
-    else element_pass<3, double, 0, false, double>(m, pc, ut, dl, nullptr, nullptr, F, st, 0, m->n_colours);
+    if (f) residual_elemlocal<3, true>(m, c, Un, Uo, f, bc, E, F, st);
+    else residual_elemlocal<3, false>(m, c, Un, Uo, f, bc, E, F, st);
   }
 }
 
@@ -808,8 +922,8 @@ static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *
   const int64_t threads = m->n_elem << D;
   k_element<D, T, 1, false, T, BS, MINB><<<(unsigned)((threads + BS - 1) / BS), BS, 0, st>>>(
       m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w, nullptr, E, c, tab, m->elem_inst);
-  k_gather_nodes<D, T><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, y,
-                                                                  fmask);
+  k_gather_nodes<D, T, false><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w,
+                                                                         nullptr, y, fmask);
   note_launches(2);
 }
 
@@ -854,7 +968,7 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
 template <typename T>
 void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *E, T *y,
                    cudaStream_t st, int variant) {
-  KCoef<T> c = kcoef<T>(pc);
+  KCoef<T> c = kcoef<T>(pc, m->dim);
   const KCoef<T> *tab = reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32);
   if (variant < 0) variant = sizeof(T) == 4 ? m->jv_variant : 0;
   if (m->dim == 2) jv_dispatch<2, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st);
@@ -867,22 +981,16 @@ template void launch_jacvec<double>(const chns_mesh *, const PhysCoef &, const d
 
 // Gauss points with a floored tau_m radicand, added to *count (all elements
 // in one launch, FP64 physics as in the residual)
-void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *ut, const double *dl,
+void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo,
                             unsigned long long *count, cudaStream_t st) {
-  KCoef<double> c = kcoef<double>(pc);
+  KCoef<double> c = kcoef<double>(pc, m->dim);
   const KCoef<double> *tab = reinterpret_cast<const KCoef<double> *>(m->coef64);
   if (m->dim == 2)
     k_element<2, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 2), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, nullptr, nullptr, count, c, tab, m->elem_inst);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst);
   else
     k_element<3, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 3), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, nullptr, nullptr, count, c, tab, m->elem_inst);
-  note_launches(1);
-}
-
-void launch_dirichlet_res(const chns_mesh *m, const double *Un, const double *bc, double *F, cudaStream_t st) {
-  int64_t n = std::max<int64_t>(std::max(m->n_wall, m->n_pins), 1);
-  k_dirichlet_res<<<grid_for(n), kBlock, 0, st>>>(m->wall, m->n_wall, m->pins, m->n_pins, m->dim, Un, bc, F);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst);
   note_launches(1);
 }
 
@@ -895,8 +1003,8 @@ chns_status upload_coef_tables(chns_mesh *m, const std::vector<PhysCoef> &pcs, c
   std::vector<KCoef<float>> a(n);
   std::vector<KCoef<double>> b(n);
   for (size_t i = 0; i < n; ++i) {
-    a[i] = kcoef<float>(pcs[i]);
-    b[i] = kcoef<double>(pcs[i]);
+    a[i] = kcoef<float>(pcs[i], m->dim);
+    b[i] = kcoef<double>(pcs[i], m->dim);
   }
   CHNS_CUDA_TRY(cudaMemcpyAsync(m->coef32, a.data(), sizeof(KCoef<float>) * n, cudaMemcpyHostToDevice, st));
   CHNS_CUDA_TRY(cudaMemcpyAsync(m->coef64, b.data(), sizeof(KCoef<double>) * n, cudaMemcpyHostToDevice, st));
@@ -921,7 +1029,7 @@ int64_t energy_blocks(const chns_mesh *m) { return (int64_t)grid_for(m->n_elem <
 
 void launch_energy(const chns_mesh *m, const PhysCoef &pc, const double *U, double *partial,
                    cudaStream_t st) {
-  KCoef<double> c = kcoef<double>(pc);
+  KCoef<double> c = kcoef<double>(pc, m->dim);
   double inv_top = 1.0 / double(int64_t(1) << m->max_level);
   unsigned g = grid_for(m->n_elem << m->dim);
   if (m->dim == 2)
