@@ -116,7 +116,8 @@ struct Coarse {
   int32_t *sent = nullptr;          // entries piece * 2^dim + corner
   DevBuf M;                         // per instance A_c -> A_c^{-1} (double), nc0 x nc0
   DevBuf Minv32;                    // per instance A_c^{-1} in float, nc0 x nc0
-  DevBuf piv;                       // Gauss-Jordan row interchanges, nc0 per instance
+  DevBuf piv;                       // Gauss-Jordan row interchanges, 3 nc0 indices per instance
+  DevBuf gj;                        // Gauss-Jordan working matrices (element precision)
   DevBuf vec;                       // coarse work vectors and operator-build partials
   DevBuf rpart;                     // restriction partials, n_pieces x 2^dim x nf doubles
   bool ready = false;

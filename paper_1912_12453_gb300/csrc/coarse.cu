@@ -34,11 +34,6 @@ inline unsigned grid_n(int64_t n) {
   return (unsigned)std::min<int64_t>(std::max<int64_t>(b, 1), 152 * 8);
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-  return v;
-}
-
 struct CGeo {
   int dim, nf, nc1;   // nc1 = 2^Lc + 1 coarse nodes per axis
   int64_t n_nodes;
@@ -374,13 +369,220 @@ __global__ void k_copy_cast(const A *__restrict__ x, int64_t n, B *__restrict__ 
   for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < n; t += int64_t(gridDim.x) * kB) y[t] = B(x[t]);
 }
 
-// In-place Gauss-Jordan inversion of each instance's n x n block (row-major)
-// with partial pivoting: pivot step k swaps the row of the largest |a_rk|,
-// r >= k, into row k (recorded in piv), scales row k by d = 1/a_kk and puts
-// d on the diagonal, and eliminates column k from the other rows, whose
-// column k becomes -a_rk d; the recorded row interchanges are undone as
-// column interchanges at the end.  No [A | I] copy: the working set is n^2
-// values (76.5 MB in float at n = 4374, inside L2).
+// Gauss-Jordan inversion of each instance's n x n block (row-major) with
+// partial pivoting, NB columns at a time.  One pivot step swaps the row of the
+// largest |a_rk|, r >= k, into row k, scales it by d = 1/a_kk, puts d on the
+// diagonal and eliminates column k from the other rows, whose column k becomes
+// -a_rk d.  NB steps change the other columns by one matrix product:
+//   A' = [r not in panel] S A + G (S A)[panel rows],
+// S the row interchanges of the panel, G (n x NB) what the steps leave in the
+// panel's own columns.  So k_gj_panel runs the NB steps on the panel alone, in
+// the registers of one block (a row per thread, two barriers a step), and
+// k_gj_update applies (S, G) to the whole matrix, from one buffer into the
+// other (in place, a row could be overwritten before another one reads it).
+// The row each line came from is carried along; the inverse's columns are put
+// back by it at the end (A^-1 = G_all S_all).
+//
+// Bound: the chain of n pivot searches and two barriers each in one block,
+// about 1 us a column in float, more in double (the panel's products run on one
+// SM's FP64 pipe).  A launch pair per column (pivot, rank-1 elimination of all
+// rows) cost 12 to 24 us per column.  Preconditioner build of a step around
+// this inverse, before -> after: n = 405 float 9.2 -> 2.1 ms, n = 750 float
+// 21.2 -> 7.9 ms, n = 4374 float 172 -> 62 ms, n = 405 double 19.7 -> 10.1 ms
+// (what is left is the probing of the matrix).
+// (abs_key: |x| as an integer of the same order, NaN below everything; the
+// search then needs no FP64 comparisons, which run on the narrow FP64 pipe)
+__device__ __forceinline__ uint64_t abs_key(float x) {
+  const uint32_t b = __float_as_uint(x) & 0x7fffffffu;
+  return b > 0x7f800000u ? 0 : b;
+}
+__device__ __forceinline__ uint64_t abs_key(double x) {
+  const uint64_t b = uint64_t(__double_as_longlong(x)) & 0x7fffffffffffffffull;
+  return b > 0x7ff0000000000000ull ? 0 : b;
+}
+__device__ __forceinline__ void warp_arg_max(uint64_t &best, int &arg) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t v = __shfl_xor_sync(FULL, best, o);
+    const int r = __shfl_xor_sync(FULL, arg, o);
+    if (v > best || (v == best && r < arg)) { best = v; arg = r; }
+  }
+}
+
+template <typename T, int NB, int R>
+__global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, int n, int k0,
+                                                   T *__restrict__ Gall, int32_t *__restrict__ permall,
+                                                   const int32_t *__restrict__ origin_in,
+                                                   int32_t *__restrict__ origin_out, int *__restrict__ bad) {
+  const T *M = Mall + int64_t(blockIdx.x) * n * n;
+  T *G = Gall + int64_t(blockIdx.x) * n * NB;
+  const int nb = min(NB, n - k0);
+  const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+  __shared__ uint64_t wv[2][32];
+  __shared__ int wr[2][32];
+  __shared__ T prow[2][NB], krow[2][NB], dinv[2];
+  __shared__ int psrc[2], ksrc[2];
+  T a[R][NB];
+  int src[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int r = threadIdx.x + i * blockDim.x;
+    src[i] = r;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) a[i][c] = r < n && c < nb ? M[int64_t(r) * n + k0 + c] : T(0);
+  }
+#pragma unroll
+  for (int kk = 0; kk < NB; ++kk) {
+    if (kk >= nb) break;
+    const int k = k0 + kk, sl = kk & 1;
+    // row of the largest |a_rk|, r >= k, the lowest of equals
+    uint64_t best = 0;
+    int arg = k;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = threadIdx.x + i * blockDim.x;
+      const uint64_t v = abs_key(a[i][kk]);
+      if (r >= k && r < n && (v > best || (v == best && r < arg))) { best = v; arg = r; }
+    }
+    warp_arg_max(best, arg);
+    if (ln == 0) { wv[sl][wid] = best; wr[sl][wid] = arg; }
+    __syncthreads();
+    best = ln < nw ? wv[sl][ln] : 0;
+    arg = ln < nw ? wr[sl][ln] : n;
+    warp_arg_max(best, arg);
+    const int p = arg;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = threadIdx.x + i * blockDim.x;
+      if (r == p) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) prow[sl][c] = a[i][c];
+        psrc[sl] = src[i];
+        const bool ok = fabs(a[i][kk]) > T(0);  // false for NaN too
+        if (!ok) *bad = 1;
+        dinv[sl] = ok ? T(1) / a[i][kk] : T(0);
+      }
+      if (r == k) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) krow[sl][c] = a[i][c];
+        ksrc[sl] = src[i];
+      }
+    }
+    __syncthreads();
+    const T d = dinv[sl];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = threadIdx.x + i * blockDim.x;
+      if (r == p && p != k) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) a[i][c] = krow[sl][c];
+        src[i] = ksrc[sl];
+      }
+      if (r == k) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) a[i][c] = c == kk ? d : prow[sl][c] * d;
+        src[i] = psrc[sl];
+      } else {
+        const T fr = -a[i][kk] * d;
+#pragma unroll
+        for (int c = 0; c < NB; ++c) a[i][c] = c == kk ? fr : fma(fr, prow[sl][c], a[i][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int r = threadIdx.x + i * blockDim.x;
+    if (r >= n) continue;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) G[int64_t(r) * NB + c] = a[i][c];
+    const int64_t o = int64_t(blockIdx.x) * n;
+    permall[o + r] = src[i];
+    origin_out[o + r] = origin_in[o + src[i]];
+  }
+}
+
+// out = [r not in panel] S in + G (S in)[panel rows]; the panel's own columns
+// become G.  A block of 256 threads computes a TS x TS tile (TS / 16 squared
+// values per thread); blockIdx.z: instance.
+template <typename T, int NB, int TS>
+__global__ void __launch_bounds__(256) k_gj_update(const T *__restrict__ inall, T *__restrict__ outall, int n, int k0,
+                                                   const T *__restrict__ Gall, const int32_t *__restrict__ permall) {
+  constexpr int V = TS / 16;
+  const T *in = inall + int64_t(blockIdx.z) * n * n;
+  T *out = outall + int64_t(blockIdx.z) * n * n;
+  const T *G = Gall + int64_t(blockIdx.z) * n * NB;
+  const int32_t *perm = permall + int64_t(blockIdx.z) * n;
+  const int nb = min(NB, n - k0);
+  const int r0 = blockIdx.y * TS, j0 = blockIdx.x * TS;
+  __shared__ T g[TS][NB + 1], u[NB][TS];
+  for (int t = threadIdx.x; t < TS * NB; t += 256) {
+    const int r = t / NB, c = t % NB;
+    g[r][c] = r0 + r < n && c < nb ? G[int64_t(r0 + r) * NB + c] : T(0);
+  }
+  for (int t = threadIdx.x; t < NB * TS; t += 256) {
+    const int c = t / TS, j = t % TS;
+    u[c][j] = c < nb && j0 + j < n ? in[int64_t(perm[k0 + c]) * n + j0 + j] : T(0);
+  }
+  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+  T acc[V][V];
+#pragma unroll
+  for (int y = 0; y < V; ++y) {
+    const int r = r0 + ty + 16 * y;
+    const bool row = r < n && (r < k0 || r >= k0 + nb);
+    const int64_t b = row ? int64_t(perm[r]) * n : 0;
+#pragma unroll
+    for (int x = 0; x < V; ++x) {
+      const int j = j0 + tx + 16 * x;
+      acc[y][x] = row && j < n ? in[b + j] : T(0);
+    }
+  }
+  __syncthreads();
+#pragma unroll 8
+  for (int c = 0; c < NB; ++c) {
+    T gr[V], uc[V];
+#pragma unroll
+    for (int y = 0; y < V; ++y) gr[y] = g[ty + 16 * y][c];
+#pragma unroll
+    for (int x = 0; x < V; ++x) uc[x] = u[c][tx + 16 * x];
+#pragma unroll
+    for (int y = 0; y < V; ++y)
+#pragma unroll
+      for (int x = 0; x < V; ++x) acc[y][x] = fma(gr[y], uc[x], acc[y][x]);
+  }
+#pragma unroll
+  for (int y = 0; y < V; ++y) {
+    const int r = r0 + ty + 16 * y;
+    if (r >= n) continue;
+#pragma unroll
+    for (int x = 0; x < V; ++x) {
+      const int j = j0 + tx + 16 * x;
+      if (j >= n) continue;
+      out[int64_t(r) * n + j] = j >= k0 && j < k0 + nb ? g[ty + 16 * y][j - k0] : acc[y][x];
+    }
+  }
+}
+
+__global__ void k_gj_init(int32_t *__restrict__ origin, int64_t n, int n_inst) {
+  for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < n * n_inst; t += int64_t(gridDim.x) * kB)
+    origin[t] = int32_t(t % n);
+}
+
+// the inverse's columns: column origin[j] is column j of the eliminated matrix
+template <typename T, typename D1, typename D2>
+__global__ void k_gj_columns(const T *__restrict__ in, int64_t n, int64_t total, const int32_t *__restrict__ origin,
+                             D1 *__restrict__ a, D2 *__restrict__ b) {
+  for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < total; t += int64_t(gridDim.x) * kB) {
+    const int64_t row = t / n, inst = row / n;
+    const int64_t q = row * n + origin[inst * n + t % n];
+    a[q] = D1(in[t]);
+    b[q] = D2(in[t]);
+  }
+}
+
+// The column-by-column form for matrices beyond the panel kernel's rows (n >
+// 5120: a coarse level of 4 in 3D, 5 in 2D): two launches per column, in place.
+// Pivot step k: the row interchange is recorded in piv and undone as a column
+// interchange at the end.
 template <typename T>
 __global__ void k_gj_pivot(T *__restrict__ Mall, int64_t n, int64_t k, T *__restrict__ colall,
                            int32_t *__restrict__ pivall, int *__restrict__ bad) {
@@ -469,8 +671,10 @@ __global__ void k_gj_unswap(T *__restrict__ Mall, int64_t n, const int32_t *__re
   }
 }
 
+constexpr int64_t kPanelRows = 5120;  // rows the panel kernel holds in registers
+
 template <typename T>
-void gauss_jordan(T *M, int64_t n, int n_inst, T *col, int32_t *piv, int *bad, cudaStream_t st) {
+void gauss_jordan_columns(T *M, int64_t n, int n_inst, T *col, int32_t *piv, int *bad, cudaStream_t st) {
   const dim3 ge((unsigned)((n + kB - 1) / kB), (unsigned)((n + kRowsGJ - 1) / kRowsGJ), (unsigned)n_inst);
   for (int64_t k = 0; k < n; ++k) {
     k_gj_pivot<T><<<n_inst, 1024, 0, st>>>(M, n, k, col, piv, bad);
@@ -479,6 +683,42 @@ void gauss_jordan(T *M, int64_t n, int n_inst, T *col, int32_t *piv, int *bad, c
   k_gj_unswap<T><<<grid_n(n * n_inst), kB, 0, st>>>(M, n, piv, n_inst);
   note_launches(int(2 * n + 1));
 }
+
+// panels of A (buf0), ping-pong with buf1; returns the buffer that holds the
+// eliminated matrix; idx: 3 n n_inst indices, the last n n_inst (or the middle
+// ones: *origin) say which column of the inverse each column is
+template <typename T, int NB, int R>
+T *gj_panels(T *buf0, T *buf1, int64_t n, int n_inst, T *G, int32_t *idx, int32_t **origin, int *bad,
+             cudaStream_t st) {
+  constexpr int TS = sizeof(T) == 8 ? 32 : 64;
+  const int threads = int(((n + R - 1) / R + 31) / 32 * 32);
+  const unsigned tiles = (unsigned)((n + TS - 1) / TS);
+  int32_t *perm = idx, *o0 = idx + n * n_inst, *o1 = idx + 2 * n * n_inst;
+  k_gj_init<<<grid_n(n * n_inst), kB, 0, st>>>(o0, n, n_inst);
+  for (int64_t k = 0; k < n; k += NB) {
+    k_gj_panel<T, NB, R><<<n_inst, threads, 0, st>>>(buf0, int(n), int(k), G, perm, o0, o1, bad);
+    k_gj_update<T, NB, TS><<<dim3(tiles, tiles, (unsigned)n_inst), 256, 0, st>>>(buf0, buf1, int(n), int(k), G, perm);
+    std::swap(buf0, buf1);
+    std::swap(o0, o1);
+    note_launches(2);
+  }
+  note_launches(1);
+  *origin = o0;
+  return buf0;
+}
+
+// Panel widths: a row's NB values per thread and R rows per thread have to
+// stay in the 64 registers of a 1024-thread block; a wider panel means fewer
+// passes over the matrix, so the widest that fits.
+template <typename T>
+T *gauss_jordan_panels(T *buf0, T *buf1, int64_t n, int n_inst, T *G, int32_t *idx, int32_t **origin, int *bad,
+                       cudaStream_t st) {
+  constexpr bool F = sizeof(T) == 4;
+  if (n <= 1024) return gj_panels<T, F ? 32 : 8, 1>(buf0, buf1, n, n_inst, G, idx, origin, bad, st);
+  if (n <= 2048) return gj_panels<T, F ? 16 : 8, 2>(buf0, buf1, n, n_inst, G, idx, origin, bad, st);
+  return gj_panels<T, F ? 8 : 4, 5>(buf0, buf1, n, n_inst, G, idx, origin, bad, st);
+}
+constexpr int kPanelMax = 32;  // widest panel
 
 }  // namespace
 
@@ -506,6 +746,7 @@ void Coarse::release() {
   M.release();
   Minv32.release();
   piv.release();
+  gj.release();
   vec.release();
   rpart.release();
   level = -1;
@@ -651,7 +892,7 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   C.ncn = ncn_all;
   C.nc = ncn_all * nf;
   TRY_CHNS(C.M.ensure(sizeof(double) * C.nc0 * C.nc0 * ni));
-  TRY_CHNS(C.piv.ensure(sizeof(int32_t) * C.nc0 * ni));
+  TRY_CHNS(C.piv.ensure(sizeof(int32_t) * 3 * C.nc0 * ni));
   TRY_CHNS(C.Minv32.ensure(sizeof(float) * C.nc0 * C.nc0 * ni));
   TRY_CHNS(C.vec.ensure(sizeof(double) * (3 * C.nc + 8 + C.ncn * kChunks * 8 * nf)));
   TRY_CHNS(C.rpart.ensure(sizeof(double) * std::max<int64_t>(np, 1) * (1 << dim) * nf));
@@ -687,17 +928,27 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, T *w, T *y, cudaSt
   // float resolves: per-field errors of the applied inverse ~1e-6 at
   // cond(A_c) ~ 1e9), the FP64 path in double.  Both copies are kept: M in
   // double, Minv32 in float.
-  void *colv = C.vec.as<double>() + 2 * C.nc;  // nc0 per instance
   int *bad = reinterpret_cast<int *>(C.vec.as<double>() + 3 * C.nc);
   int32_t *piv = C.piv.as<int32_t>();
   float *M32 = C.Minv32.as<float>();
   CHNS_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), st));
-  if (sizeof(T) == sizeof(float)) {
+  if (nc0 <= kPanelRows) {
+    // two matrices to go back and forth between, and the panel's columns
+    const int64_t np = nc0 * kPanelMax * C.n_inst;
+    TRY_CHNS(C.gj.ensure(sizeof(T) * (2 * nn + np)));
+    T *b0 = C.gj.as<T>();
+    int32_t *origin = nullptr;
+    k_copy_cast<double, T><<<grid_n(nn), kB, 0, st>>>(M, nn, b0);
+    const T *r = gauss_jordan_panels<T>(b0, b0 + nn, nc0, C.n_inst, b0 + 2 * nn, piv, &origin, bad, st);
+    k_gj_columns<T, double, float><<<grid_n(nn), kB, 0, st>>>(r, nc0, nn, origin, M, M32);
+  } else if (sizeof(T) == sizeof(float)) {
+    void *colv = C.vec.as<double>() + 2 * C.nc;  // nc0 per instance
     k_copy_cast<double, float><<<grid_n(nn), kB, 0, st>>>(M, nn, M32);
-    gauss_jordan<float>(M32, nc0, C.n_inst, static_cast<float *>(colv), piv, bad, st);
+    gauss_jordan_columns<float>(M32, nc0, C.n_inst, static_cast<float *>(colv), piv, bad, st);
     k_copy_cast<float, double><<<grid_n(nn), kB, 0, st>>>(M32, nn, M);
   } else {
-    gauss_jordan<double>(M, nc0, C.n_inst, static_cast<double *>(colv), piv, bad, st);
+    void *colv = C.vec.as<double>() + 2 * C.nc;
+    gauss_jordan_columns<double>(M, nc0, C.n_inst, static_cast<double *>(colv), piv, bad, st);
     k_copy_cast<double, float><<<grid_n(nn), kB, 0, st>>>(M, nn, M32);
   }
   note_launches(2);
