@@ -68,11 +68,11 @@ chns_status prepare(chns_mesh *m, const double *Un, const double *Uo, cudaStream
   return check_launch();
 }
 
-// element-local buffer of precision T (n_elem * 2^dim * nf values)
+// element-local buffer of precision T (n_elem * 2^dim * nf values a direction)
 template <typename T>
-chns_status ensure_ebuf(chns_mesh *m, T **E) {
+chns_status ensure_ebuf(chns_mesh *m, T **E, int nv) {
   DevBuf &b = sizeof(T) == 8 ? m->ws.e64 : m->ws.e32;
-  TRY(b.ensure(sizeof(T) * (m->n_elem << m->dim) * m->nf));
+  TRY(b.ensure(sizeof(T) * (m->n_elem << m->dim) * m->nf * nv));
   *E = b.as<T>();
   return CHNS_OK;
 }
@@ -87,43 +87,48 @@ chns_status residual_into(chns_mesh *m, const PhysCoef &pc, const double *Un, co
 
 template <typename T>
 chns_status jacvec_prepared(chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *y,
-                            cudaStream_t st) {
+                            cudaStream_t st, int nv) {
   T *E = nullptr;
-  TRY(ensure_ebuf<T>(m, &E));
-  launch_jacvec<T>(m, pc, ut, dl, w, E, y, st);
+  TRY(ensure_ebuf<T>(m, &E, nv));
+  launch_jacvec<T>(m, pc, ut, dl, w, E, y, st, -1, nv);
   return check_launch();
+}
+
+int probe_batch(const chns_mesh *m, size_t elem, size_t extra, int total) {
+  const size_t per = elem * size_t(m->nf) * (2 * size_t(m->n_nodes) + (size_t(m->n_elem) << m->dim)) + extra;
+  return int(std::max<size_t>(1, std::min<size_t>(size_t(total), (size_t(64) << 20) / per)));
 }
 template chns_status prepare<float>(chns_mesh *, const double *, const double *, cudaStream_t, float **, float **);
 template chns_status prepare<double>(chns_mesh *, const double *, const double *, cudaStream_t, double **, double **);
-template chns_status ensure_ebuf<float>(chns_mesh *, float **);
-template chns_status ensure_ebuf<double>(chns_mesh *, double **);
+template chns_status ensure_ebuf<float>(chns_mesh *, float **, int);
+template chns_status ensure_ebuf<double>(chns_mesh *, double **, int);
 template chns_status jacvec_prepared<float>(chns_mesh *, const PhysCoef &, const float *, const float *, const float *,
-                                            float *, cudaStream_t);
+                                            float *, cudaStream_t, int);
 template chns_status jacvec_prepared<double>(chns_mesh *, const PhysCoef &, const double *, const double *,
-                                             const double *, double *, cudaStream_t);
+                                             const double *, double *, cudaStream_t, int);
 
 // ---------------------------------------------------------------- block-Jacobi by probing
 // The nodal (nf x nf) diagonal blocks of J are read off J applied to the
 // indicator of one field on the nodes of one node colour: nodes of a colour
-// never share an element, so each probed node sees only its own block.
+// never share an element, so each probed node sees only its own block.  Probes
+// go through J.w in batches: one by one they were five launches each, 48 on a
+// uniform octree and more on an adaptive one, of a few us of work.
 template <typename T>
 chns_status build_block_jacobi(chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, DevBuf &out,
                                cudaStream_t st, double scale) {
   Workspace &ws = m->ws;
-  const int nf = m->nf;
+  const int nf = m->nf, total = m->n_node_colours * nf;
   const int64_t n = m->n_nodes * nf;
+  const int batch = probe_batch(m, sizeof(T), 0, total);
   TRY(out.ensure(sizeof(T) * m->n_nodes * nf * nf + 16));
-  TRY(ws.wv.ensure(sizeof(T) * n));
-  TRY(ws.yv.ensure(sizeof(T) * n));
+  TRY(ws.wv.ensure(sizeof(T) * n * batch));
+  TRY(ws.yv.ensure(sizeof(T) * n * batch));
   T *w = ws.wv.as<T>(), *y = ws.yv.as<T>(), *B = out.as<T>();
-  for (int c = 0; c < m->n_node_colours; ++c) {
-    int64_t b = m->node_colour_start[c], e = m->node_colour_start[c + 1];
-    for (int f = 0; f < nf; ++f) {
-      CHNS_CUDA_TRY(cudaMemsetAsync(w, 0, sizeof(T) * n, st));
-      probe_set<T>(m->node_perm + b, e - b, nf, f, w, st);
-      TRY(jacvec_prepared<T>(m, pc, ut, dl, w, y, st));
-      probe_get<T>(m->node_perm + b, e - b, nf, f, y, B, st);
-    }
+  for (int v0 = 0; v0 < total; v0 += batch) {
+    const int nv = std::min(batch, total - v0);
+    probe_set<T>(m->node_colour, m->n_nodes, nf, v0, nv, w, st);
+    TRY(jacvec_prepared<T>(m, pc, ut, dl, w, y, st, nv));
+    probe_get<T>(m->node_colour, m->n_nodes, nf, v0, nv, y, B, st);
   }
   int *bad = reinterpret_cast<int *>(reinterpret_cast<char *>(B) + sizeof(T) * m->n_nodes * nf * nf);
   CHNS_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), st));
@@ -540,19 +545,15 @@ struct JvCtx {
 };
 
 template <typename T>
-chns_status jv_callback(void *ctx, const T *w, T *y) {
+chns_status jv_callback(void *ctx, const T *w, T *y, int nv) {
   JvCtx<T> *c = static_cast<JvCtx<T> *>(ctx);
-  return jacvec_prepared<T>(c->m, *c->pc, c->ut, c->dl, w, y, c->st);
+  return jacvec_prepared<T>(c->m, *c->pc, c->ut, c->dl, w, y, c->st, nv);
 }
 
 template <typename T>
 chns_status build_coarse_operator(chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, cudaStream_t st) {
-  Workspace &ws = m->ws;
-  const int64_t n = m->n_nodes * m->nf;
-  TRY(ws.wv.ensure(sizeof(T) * n));
-  TRY(ws.yv.ensure(sizeof(T) * n));
   JvCtx<T> ctx{m, &pc, ut, dl, st};
-  return coarse_build<T>(m, &jv_callback<T>, &ctx, ws.wv.as<T>(), ws.yv.as<T>(), st);
+  return coarse_build<T>(m, &jv_callback<T>, &ctx, st);
 }
 
 // An FP32-Krylov Newton iteration must cut ||F|| by at least this factor;
@@ -993,6 +994,7 @@ void chns_mesh_destroy(chns_mesh *m) {
   cudaFree(m->hang);
   cudaFree(m->wall);
   cudaFree(m->node_perm);
+  cudaFree(m->node_colour);
   cudaFree(m->gptr);
   cudaFree(m->gent);
   cudaFree(m->nflag);

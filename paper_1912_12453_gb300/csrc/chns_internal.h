@@ -118,7 +118,13 @@ struct Coarse {
   DevBuf Minv32;                    // per instance A_c^{-1} in float, nc0 x nc0
   DevBuf piv;                       // Gauss-Jordan row interchanges, 3 nc0 indices per instance
   DevBuf gj;                        // Gauss-Jordan working matrices (element precision)
-  DevBuf vec;                       // coarse work vectors and operator-build partials
+  DevBuf cpart;                     // operator-build partials of a batch of probes
+  int n_chunks = 0;                 // pieces of the longest restriction list
+  // the coarse grid is the mesh itself (P = I): the operator and its inverse
+  // are in the mesh's node order, cinv[coarse node] is its mesh node
+  bool direct = false;
+  int32_t *cinv = nullptr;
+  DevBuf vec;                       // coarse work vectors
   DevBuf rpart;                     // restriction partials, n_pieces x 2^dim x nf doubles
   bool ready = false;
   ~Coarse();
@@ -159,6 +165,7 @@ struct chns_mesh {
   int32_t *hang = nullptr;             // n_hang * 4 parent nodes (-1 padded for edge midpoints)
   int32_t *wall = nullptr;             // n_wall node indices on the box boundary
   int32_t *node_perm = nullptr;        // n_nodes node indices grouped by node colour
+  uint8_t *node_colour = nullptr;      // n_nodes: the node's colour (at most 256)
   // node gather of element-local J.w contributions: the (element, corner)
   // slots feeding node i are gent[gptr[i] .. gptr[i+1]), each slot e*nc+c
   // with its hanging-node weight in the top two bits (0: 1, 1: 1/2, 2: 1/4),

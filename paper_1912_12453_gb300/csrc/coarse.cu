@@ -21,6 +21,7 @@
 
 #include "chns_internal.h"
 #include "coarse.h"
+#include "solver.h"
 
 namespace chns {
 
@@ -40,6 +41,7 @@ struct CGeo {
   int64_t ncn_inst;   // coarse nodes per instance
   int64_t nc0;        // coarse unknowns per instance
   int64_t ncell_inst; // coarse cells per instance, (nc1 - 1)^dim
+  int direct;         // the coarse grid is the mesh: unknowns in node order
 };
 
 // 16 bytes of T
@@ -70,11 +72,14 @@ __device__ __forceinline__ int lin(const CGeo &g, const int *c) {
   return idx;
 }
 
-// probing vector: field f = sum of the coarse hats of colour k; other fields 0
+// probing vectors v0 .. v0 + gridDim.y - 1; number v = k NF + f: field f = sum
+// of the coarse hats of colour k; other fields 0
 template <typename T, int NF, int DIM>
-__global__ void __launch_bounds__(kB) k_probe_coarse(CGeo g, const float *__restrict__ pos, int k, int f,
+__global__ void __launch_bounds__(kB) k_probe_coarse(CGeo g, const float *__restrict__ pos, int v0,
                                                      T *__restrict__ w) {
-  int kk[3] = {k % 3, (k / 3) % 3, k / 9};
+  const int k = (v0 + int(blockIdx.y)) / NF, f = (v0 + int(blockIdx.y)) % NF;
+  const int kk[3] = {k % 3, (k / 3) % 3, k / 9};
+  w += blockIdx.y * g.n_nodes * NF;
   for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < g.n_nodes; i += int64_t(gridDim.x) * kB) {
     int b[3];
     float t[3];
@@ -113,77 +118,63 @@ __device__ __forceinline__ bool slot_owner(const CGeo &g, const int *cpc, const 
   return ok;
 }
 
-constexpr int kChunks = 16;
+constexpr int kChunk = 64;
 
-// Block (c', sl) takes the sl-th of kChunks slices of the restriction list of
-// coarse row node c' and, for the probed colour k, sums P[i, c'] y[i, q] per
-// owner slot (the owner of mesh node i: the nearest coarse node of colour k).
-// Sums in T within the block (fixed order), one partial per slice.
-template <typename T, int NF>
-__global__ void __launch_bounds__(kB) k_gather_coarse(CGeo g, const int64_t *__restrict__ rstart,
-                                                      const int32_t *__restrict__ rnode,
-                                                      const float *__restrict__ rw, const float *__restrict__ pos,
-                                                      int k, const T *__restrict__ y, double *__restrict__ part) {
-  const int cp = blockIdx.x, sl = blockIdx.y;
-  int cpc[3] = {0, 0, 0}, kk[3] = {k % 3, (k / 3) % 3, k / 9};
-  {
-    int r = int(cp % g.ncn_inst);
-    for (int a = 0; a < g.dim; ++a) { cpc[a] = r % g.nc1; r /= g.nc1; }
-  }
-  T acc[8][NF];
-#pragma unroll
-  for (int s = 0; s < 8; ++s)
-#pragma unroll
-    for (int q = 0; q < NF; ++q) acc[s][q] = T(0);
-  const int64_t b0 = rstart[cp], len = rstart[cp + 1] - b0;
-  const int64_t lo = b0 + len * sl / kChunks, hi = b0 + len * (sl + 1) / kChunks;
-  for (int64_t e = lo + threadIdx.x; e < hi; e += kB) {
-    const int64_t i = rnode[e];
-    const T wgt = T(rw[e]);
-    int slot = 0;
+// Block (c', sl, v) takes the sl-th piece of kChunk entries of the restriction
+// list of coarse row node c' and, for probe v (colour k), sums P[i, c'] y[i, q]
+// per owner slot s (the owner of mesh node i: the nearest coarse node of
+// colour k), in list order: the threads first find the entries' slots
+// together, then thread (s, q) adds up the entries of its slot.  A block of
+// 256 threads with 48 sums each, reduced over the block, spent its time on the
+// reduction: most lists hold 64 to 125 entries.
+template <typename T, int NF, int DIM>
+__global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int64_t *__restrict__ rstart,
+                                                          const int32_t *__restrict__ rnode,
+                                                          const float *__restrict__ rw, const float *__restrict__ pos,
+                                                          int v0, const T *__restrict__ y, double *__restrict__ part) {
+  constexpr int NS = 1 << DIM;
+  static_assert(NS * NF <= kChunk, "one sum per thread");
+  const int cp = blockIdx.x, sl = blockIdx.y, k = (v0 + int(blockIdx.z)) / NF;
+  const int kk[3] = {k % 3, (k / 3) % 3, k / 9};
+  __shared__ int32_t node[kChunk], slot[kChunk];
+  __shared__ T wgt[kChunk];
+  y += blockIdx.z * g.n_nodes * NF;
+  const int64_t b = rstart[cp] + int64_t(sl) * kChunk;
+  const int cnt = int(min(int64_t(kChunk), rstart[cp + 1] - b));
+  if (int(threadIdx.x) < cnt) {
+    const int64_t i = rnode[b + threadIdx.x];
+    int r = int(cp % g.ncn_inst), s = 0;
     bool ok = true;
-    for (int a = 0; a < g.dim; ++a) {
-      const float p = pos[i * g.dim + a];
-      int o = kk[a] + 3 * (int)floorf((p - float(kk[a])) / 3.0f + 0.5f);
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      const int cpc = r % g.nc1;
+      r /= g.nc1;
+      const float p = pos[i * DIM + a];
+      const int o = kk[a] + 3 * (int)floorf((p - float(kk[a])) / 3.0f + 0.5f);
       if (o < 0 || o >= g.nc1) ok = false;
-      if (o > cpc[a]) slot |= 1 << a;
+      if (o > cpc) s |= 1 << a;
     }
-    if (!ok) continue;
-    T yq[NF];
-#pragma unroll
-    for (int q = 0; q < NF; ++q) yq[q] = y[i * NF + q];
-#pragma unroll
-    for (int s = 0; s < 8; ++s)
-      if (s == slot)
-#pragma unroll
-        for (int q = 0; q < NF; ++q) acc[s][q] = fma(wgt, yq[q], acc[s][q]);
+    node[threadIdx.x] = int32_t(i);
+    slot[threadIdx.x] = ok ? s : -1;
+    wgt[threadIdx.x] = T(rw[b + threadIdx.x]);
   }
-  __shared__ T red[kB / 32][8 * NF];
-  const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 0; s < 8; ++s)
-#pragma unroll
-    for (int q = 0; q < NF; ++q) {
-      const T v = warp_sum_t(acc[s][q]);
-      if (ln == 0) red[wid][s * NF + q] = v;
-    }
   __syncthreads();
-  for (int t = threadIdx.x; t < 8 * NF; t += kB) {
-    T v = T(0);
-#pragma unroll
-    for (int w = 0; w < kB / 32; ++w) v += red[w][t];
-    part[(int64_t(cp) * kChunks + sl) * 8 * NF + t] = double(v);
-  }
+  const int s = threadIdx.x / NF, q = threadIdx.x % NF;
+  if (s >= NS) return;
+  T acc = T(0);
+  for (int e = 0; e < cnt; ++e)
+    if (slot[e] == s) acc = fma(wgt[e], y[int64_t(node[e]) * NF + q], acc);
+  part[((blockIdx.z * int64_t(gridDim.x) + cp) * gridDim.y + sl) * NS * NF + threadIdx.x] = double(acc);
 }
 
-// A[(c', q), (owner(s), f)] = sum of the slices, in slice order
-__global__ void k_gather_sum(CGeo g, int k, int f, const double *__restrict__ part, double *__restrict__ A,
+// A[(c', q), (owner(s), f)] = sum of the pieces, in list order
+__global__ void k_gather_sum(CGeo g, int v0, int n_chunks, const double *__restrict__ part, double *__restrict__ A,
                              int64_t ldA, int64_t ncn) {
   const int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x;
-  const int nf = g.nf;
-  if (t >= ncn * 8 * nf) return;
-  const int cp = int(t / (8 * nf)), s = int((t / nf) % 8), q = int(t % nf);
-  if (s >= (1 << g.dim)) return;
+  const int nf = g.nf, ns = 1 << g.dim, v = v0 + blockIdx.y, k = v / nf, f = v % nf;
+  if (t >= ncn * ns * nf) return;
+  const int64_t cp = t / (ns * nf);
+  const int s = int((t / nf) % ns), q = int(t % nf);
   const int64_t inst = cp / g.ncn_inst, lcp = cp % g.ncn_inst;
   int cpc[3] = {0, 0, 0}, kk[3] = {k % 3, (k / 3) % 3, k / 9}, oc[3];
   {
@@ -191,10 +182,36 @@ __global__ void k_gather_sum(CGeo g, int k, int f, const double *__restrict__ pa
     for (int a = 0; a < g.dim; ++a) { cpc[a] = r % g.nc1; r /= g.nc1; }
   }
   if (!slot_owner(g, cpc, kk, s, oc)) return;
-  double v = 0.0;
-  for (int sl = 0; sl < kChunks; ++sl) v += part[((int64_t(cp) * kChunks + sl) * 8 + s) * nf + q];
+  double sum = 0.0;
+  for (int sl = 0; sl < n_chunks; ++sl)
+    sum += part[(((blockIdx.y * ncn + cp) * n_chunks + sl) * ns + s) * nf + q];
   double *Ai = A + inst * g.nc0 * ldA;
-  Ai[(lcp * nf + q) * ldA + int64_t(lin(g, oc)) * nf + f] = v;
+  Ai[(lcp * nf + q) * ldA + int64_t(lin(g, oc)) * nf + f] = sum;
+}
+
+// The same for a coarse grid that is the mesh: row (i, q) of A, in the mesh's
+// node order, gets y[i, q] in the column of the probed node next to node i
+template <typename T, int NF, int DIM>
+__global__ void __launch_bounds__(kB) k_collect_direct(CGeo g, const float *__restrict__ pos,
+                                                       const int32_t *__restrict__ cinv, int v0,
+                                                       const T *__restrict__ y, double *__restrict__ A) {
+  const int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x;
+  if (i >= g.n_nodes) return;
+  const int k = (v0 + int(blockIdx.y)) / NF, f = (v0 + int(blockIdx.y)) % NF;
+  const int kk[3] = {k % 3, (k / 3) % 3, k / 9};
+  int oc[3];
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) {
+    const int c = int(pos[i * DIM + a]);
+    int d = (kk[a] - c % 3 + 3) % 3;  // 0, 1 or 2 = -1
+    oc[a] = c + (d == 2 ? -1 : d);
+    if (oc[a] < 0 || oc[a] >= g.nc1) return;
+  }
+  const int64_t inst = i / g.ncn_inst, li = i % g.ncn_inst, lo = cinv[inst * g.ncn_inst + lin(g, oc)] % g.ncn_inst;
+  const T *yi = y + (blockIdx.y * g.n_nodes + i) * NF;
+  double *Ai = A + inst * g.nc0 * g.nc0 + lo * NF + f;
+#pragma unroll
+  for (int q = 0; q < NF; ++q) Ai[(li * NF + q) * g.nc0] = double(yi[q]);
 }
 
 constexpr int kPiece = 1024;
@@ -313,7 +330,10 @@ __global__ void __launch_bounds__(kB) k_block_prolong(CGeo g, const float *__res
     T x[NF], acc[NF];
 #pragma unroll
     for (int q = 0; q < NF; ++q) { x[q] = v[i * NF + q]; acc[q] = T(0); }
-    if (zc) {
+    if (zc && g.direct) {
+#pragma unroll
+      for (int q = 0; q < NF; ++q) acc[q] = zc[i * NF + q];
+    } else if (zc) {
       int b[3];
       float tf[3];
       locate(g, pos + i * DIM, b, tf);
@@ -747,6 +767,11 @@ void Coarse::release() {
   Minv32.release();
   piv.release();
   gj.release();
+  cpart.release();
+  cudaFree(cinv);
+  cinv = nullptr;
+  direct = false;
+  n_chunks = 0;
   vec.release();
   rpart.release();
   level = -1;
@@ -800,6 +825,17 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   std::vector<int64_t> cnt(ncn_all + 1, 0);
   for (int64_t i = 0; i < m->n_nodes; ++i) corners(i, [&](int64_t idx, double) { cnt[idx + 1]++; });
   for (int64_t c = 0; c < ncn_all; ++c) cnt[c + 1] += cnt[c];
+  int64_t longest = 0;
+  for (int64_t c = 0; c < ncn_all; ++c) longest = std::max(longest, cnt[c + 1] - cnt[c]);
+  C.n_chunks = int((longest + kChunk - 1) / kChunk);
+  C.direct = m->uniform && Lc == m->min_level;
+  if (C.direct) {
+    // node i <-> coarse node (the corners of a node on the coarse grid: itself)
+    std::vector<int32_t> cinv(ncn_all);
+    for (int64_t i = 0; i < m->n_nodes; ++i) corners(i, [&](int64_t idx, double) { cinv[idx] = (int32_t)i; });
+    CHNS_CUDA_TRY(cudaMalloc(&C.cinv, sizeof(int32_t) * cinv.size()));
+    CHNS_CUDA_TRY(cudaMemcpy(C.cinv, cinv.data(), sizeof(int32_t) * cinv.size(), cudaMemcpyHostToDevice));
+  }
   std::vector<int32_t> rnode(cnt[ncn_all]);
   std::vector<float> rw(cnt[ncn_all]);
   std::vector<int64_t> fill(cnt.begin(), cnt.end() - 1);
@@ -894,35 +930,56 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   TRY_CHNS(C.M.ensure(sizeof(double) * C.nc0 * C.nc0 * ni));
   TRY_CHNS(C.piv.ensure(sizeof(int32_t) * 3 * C.nc0 * ni));
   TRY_CHNS(C.Minv32.ensure(sizeof(float) * C.nc0 * C.nc0 * ni));
-  TRY_CHNS(C.vec.ensure(sizeof(double) * (3 * C.nc + 8 + C.ncn * kChunks * 8 * nf)));
+  TRY_CHNS(C.vec.ensure(sizeof(double) * (3 * C.nc + 8)));
   TRY_CHNS(C.rpart.ensure(sizeof(double) * std::max<int64_t>(np, 1) * (1 << dim) * nf));
   return CHNS_OK;
 }
 
 template <typename T>
-chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, T *w, T *y, cudaStream_t st) {
+chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
   Coarse &C = m->coarse;
+  Workspace &ws = m->ws;
   const int nf = m->nf, dim = m->dim;
-  CGeo g{dim, nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst};
+  CGeo g{dim, nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst, C.direct ? 1 : 0};
   double *M = C.M.as<double>();
-  const int64_t nc0 = C.nc0, nn = nc0 * nc0 * C.n_inst;
+  const int64_t nc0 = C.nc0, nn = nc0 * nc0 * C.n_inst, n = m->n_nodes * nf;
   CHNS_CUDA_TRY(cudaMemsetAsync(M, 0, sizeof(double) * nn, st));
-  const int ncol = dim == 2 ? 9 : 27;
-  double *part = C.vec.as<double>() + 3 * C.nc + 8;
-  for (int k = 0; k < ncol; ++k)
-    for (int f = 0; f < nf; ++f) {
-      if (dim == 2) k_probe_coarse<T, 5, 2><<<grid_n(m->n_nodes), kB, 0, st>>>(g, C.pos, k, f, w);
-      else k_probe_coarse<T, 6, 3><<<grid_n(m->n_nodes), kB, 0, st>>>(g, C.pos, k, f, w);
+  // the probes (9 colours in 2D, 27 in 3D, times the fields) go through J.w in
+  // batches: 45 or 162 times five launches otherwise, most of them too small to
+  // fill the GPU.  With the batches of the nodal blocks, one CN step: FP64 of
+  // the 2D droplet 18.3 -> 9.1 ms, multigrid of the level-5 3D droplet 22.5 ->
+  // 12.6 ms
+  const int total = (dim == 2 ? 9 : 27) * nf;
+  const size_t piece = C.direct ? 0 : sizeof(double) * size_t(C.ncn) * C.n_chunks * (size_t(1) << dim) * nf;
+  const int batch = probe_batch(m, sizeof(T), piece, total);
+  TRY_CHNS(ws.wv.ensure(sizeof(T) * n * batch));
+  TRY_CHNS(ws.yv.ensure(sizeof(T) * n * batch));
+  TRY_CHNS(C.cpart.ensure(piece * batch));
+  T *w = ws.wv.as<T>(), *y = ws.yv.as<T>();
+  double *part = C.cpart.as<double>();
+  for (int v0 = 0; v0 < total; v0 += batch) {
+    const unsigned nv = (unsigned)std::min(batch, total - v0);
+    const dim3 gp(grid_n(m->n_nodes), nv);
+    if (dim == 2) k_probe_coarse<T, 5, 2><<<gp, kB, 0, st>>>(g, C.pos, v0, w);
+    else k_probe_coarse<T, 6, 3><<<gp, kB, 0, st>>>(g, C.pos, v0, w);
+    note_launches(1);
+    TRY_CHNS(jv(ctx, w, y, int(nv)));
+    if (C.direct) {
+      const dim3 gd((unsigned)((m->n_nodes + kB - 1) / kB), nv);
+      if (dim == 2) k_collect_direct<T, 5, 2><<<gd, kB, 0, st>>>(g, C.pos, C.cinv, v0, y, M);
+      else k_collect_direct<T, 6, 3><<<gd, kB, 0, st>>>(g, C.pos, C.cinv, v0, y, M);
       note_launches(1);
-      TRY_CHNS(jv(ctx, w, y));
-      dim3 gr((unsigned)C.ncn, kChunks);
-      if (nf == 5)
-        k_gather_coarse<T, 5><<<gr, kB, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, k, y, part);
-      else
-        k_gather_coarse<T, 6><<<gr, kB, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, k, y, part);
-      k_gather_sum<<<(unsigned)((C.ncn * 8 * nf + kB - 1) / kB), kB, 0, st>>>(g, k, f, part, M, nc0, C.ncn);
-      note_launches(2);
+      continue;
     }
+    const dim3 gr((unsigned)C.ncn, (unsigned)C.n_chunks, nv);
+    if (dim == 2)
+      k_gather_coarse<T, 5, 2><<<gr, kChunk, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, v0, y, part);
+    else
+      k_gather_coarse<T, 6, 3><<<gr, kChunk, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, v0, y, part);
+    const dim3 gs((unsigned)((C.ncn * (nf << dim) + kB - 1) / kB), nv);
+    k_gather_sum<<<gs, kB, 0, st>>>(g, v0, C.n_chunks, part, M, nc0, C.ncn);
+    note_launches(2);
+  }
   // A_c^{-1} per instance, in the element precision: the FP32 path inverts
   // in float (A_c is ill-conditioned along a pressure direction only, which
   // float resolves: per-field errors of the applied inverse ~1e-6 at
@@ -961,35 +1018,41 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, T *w, T *y, cudaSt
   C.ready = true;
   return CHNS_OK;
 }
-template chns_status coarse_build<float>(chns_mesh *, JvFn<float>, void *, float *, float *, cudaStream_t);
-template chns_status coarse_build<double>(chns_mesh *, JvFn<double>, void *, double *, double *, cudaStream_t);
+template chns_status coarse_build<float>(chns_mesh *, JvFn<float>, void *, cudaStream_t);
+template chns_status coarse_build<double>(chns_mesh *, JvFn<double>, void *, cudaStream_t);
 
-// z = B^{-1} v (+ P A_c^{-1} R v when the coarse space is ready and wanted)
+// z = B^{-1} v (+ P A_c^{-1} R v when the coarse space is ready and wanted).  On
+// a coarse grid that is the mesh, P and R are the identity and the inverse is
+// in node order: without a block term the apply is one product.
 template <typename T>
 void precond_apply(chns_mesh *m, const T *Binv, bool coarse, const T *v, T *z, cudaStream_t st) {
   Coarse &C = m->coarse;
   const bool use = coarse && C.ready;
-  CGeo g{m->dim, m->nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst};
-  T *rc = nullptr, *zc = nullptr;
+  CGeo g{m->dim, m->nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst, C.direct ? 1 : 0};
+  const T *zc = nullptr;
   if (use) {
-    rc = reinterpret_cast<T *>(C.vec.as<double>());
-    zc = reinterpret_cast<T *>(C.vec.as<double>() + C.nc);
-    T *part = reinterpret_cast<T *>(C.rpart.as<double>());
-    const unsigned np = (unsigned)C.n_pieces;
-    const unsigned gs = (unsigned)((C.nc * 32 + kB - 1) / kB);
-    if (m->dim == 2)
-      k_restrict_cells<T, 5, 2><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
-    else
-      k_restrict_cells<T, 6, 3><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
-    k_restrict_sum<T><<<gs, kB, 0, st>>>(C.nc, m->nf, C.sptr, C.sent, part, rc);
+    const T *rc = v;
+    T *out = C.direct && !Binv ? z : reinterpret_cast<T *>(C.vec.as<double>() + C.nc);
+    if (!C.direct) {
+      T *r = reinterpret_cast<T *>(C.vec.as<double>());
+      T *part = reinterpret_cast<T *>(C.rpart.as<double>());
+      const unsigned np = (unsigned)C.n_pieces;
+      const unsigned gs = (unsigned)((C.nc * 32 + kB - 1) / kB);
+      if (m->dim == 2)
+        k_restrict_cells<T, 5, 2><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
+      else
+        k_restrict_cells<T, 6, 3><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
+      k_restrict_sum<T><<<gs, kB, 0, st>>>(C.nc, m->nf, C.sptr, C.sent, part, r);
+      note_launches(2);
+      rc = r;
+    }
+    const T *Mi = sizeof(T) == sizeof(float) ? reinterpret_cast<const T *>(C.Minv32.as<float>())
+                                             : reinterpret_cast<const T *>(C.M.as<double>());
     const unsigned gm = (unsigned)((C.nc * 32 + kB - 1) / kB);
-    if (sizeof(T) == sizeof(float))
-      k_coarse_matvec<T><<<gm, kB, 0, st>>>(reinterpret_cast<const T *>(C.Minv32.as<float>()), C.nc0,
-                                            C.nc0 * C.nc0, C.nc, C.nc0, rc, zc);
-    else
-      k_coarse_matvec<T><<<gm, kB, 0, st>>>(reinterpret_cast<const T *>(C.M.as<double>()), C.nc0,
-                                            C.nc0 * C.nc0, C.nc, C.nc0, rc, zc);
-    note_launches(3);
+    k_coarse_matvec<T><<<gm, kB, 0, st>>>(Mi, C.nc0, C.nc0 * C.nc0, C.nc, C.nc0, rc, out);
+    note_launches(1);
+    if (out == z) return;
+    zc = out;
   }
   const int32_t *ni = (use && m->n_inst > 1) ? m->node_inst : nullptr;
   if (m->dim == 2) k_block_prolong<T, 5, 2><<<grid_n(m->n_nodes), kB, 0, st>>>(g, C.pos, ni, Binv, v, zc, z);

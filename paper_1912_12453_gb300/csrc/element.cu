@@ -513,16 +513,21 @@ KCoef<T> kcoef(const PhysCoef &p, int dim) {
 // is floored (O = unsigned long long, one counter); MODE 3: J.w scattered into
 // the node vector (one launch per element colour).  MODE 0 and 2 read the
 // states themselves (ut = U_new, dl = U_old: they are evaluated once per
-// state), the J.w modes the prepared averages and increments.  BS, MINB:
-// block size and minimum resident blocks per SM (the register budget).
+// state), the J.w modes the prepared averages and increments.  MODE 1 takes
+// gridDim.y directions at a time (w and out at strides).  BS, MINB: block size
+// and minimum resident blocks per SM (the register budget).
 template <int D, typename T, int MODE, bool HASF, typename O, int BS = 128, int MINB = 6>
 __global__ void __launch_bounds__(BS, MINB) k_element(
     const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
     const int32_t *__restrict__ hang, int64_t e_begin, int64_t e_end,
     const T *__restrict__ ut, const T *__restrict__ dl, const T *__restrict__ w,
     const T *__restrict__ f, O *__restrict__ out, KCoef<T> c0, const KCoef<T> *__restrict__ tab,
-    const uint16_t *__restrict__ einst) {
+    const uint16_t *__restrict__ einst, int64_t wstride, int64_t ostride) {
   constexpr int NC = 1 << D, NF = D + 3, ND = D + 1;
+  if (MODE == 1) {
+    w += blockIdx.y * wstride;
+    out += blockIdx.y * ostride;
+  }
   constexpr bool UNIT = sizeof(T) == 4, RAW = MODE == 0 || MODE == 2;
   static_assert(!(UNIT && RAW), "the residual is in double");
   const int lc = threadIdx.x & (NC - 1);
@@ -697,8 +702,11 @@ __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict_
                                                       const int32_t *__restrict__ gent,
                                                       const uint8_t *__restrict__ nflag, int64_t n_nodes,
                                                       const T *__restrict__ E, const T *w, const T *bc, T *y,
-                                                      uint32_t fmask) {
+                                                      uint32_t fmask, int64_t estride) {
   constexpr int NF = D + 3, G = 8;
+  E += blockIdx.y * estride;  // gridDim.y directions, one vector after another
+  w += blockIdx.y * n_nodes * NF;
+  y += blockIdx.y * n_nodes * NF;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n_nodes; i += int64_t(gridDim.x) * blockDim.x) {
     T acc[NF];
 #pragma unroll
@@ -885,9 +893,9 @@ static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const
                                const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
   k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks><<<grid_elem(m->n_elem << D), kElemBlock, 0, st>>>(
       m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
-      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst);
+      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0);
   k_gather_nodes<D, double, true><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
-                                                                             Un, bc, F, 0xffu);
+                                                                             Un, bc, F, 0xffu, 0);
   note_launches(2);
 }
 
@@ -918,12 +926,14 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 //   6: as 0 with 128-thread blocks, 4 per SM (up to 128 registers)
 template <int D, typename T, int BS, int MINB>
 static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
-                         const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st) {
-  const int64_t threads = m->n_elem << D;
-  k_element<D, T, 1, false, T, BS, MINB><<<(unsigned)((threads + BS - 1) / BS), BS, 0, st>>>(
-      m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w, nullptr, E, c, tab, m->elem_inst);
-  k_gather_nodes<D, T, false><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w,
-                                                                         nullptr, y, fmask);
+                         const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
+  constexpr int NF = D + 3;
+  const int64_t threads = m->n_elem << D, es = threads * NF;
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_nodes(m->n_nodes), (unsigned)nv);
+  k_element<D, T, 1, false, T, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
+                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, es);
+  k_gather_nodes<D, T, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
+                                                     es);
   note_launches(2);
 }
 
@@ -935,7 +945,7 @@ static void jv_colours(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
     const int64_t b = m->colour_start[col], e = m->colour_start[col + 1];
     if (e <= b) continue;
     k_element<D, T, 3, false, T><<<grid_elem((e - b) << D), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, b, e, ut, dl, w, nullptr, y, c, tab, m->elem_inst);
+        m->conn, m->level, m->hang, b, e, ut, dl, w, nullptr, y, c, tab, m->elem_inst, 0, 0);
     note_launches(1);
   }
   k_fix_rows<D, T><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->nflag, m->n_nodes, w, y, fmask);
@@ -944,40 +954,41 @@ static void jv_colours(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
 
 template <int D, typename T>
 static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
-                        const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st) {
+                        const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
+  if (nv > 1 && variant == 4) variant = 0;  // the colour schedule takes one direction at a time
   if constexpr (sizeof(T) == 4) {
     switch (variant) {
-      case 1: jv_elemlocal<D, T, 256, 3>(m, c, tab, ut, dl, w, E, y, fmask, st); return;
-      case 2: jv_elemlocal<D, T, 64, 12>(m, c, tab, ut, dl, w, E, y, fmask, st); return;
-      case 3: jv_elemlocal<D, T, 128, 8>(m, c, tab, ut, dl, w, E, y, fmask, st); return;
+      case 1: jv_elemlocal<D, T, 256, 3>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
+      case 2: jv_elemlocal<D, T, 64, 12>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
+      case 3: jv_elemlocal<D, T, 128, 8>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
       case 4: jv_colours<D, T>(m, c, tab, ut, dl, w, y, fmask, st); return;
-      case 5: jv_elemlocal<D, T, 128, 5>(m, c, tab, ut, dl, w, E, y, fmask, st); return;
-      case 6: jv_elemlocal<D, T, 128, 4>(m, c, tab, ut, dl, w, E, y, fmask, st); return;
+      case 5: jv_elemlocal<D, T, 128, 5>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
+      case 6: jv_elemlocal<D, T, 128, 4>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
       default: break;
     }
   }
   if constexpr (sizeof(T) == 8) {
     // FP64: bound by the narrow FP64 pipe, so occupancy matters less than
     // the register spills a 6-blocks-per-SM budget causes
-    jv_elemlocal<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, y, fmask, st);
+    jv_elemlocal<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
   } else {
-    jv_elemlocal<D, T, 128, 6>(m, c, tab, ut, dl, w, E, y, fmask, st);
+    jv_elemlocal<D, T, 128, 6>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
   }
 }
 
 template <typename T>
 void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *E, T *y,
-                   cudaStream_t st, int variant) {
+                   cudaStream_t st, int variant, int nv) {
   KCoef<T> c = kcoef<T>(pc, m->dim);
   const KCoef<T> *tab = reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32);
   if (variant < 0) variant = sizeof(T) == 4 ? m->jv_variant : 0;
-  if (m->dim == 2) jv_dispatch<2, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st);
-  else jv_dispatch<3, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st);
+  if (m->dim == 2) jv_dispatch<2, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
+  else jv_dispatch<3, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
 }
 template void launch_jacvec<float>(const chns_mesh *, const PhysCoef &, const float *, const float *,
-                                   const float *, float *, float *, cudaStream_t, int);
+                                   const float *, float *, float *, cudaStream_t, int, int);
 template void launch_jacvec<double>(const chns_mesh *, const PhysCoef &, const double *, const double *,
-                                    const double *, double *, double *, cudaStream_t, int);
+                                    const double *, double *, double *, cudaStream_t, int, int);
 
 // Gauss points with a floored tau_m radicand, added to *count (all elements
 // in one launch, FP64 physics as in the residual)
@@ -987,10 +998,10 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
   const KCoef<double> *tab = reinterpret_cast<const KCoef<double> *>(m->coef64);
   if (m->dim == 2)
     k_element<2, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 2), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0);
   else
     k_element<3, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 3), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0);
   note_launches(1);
 }
 

@@ -16,11 +16,12 @@ void launch_prep(const chns_mesh *m, const double *Un, const double *Uo, T *ut, 
 void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const double *f,
                      const double *bc, double *E, double *F, cudaStream_t st);
 // J.w with schedule `variant` (-1: the mesh's tuned schedule for float,
-// schedule 0 for double); see element.cu for the schedules
+// schedule 0 for double); see element.cu for the schedules.  nv directions at
+// a time: w and y hold nv vectors one after another, E nv element-local buffers
 constexpr int kJacvecVariants = 7;
 template <typename T>
 void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *E, T *y,
-                   cudaStream_t st, int variant = -1);
+                   cudaStream_t st, int variant = -1, int nv = 1);
 void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo,
                             unsigned long long *count, cudaStream_t st);
 int64_t energy_blocks(const chns_mesh *m);

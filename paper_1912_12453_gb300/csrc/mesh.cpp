@@ -479,6 +479,8 @@ chns_status build_mesh(int dim, int64_t n, const uint8_t *level, const uint32_t 
   m->inst_node_start = {0, n_nodes};
   m->inst_max_level = {max_level};
   if ((st = upload(&m->node_perm, nperm)) != CHNS_OK) return st;
+  const std::vector<uint8_t> ncol8(ncol.begin(), ncol.end());
+  if ((st = upload(&m->node_colour, ncol8)) != CHNS_OK) return st;
   return CHNS_OK;
 }
 
@@ -700,7 +702,13 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   // node colours: colour c of the union = colour c of every instance
   u->node_colour_start.assign(n_ncol + 1, 0);
   std::vector<std::vector<int32_t>> hperm(ms.size());
-  for (size_t i = 0; i < ms.size(); ++i) hperm[i] = download(ms[i]->node_perm, size_t(ms[i]->n_nodes));
+  std::vector<uint8_t> ncol8;
+  ncol8.reserve(size_t(n_nodes));
+  for (size_t i = 0; i < ms.size(); ++i) {
+    hperm[i] = download(ms[i]->node_perm, size_t(ms[i]->n_nodes));
+    const std::vector<uint8_t> c8 = download(ms[i]->node_colour, size_t(ms[i]->n_nodes));
+    ncol8.insert(ncol8.end(), c8.begin(), c8.end());
+  }
   for (int c = 0; c < n_ncol; ++c) {
     for (size_t i = 0; i < ms.size(); ++i) {
       const chns_mesh *m = ms[i];
@@ -721,6 +729,7 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   if ((st = upload(&u->wall, wall)) != CHNS_OK) return st;
   if ((st = upload(&u->pins, pins)) != CHNS_OK) return st;
   if ((st = upload(&u->node_perm, nperm)) != CHNS_OK) return st;
+  if ((st = upload(&u->node_colour, ncol8)) != CHNS_OK) return st;
   if ((st = upload(&u->elem_inst, einst)) != CHNS_OK) return st;
   if ((st = upload(&u->node_inst, ninst)) != CHNS_OK) return st;
   return CHNS_OK;

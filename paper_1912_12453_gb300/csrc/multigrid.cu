@@ -528,7 +528,7 @@ static void launch_inject(const chns_mesh *c, const int32_t *inj, const T *utf, 
 }
 
 template <typename T>
-static chns_status jv_level(void *ctx, const T *w, T *y);
+static chns_status jv_level(void *ctx, const T *w, T *y, int nv);
 
 namespace {
 template <typename T>
@@ -541,9 +541,9 @@ struct LevelCtx {
 }  // namespace
 
 template <typename T>
-static chns_status jv_level(void *ctx, const T *w, T *y) {
+static chns_status jv_level(void *ctx, const T *w, T *y, int nv) {
   LevelCtx<T> *c = static_cast<LevelCtx<T> *>(ctx);
-  return jacvec_prepared<T>(c->m, *c->pc, c->ut, c->dl, w, y, c->st);
+  return jacvec_prepared<T>(c->m, *c->pc, c->ut, c->dl, w, y, c->st, nv);
 }
 
 template <typename T>
@@ -594,10 +594,8 @@ chns_status mg_build(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
       TRY_MG(build_block_jacobi<T>(c, pc, ut, dl, L.binv[P], st, omega));
     } else {
       // bottom: dense inverse of the level's own operator (coarse grid = this mesh)
-      TRY_MG(c->ws.wv.ensure(sizeof(T) * n));
-      TRY_MG(c->ws.yv.ensure(sizeof(T) * n));
       LevelCtx<T> ctx{c, &pc, ut, dl, st};
-      TRY_MG(coarse_build<T>(c, &jv_level<T>, &ctx, c->ws.wv.as<T>(), c->ws.yv.as<T>(), st));
+      TRY_MG(coarse_build<T>(c, &jv_level<T>, &ctx, st));
     }
   }
   G.ready[P] = true;

@@ -326,21 +326,28 @@ __global__ void k_mask_field(double *__restrict__ y, int64_t n_nodes, int nf, in
     y[t] = (t % nf == k) ? s * y[t] : 0.0;
 }
 
-// probing vector: 1 in field f of the nodes of one node colour
+// probing vectors v0 .. v0 + gridDim.y - 1, one after another; number v = c nf
+// + f is 1 in field f of the nodes of colour c, 0 elsewhere
 template <typename T>
-__global__ void k_probe_set(const int32_t *__restrict__ nodes, int64_t cnt, int nf, int f, T *__restrict__ w) {
-  int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x;
-  if (i < cnt) w[int64_t(nodes[i]) * nf + f] = T(1);
+__global__ void k_probe_set(const uint8_t *__restrict__ colour, int64_t n_nodes, int nf, int v0, T *__restrict__ w) {
+  const int v = v0 + blockIdx.y, c = v / nf, f = v % nf;
+  w += blockIdx.y * n_nodes * nf;
+  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n_nodes; i += int64_t(gridDim.x) * kB) {
+    const bool on = colour[i] == c;
+    for (int q = 0; q < nf; ++q) w[i * nf + q] = on && q == f ? T(1) : T(0);
+  }
 }
 
-// B[a][r][f] = y[a*nf + r] for the probed nodes
+// B[a][r][f] = y[a*nf + r] of the probe that was 1 in field f of node a, for
+// the probes v0 .. v0 + nv - 1
 template <typename T>
-__global__ void k_probe_get(const int32_t *__restrict__ nodes, int64_t cnt, int nf, int f,
+__global__ void k_probe_get(const uint8_t *__restrict__ colour, int64_t n_nodes, int nf, int v0, int nv,
                             const T *__restrict__ y, T *__restrict__ B) {
-  int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x;
-  if (i < cnt) {
-    int64_t a = nodes[i];
-    for (int r = 0; r < nf; ++r) B[(a * nf + r) * nf + f] = y[a * nf + r];
+  for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < n_nodes * nf; t += int64_t(gridDim.x) * kB) {
+    const int64_t a = t / nf;
+    const int f = int(t % nf), v = colour[a] * nf + f - v0;
+    if (v < 0 || v >= nv) continue;
+    for (int r = 0; r < nf; ++r) B[(a * nf + r) * nf + f] = y[(v * n_nodes + a) * nf + r];
   }
 }
 
@@ -497,17 +504,19 @@ void vec_mask_field(double *y, int64_t n_nodes, int nf, int k, double s, cudaStr
 }
 
 template <typename T>
-void probe_set(const int32_t *nodes, int64_t cnt, int nf, int f, T *w, cudaStream_t st) {
-  if (cnt > 0) { k_probe_set<T><<<(unsigned)((cnt + kB - 1) / kB), kB, 0, st>>>(nodes, cnt, nf, f, w); note_launches(1); }
+void probe_set(const uint8_t *colour, int64_t n_nodes, int nf, int v0, int nv, T *w, cudaStream_t st) {
+  k_probe_set<T><<<dim3(grid_n(n_nodes), (unsigned)nv), kB, 0, st>>>(colour, n_nodes, nf, v0, w);
+  note_launches(1);
 }
 template <typename T>
-void probe_get(const int32_t *nodes, int64_t cnt, int nf, int f, const T *y, T *B, cudaStream_t st) {
-  if (cnt > 0) { k_probe_get<T><<<(unsigned)((cnt + kB - 1) / kB), kB, 0, st>>>(nodes, cnt, nf, f, y, B); note_launches(1); }
+void probe_get(const uint8_t *colour, int64_t n_nodes, int nf, int v0, int nv, const T *y, T *B, cudaStream_t st) {
+  k_probe_get<T><<<grid_n(n_nodes * nf), kB, 0, st>>>(colour, n_nodes, nf, v0, nv, y, B);
+  note_launches(1);
 }
-template void probe_set<float>(const int32_t *, int64_t, int, int, float *, cudaStream_t);
-template void probe_set<double>(const int32_t *, int64_t, int, int, double *, cudaStream_t);
-template void probe_get<float>(const int32_t *, int64_t, int, int, const float *, float *, cudaStream_t);
-template void probe_get<double>(const int32_t *, int64_t, int, int, const double *, double *, cudaStream_t);
+template void probe_set<float>(const uint8_t *, int64_t, int, int, int, float *, cudaStream_t);
+template void probe_set<double>(const uint8_t *, int64_t, int, int, int, double *, cudaStream_t);
+template void probe_get<float>(const uint8_t *, int64_t, int, int, int, const float *, float *, cudaStream_t);
+template void probe_get<double>(const uint8_t *, int64_t, int, int, int, const double *, double *, cudaStream_t);
 
 template <typename T>
 void invert_blocks(T *B, int64_t n_nodes, int nf, int *bad, double scale, cudaStream_t st) {

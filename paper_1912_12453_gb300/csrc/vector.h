@@ -47,10 +47,12 @@ void vec_div_field(const double *r, const double *d, double *z, int64_t n_nodes,
 void vec_mask_fields(double *y, int64_t n_nodes, int nf, uint32_t fmask, cudaStream_t st);
 // *res = max_i |x_i - y_i| (partial: red_blocks() doubles)
 void vec_maxabs_diff(const double *x, const double *y, int64_t n, double *partial, double *res, cudaStream_t st);
+// nv probing vectors from number v0 on (number c nf + f: 1 in field f of the
+// nodes of colour c), and the columns of the nodal blocks they read off
 template <typename T>
-void probe_set(const int32_t *nodes, int64_t cnt, int nf, int f, T *w, cudaStream_t st);
+void probe_set(const uint8_t *colour, int64_t n_nodes, int nf, int v0, int nv, T *w, cudaStream_t st);
 template <typename T>
-void probe_get(const int32_t *nodes, int64_t cnt, int nf, int f, const T *y, T *B, cudaStream_t st);
+void probe_get(const uint8_t *colour, int64_t n_nodes, int nf, int v0, int nv, const T *y, T *B, cudaStream_t st);
 // B <- scale * B^{-1} for each nf x nf nodal block
 template <typename T>
 void invert_blocks(T *B, int64_t n_nodes, int nf, int *bad, double scale, cudaStream_t st);
