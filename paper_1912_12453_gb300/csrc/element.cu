@@ -674,6 +674,76 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   }
 }
 
+// ---------------------------------------------------------------- mass matrix
+// Scalar corner value through the hanging constraint, field at offset k of
+// node blocks of S values
+template <int S>
+__device__ __forceinline__ double gather1(int cn, const int32_t *__restrict__ hang, const double *__restrict__ u,
+                                          int k) {
+  if (cn >= 0) return __ldg(u + int64_t(cn) * S + k);
+  const int4 p = reinterpret_cast<const int4 *>(hang)[-cn - 1];
+  const double a = __ldg(u + int64_t(p.x) * S + k) + __ldg(u + int64_t(p.y) * S + k);
+  if (p.z < 0) return 0.5 * a;
+  return 0.25 * (a + (__ldg(u + int64_t(p.z) * S + k) + __ldg(u + int64_t(p.w) * S + k)));
+}
+
+// Element-local part of the Q1 mass matrix times p' = z + *beta p (a scalar
+// per node) into the slots E.  With the 2-point Gauss rule the element matrix
+// is the product over the axes of (h/6) [2 1; 1 2]: u + o/2 per axis and one
+// factor W (2/3)^D, nine FP64 instructions a lane.  The J.w of all fields took
+// 72 times a full apply (1.27 ms on 77,932 leaves) for the same product.
+template <int D>
+__global__ void __launch_bounds__(256) k_mass(const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
+                                              const int32_t *__restrict__ hang, int64_t n_elem,
+                                              const double *__restrict__ z, const double *__restrict__ p,
+                                              const double *__restrict__ beta, const int *__restrict__ done, double W0,
+                                              double *__restrict__ E) {
+  if (done && *done) return;
+  constexpr int NC = 1 << D;
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  int64_t e = t >> D;
+  const bool active = e < n_elem;
+  if (!active) e = n_elem - 1;
+  const int cn = conn[e * NC + (threadIdx.x & (NC - 1))];
+  double u = gather1<1>(cn, hang, z, 0);
+  if (p) u = fma(*beta, gather1<1>(cn, hang, p, 0), u);
+#pragma unroll
+  for (int a = 0; a < D; ++a) u = fma(0.5, __shfl_xor_sync(FULL, u, 1 << a), u);
+  if (active) E[t] = scale2(W0 * (D == 2 ? 4.0 / 9.0 : 8.0 / 27.0), -D * int(level[e])) * u;
+}
+
+// Element-local part of the chemical-potential row at U_new = U_old = U:
+// (N, psi'(phi) - mu) + Cn^2 (grad N, grad phi)
+template <int D>
+__global__ void __launch_bounds__(256) k_mu_row(const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
+                                                const int32_t *__restrict__ hang, int64_t n_elem,
+                                                const double *__restrict__ U, KCoef<double> c,
+                                                double *__restrict__ E) {
+  constexpr int NC = 1 << D, NF = D + 3;
+  const int lc = threadIdx.x & (NC - 1);
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  int64_t e = t >> D;
+  const bool active = e < n_elem;
+  if (!active) e = n_elem - 1;
+  const int cn = conn[e * NC + lc], l = level[e];
+  Stage<D, double> s;
+  s.v = CAD<D>;
+  s.cS = scale2(c.cS0, -D * l);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const bool neg = !((lc >> a) & 1);
+    s.sg[a] = flip_if(scale2(c.sg0[a], l), neg);
+    s.cV[a] = flip_if(scale2(c.cV0[a], (1 - D) * l), neg);
+  }
+  double phi, g[D];
+  ip_vg<D>(gather1<NF>(cn, hang, U, D + 1), s, phi, g);
+  const double mu = ip_v<D>(gather1<NF>(cn, hang, U, D + 2)) * CAD<D>;
+#pragma unroll
+  for (int a = 0; a < D; ++a) g[a] *= c.Cn2;
+  const double r = contract<D>(phi * fma(phi, phi, -1.0) - mu, g, s);
+  if (active) E[t] = r;
+}
+
 // ---------------------------------------------------------------- node kernels
 // v~ = (U_new + U_old)/2 for all fields; increments of v and phi
 template <int D, typename T>
@@ -1002,6 +1072,23 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
   else
     k_element<3, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 3), kElemBlock, 0, st>>>(
         m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0);
+  note_launches(1);
+}
+
+void launch_mass(const chns_mesh *m, const PhysCoef &pc, const double *z, const double *p, const double *beta,
+                 const int *done, double *E, cudaStream_t st) {
+  const KCoef<double> c = kcoef<double>(pc, m->dim);
+  const unsigned g = grid_for(m->n_elem << m->dim);
+  if (m->dim == 2) k_mass<2><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, c.W0, E);
+  else k_mass<3><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, c.W0, E);
+  note_launches(1);
+}
+
+void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st) {
+  const KCoef<double> c = kcoef<double>(pc, m->dim);
+  const unsigned g = grid_for(m->n_elem << m->dim);
+  if (m->dim == 2) k_mu_row<2><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, U, c, E);
+  else k_mu_row<3><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, U, c, E);
   note_launches(1);
 }
 

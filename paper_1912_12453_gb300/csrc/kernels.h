@@ -24,6 +24,12 @@ void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T 
                    cudaStream_t st, int variant = -1, int nv = 1);
 void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo,
                             unsigned long long *count, cudaStream_t st);
+// scalar Q1 mass matrix times z + *beta p (p nullable: z), and the
+// chemical-potential row of U, into element-local slots (n_elem * 2^dim
+// doubles); launch_mass does nothing once *done (nullable) is set
+void launch_mass(const chns_mesh *m, const PhysCoef &pc, const double *z, const double *p, const double *beta,
+                 const int *done, double *E, cudaStream_t st);
+void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st);
 int64_t energy_blocks(const chns_mesh *m);
 // per-instance element coefficients of a batched (union) mesh
 chns_status upload_coef_tables(chns_mesh *m, const std::vector<PhysCoef> &pcs, cudaStream_t st);
