@@ -888,17 +888,15 @@ chns_status step_impl(chns_mesh *m, const chns_params *p, const chns_solver_opts
 chns_status energy_mass_impl(chns_mesh *m, const chns_params *p, const double *U, double out[3],
                              cudaStream_t st) {
   PhysCoef pc = make_coef(*p, m->lo, m->hi);
-  int64_t nb = energy_blocks(m);
-  TRY(m->ws.red.ensure(sizeof(double) * std::max<int64_t>(3 * nb, (kMaxRestart + 16) * red_blocks())));
-  launch_energy(m, pc, U, m->ws.red.as<double>(), st);
+  Workspace &ws = m->ws;
+  TRY(ws.red.ensure(sizeof(double) * std::max<int64_t>(3 * energy_blocks(m), (kMaxRestart + 16) * red_blocks())));
+  TRY(ws.hdev.ensure(sizeof(double) * 8 * kHessSlot));
+  TRY(ensure_pinned(ws));
+  launch_energy(m, pc, U, ws.red.as<double>(), ws.hdev.as<double>(), st);
   TRY(check_launch());
-  std::vector<double> h(3 * nb);
-  CHNS_CUDA_TRY(cudaMemcpyAsync(h.data(), m->ws.red.as<double>(), sizeof(double) * 3 * nb,
-                                cudaMemcpyDeviceToHost, st));
+  CHNS_CUDA_TRY(cudaMemcpyAsync(ws.hpinned, ws.hdev.as<double>(), sizeof(double) * 3, cudaMemcpyDeviceToHost, st));
   CHNS_CUDA_TRY(cudaStreamSynchronize(st));
-  out[0] = out[1] = out[2] = 0.0;
-  for (int64_t b = 0; b < nb; ++b)
-    for (int k = 0; k < 3; ++k) out[k] += h[b * 3 + k];
+  for (int k = 0; k < 3; ++k) out[k] = ws.hpinned[k];
   return CHNS_OK;
 }
 

@@ -39,31 +39,6 @@ static __device__ __align__(256) double g_partials[kMaxBlocks * 3];
 std::mutex g_mu;
 double *g_addr[kMaxDevices] = {nullptr};
 
-// out[k] = sum over blocks b of g_partials[b * 3 + k] in a fixed order: one
-// block of 256 threads, thread t sums the blocks t, t + 256, ... in
-// increasing order, then a fixed shuffle tree per warp and a fixed sum over
-// the warps.  Deterministic; the order differs from chns_energy_mass's host
-// loop only by rounding.
-constexpr int kSumThreads = 256;
-__global__ void __launch_bounds__(kSumThreads) k_sum3(int64_t nb, double *__restrict__ out) {
-  double s[3] = {0.0, 0.0, 0.0};
-  for (int64_t b = threadIdx.x; b < nb; b += kSumThreads)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) s[k] += g_partials[b * 3 + k];
-  __shared__ double part[3][kSumThreads / 32];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
-    if ((threadIdx.x & 31) == 0) part[k][threadIdx.x >> 5] = s[k];
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0.0;
-    for (int w = 0; w < kSumThreads / 32; ++w) t += part[threadIdx.x][w];
-    out[threadIdx.x] = t;
-  }
-}
-
 chns_status scratch_address(double **p) {
   int dev = 0;
   CHNS_CUDA_TRY(cudaGetDevice(&dev));
@@ -89,7 +64,7 @@ extern "C" chns_status chns_energy_mass_noalloc(const chns_mesh *m, const chns_p
   chns_status ps = check_params(m, p);  // the same checks as chns_energy_mass
   if (ps != CHNS_OK) return ps;
   if (!U || !out3) { set_error("null argument"); return CHNS_ERR_ARG; }
-  const int64_t nb = energy_blocks(m);
+  const int64_t nb = ((m->n_elem << m->dim) + 255) / 256;  // the limit is stated in leaves, whatever the grid uses
   if (nb > kMaxBlocks) {
     set_error("mesh too large for chns_energy_mass_noalloc: %lld elements need %lld reduction blocks, "
               "the fixed scratch holds %lld (at most %lld leaves in 3D, %lld in 2D)",
@@ -105,9 +80,7 @@ extern "C" chns_status chns_energy_mass_noalloc(const chns_mesh *m, const chns_p
   if (s != CHNS_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   PhysCoef pc = make_coef(*p, m->lo, m->hi);
-  launch_energy(m, pc, U, scratch, st);
-  k_sum3<<<1, kSumThreads, 0, st>>>(nb, out3);
-  note_launches(1);
+  launch_energy(m, pc, U, scratch, out3, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error("kernel launch failed: %s", cudaGetErrorString(e)); return CHNS_ERR_CUDA; }
   return CHNS_OK;
