@@ -177,9 +177,11 @@ chns_status chns_mesh_check(const chns_mesh *mesh);
  * chns_solver_opts.autotune): variant in [0, 7) fixes it (and marks the mesh
  * tuned); times_ms (host, nullable, 7 entries) receives the autotuner's
  * median time per schedule, negative where none was measured.  Schedules:
- * 0-3, 5, 6 element-local buffer + node gather with (block size, blocks per
- * SM) = (128, 6), (256, 3), (64, 12), (128, 8), -, (128, 5), (128, 4); 4
- * element colours with in-place adds.  variant = -1 only reads. */
+ * 0-3 element-local buffer + node gather, two Gauss points per lane, with
+ * (block size, blocks per SM) = (64, 7), (128, 3), (64, 6), (128, 4) (as 5 on a
+ * batch's union mesh); 5, 6 the same with one Gauss point per lane, (128, 5)
+ * and (128, 6); 4 element colours with in-place adds.  variant = -1 only
+ * reads. */
 chns_status chns_mesh_jacvec_schedule(chns_mesh *mesh, int variant, int *current, double *times_ms);
 
 void chns_mesh_destroy(chns_mesh *mesh);

@@ -15,6 +15,7 @@
 // numbers (value, derivative along w).
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 
 #include "chns_internal.h"
 #include "kernels.h"
@@ -25,16 +26,49 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// ---------------------------------------------------------------- packed pairs
+// Two floats in a register pair: one packed instruction (sm_100 and later)
+// does what two scalar ones do in one issue slot.
+struct F2 {
+  unsigned long long v;
+  F2() = default;
+  __device__ __forceinline__ explicit F2(float a) : F2(a, a) {}
+  __device__ __forceinline__ F2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+  __device__ __forceinline__ float lo() const { return __uint_as_float(unsigned(v)); }
+  __device__ __forceinline__ float hi() const { return __uint_as_float(unsigned(v >> 32)); }
+};
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 &operator*=(F2 &a, F2 b) { return a = a * b; }
+
 // ---------------------------------------------------------------- dual numbers
-// mad(a, b, c) = a b + c, one rounding per scalar fma
+// mad(a, b, c) = a b + c, one rounding per fma
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
 
 template <typename T>
 struct Dl {
   T v, d;
   __device__ __forceinline__ Dl() {}
-  __device__ __forceinline__ Dl(T a) : v(a), d(T(0)) {}
+  __device__ __forceinline__ explicit Dl(T a) : v(a), d(T(0.0f)) {}
   __device__ __forceinline__ Dl(T a, T b) : v(a), d(b) {}
 };
 template <typename T> __device__ __forceinline__ Dl<T> operator+(Dl<T> a, Dl<T> b) { return Dl<T>(a.v + b.v, a.d + b.d); }
@@ -52,26 +86,45 @@ template <typename T> __device__ __forceinline__ Dl<T> madc(Dl<T> a, T b, T c) {
 template <typename T> __device__ __forceinline__ Dl<T> madc(Dl<T> a, Dl<T> b, T c) {
   return Dl<T>(mad(a.v, b.v, c), mad(a.d, b.v, a.v * b.d));
 }
-__device__ __forceinline__ float madc(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double madc(double a, double b, double c) { return fma(a, b, c); }
+template <typename T> __device__ __forceinline__ T madc(T a, T b, T c) { return mad(a, b, c); }
 template <typename T> __device__ __forceinline__ Dl<T> subc(Dl<T> a, T b) { return Dl<T>(a.v - b, a.d); }
 template <typename T> __device__ __forceinline__ T subc(T a, T b) { return a - b; }
 template <typename T> __device__ __forceinline__ T val(Dl<T> a) { return a.v; }
 __device__ __forceinline__ float val(float a) { return a; }
 __device__ __forceinline__ double val(double a) { return a; }
 
-__device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
-__device__ __forceinline__ float rcp_(float x) { return 1.0f / x; }
-__device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
-template <typename T> __device__ __forceinline__ Dl<T> rcp_(Dl<T> a) {
-  T r = rcp_(a.v);
-  return Dl<T>(r, -a.d * r * r);
+// conditions: one per number, two per pair
+struct B2 { bool lo, hi; };
+template <typename T> struct Cond { using type = bool; };
+template <> struct Cond<F2> { using type = B2; };
+template <typename T> __device__ __forceinline__ bool abs_le1(T x) { return fabs(x) <= T(1); }
+__device__ __forceinline__ B2 abs_le1(F2 x) { return {fabsf(x.lo()) <= 1.0f, fabsf(x.hi()) <= 1.0f}; }
+template <typename T> __device__ __forceinline__ bool less(T a, T b) { return a < b; }
+__device__ __forceinline__ B2 less(F2 a, F2 b) { return {a.lo() < b.lo(), a.hi() < b.hi()}; }
+template <typename T> __device__ __forceinline__ T sign1(T x) { return x > T(0) ? T(1) : T(-1); }
+__device__ __forceinline__ F2 sign1(F2 x) { return F2(sign1(x.lo()), sign1(x.hi())); }
+__device__ __forceinline__ float sel(bool c, float a, float b) { return c ? a : b; }
+__device__ __forceinline__ double sel(bool c, double a, double b) { return c ? a : b; }
+__device__ __forceinline__ F2 sel(B2 c, F2 a, F2 b) { return F2(c.lo ? a.lo() : b.lo(), c.hi ? a.hi() : b.hi()); }
+template <typename C, typename T> __device__ __forceinline__ Dl<T> sel(C c, Dl<T> a, Dl<T> b) {
+  return Dl<T>(sel(c, a.v, b.v), sel(c, a.d, b.d));
 }
-// rad^(-1/2) and its derivative -1/2 rad^(-3/2) rad'
-template <typename T> __device__ __forceinline__ Dl<T> rsqrt_(Dl<T> a) {
-  T r = rsqrt_(a.v);
-  return Dl<T>(r, T(-0.5) * a.d * r * r * r);
+
+// -1/x and -x^(-1/2) (negated: the weak form below then needs no negation of a pair)
+__device__ __forceinline__ float nrcp_(float x) { return -(1.0f / x); }
+__device__ __forceinline__ double nrcp_(double x) { return -(1.0 / x); }
+__device__ __forceinline__ F2 nrcp_(F2 x) { return F2(nrcp_(x.lo()), nrcp_(x.hi())); }
+template <typename T> __device__ __forceinline__ Dl<T> nrcp_(Dl<T> a) {
+  const T r = nrcp_(a.v);
+  return Dl<T>(r, a.d * (r * r));
+}
+__device__ __forceinline__ float nrsqrt_(float x) { return -rsqrtf(x); }
+__device__ __forceinline__ double nrsqrt_(double x) { return -rsqrt(x); }
+__device__ __forceinline__ F2 nrsqrt_(F2 x) { return F2(nrsqrt_(x.lo()), nrsqrt_(x.hi())); }
+// derivative 1/2 x^(-3/2) x' = -1/2 r^3 x' with r = -x^(-1/2)
+template <typename T> __device__ __forceinline__ Dl<T> nrsqrt_(Dl<T> a) {
+  const T r = nrsqrt_(a.v);
+  return Dl<T>(r, (a.d * T(-0.5f)) * (r * r) * r);
 }
 
 // x 2^k, exact.  In double on the exponent bits: the FP64 pipe issues one
@@ -327,16 +380,20 @@ struct GpIn {
 };
 
 // Everything that depends only on the parameters and the box is folded on the
-// host; what depends on the leaf is a power of two of its level.
+// host; what depends on the leaf is a power of two of its level.  Some are
+// kept negated (n...): a pair has no negation for free.
 template <typename T>
-struct KCoef {
+struct KPhys {
   T inv_dt, four_dt2, alpha, beta;
-  T gRe, xRe;              // eta / Re = gRe phi* + xRe
+  T ngRe, gRe, xRe;        // eta / Re = gRe phi* + xRe
   T jcP;                   // J / Pe = jcP grad mu
-  T inv_We, CnWe, inv_PeCn, Cn2;
-  T gFr[3];                // gravity / Fr
+  T inv_We, ninv_We, CnWe, nCnWe, inv_PeCn, Cn2;
+  T ngFr[3];               // - gravity / Fr
+};
+template <typename T>
+struct KCoef : KPhys<T> {
   // geometry of a leaf of level 0; a leaf of level l has these times a power of 2^l
-  T G0[3];                 // G = 4 / ext^2
+  T nG0[3];                // - G = - 4 / ext^2
   T CIGG0, inv_trG0;       // C_I G:G and 1 / tr G
   T sg0[3], sh0[3], cS0, cV0[3];  // Stage without the signs
   T W0;                    // prod ext / 2
@@ -369,44 +426,47 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 // after: residual of the level-6 octree (262,144 leaves) 2.34 -> 1.41 ms, FP64
 // J.w of 77,932 adaptive leaves 1.27 -> 0.79 ms, FP32 J.w of the level-6 octree
 // 132 -> 116 us (element kernel alone 88 -> 69 us).
-template <int D, bool HASF, typename T, typename S>
-__device__ __forceinline__ void gp_physics(const KCoef<T> &c, const T *G, T CI_GG, T inv_trG, T CnWeH,
-                                           const GpIn<D, S> &q, const T *f, S *Sq, S (*Vq)[D], bool &floored) {
+//
+// nG, CI_GG, inv_trG, CnWeH come per leaf; T is the number type (a pair: two
+// Gauss points), S is T or its dual.
+template <int D, bool HASF, typename T, typename S, typename C>
+__device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T inv_trG, T CnWeH,
+                                           const GpIn<D, S> &q, const T *f, S *Sq, S (*Vq)[D],
+                                           typename Cond<T>::type &floored) {
   // phi* clip (Eq. phi_for_density) and mixture properties at t_{k+1}
   const T pn = val(q.phin);
-  const bool inside = fabs(pn) <= T(1);
-  const S phis = inside ? q.phin : S(pn > T(0) ? T(1) : T(-1));
+  const auto inside = abs_le1(pn);
+  const S phis = sel(inside, q.phin, S(sign1(pn)));
   const S rho = madc(phis, c.alpha, c.beta);
   const S etaRe = madc(phis, c.gRe, c.xRe);
-  const S inv_rho = rcp_(rho);
+  const S ninv_rho = nrcp_(rho);
   S cm[D], cR[D];  // c_j and c_j - d_j eta / Re
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     cm[j] = mad(rho, q.vt[j], q.dmut[j] * c.jcP);
-    const S de = inside ? q.dphin[j] * c.gRe : S(T(0));
-    cR[j] = cm[j] - de;
+    cR[j] = cm[j] + sel(inside, q.dphin[j] * c.ngRe, S(T(0.0f)));
   }
   // tau_m, tau_c with G = diag(4/h^2); radicand floored at 4/dt^2
-  S vGc = (q.vt[0] * cm[0]) * G[0];
+  S nvGc = (q.vt[0] * cm[0]) * nG[0];
 #pragma unroll
-  for (int i = 1; i < D; ++i) vGc = mad(q.vt[i] * cm[i], G[i], vGc);
-  const S visc = etaRe * inv_rho;
-  S rad = mad(inv_rho, vGc, madc(visc * visc, CI_GG, c.four_dt2));
-  floored = val(rad) < c.four_dt2;
-  if (floored) rad = S(c.four_dt2);
-  const S tau = rsqrt_(rad);
+  for (int i = 1; i < D; ++i) nvGc = mad(q.vt[i] * cm[i], nG[i], nvGc);
+  const S nvisc = etaRe * ninv_rho;
+  S rad = mad(ninv_rho, nvGc, madc(nvisc * nvisc, CI_GG, c.four_dt2));
+  floored = less(val(rad), c.four_dt2);
+  rad = sel(floored, S(c.four_dt2), rad);
+  const S ntau = nrsqrt_(rad);
   // strong residuals
-  S A[D], t[D];
+  S A[D], nt[D];  // nt = - tau_m R_m
   S divv = q.dvt[0][0];
 #pragma unroll
   for (int i = 1; i < D; ++i) divv = divv + q.dvt[i][i];
   if (HASF) divv = subc(divv, f[D]);  // R_c
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    A[i] = rho * madc(q.dv[i], c.inv_dt, -c.gFr[i]);
+    A[i] = rho * madc(q.dv[i], c.inv_dt, c.ngFr[i]);
     if (HASF) A[i] = subc(A[i], f[i]);
     S R = mad(q.dpt[i], c.inv_We, A[i]);
-    S cap = D == 2 ? q.hphit[0] * q.dphit[1 - i] : S(T(0));
+    S cap = D == 2 ? q.hphit[0] * q.dphit[1 - i] : S(T(0.0f));
     if (D == 3) {
       const int j0 = i == 0 ? 1 : 0, j1 = i == 2 ? 1 : 2;
       cap = mad(q.hphit[hidx<D>(i, j0)], q.dphit[j0], q.hphit[hidx<D>(i, j1)] * q.dphit[j1 < D ? j1 : 0]);
@@ -414,23 +474,23 @@ __device__ __forceinline__ void gp_physics(const KCoef<T> &c, const T *G, T CI_G
     R = mad(cap, CnWeH, R);
 #pragma unroll
     for (int j = 0; j < D; ++j) R = mad(q.dvt[i][j], cR[j], R);
-    t[i] = tau * R;
+    nt[i] = ntau * R;
   }
   // momentum rows
-  const S tau_c = (rad * tau) * inv_trG;
-  const S diag = (rho * tau_c * divv - q.pt) * c.inv_We;
+  const S ntau_c = (rad * ntau) * inv_trG;
+  const S diag = mad(rho * ntau_c, divv, q.pt) * c.ninv_We;
 #pragma unroll
-  for (int j = 0; j < D; ++j) cm[j] = cm[j] - t[j];
+  for (int j = 0; j < D; ++j) cm[j] = cm[j] + nt[j];
   S cphi[D];
 #pragma unroll
-  for (int i = 0; i < D; ++i) cphi[i] = q.dphit[i] * (-c.CnWe);
+  for (int i = 0; i < D; ++i) cphi[i] = q.dphit[i] * c.nCnWe;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     S Si = A[i];
 #pragma unroll
     for (int j = 0; j < D; ++j) Si = mad(q.dvt[i][j], cm[j], Si);
     Sq[i] = Si;
-    Vq[D][i] = t[i] * inv_rho;  // PSPG; tau_m R_m / rho
+    Vq[D][i] = nt[i] * ninv_rho;  // PSPG; tau_m R_m / rho
   }
 #pragma unroll
   for (int i = 0; i < D; ++i)
@@ -445,10 +505,11 @@ __device__ __forceinline__ void gp_physics(const KCoef<T> &c, const T *G, T CI_G
   Sq[D] = divv;
   // Cahn-Hilliard row
   Sq[D + 1] = q.dphi * c.inv_dt;
+  const S nphi = q.phit * T(-1.0f);
 #pragma unroll
-  for (int i = 0; i < D; ++i) Vq[D + 1][i] = q.dmut[i] * c.inv_PeCn - q.vt[i] * q.phit;
+  for (int i = 0; i < D; ++i) Vq[D + 1][i] = mad(q.vt[i], nphi, q.dmut[i] * c.inv_PeCn);
   // chemical-potential row, psi'(phi~) = phi~^3 - phi~
-  Sq[D + 2] = q.phit * madc(q.phit, q.phit, T(-1)) - q.mut;
+  Sq[D + 2] = q.phit * madc(q.phit, q.phit, T(-1.0f)) - q.mut;
 #pragma unroll
   for (int i = 0; i < D; ++i) Vq[D + 2][i] = q.dphit[i] * c.Cn2;
   if (HASF) {
@@ -477,14 +538,15 @@ KCoef<T> kcoef(const PhysCoef &p, int dim) {
   KCoef<T> c;
   c.inv_dt = T(p.inv_dt); c.four_dt2 = T(p.four_dt2);
   c.alpha = T(p.alpha); c.beta = T(p.beta);
-  c.gRe = T(p.gamma * p.inv_Re); c.xRe = T(p.xi * p.inv_Re);
+  c.gRe = T(p.gamma * p.inv_Re); c.ngRe = -c.gRe; c.xRe = T(p.xi * p.inv_Re);
   c.jcP = T(p.jc * p.inv_Pe);
-  c.inv_We = T(p.inv_We); c.CnWe = T(p.CnWe); c.inv_PeCn = T(p.inv_PeCn); c.Cn2 = T(p.Cn2);
+  c.inv_We = T(p.inv_We); c.ninv_We = -c.inv_We; c.CnWe = T(p.CnWe); c.nCnWe = -c.CnWe;
+  c.inv_PeCn = T(p.inv_PeCn); c.Cn2 = T(p.Cn2);
   double trG = 0.0, GG = 0.0, W = 1.0;
   for (int a = 0; a < 3; ++a) {
-    c.gFr[a] = T(p.g[a] * p.inv_Fr);
+    c.ngFr[a] = T(-p.g[a] * p.inv_Fr);
     const double G = 4.0 / (p.ext[a] * p.ext[a]);
-    c.G0[a] = T(G);
+    c.nG0[a] = T(-G);
     if (a < dim) {
       trG += G;
       GG += G * G;
@@ -558,7 +620,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   // geometry of this leaf
   const int l = level[e];
   Stage<D, T> s;
-  T G[D];
+  T nG[D];
   s.v = T((RAW ? 0.5 : 1.0) * CAD<D>);
   s.cS = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
 #pragma unroll
@@ -567,7 +629,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     s.sg[a] = flip_if(scale2(c.sg0[a], l - (RAW ? 1 : 0)), neg);
     s.sh[a] = UNIT ? flip_if(scale2(c.sh0[a], l), neg) : T(0);
     s.cV[a] = flip_if(scale2(c.cV0[a], (1 - D) * l - (RAW ? 0 : 1)), neg);
-    G[a] = scale2(c.G0[a], 2 * l);
+    nG[a] = scale2(c.nG0[a], 2 * l);
   }
   const T CI_GG = scale2(c.CIGG0, 4 * l), inv_trG = scale2(c.inv_trG0, -2 * l);
   // d_a d_b = sg_a sg_b / CA^D (half of it with the halved factors)
@@ -608,7 +670,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     q.dphi = T(2) * dphiq;
     q.phin = A.phit + dphiq;
     T Sq[NF], Vq[NF][D];
-    gp_physics<D, HASF, T, T>(c, G, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    gp_physics<D, HASF, T, T>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
     if constexpr (MODE == 2) {
       const unsigned b = __ballot_sync(FULL, floored && active);
       if ((threadIdx.x & 31) == 0 && b) atomicAdd(reinterpret_cast<unsigned long long *>(out), (unsigned long long)__popc(b));
@@ -642,7 +704,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     q.dphi = Dl<T>(dphiq, two * B.phit);
     q.phin = Dl<T>(mad(hf, dphiq, A.phit), two * B.phit);
     Dl<T> Sq[NF], Vq[NF][D];
-    gp_physics<D, HASF, T, Dl<T>>(c, G, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    gp_physics<D, HASF, T, Dl<T>>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
       T Vk[D];
@@ -668,6 +730,217 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     } else if (active) {
       scatter<NF>(cn, hang, out, r);
     }
+  }
+}
+
+// ---------------------------------------------------------------- J.w in float, two Gauss points a lane
+// As k_element MODE 1, with 2^(D-1) lanes per leaf: lane c holds the corners c
+// and c + 2^(D-1) (the last axis' bit) and the two Gauss points of that pair.
+// All arithmetic of the pair is packed, the last axis' stage stays in the lane.
+// Bound by issue slots with one point a lane (896 instructions per Gauss point:
+// 586 of arithmetic, 125 shuffles): packing halves the arithmetic's slots, the
+// in-lane axis half of the shuffles.  One apply, before -> after: level-6 octree
+// 117 -> 98 us, 1,375,648 adaptive leaves 631 -> 585 us.
+template <int D>
+struct Stage2 {
+  F2 sg[D - 1];  // derivative factors of the lane axes, both halves
+  F2 sh[D - 1];  // the same for UNIT data
+  float sgl, shl;  // last axis: + for both halves (own - other, signed)
+  F2 cS, cV[D - 1];
+  float cVl;
+};
+
+__device__ __forceinline__ F2 shfl2(F2 x, int m) {
+  return F2(__shfl_xor_sync(FULL, x.lo(), m), __shfl_xor_sync(FULL, x.hi(), m));
+}
+template <bool UNIT>
+__device__ __forceinline__ F2 st_mix2(F2 u, F2 o) {
+  constexpr float ca = 0.5f + 0.28867513459481288225f, cb = 0.5f - 0.28867513459481288225f;
+  if (UNIT) return mad(F2(ca), u, F2(cb) * o);
+  return mad(F2(float(TB)), o, u);
+}
+template <bool UNIT>
+__device__ __forceinline__ void st_vd2(F2 u, int m, F2 &v, F2 &d) {
+  const F2 o = shfl2(u, m);
+  v = st_mix2<UNIT>(u, o);
+  d = u - o;
+}
+template <bool UNIT>
+__device__ __forceinline__ F2 st_v2(F2 u, int m) { return st_mix2<UNIT>(u, shfl2(u, m)); }
+// the last axis, within the pair
+template <bool UNIT>
+__device__ __forceinline__ F2 in_v(F2 u) {
+  return F2(st_mix<UNIT>(u.lo(), u.hi()), st_mix<UNIT>(u.hi(), u.lo()));
+}
+__device__ __forceinline__ F2 in_d(F2 u, float f) { return F2((u.hi() - u.lo()) * f); }
+
+template <int D>
+__device__ __forceinline__ F2 ip_v2(F2 u) {
+  F2 a = st_v2<false>(u, 1);
+  if (D == 3) a = st_v2<false>(a, 2);
+  return in_v<false>(a) * F2(float(CAD<D>));
+}
+
+template <int D, bool UNIT = false>
+__device__ __forceinline__ void ip_vg2(F2 u, const Stage2<D> &s, F2 &v, F2 *g) {
+  const F2 *f = UNIT ? s.sh : s.sg;
+  const float fl = UNIT ? s.shl : s.sgl;
+  F2 A, Bx;
+  st_vd2<UNIT>(u, 1, A, Bx);
+  if (D == 2) {
+    v = in_v<UNIT>(A);
+    g[D - 1] = in_d(A, fl);
+    g[0] = in_v<UNIT>(Bx) * f[0];
+  } else {
+    F2 AA, AB;
+    st_vd2<UNIT>(A, 2, AA, AB);
+    const F2 BA = st_v2<UNIT>(Bx, 2);
+    v = in_v<UNIT>(AA);
+    g[D - 1] = in_d(AA, fl);
+    g[1] = in_v<UNIT>(AB) * f[D - 2];
+    g[0] = in_v<UNIT>(BA) * f[0];
+  }
+  if (!UNIT) v *= F2(float(CAD<D>));
+}
+
+template <int D, bool UNIT = false>
+__device__ __forceinline__ void ip_full2(F2 u, const Stage2<D> &s, F2 &v, F2 *g, F2 *hs) {
+  const F2 *f = UNIT ? s.sh : s.sg;
+  const float fl = UNIT ? s.shl : s.sgl;
+  F2 A, Bx;
+  st_vd2<UNIT>(u, 1, A, Bx);
+  if (D == 2) {
+    v = in_v<UNIT>(A);
+    g[D - 1] = in_d(A, fl);
+    g[0] = in_v<UNIT>(Bx) * f[0];
+    hs[0] = in_d(Bx, fl) * f[0];
+  } else {
+    F2 AA, AB, BA, BB;
+    st_vd2<UNIT>(A, 2, AA, AB);
+    st_vd2<UNIT>(Bx, 2, BA, BB);
+    v = in_v<UNIT>(AA);
+    g[D - 1] = in_d(AA, fl);
+    g[1] = in_v<UNIT>(AB) * f[D - 2];
+    hs[2] = in_d(AB, fl) * f[D - 2];
+    g[0] = in_v<UNIT>(BA) * f[0];
+    hs[1] = in_d(BA, fl) * f[0];
+    hs[0] = in_v<UNIT>(BB) * (f[0] * f[D - 2]);
+  }
+  if (!UNIT) v *= F2(float(CAD<D>));
+}
+
+template <int D>
+__device__ __forceinline__ F2 contract2(F2 S, const F2 *V, const Stage2<D> &s) {
+  const F2 tb{float(TB)}, ntb{float(-TB)};
+  S *= s.cS;
+  const float t = (V[D - 1].lo() + V[D - 1].hi()) * s.cVl;
+  F2 X(fmaf(float(TB), S.hi(), S.lo()) - t, fmaf(float(TB), S.lo(), S.hi()) + t);
+  F2 Y0 = in_v<false>(V[0] * s.cV[0]);
+  if (D == 3) {
+    const F2 Y1 = in_v<false>(V[1] * s.cV[D - 2]);
+    X = (X + Y1) - shfl2(mad(ntb, X, Y1), 2);
+    Y0 = mad(tb, shfl2(Y0, 2), Y0);
+  }
+  return (X + Y0) - shfl2(mad(ntb, X, Y0), 1);
+}
+
+template <int D>
+__device__ __forceinline__ void interp_state2(const F2 *u, const Stage2<D> &s, Interp<D, F2> &I) {
+#pragma unroll
+  for (int i = 0; i < D; ++i) ip_vg2<D>(u[i], s, I.vt[i], I.dvt[i]);
+  ip_vg2<D>(u[D], s, I.pt, I.dpt);
+  ip_full2<D, true>(u[D + 1], s, I.phit, I.dphit, I.hphit);
+  ip_vg2<D>(u[D + 2], s, I.mut, I.dmut);
+}
+
+template <int N>
+__device__ __forceinline__ void gather_pair(int c0, int c1, const int32_t *__restrict__ hang,
+                                            const float *__restrict__ src, F2 *out) {
+  float a[N], b[N];
+  gather<N>(c0, hang, src, a);
+  gather<N>(c1, hang, src, b);
+#pragma unroll
+  for (int k = 0; k < N; ++k) out[k] = F2(a[k], b[k]);
+}
+
+template <int D, int BS, int MINB>
+__global__ void __launch_bounds__(BS, MINB) k_jv_pair(
+    const int32_t *__restrict__ conn, const uint8_t *__restrict__ level, const int32_t *__restrict__ hang,
+    int64_t n_elem, const float *__restrict__ ut, const float *__restrict__ dl, const float *__restrict__ w,
+    float *__restrict__ out, const __grid_constant__ KCoef<float> c, const __grid_constant__ KPhys<F2> cp,
+    int64_t wstride, int64_t ostride) {
+  constexpr int NL = 1 << (D - 1), NC = 2 * NL, NF = D + 3, ND = D + 1;
+  w += blockIdx.y * wstride;
+  out += blockIdx.y * ostride;
+  const int lc = threadIdx.x & (NL - 1);
+  int64_t e = (int64_t(blockIdx.x) * BS + threadIdx.x) >> (D - 1);
+  const bool active = e < n_elem;
+  if (!active) e = n_elem - 1;
+  const int c0 = conn[e * NC + lc], c1 = conn[e * NC + lc + NL], l = level[e];
+  F2 u[NF], d[ND], wn[NF];
+  gather_pair<NF>(c0, c1, hang, ut, u);
+  gather_pair<ND>(c0, c1, hang, dl, d);
+  gather_pair<NF>(c0, c1, hang, w, wn);
+
+  Stage2<D> s;
+  F2 nG[D];
+#pragma unroll
+  for (int a = 0; a < D - 1; ++a) {
+    const bool neg = !((lc >> a) & 1);
+    s.sg[a] = F2(flip_if(scale2(c.sg0[a], l), neg));
+    s.sh[a] = F2(flip_if(scale2(c.sh0[a], l), neg));
+    s.cV[a] = F2(flip_if(scale2(c.cV0[a], (1 - D) * l - 1), neg));
+  }
+  s.sgl = scale2(c.sg0[D - 1], l);
+  s.shl = scale2(c.sh0[D - 1], l);
+  s.cVl = scale2(c.cV0[D - 1], (1 - D) * l - 1);
+  s.cS = F2(scale2(c.cS0, -D * l - 1));
+#pragma unroll
+  for (int a = 0; a < D; ++a) nG[a] = F2(scale2(c.nG0[a], 2 * l));
+  const F2 CI_GG(scale2(c.CIGG0, 4 * l)), inv_trG(scale2(c.inv_trG0, -2 * l));
+
+  Interp<D, F2> A, B;
+  interp_state2<D>(u, s, A);
+  interp_state2<D>(wn, s, B);
+  F2 dphi, dphig[D];
+  ip_vg2<D, true>(d[D], s, dphi, dphig);
+  GpIn<D, Dl<F2>> q;
+  const F2 two(2.0f), hf(0.5f);
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    q.vt[i] = Dl<F2>(A.vt[i], B.vt[i]);
+    q.dv[i] = Dl<F2>(ip_v2<D>(d[i]), two * B.vt[i]);
+    q.dpt[i] = Dl<F2>(A.dpt[i], B.dpt[i]);
+    q.dphit[i] = Dl<F2>(A.dphit[i], B.dphit[i]);
+    q.dmut[i] = Dl<F2>(A.dmut[i], B.dmut[i]);
+    q.dphin[i] = Dl<F2>(mad(hf, dphig[i], A.dphit[i]), two * B.dphit[i]);
+#pragma unroll
+    for (int j = 0; j < D; ++j) q.dvt[i][j] = Dl<F2>(A.dvt[i][j], B.dvt[i][j]);
+  }
+#pragma unroll
+  for (int k = 0; k < (D == 3 ? 3 : 1); ++k) q.hphit[k] = Dl<F2>(A.hphit[k], B.hphit[k]);
+  q.pt = Dl<F2>(A.pt, B.pt);
+  q.phit = Dl<F2>(A.phit, B.phit);
+  q.mut = Dl<F2>(A.mut, B.mut);
+  q.dphi = Dl<F2>(dphi, two * B.phit);
+  q.phin = Dl<F2>(mad(hf, dphi, A.phit), two * B.phit);
+  Dl<F2> Sq[NF], Vq[NF][D];
+  B2 floored;
+  gp_physics<D, false, F2, Dl<F2>>(cp, nG, CI_GG, inv_trG, cp.CnWe, q, static_cast<const F2 *>(nullptr), Sq, Vq,
+                                   floored);
+  float r0[NF], r1[NF];
+#pragma unroll
+  for (int k = 0; k < NF; ++k) {
+    F2 Vk[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) Vk[j] = Vq[k][j].d;
+    const F2 r = contract2<D>(Sq[k].d, Vk, s);
+    r0[k] = r.lo();
+    r1[k] = r.hi();
+  }
+  if (active) {
+    store_block<NF>(out + (e * NC + lc) * NF, r0);
+    store_block<NF>(out + (e * NC + lc + NL) * NF, r1);
   }
 }
 
@@ -1004,18 +1277,19 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 }
 
 // J.w schedules (chosen per mesh by the autotuner, FP32 only; FP64 always
-// uses schedule 0):
-//   0: all elements at once into the element-local buffer E (n_elem * 2^dim
-//      * nf values of T), 128-thread blocks, 6 per SM; then the node gather
-//      with the constrained rows (no colouring, no output zeroing)
-//   1: as 0 with 256-thread blocks, 3 per SM
-//   2: as 0 with 64-thread blocks, 12 per SM
-//   3: as 0 with 128-thread blocks, 8 per SM (at most 64 registers)
+// uses the element-local buffer with 128-thread blocks, 3 per SM):
+//   0-3: two Gauss points per lane (k_jv_pair), all elements at once into the
+//      element-local buffer E (n_elem * 2^dim * nf values), then the node
+//      gather with the constrained rows; (threads, blocks per SM) = (64, 7),
+//      (128, 3), (64, 6), (128, 4).  0 is the default: 14 warps an SM hide the
+//      scattered loads of an adaptive mesh better than 12 (585 against 661 us
+//      on 1,375,648 leaves) and cost 4 % on a uniform one (97.7 against 93.8)
 //   4: element colours one launch after another, each element adding its
 //      contributions into y (disjoint nodes within a colour; no E buffer),
 //      then the constrained rows
-//   5: as 0 with 128-thread blocks, 5 per SM (up to 102 registers)
-//   6: as 0 with 128-thread blocks, 4 per SM (up to 128 registers)
+//   5, 6: as 0 with one Gauss point per lane, 128 threads, 5 and 6 per SM; 5 is
+//      what a batch's union mesh uses (each element has its own coefficients,
+//      which as pairs would take twice the registers)
 template <int D, typename T, int BS, int MINB>
 static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
                          const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
@@ -1026,6 +1300,35 @@ static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *
                                                             nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, es);
   k_gather_nodes<D, T, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
                                                      es);
+  note_launches(2);
+}
+
+static F2 host_pair(float a) {
+  uint32_t b;
+  std::memcpy(&b, &a, 4);
+  F2 p;
+  p.v = (uint64_t(b) << 32) | b;
+  return p;
+}
+static KPhys<F2> pair_coef(const KPhys<float> &c) {
+  KPhys<F2> p;
+  static_assert(sizeof(KPhys<F2>) == 2 * sizeof(KPhys<float>), "plain arrays of constants");
+  const float *x = reinterpret_cast<const float *>(&c);
+  F2 *y = reinterpret_cast<F2 *>(&p);
+  for (size_t k = 0; k < sizeof(KPhys<float>) / 4; ++k) y[k] = host_pair(x[k]);
+  return p;
+}
+
+template <int D, int BS, int MINB>
+static void jv_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut, const float *dl, const float *w,
+                    float *E, float *y, uint32_t fmask, cudaStream_t st, int nv) {
+  constexpr int NF = D + 3;
+  const int64_t threads = m->n_elem << (D - 1), es = (m->n_elem << D) * NF;
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_nodes(m->n_nodes), (unsigned)nv);
+  k_jv_pair<D, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
+                                            m->n_nodes * NF, es);
+  k_gather_nodes<D, float, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y,
+                                                         fmask, es);
   note_launches(2);
 }
 
@@ -1049,14 +1352,17 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
                         const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
   if (nv > 1 && variant == 4) variant = 0;  // the colour schedule takes one direction at a time
   if constexpr (sizeof(T) == 4) {
+    if (!tab) switch (variant) {
+        case 0: jv_pair<D, 64, 7>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
+        case 1: jv_pair<D, 128, 3>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
+        case 2: jv_pair<D, 64, 6>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
+        case 3: jv_pair<D, 128, 4>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
+        default: break;
+      }
     switch (variant) {
-      case 1: jv_elemlocal<D, T, 256, 3>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
-      case 2: jv_elemlocal<D, T, 64, 12>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
-      case 3: jv_elemlocal<D, T, 128, 8>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
       case 4: jv_colours<D, T>(m, c, tab, ut, dl, w, y, fmask, st); return;
-      case 5: jv_elemlocal<D, T, 128, 5>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
-      case 6: jv_elemlocal<D, T, 128, 4>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
-      default: break;
+      case 6: jv_elemlocal<D, T, 128, 6>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
+      default: break;  // 5, and the pair schedules on a batch's union mesh
     }
   }
   if constexpr (sizeof(T) == 8) {
@@ -1064,7 +1370,7 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
     // the register spills a 6-blocks-per-SM budget causes
     jv_elemlocal<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
   } else {
-    jv_elemlocal<D, T, 128, 6>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
+    jv_elemlocal<D, T, 128, 5>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
   }
 }
 
