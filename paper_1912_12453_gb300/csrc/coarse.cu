@@ -451,9 +451,11 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
 #pragma unroll
     for (int c = 0; c < NB; ++c) a[i][c] = r < n && c < nb ? M[int64_t(r) * n + k0 + c] : T(0);
   }
-#pragma unroll
-  for (int kk = 0; kk < NB; ++kk) {
-    if (kk >= nb) break;
+  // The loop stays rolled (unrolled it is 80 KB of code that runs once): the
+  // current column is always a[.][0], each step writes its results one place
+  // down and the finished column to the end.
+#pragma unroll 1
+  for (int kk = 0; kk < nb; ++kk) {
     const int k = k0 + kk, sl = kk & 1;
     // row of the largest |a_rk|, r >= k, the lowest of equals
     uint64_t best = 0;
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       const int r = threadIdx.x + i * blockDim.x;
-      const uint64_t v = abs_key(a[i][kk]);
+      const uint64_t v = abs_key(a[i][0]);
       if (r >= k && r < n && (v > best || (v == best && r < arg))) { best = v; arg = r; }
     }
     warp_arg_max(best, arg);
@@ -478,9 +480,9 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
 #pragma unroll
         for (int c = 0; c < NB; ++c) prow[sl][c] = a[i][c];
         psrc[sl] = src[i];
-        const bool ok = fabs(a[i][kk]) > T(0);  // false for NaN too
+        const bool ok = fabs(a[i][0]) > T(0);  // false for NaN too
         if (!ok) *bad = 1;
-        dinv[sl] = ok ? T(1) / a[i][kk] : T(0);
+        dinv[sl] = ok ? T(1) / a[i][0] : T(0);
       }
       if (r == k) {
 #pragma unroll
@@ -498,23 +500,23 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
         for (int c = 0; c < NB; ++c) a[i][c] = krow[sl][c];
         src[i] = ksrc[sl];
       }
-      if (r == k) {
+      // row k: prow d; the others: a - (a_k d) prow
+      const bool piv = r == k;
+      if (piv) src[i] = psrc[sl];
+      const T fr = piv ? d : -a[i][0] * d;
 #pragma unroll
-        for (int c = 0; c < NB; ++c) a[i][c] = c == kk ? d : prow[sl][c] * d;
-        src[i] = psrc[sl];
-      } else {
-        const T fr = -a[i][kk] * d;
-#pragma unroll
-        for (int c = 0; c < NB; ++c) a[i][c] = c == kk ? fr : fma(fr, prow[sl][c], a[i][c]);
-      }
+      for (int c = 1; c < NB; ++c) a[i][c - 1] = fma(fr, prow[sl][c], piv ? T(0) : a[i][c]);
+      a[i][NB - 1] = fr;
     }
   }
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     const int r = threadIdx.x + i * blockDim.x;
     if (r >= n) continue;
+    // a narrow last panel: its nb columns have moved to the end
 #pragma unroll
-    for (int c = 0; c < NB; ++c) G[int64_t(r) * NB + c] = a[i][c];
+    for (int c = 0; c < NB; ++c)
+      if (c >= NB - nb) G[int64_t(r) * NB + c - (NB - nb)] = a[i][c];
     const int64_t o = int64_t(blockIdx.x) * n;
     permall[o + r] = src[i];
     origin_out[o + r] = origin_in[o + src[i]];
