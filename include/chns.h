@@ -178,7 +178,7 @@ chns_status chns_mesh_check(const chns_mesh *mesh);
  * tuned); times_ms (host, nullable, 7 entries) receives the autotuner's
  * median time per schedule, negative where none was measured.  Schedules:
  * 0-3 element-local buffer + node gather, two Gauss points per lane, with
- * (block size, blocks per SM) = (64, 7), (128, 3), (64, 6), (128, 4) (as 5 on a
+ * (block size, blocks per SM) = (64, 8), (128, 3), (64, 6), (128, 4) (as 5 on a
  * batch's union mesh); 5, 6 the same with one Gauss point per lane, (128, 5)
  * and (128, 6); 4 element colours with in-place adds.  variant = -1 only
  * reads. */

@@ -20,7 +20,7 @@ CHNS_FP32_BULK = 1
 CHNS_PC_TWO_LEVEL = 0
 CHNS_PC_MULTIGRID = 1
 # FP32 J.w schedules the autotuner chooses among (StepStats.jacvec_variant)
-JACVEC_VARIANTS = ["element-local buffer + node gather, two Gauss points per lane, 64-thread blocks, 7/SM",
+JACVEC_VARIANTS = ["element-local buffer + node gather, two Gauss points per lane, 64-thread blocks, 8/SM",
                    "element-local buffer + node gather, two Gauss points per lane, 128-thread blocks, 3/SM",
                    "element-local buffer + node gather, two Gauss points per lane, 64-thread blocks, 6/SM",
                    "element-local buffer + node gather, two Gauss points per lane, 128-thread blocks, 4/SM",

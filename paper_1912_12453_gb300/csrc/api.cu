@@ -987,6 +987,7 @@ void chns_mesh_destroy(chns_mesh *m) {
   cudaGetDevice(&prev);
   cudaSetDevice(m->device);
   cudaFree(m->conn);
+  cudaFree(m->elem_perm);
   cudaFree(m->level);
   cudaFree(m->anchor);
   cudaFree(m->hang);

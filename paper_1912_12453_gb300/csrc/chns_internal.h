@@ -139,7 +139,7 @@ struct chns_mesh {
   int64_t n_elem = 0, n_nodes = 0, n_hang = 0;
   bool uniform = false;
   int n_colours = 0;
-  std::vector<int64_t> colour_start;   // n_colours + 1, elements are stored colour by colour
+  std::vector<int64_t> colour_start;   // n_colours + 1: ranges of the colours in elem_perm
   int n_node_colours = 0;
   std::vector<int64_t> node_colour_start;  // nodes of each node colour (for probing)
   int64_t origin = -1;                 // node at the box origin (pressure pin)
@@ -158,7 +158,9 @@ struct chns_mesh {
   std::vector<int64_t> node_xyz;       // host: n_nodes * dim integer coordinates
   std::vector<uint8_t> leaf_level;     // host: the leaves as given (Morton order), plain meshes
   std::vector<uint32_t> leaf_anchor;   // host: n_elem * dim
-  // device arrays
+  // device arrays; elements in the order of the leaves (Morton order, a union
+  // mesh: instance by instance)
+  int32_t *elem_perm = nullptr;        // n_elem element indices grouped by colour
   int32_t *conn = nullptr;             // n_elem * nc: node index, or -(h+1) for hanging corner h
   uint8_t *level = nullptr;            // n_elem
   uint32_t *anchor = nullptr;          // n_elem * dim

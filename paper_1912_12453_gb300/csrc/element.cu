@@ -570,7 +570,8 @@ KCoef<T> kcoef(const PhysCoef &p, int dim) {
 // MODE 0: residual into the element-local slots; MODE 1: J.w into the
 // element-local slots; MODE 2: count of the Gauss points whose tau_m radicand
 // is floored (O = unsigned long long, one counter); MODE 3: J.w scattered into
-// the node vector (one launch per element colour).  MODE 0 and 2 read the
+// the node vector (one launch per element colour,
+// elements eperm[e_begin..e_end)).  MODE 0 and 2 read the
 // states themselves (ut = U_new, dl = U_old: they are evaluated once per
 // state), the J.w modes the prepared averages and increments.  MODE 1 takes
 // gridDim.y directions at a time (w and out at strides).  BS, MINB: block size
@@ -581,7 +582,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     const int32_t *__restrict__ hang, int64_t e_begin, int64_t e_end,
     const T *__restrict__ ut, const T *__restrict__ dl, const T *__restrict__ w,
     const T *__restrict__ f, O *__restrict__ out, KCoef<T> c0, const KCoef<T> *__restrict__ tab,
-    const uint16_t *__restrict__ einst, int64_t wstride, int64_t ostride) {
+    const uint16_t *__restrict__ einst, int64_t wstride, int64_t ostride, const int32_t *__restrict__ eperm) {
   constexpr int NC = 1 << D, NF = D + 3, ND = D + 1;
   if (MODE == 1) {
     w += blockIdx.y * wstride;
@@ -593,6 +594,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   int64_t e = e_begin + ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> D);
   const bool active = e < e_end;
   if (!active) e = e_end - 1;  // keep the lanes alive for the shuffles
+  if (MODE == 3) e = eperm[e];
   const int cn = conn[e * NC + lc];
   // batched meshes: the coefficients of the element's own problem instance
   const KCoef<T> c = tab ? tab[einst[e]] : c0;
@@ -863,41 +865,20 @@ __device__ __forceinline__ void gather_pair(int c0, int c1, const int32_t *__res
   for (int k = 0; k < N; ++k) out[k] = F2(a[k], b[k]);
 }
 
-template <int D, int BS, int MINB>
-__global__ void __launch_bounds__(BS, MINB) k_jv_pair(
-    const int32_t *__restrict__ conn, const uint8_t *__restrict__ level, const int32_t *__restrict__ hang,
-    int64_t n_elem, const float *__restrict__ ut, const float *__restrict__ dl, const float *__restrict__ w,
-    float *__restrict__ out, const __grid_constant__ KCoef<float> c, const __grid_constant__ KPhys<F2> cp,
-    int64_t wstride, int64_t ostride) {
-  constexpr int NL = 1 << (D - 1), NC = 2 * NL, NF = D + 3, ND = D + 1;
-  w += blockIdx.y * wstride;
-  out += blockIdx.y * ostride;
-  const int lc = threadIdx.x & (NL - 1);
-  int64_t e = (int64_t(blockIdx.x) * BS + threadIdx.x) >> (D - 1);
-  const bool active = e < n_elem;
-  if (!active) e = n_elem - 1;
-  const int c0 = conn[e * NC + lc], c1 = conn[e * NC + lc + NL], l = level[e];
-  F2 u[NF], d[ND], wn[NF];
-  gather_pair<NF>(c0, c1, hang, ut, u);
-  gather_pair<ND>(c0, c1, hang, dl, d);
-  gather_pair<NF>(c0, c1, hang, w, wn);
-
+// J.w of one leaf: u, d, wn hold the lane's two corners, r0, r1 their rows
+template <int D>
+__device__ __forceinline__ void pair_leaf(const KCoef<float> &c, const KPhys<F2> &cp, int lc, int l, const F2 *u,
+                                          const F2 *d, const F2 *wn, float *r0, float *r1) {
+  constexpr int NF = D + 3;
   Stage2<D> s;
-  F2 nG[D];
 #pragma unroll
   for (int a = 0; a < D - 1; ++a) {
     const bool neg = !((lc >> a) & 1);
     s.sg[a] = F2(flip_if(scale2(c.sg0[a], l), neg));
     s.sh[a] = F2(flip_if(scale2(c.sh0[a], l), neg));
-    s.cV[a] = F2(flip_if(scale2(c.cV0[a], (1 - D) * l - 1), neg));
   }
   s.sgl = scale2(c.sg0[D - 1], l);
   s.shl = scale2(c.sh0[D - 1], l);
-  s.cVl = scale2(c.cV0[D - 1], (1 - D) * l - 1);
-  s.cS = F2(scale2(c.cS0, -D * l - 1));
-#pragma unroll
-  for (int a = 0; a < D; ++a) nG[a] = F2(scale2(c.nG0[a], 2 * l));
-  const F2 CI_GG(scale2(c.CIGG0, 4 * l)), inv_trG(scale2(c.inv_trG0, -2 * l));
 
   Interp<D, F2> A, B;
   interp_state2<D>(u, s, A);
@@ -924,11 +905,23 @@ __global__ void __launch_bounds__(BS, MINB) k_jv_pair(
   q.mut = Dl<F2>(A.mut, B.mut);
   q.dphi = Dl<F2>(dphi, two * B.phit);
   q.phin = Dl<F2>(mad(hf, dphi, A.phit), two * B.phit);
+  // the leaf's factors are made where they are used: kept from the start they
+  // would sit in registers through the interpolation
+  asm volatile("" : "+r"(l));
+  F2 nG[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) nG[a] = F2(scale2(c.nG0[a], 2 * l));
+  const F2 CI_GG(scale2(c.CIGG0, 4 * l)), inv_trG(scale2(c.inv_trG0, -2 * l));
   Dl<F2> Sq[NF], Vq[NF][D];
   B2 floored;
   gp_physics<D, false, F2, Dl<F2>>(cp, nG, CI_GG, inv_trG, cp.CnWe, q, static_cast<const F2 *>(nullptr), Sq, Vq,
                                    floored);
-  float r0[NF], r1[NF];
+  asm volatile("" : "+r"(l));
+#pragma unroll
+  for (int a = 0; a < D - 1; ++a)
+    s.cV[a] = F2(flip_if(scale2(c.cV0[a], (1 - D) * l - 1), !((lc >> a) & 1)));
+  s.cVl = scale2(c.cV0[D - 1], (1 - D) * l - 1);
+  s.cS = F2(scale2(c.cS0, -D * l - 1));
 #pragma unroll
   for (int k = 0; k < NF; ++k) {
     F2 Vk[D];
@@ -938,6 +931,28 @@ __global__ void __launch_bounds__(BS, MINB) k_jv_pair(
     r0[k] = r.lo();
     r1[k] = r.hi();
   }
+}
+
+template <int D, int BS, int MINB>
+__global__ void __launch_bounds__(BS, MINB) k_jv_pair(
+    const int32_t *__restrict__ conn, const uint8_t *__restrict__ level, const int32_t *__restrict__ hang,
+    int64_t n_elem, const float *__restrict__ ut, const float *__restrict__ dl, const float *__restrict__ w,
+    float *__restrict__ out, const __grid_constant__ KCoef<float> c, const __grid_constant__ KPhys<F2> cp,
+    int64_t wstride, int64_t ostride) {
+  constexpr int NL = 1 << (D - 1), NC = 2 * NL, NF = D + 3, ND = D + 1;
+  w += blockIdx.y * wstride;
+  out += blockIdx.y * ostride;
+  const int lc = threadIdx.x & (NL - 1);
+  int64_t e = (int64_t(blockIdx.x) * BS + threadIdx.x) >> (D - 1);
+  const bool active = e < n_elem;
+  if (!active) e = n_elem - 1;
+  const int c0 = conn[e * NC + lc], c1 = conn[e * NC + lc + NL], l = level[e];
+  F2 u[NF], d[ND], wn[NF];
+  gather_pair<NF>(c0, c1, hang, ut, u);
+  gather_pair<ND>(c0, c1, hang, dl, d);
+  gather_pair<NF>(c0, c1, hang, w, wn);
+  float r0[NF], r1[NF];
+  pair_leaf<D>(c, cp, lc, l, u, d, wn, r0, r1);
   if (active) {
     store_block<NF>(out + (e * NC + lc) * NF, r0);
     store_block<NF>(out + (e * NC + lc + NL) * NF, r1);
@@ -1034,52 +1049,55 @@ __global__ void k_prep(const double *__restrict__ Un, const double *__restrict__
 
 // y[i] = sum over the slots of node i of weight * E[slot] (fixed order), then
 // the constrained rows (wall velocities, the pinned pressure): y = w for J.w,
-// y = w - bc for the residual (RES: w = U_new, bc nullable).  The slots of a
-// node are fetched eight at a time (independent loads), then added in list
-// order.
+// y = w - bc for the residual (RES: w = U_new, bc nullable).  A thread per pair
+// of values (3D) or per value (2D) of a node, the threads of a node side by
+// side: a warp's load then touches a third (a fifth) of the slots, and as many
+// fewer cache lines, than with a thread per node.  Slots are fetched eight at a
+// time (independent loads), then added in list order.
 template <int D, typename T, bool RES>
 __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict__ gptr,
                                                       const int32_t *__restrict__ gent,
                                                       const uint8_t *__restrict__ nflag, int64_t n_nodes,
                                                       const T *__restrict__ E, const T *w, const T *bc, T *y,
                                                       uint32_t fmask, int64_t estride) {
-  constexpr int NF = D + 3, G = 8;
+  constexpr int NF = D + 3, G = 8, L = NF % 2 == 0 ? 2 : 1, NP = NF / L;
   E += blockIdx.y * estride;  // gridDim.y directions, one vector after another
   w += blockIdx.y * n_nodes * NF;
   y += blockIdx.y * n_nodes * NF;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n_nodes; i += int64_t(gridDim.x) * blockDim.x) {
-    T acc[NF];
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (t >= n_nodes * NP) return;
+  const unsigned i = unsigned(t / NP);
+  const int k0 = int(t - int64_t(i) * NP) * L;
+  T acc[L];
 #pragma unroll
-    for (int k = 0; k < NF; ++k) acc[k] = T(0);
-    const int p0 = gptr[i], p1 = gptr[i + 1];
-    for (int pb = p0; pb < p1; pb += G) {
-      uint32_t ent[G];
+  for (int k = 0; k < L; ++k) acc[k] = T(0);
+  const int p0 = gptr[i], p1 = gptr[i + 1];
+  const unsigned fl = nflag[i];
+  for (int pb = p0; pb < p1; pb += G) {
+    uint32_t ent[G];
 #pragma unroll
-      for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
-      T v[G][NF];
+    for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
+    T v[G][L];
 #pragma unroll
-      for (int g = 0; g < G; ++g)
-        if (ent[g] != 0xffffffffu) load_block<NF>(E + int64_t(ent[g] & 0x3fffffffu) * NF, v[g]);
+    for (int g = 0; g < G; ++g)
+      if (ent[g] != 0xffffffffu) load_block<L>(E + int64_t(ent[g] & 0x3fffffffu) * NF + k0, v[g]);
 #pragma unroll
-      for (int g = 0; g < G; ++g)
-        if (ent[g] != 0xffffffffu) {
-          const uint32_t code = ent[g] >> 30;
-          const T wt = code == 0 ? T(1) : (code == 1 ? T(0.5) : T(0.25));
+    for (int g = 0; g < G; ++g)
+      if (ent[g] != 0xffffffffu) {
+        const uint32_t code = ent[g] >> 30;
+        const T wt = code == 0 ? T(1) : (code == 1 ? T(0.5) : T(0.25));
 #pragma unroll
-          for (int k = 0; k < NF; ++k) acc[k] = fma(wt, v[g][k], acc[k]);
-        }
-    }
-    const uint8_t fl = nflag[i];
-    if (fl & 1)
-#pragma unroll
-      for (int k = 0; k < D; ++k) acc[k] = w[i * NF + k] - (RES && bc ? bc[i * NF + k] : T(0));
-    if (fl & 2) acc[D] = w[i * NF + D] - (RES && bc ? bc[i * NF + D] : T(0));
-    if (!RES && fmask != 0xffu)
-#pragma unroll
-      for (int k = 0; k < NF; ++k)
-        if (!((fmask >> k) & 1u)) acc[k] = w[i * NF + k];
-    store_block<NF>(y + i * NF, acc);
+        for (int k = 0; k < L; ++k) acc[k] = fma(wt, v[g][k], acc[k]);
+      }
   }
+#pragma unroll
+  for (int k = 0; k < L; ++k) {
+    const int q = k0 + k;
+    if (((fl & 1) && q < D) || ((fl & 2) && q == D))
+      acc[k] = w[int64_t(i) * NF + q] - (RES && bc ? bc[int64_t(i) * NF + q] : T(0));
+    else if (!RES && !((fmask >> q) & 1u)) acc[k] = w[int64_t(i) * NF + q];
+  }
+  store_block<L>(y + int64_t(i) * NF + k0, acc);
 }
 
 // J.w by colour scatter: the constrained rows and the rows of fields outside
@@ -1238,6 +1256,11 @@ inline unsigned grid_nodes(int64_t n) {
 }
 }  // namespace
 
+namespace {
+template <int D>
+unsigned grid_gather(int64_t n_nodes) { return grid_for(n_nodes * (D == 3 ? 3 : 5)); }
+}  // namespace
+
 template <typename T>
 void launch_prep(const chns_mesh *m, const double *Un, const double *Uo, T *ut, T *dl, cudaStream_t st) {
   if (m->dim == 2) { k_prep<2, T><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(Un, Uo, m->n_nodes, ut, dl); note_launches(1); }
@@ -1258,8 +1281,8 @@ static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const
                                const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
   k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks><<<grid_elem(m->n_elem << D), kElemBlock, 0, st>>>(
       m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
-      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0);
-  k_gather_nodes<D, double, true><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
+      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0, nullptr);
+  k_gather_nodes<D, double, true><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
                                                                              Un, bc, F, 0xffu, 0);
   note_launches(2);
 }
@@ -1280,7 +1303,7 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 // uses the element-local buffer with 128-thread blocks, 3 per SM):
 //   0-3: two Gauss points per lane (k_jv_pair), all elements at once into the
 //      element-local buffer E (n_elem * 2^dim * nf values), then the node
-//      gather with the constrained rows; (threads, blocks per SM) = (64, 7),
+//      gather with the constrained rows; (threads, blocks per SM) = (64, 8),
 //      (128, 3), (64, 6), (128, 4).  0 is the default: 14 warps an SM hide the
 //      scattered loads of an adaptive mesh better than 12 (585 against 661 us
 //      on 1,375,648 leaves) and cost 4 % on a uniform one (97.7 against 93.8)
@@ -1295,9 +1318,10 @@ static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *
                          const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << D, es = threads * NF;
-  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_nodes(m->n_nodes), (unsigned)nv);
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
   k_element<D, T, 1, false, T, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
-                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, es);
+                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, es,
+                                                            nullptr);
   k_gather_nodes<D, T, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
                                                      es);
   note_launches(2);
@@ -1324,7 +1348,7 @@ static void jv_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut, 
                     float *E, float *y, uint32_t fmask, cudaStream_t st, int nv) {
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << (D - 1), es = (m->n_elem << D) * NF;
-  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_nodes(m->n_nodes), (unsigned)nv);
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
   k_jv_pair<D, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
                                             m->n_nodes * NF, es);
   k_gather_nodes<D, float, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y,
@@ -1340,7 +1364,7 @@ static void jv_colours(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
     const int64_t b = m->colour_start[col], e = m->colour_start[col + 1];
     if (e <= b) continue;
     k_element<D, T, 3, false, T><<<grid_elem((e - b) << D), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, b, e, ut, dl, w, nullptr, y, c, tab, m->elem_inst, 0, 0);
+        m->conn, m->level, m->hang, b, e, ut, dl, w, nullptr, y, c, tab, m->elem_inst, 0, 0, m->elem_perm);
     note_launches(1);
   }
   k_fix_rows<D, T><<<grid_nodes(m->n_nodes), kBlock, 0, st>>>(m->nflag, m->n_nodes, w, y, fmask);
@@ -1353,7 +1377,7 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
   if (nv > 1 && variant == 4) variant = 0;  // the colour schedule takes one direction at a time
   if constexpr (sizeof(T) == 4) {
     if (!tab) switch (variant) {
-        case 0: jv_pair<D, 64, 7>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
+        case 0: jv_pair<D, 64, 8>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
         case 1: jv_pair<D, 128, 3>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
         case 2: jv_pair<D, 64, 6>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
         case 3: jv_pair<D, 128, 4>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
@@ -1396,10 +1420,12 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
   const KCoef<double> *tab = reinterpret_cast<const KCoef<double> *>(m->coef64);
   if (m->dim == 2)
     k_element<2, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 2), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0,
+        nullptr);
   else
     k_element<3, double, 2, false, unsigned long long><<<grid_elem(m->n_elem << 3), kElemBlock, 0, st>>>(
-        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0);
+        m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, nullptr, count, c, tab, m->elem_inst, 0, 0,
+        nullptr);
   note_launches(1);
 }
 
@@ -1451,7 +1477,7 @@ chns_status copy_coef_tables(const chns_mesh *src, chns_mesh *dst) {
   return CHNS_OK;
 }
 
-int64_t energy_blocks(const chns_mesh *m) { return std::min<int64_t>(grid_for(m->n_elem << m->dim), 152 * 6); }
+int64_t energy_blocks(const chns_mesh *m) { return std::min<int64_t>(grid_for(m->n_elem << m->dim), 152 * 4); }
 
 void launch_energy(const chns_mesh *m, const PhysCoef &pc, const double *U, double *partial, double *out3,
                    cudaStream_t st) {

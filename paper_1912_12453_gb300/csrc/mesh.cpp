@@ -395,24 +395,17 @@ chns_status build_mesh(int dim, int64_t n, const uint8_t *level, const uint32_t 
       n_col = std::max(n_col, c + 1);
     }
   }
-  // elements sorted by colour, Morton order within a colour (counting sort)
+  // elements grouped by colour, Morton order within a colour (counting sort);
+  // the element arrays themselves stay in Morton order: neighbouring lanes and
+  // blocks then share nodes, which colour order rules out by construction
   m->n_colours = n_col;
   m->colour_start.assign(n_col + 1, 0);
   for (int64_t e = 0; e < n; ++e) m->colour_start[ecol[e] + 1]++;
   for (int c = 0; c < n_col; ++c) m->colour_start[c + 1] += m->colour_start[c];
-  std::vector<int64_t> order(n);
+  std::vector<int32_t> eperm(n);
   {
     std::vector<int64_t> at(m->colour_start.begin(), m->colour_start.end() - 1);
-    for (int64_t e = 0; e < n; ++e) order[at[ecol[e]]++] = e;
-  }
-  std::vector<int32_t> conn_s(size_t(n) * nc);
-  std::vector<uint8_t> lev_s(n);
-  std::vector<uint32_t> anc_s(size_t(n) * dim);
-  for (int64_t i = 0; i < n; ++i) {
-    int64_t e = order[i];
-    for (int c = 0; c < nc; ++c) conn_s[i * nc + c] = conn[e * nc + c];
-    lev_s[i] = level[e];
-    for (int a = 0; a < dim; ++a) anc_s[i * dim + a] = anchor[e * dim + a];
+    for (int64_t e = 0; e < n; ++e) eperm[at[ecol[e]]++] = (int32_t)e;
   }
 
   // --- node colouring: nodes of one colour never share an element footprint
@@ -464,9 +457,10 @@ chns_status build_mesh(int dim, int64_t n, const uint8_t *level, const uint32_t 
 
   chns_status st;
   CHNS_CUDA_TRY(cudaGetDevice(&m->device));
-  if ((st = upload(&m->conn, conn_s)) != CHNS_OK) return st;
-  if ((st = upload(&m->level, lev_s)) != CHNS_OK) return st;
-  if ((st = upload(&m->anchor, anc_s)) != CHNS_OK) return st;
+  if ((st = upload(&m->conn, conn)) != CHNS_OK) return st;
+  if ((st = upload(&m->level, m->leaf_level)) != CHNS_OK) return st;
+  if ((st = upload(&m->anchor, m->leaf_anchor)) != CHNS_OK) return st;
+  if ((st = upload(&m->elem_perm, eperm)) != CHNS_OK) return st;
   if ((st = upload(&m->hang, hang_dev)) != CHNS_OK) return st;
   if ((st = upload(&m->wall, wall)) != CHNS_OK) return st;
   {
@@ -558,11 +552,18 @@ chns_status validate_mesh(const chns_mesh *m) {
     set_error("colour ranges do not cover the elements");
     return CHNS_ERR_MESH;
   }
+  const std::vector<int32_t> eperm = download(m->elem_perm, size_t(m->n_elem));
+  std::vector<uint8_t> listed(size_t(m->n_elem), 0);
+  for (int32_t e : eperm) {
+    if (e < 0 || e >= m->n_elem || listed[e]) { set_error("colour lists do not hold every element once"); return CHNS_ERR_MESH; }
+    listed[e] = 1;
+  }
   std::vector<int64_t> owner(size_t(m->n_nodes), -1);
   std::vector<int> owner_col(size_t(m->n_nodes), -1);
   for (int c = 0; c < m->n_colours; ++c)
-    for (int64_t e = m->colour_start[c]; e < m->colour_start[c + 1]; ++e)
+    for (int64_t p = m->colour_start[c]; p < m->colour_start[c + 1]; ++p)
       for (int k = 0; k < nc; ++k) {
+        const int64_t e = eperm[p];
         const int32_t v = conn[e * nc + k];
         int32_t fp[4] = {v, -1, -1, -1};
         if (v < 0) std::memcpy(fp, &hang[size_t(-v - 1) * 4], sizeof(fp));
@@ -654,8 +655,8 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   u->uniform = true;
   for (auto *m : ms)
     if (!m->uniform || m->min_level != ms[0]->min_level) u->uniform = false;
-  // elements colour by colour, instance by instance
-  std::vector<int32_t> conn;
+  // elements instance by instance, and the colour lists
+  std::vector<int32_t> conn, eperm;
   std::vector<uint8_t> lev;
   std::vector<uint32_t> anc;
   std::vector<uint16_t> einst;
@@ -663,31 +664,31 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   lev.reserve(n_elem);
   anc.reserve(size_t(n_elem) * dim);
   einst.reserve(n_elem);
-  std::vector<std::vector<int32_t>> hconn(ms.size());
-  std::vector<std::vector<uint8_t>> hlev(ms.size());
-  std::vector<std::vector<uint32_t>> hanc(ms.size());
+  eperm.reserve(n_elem);
+  std::vector<std::vector<int32_t>> hep(ms.size());
+  std::vector<int64_t> elem_off(ms.size() + 1, 0);
   for (size_t i = 0; i < ms.size(); ++i) {
-    hconn[i] = download(ms[i]->conn, size_t(ms[i]->n_elem) * nc);
-    hlev[i] = download(ms[i]->level, size_t(ms[i]->n_elem));
-    hanc[i] = download(ms[i]->anchor, size_t(ms[i]->n_elem) * dim);
-    u->inst_max_level.push_back(ms[i]->max_level);
+    const chns_mesh *m = ms[i];
+    elem_off[i + 1] = elem_off[i] + m->n_elem;
+    for (int32_t v : download(m->conn, size_t(m->n_elem) * nc))
+      conn.push_back(v >= 0 ? int32_t(v + node_off[i]) : int32_t(v - hang_off[i]));
+    const std::vector<uint8_t> hlev = download(m->level, size_t(m->n_elem));
+    const std::vector<uint32_t> hanc = download(m->anchor, size_t(m->n_elem) * dim);
+    lev.insert(lev.end(), hlev.begin(), hlev.end());
+    anc.insert(anc.end(), hanc.begin(), hanc.end());
+    einst.insert(einst.end(), size_t(m->n_elem), (uint16_t)i);
+    hep[i] = download(m->elem_perm, size_t(m->n_elem));
+    u->inst_max_level.push_back(m->max_level);
   }
   u->colour_start.assign(n_col + 1, 0);
   for (int c = 0; c < n_col; ++c) {
     for (size_t i = 0; i < ms.size(); ++i) {
       const chns_mesh *m = ms[i];
       if (c >= m->n_colours) continue;
-      for (int64_t e = m->colour_start[c]; e < m->colour_start[c + 1]; ++e) {
-        for (int k = 0; k < nc; ++k) {
-          int32_t v = hconn[i][e * nc + k];
-          conn.push_back(v >= 0 ? int32_t(v + node_off[i]) : int32_t(v - hang_off[i]));
-        }
-        lev.push_back(hlev[i][e]);
-        for (int a = 0; a < dim; ++a) anc.push_back(hanc[i][e * dim + a]);
-        einst.push_back((uint16_t)i);
-      }
+      for (int64_t p = m->colour_start[c]; p < m->colour_start[c + 1]; ++p)
+        eperm.push_back(int32_t(hep[i][p] + elem_off[i]));
     }
-    u->colour_start[c + 1] = (int64_t)lev.size();
+    u->colour_start[c + 1] = (int64_t)eperm.size();
   }
   std::vector<int32_t> hang, wall, pins, nperm, ninst(n_nodes);
   for (size_t i = 0; i < ms.size(); ++i) {
@@ -725,6 +726,7 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   if ((st = upload(&u->conn, conn)) != CHNS_OK) return st;
   if ((st = upload(&u->level, lev)) != CHNS_OK) return st;
   if ((st = upload(&u->anchor, anc)) != CHNS_OK) return st;
+  if ((st = upload(&u->elem_perm, eperm)) != CHNS_OK) return st;
   if ((st = upload(&u->hang, hang)) != CHNS_OK) return st;
   if ((st = upload(&u->wall, wall)) != CHNS_OK) return st;
   if ((st = upload(&u->pins, pins)) != CHNS_OK) return st;

@@ -170,24 +170,19 @@ __global__ void __launch_bounds__(kB) k_prolong_add(int64_t nf_nodes, int dim, c
 
 // ---------------------------------------------------------------- host: hierarchy
 struct Leaf {
-  uint64_t key;
   uint8_t level;
   uint32_t a[3];
 };
 
-// leaves of a built mesh, back in Morton order
+// leaves of a built mesh, in Morton order
 std::vector<Leaf> mesh_leaves(const chns_mesh *m) {
-  const std::vector<uint8_t> lev = download(m->level, size_t(m->n_elem));
-  const std::vector<uint32_t> anc = download(m->anchor, size_t(m->n_elem) * m->dim);
   std::vector<Leaf> out(m->n_elem);
   for (int64_t e = 0; e < m->n_elem; ++e) {
     Leaf &l = out[e];
-    l.level = lev[e];
+    l.level = m->leaf_level[e];
     l.a[0] = l.a[1] = l.a[2] = 0;
-    for (int d = 0; d < m->dim; ++d) l.a[d] = anc[e * m->dim + d];
-    l.key = morton(l.a, m->dim, m->max_level);
+    for (int d = 0; d < m->dim; ++d) l.a[d] = m->leaf_anchor[e * m->dim + d];
   }
-  std::sort(out.begin(), out.end(), [](const Leaf &x, const Leaf &y) { return x.key < y.key; });
   return out;
 }
 
