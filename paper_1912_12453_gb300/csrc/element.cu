@@ -1068,12 +1068,14 @@ __global__ void __launch_bounds__(256) k_prep(const double *__restrict__ Un, con
 
 // y[i] = sum over the slots of node i of weight * E[slot] (fixed order), then
 // the constrained rows (wall velocities, the pinned pressure): y = w for J.w,
-// y = w - bc for the residual (RES: w = U_new, bc nullable).  A thread per pair
+// y = w - bc for the residual (kResidual: w = U_new, bc nullable).  kDefect:
+// y = bc - J.w, the defect of bc.  A thread per pair
 // of values (3D) or per value (2D) of a node, the threads of a node side by
 // side: a warp's load then touches a third (a fifth) of the slots, and as many
 // fewer cache lines, than with a thread per node.  Slots are fetched eight at a
 // time (independent loads), then added in list order.
-template <int D, typename T, bool RES>
+enum GatherOp { kApply, kResidual, kDefect };
+template <int D, typename T, GatherOp OP>
 __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict__ gptr,
                                                       const int32_t *__restrict__ gent,
                                                       const uint8_t *__restrict__ nflag, int64_t n_nodes,
@@ -1113,10 +1115,58 @@ __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict_
   for (int k = 0; k < L; ++k) {
     const int q = k0 + k;
     if (((fl & 1) && q < D) || ((fl & 2) && q == D))
-      acc[k] = w[int64_t(i) * NF + q] - (RES && bc ? bc[int64_t(i) * NF + q] : T(0));
-    else if (!RES && !((fmask >> q) & 1u)) acc[k] = w[int64_t(i) * NF + q];
+      acc[k] = w[int64_t(i) * NF + q] - (OP == kResidual && bc ? bc[int64_t(i) * NF + q] : T(0));
+    else if (OP != kResidual && !((fmask >> q) & 1u)) acc[k] = w[int64_t(i) * NF + q];
+    if (OP == kDefect) acc[k] = bc[int64_t(i) * NF + q] - acc[k];
   }
   store_block<L>(y + int64_t(i) * NF + k0, acc);
+}
+
+// One damped nodal block-Jacobi sweep on top of the element part of J.x in E:
+// x += B (b - J.x), the node sums as in k_gather_nodes.  Eight lanes per node,
+// lane q its component q: the slots, the rows of B and the vectors are read in
+// pieces of a node's length, and the product needs six shuffles.  (A gather, then
+// a sweep with a thread per node and its 144 B block, took a launch and a pass
+// over y more.)
+template <int D, typename T>
+__global__ void __launch_bounds__(256) k_gather_smooth(const int32_t *__restrict__ gptr,
+                                                       const int32_t *__restrict__ gent,
+                                                       const uint8_t *__restrict__ nflag, int64_t n_nodes,
+                                                       const T *__restrict__ E, const T *__restrict__ b,
+                                                       const T *__restrict__ B, T *__restrict__ x, uint32_t fmask) {
+  constexpr int NF = D + 3, G = 8;
+  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  const int q = threadIdx.x & 7;
+  const bool on = (t >> 3) < n_nodes && q < NF;
+  const int64_t i = on ? t >> 3 : 0, at = i * NF + (on ? q : 0);
+  T row[NF];
+#pragma unroll
+  for (int c = 0; c < NF; ++c) row[c] = B[at * NF + c];
+  const T xi = x[at], bi = b[at];
+  const unsigned fl = nflag[i];
+  const int p0 = gptr[i], p1 = gptr[i + 1], k = int(at - i * NF);
+  T acc = T(0);
+  for (int pb = p0; pb < p1; pb += G) {
+    uint32_t ent[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
+    T v[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (ent[g] != 0xffffffffu) v[g] = E[int64_t(ent[g] & 0x3fffffffu) * NF + k];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (ent[g] != 0xffffffffu) {
+        const uint32_t code = ent[g] >> 30;
+        acc = fma(code == 0 ? T(1) : (code == 1 ? T(0.5) : T(0.25)), v[g], acc);
+      }
+  }
+  if (((fl & 1) && k < D) || ((fl & 2) && k == D) || !((fmask >> k) & 1u)) acc = xi;
+  const T r = bi - acc;
+  T s = T(0);
+#pragma unroll
+  for (int c = 0; c < NF; ++c) s = fma(row[c], __shfl_sync(FULL, r, c, 8), s);
+  if (on) x[at] = xi + s;
 }
 
 // J.w by colour scatter: the constrained rows and the rows of fields outside
@@ -1303,7 +1353,7 @@ static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const
   k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks><<<grid_elem(m->n_elem << D), kElemBlock, 0, st>>>(
       m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
       reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0, nullptr);
-  k_gather_nodes<D, double, true><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
+  k_gather_nodes<D, double, kResidual><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
                                                                              Un, bc, F, 0xffu, 0);
   note_launches(2);
 }
@@ -1335,17 +1385,15 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 //      what a batch's union mesh uses (each element has its own coefficients,
 //      which as pairs would take twice the registers)
 template <int D, typename T, int BS, int MINB>
-static void jv_elemlocal(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
-                         const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
+static void elem_local(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
+                       const T *w, T *E, cudaStream_t st, int nv) {
   constexpr int NF = D + 3;
-  const int64_t threads = m->n_elem << D, es = threads * NF;
-  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
+  const int64_t threads = m->n_elem << D;
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
   k_element<D, T, 1, false, T, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
-                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, es,
-                                                            nullptr);
-  k_gather_nodes<D, T, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
-                                                     es);
-  note_launches(2);
+                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF,
+                                                            threads * NF, nullptr);
+  note_launches(1);
 }
 
 static F2 host_pair(float a) {
@@ -1365,16 +1413,14 @@ static KPhys<F2> pair_coef(const KPhys<float> &c) {
 }
 
 template <int D, int BS, int MINB>
-static void jv_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut, const float *dl, const float *w,
-                    float *E, float *y, uint32_t fmask, cudaStream_t st, int nv) {
+static void elem_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut, const float *dl, const float *w,
+                      float *E, cudaStream_t st, int nv) {
   constexpr int NF = D + 3;
-  const int64_t threads = m->n_elem << (D - 1), es = (m->n_elem << D) * NF;
-  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv), gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
+  const int64_t threads = m->n_elem << (D - 1);
+  const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
   k_jv_pair<D, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
-                                            m->n_nodes * NF, es);
-  k_gather_nodes<D, float, false><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y,
-                                                         fmask, es);
-  note_launches(2);
+                                            m->n_nodes * NF, (m->n_elem << D) * NF);
+  note_launches(1);
 }
 
 template <int D, typename T>
@@ -1392,31 +1438,57 @@ static void jv_colours(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
   note_launches(1);
 }
 
+// element part of J.w into E (any schedule but the colours)
 template <int D, typename T>
-static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
-                        const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
-  if (nv > 1 && variant == 4) variant = 0;  // the colour schedule takes one direction at a time
-  if constexpr (sizeof(T) == 4) {
-    if (!tab) switch (variant) {
-        case 0: jv_pair<D, 64, 8>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
-        case 1: jv_pair<D, 128, 3>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
-        case 2: jv_pair<D, 64, 6>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
-        case 3: jv_pair<D, 128, 4>(m, c, ut, dl, w, E, y, fmask, st, nv); return;
-        default: break;
-      }
-    switch (variant) {
-      case 4: jv_colours<D, T>(m, c, tab, ut, dl, w, y, fmask, st); return;
-      case 6: jv_elemlocal<D, T, 128, 6>(m, c, tab, ut, dl, w, E, y, fmask, st, nv); return;
-      default: break;  // 5, and the pair schedules on a batch's union mesh
-    }
-  }
+static void elem_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+                          const T *dl, const T *w, T *E, cudaStream_t st, int nv) {
   if constexpr (sizeof(T) == 8) {
     // FP64: bound by the narrow FP64 pipe, so occupancy matters less than
     // the register spills a 6-blocks-per-SM budget causes
-    jv_elemlocal<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
+    elem_local<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, st, nv);
   } else {
-    jv_elemlocal<D, T, 128, 5>(m, c, tab, ut, dl, w, E, y, fmask, st, nv);
+    if (!tab) switch (variant) {
+        case 0: elem_pair<D, 64, 8>(m, c, ut, dl, w, E, st, nv); return;
+        case 1: elem_pair<D, 128, 3>(m, c, ut, dl, w, E, st, nv); return;
+        case 2: elem_pair<D, 64, 6>(m, c, ut, dl, w, E, st, nv); return;
+        case 3: elem_pair<D, 128, 4>(m, c, ut, dl, w, E, st, nv); return;
+        default: break;
+      }
+    if (variant == 6) elem_local<D, T, 128, 6>(m, c, tab, ut, dl, w, E, st, nv);
+    else elem_local<D, T, 128, 5>(m, c, tab, ut, dl, w, E, st, nv);  // 5, and the pair schedules on a union mesh
   }
+}
+
+template <int D, typename T>
+static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+                        const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
+  if constexpr (sizeof(T) == 4) {
+    if (variant == 4 && nv == 1) {
+      jv_colours<D, T>(m, c, tab, ut, dl, w, y, fmask, st);
+      return;
+    }
+    if (variant == 4) variant = 0;  // the colour schedule takes one direction at a time
+  }
+  elem_dispatch<D, T>(m, variant, c, tab, ut, dl, w, E, st, nv);
+  const dim3 gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
+  k_gather_nodes<D, T, kApply><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
+                                                      (m->n_elem << D) * (D + 3));
+  note_launches(1);
+}
+
+// r = b - J x, and x += B (b - J x): the element part, then one node kernel.
+// The colour schedule, which has no element-local buffer, is not used here.
+template <int D, typename T>
+static void jv_defect(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+                      const T *dl, const T *b, const T *B, T *E, T *x, T *r, uint32_t fmask, cudaStream_t st) {
+  elem_dispatch<D, T>(m, variant == 4 ? 0 : variant, c, tab, ut, dl, x, E, st, 1);
+  if (r)
+    k_gather_nodes<D, T, kDefect><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag,
+                                                                                m->n_nodes, E, x, b, r, fmask, 0);
+  else
+    k_gather_smooth<D, T><<<grid_for(m->n_nodes * 8), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, b,
+                                                                       B, x, fmask);
+  note_launches(1);
 }
 
 template <typename T>
@@ -1432,6 +1504,21 @@ template void launch_jacvec<float>(const chns_mesh *, const PhysCoef &, const fl
                                    const float *, float *, float *, cudaStream_t, int, int);
 template void launch_jacvec<double>(const chns_mesh *, const PhysCoef &, const double *, const double *,
                                     const double *, double *, double *, cudaStream_t, int, int);
+
+template <typename T>
+void launch_jacvec_defect(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *b, const T *B,
+                          T *E, T *x, T *r, cudaStream_t st) {
+  const KCoef<T> c = kcoef<T>(pc, m->dim);
+  const KCoef<T> *tab = reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32);
+  const int variant = sizeof(T) == 4 ? m->jv_variant : 0;
+  if (m->dim == 2) jv_defect<2, T>(m, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
+  else jv_defect<3, T>(m, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
+}
+template void launch_jacvec_defect<float>(const chns_mesh *, const PhysCoef &, const float *, const float *,
+                                          const float *, const float *, float *, float *, float *, cudaStream_t);
+template void launch_jacvec_defect<double>(const chns_mesh *, const PhysCoef &, const double *, const double *,
+                                           const double *, const double *, double *, double *, double *,
+                                           cudaStream_t);
 
 // Gauss points with a floored tau_m radicand, added to *count (all elements
 // in one launch, FP64 physics as in the residual)

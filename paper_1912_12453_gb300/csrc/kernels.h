@@ -22,6 +22,11 @@ constexpr int kJacvecVariants = 7;
 template <typename T>
 void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *E, T *y,
                    cudaStream_t st, int variant = -1, int nv = 1);
+// r = b - J x (r given), or one block-Jacobi sweep x += B (b - J x) with the
+// nodal blocks B; E: the element-local buffer
+template <typename T>
+void launch_jacvec_defect(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *b, const T *B,
+                          T *E, T *x, T *r, cudaStream_t st);
 void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo,
                             unsigned long long *count, cudaStream_t st);
 // scalar Q1 mass matrix times z + *beta p (p nullable: z), and the

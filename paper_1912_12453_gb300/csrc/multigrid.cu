@@ -78,67 +78,83 @@ __global__ void k_inject(int64_t n, const int32_t *__restrict__ inj, const T *__
   }
 }
 
+// Eight lanes per node in the kernels below, lane q the node's component q:
+// vectors, list entries and block rows are read in pieces of a node's length,
+// and small levels get eight times the threads.
+constexpr int kLanes = 8;
+inline unsigned grid_lanes(int64_t nodes) { return (unsigned)((nodes * kLanes + kB - 1) / kB); }
+
+// lane q: sum_c B[q][c] r_c, r_c from lane c
 template <typename T, int NF>
-__device__ __forceinline__ void block_mv(const T *__restrict__ B, int64_t i, const T *r, T *out) {
-  const T *b = B + i * NF * NF;
+__device__ __forceinline__ T block_row(const T *row, T r) {
+  T s = T(0);
 #pragma unroll
-  for (int q = 0; q < NF; ++q) {
-    T s = T(0);
-#pragma unroll
-    for (int c = 0; c < NF; ++c) s = fma(b[q * NF + c], r[c], s);
-    out[q] = s;
-  }
+  for (int c = 0; c < NF; ++c) s = fma(row[c], __shfl_sync(0xffffffffu, r, c, kLanes), s);
+  return s;
 }
 
-// x = B b (y == nullptr), or x += B (b - y): one damped block-Jacobi sweep
+// x = B b: the first damped block-Jacobi sweep
 template <typename T, int NF>
 __global__ void __launch_bounds__(kB) k_smooth(int64_t n, const T *__restrict__ B, const T *__restrict__ b,
-                                               const T *__restrict__ y, T *__restrict__ x) {
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
-    T r[NF], d[NF];
+                                               T *__restrict__ x) {
+  const int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x;
+  const int q = threadIdx.x % kLanes;
+  const bool on = t / kLanes < n && q < NF;
+  const int64_t at = on ? t / kLanes * NF + q : 0;
+  T row[NF];
 #pragma unroll
-    for (int k = 0; k < NF; ++k) r[k] = y ? b[i * NF + k] - y[i * NF + k] : b[i * NF + k];
-    block_mv<T, NF>(B, i, r, d);
-#pragma unroll
-    for (int k = 0; k < NF; ++k) x[i * NF + k] = y ? x[i * NF + k] + d[k] : d[k];
-  }
+  for (int c = 0; c < NF; ++c) row[c] = B[at * NF + c];
+  const T s = block_row<T, NF>(row, b[at]);
+  if (on) x[at] = s;
 }
 
-// bc[j] = sum over the restriction list of coarse node j of w (b - y)[i];
-// zero in the constrained rows of the coarse level.  Eight lanes per coarse
-// node (lane s takes the list entries s, s + 8, ...), then a fixed xor
-// butterfly over the eight lanes: deterministic, and eight times the
-// parallelism of a thread per coarse node on these short scattered lists.
-constexpr int kRLanes = 8;
+// bc[j] = sum over the restriction list of coarse node j of w r[i] (r: the
+// defect of the finer level), zero in the constrained rows of the coarse level;
+// with B also the coarse level's first sweep x = B bc.  Lane s takes the list
+// entries s, s + 8, ..., then a fixed xor butterfly over the eight lanes:
+// deterministic, and eight times the parallelism of a thread per coarse node on
+// these short scattered lists.
 template <typename T, int NF>
-__global__ void __launch_bounds__(kB) k_restrict_res(int64_t nc, int dim, const int32_t *__restrict__ rptr,
-                                                     const int32_t *__restrict__ rcol, const float *__restrict__ rw,
-                                                     const T *__restrict__ b, const T *__restrict__ y,
-                                                     const uint8_t *__restrict__ cflag, T *__restrict__ bc) {
-  const int64_t j = (blockIdx.x * int64_t(kB) + threadIdx.x) / kRLanes;
-  const int sub = threadIdx.x % kRLanes;
+__global__ void __launch_bounds__(kB) k_restrict(int64_t nc, int dim, const int32_t *__restrict__ rptr,
+                                                 const int32_t *__restrict__ rcol, const float *__restrict__ rw,
+                                                 const T *__restrict__ r, const uint8_t *__restrict__ cflag,
+                                                 T *__restrict__ bc, const T *__restrict__ B, T *__restrict__ x) {
+  const int64_t j0 = (blockIdx.x * int64_t(kB) + threadIdx.x) / kLanes;
+  const int sub = threadIdx.x % kLanes;
+  const bool on = j0 < nc;
+  const int64_t j = on ? j0 : 0;
+  T row[NF];
+  if (B)
+#pragma unroll
+    for (int c = 0; c < NF; ++c) row[c] = B[(j * NF + (sub < NF ? sub : 0)) * NF + c];
   T acc[NF];
 #pragma unroll
   for (int k = 0; k < NF; ++k) acc[k] = T(0);
-  if (j < nc) {
-    for (int e = rptr[j] + sub; e < rptr[j + 1]; e += kRLanes) {
+  if (on) {
+    const int e1 = rptr[j + 1];
+#pragma unroll 4
+    for (int e = rptr[j] + sub; e < e1; e += kLanes) {
       const int64_t i = rcol[e];
       const T w = T(rw[e]);
 #pragma unroll
-      for (int k = 0; k < NF; ++k) acc[k] = fma(w, b[i * NF + k] - y[i * NF + k], acc[k]);
+      for (int k = 0; k < NF; ++k) acc[k] = fma(w, r[i * NF + k], acc[k]);
     }
   }
 #pragma unroll
   for (int k = 0; k < NF; ++k)
 #pragma unroll
-    for (int o = kRLanes / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-  if (j < nc && sub == 0) {
-    const uint8_t fl = cflag[j];
-    if (fl & 1)
-      for (int k = 0; k < dim; ++k) acc[k] = T(0);
-    if (fl & 2) acc[dim] = T(0);
+    for (int o = kLanes / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+  const uint8_t fl = cflag[j];
+  T own = T(0), s = T(0);
 #pragma unroll
-    for (int k = 0; k < NF; ++k) bc[j * NF + k] = acc[k];
+  for (int k = 0; k < NF; ++k) {
+    if (((fl & 1) && k < dim) || ((fl & 2) && k == dim)) acc[k] = T(0);
+    if (k == sub) own = acc[k];
+    if (B) s = fma(row[k], acc[k], s);
+  }
+  if (on && sub < NF) {
+    bc[j * NF + sub] = own;
+    if (B) x[j * NF + sub] = s;
   }
 }
 
@@ -149,23 +165,17 @@ __global__ void __launch_bounds__(kB) k_prolong_add(int64_t nf_nodes, int dim, c
                                                     const int32_t *__restrict__ pcol, const float *__restrict__ pw,
                                                     const T *__restrict__ xc, const uint8_t *__restrict__ fflag,
                                                     T *__restrict__ x) {
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < nf_nodes; i += int64_t(gridDim.x) * kB) {
-    T acc[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) acc[k] = T(0);
-    for (int e = pptr[i]; e < pptr[i + 1]; ++e) {
-      const int64_t j = pcol[e];
-      const T w = T(pw[e]);
-#pragma unroll
-      for (int k = 0; k < NF; ++k) acc[k] = fma(w, xc[j * NF + k], acc[k]);
-    }
-    const uint8_t fl = fflag[i];
-    if (fl & 1)
-      for (int k = 0; k < dim; ++k) acc[k] = T(0);
-    if (fl & 2) acc[dim] = T(0);
-#pragma unroll
-    for (int k = 0; k < NF; ++k) x[i * NF + k] += acc[k];
-  }
+  const int64_t i = (blockIdx.x * int64_t(kB) + threadIdx.x) / kLanes;
+  const int q = threadIdx.x % kLanes;
+  if (i >= nf_nodes || q >= NF) return;
+  const T xi = x[i * NF + q];
+  const uint8_t fl = fflag[i];
+  T acc = T(0);
+  const int e1 = pptr[i + 1];
+#pragma unroll 8
+  for (int e = pptr[i]; e < e1; ++e) acc = fma(T(pw[e]), xc[int64_t(pcol[e]) * NF + q], acc);
+  if (((fl & 1) && q < dim) || ((fl & 2) && q == dim)) acc = T(0);
+  x[i * NF + q] = xi + acc;
 }
 
 // ---------------------------------------------------------------- host: hierarchy
@@ -609,31 +619,36 @@ chns_status mg_apply(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
   constexpr int P = prec_index<T>();
   auto UT = [&](int l) -> const T * { return l == 0 ? ut0 : G.lv[l].ut[P].as<T>(); };
   auto DL = [&](int l) -> const T * { return l == 0 ? dl0 : G.lv[l].dl[P].as<T>(); };
-  auto smooth_k = [&](int l, const T *y) {
-    chns_mesh *c = G.lv[l].mesh;
-    const T *Bi = G.lv[l].binv[P].as<T>();
-    if (c->nf == 5) k_smooth<T, 5><<<grid_n(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(l), y, X(l));
-    else k_smooth<T, 6><<<grid_n(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(l), y, X(l));
-    note_launches(1);
+  auto E = [&](int l) -> T * {  // allocated by mg_build
+    Workspace &ws = G.lv[l].mesh->ws;
+    return sizeof(T) == 8 ? ws.e64.as<T>() : ws.e32.as<T>();
   };
-  // down
+  // one sweep x += B (b - A x), or the defect y = b - A x: two launches
+  auto sweep = [&](int l, T *y) {
+    launch_jacvec_defect<T>(G.lv[l].mesh, pc, UT(l), DL(l), B(l), G.lv[l].binv[P].as<T>(), E(l), X(l), y, st);
+  };
+  // down; the first sweep of a coarse level (x = B b) rides on the restriction
+  if (nl > 1) {
+    chns_mesh *c = G.lv[0].mesh;
+    const T *Bi = G.lv[0].binv[P].as<T>();
+    if (c->nf == 5) k_smooth<T, 5><<<grid_lanes(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(0), X(0));
+    else k_smooth<T, 6><<<grid_lanes(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(0), X(0));
+    note_launches(1);
+  }
   for (int l = 0; l + 1 < nl; ++l) {
-    chns_mesh *c = G.lv[l].mesh;
     T *y = G.lv[l].y.as<T>();
-    smooth_k(l, nullptr);
-    for (int s = 1; s < nu; ++s) {
-      TRY_MG(jacvec_prepared<T>(c, pc, UT(l), DL(l), X(l), y, st));
-      smooth_k(l, y);
-    }
-    TRY_MG(jacvec_prepared<T>(c, pc, UT(l), DL(l), X(l), y, st));
+    for (int s = 1; s < nu; ++s) sweep(l, nullptr);
+    sweep(l, y);
     const MgLevel &Lc = G.lv[l + 1];
     chns_mesh *cc = Lc.mesh;
     T *bc = G.lv[l + 1].b.as<T>();
-    const unsigned gr = (unsigned)((cc->n_nodes * kRLanes + kB - 1) / kB);  // every coarse node one pass
-    if (c->nf == 5)
-      k_restrict_res<T, 5><<<gr, kB, 0, st>>>(cc->n_nodes, c->dim, Lc.rptr, Lc.rcol, Lc.rw, B(l), y, cc->nflag, bc);
+    const T *Bi = l + 2 < nl ? G.lv[l + 1].binv[P].as<T>() : nullptr;
+    T *xc = Bi ? X(l + 1) : nullptr;
+    const unsigned gr = grid_lanes(cc->n_nodes);
+    if (cc->nf == 5)
+      k_restrict<T, 5><<<gr, kB, 0, st>>>(cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
     else
-      k_restrict_res<T, 6><<<gr, kB, 0, st>>>(cc->n_nodes, c->dim, Lc.rptr, Lc.rcol, Lc.rw, B(l), y, cc->nflag, bc);
+      k_restrict<T, 6><<<gr, kB, 0, st>>>(cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
     note_launches(1);
   }
   // bottom: exact solve
@@ -642,20 +657,15 @@ chns_status mg_apply(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
   for (int l = nl - 2; l >= 0; --l) {
     chns_mesh *c = G.lv[l].mesh;
     const MgLevel &Lc = G.lv[l + 1];
-    T *y = G.lv[l].y.as<T>();
+    const unsigned gp = grid_lanes(c->n_nodes);
     if (c->nf == 5)
-      k_prolong_add<T, 5><<<grid_n(c->n_nodes), kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1),
-                                                             c->nflag, X(l));
+      k_prolong_add<T, 5><<<gp, kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
     else
-      k_prolong_add<T, 6><<<grid_n(c->n_nodes), kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1),
-                                                             c->nflag, X(l));
+      k_prolong_add<T, 6><<<gp, kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
     note_launches(1);
-    for (int s = 0; s < nu; ++s) {
-      TRY_MG(jacvec_prepared<T>(c, pc, UT(l), DL(l), X(l), y, st));
-      smooth_k(l, y);
-    }
+    for (int s = 0; s < nu; ++s) sweep(l, nullptr);
   }
-  return CHNS_OK;
+  return check_launch();
 }
 
 template chns_status mg_update_state<float>(chns_mesh *, const float *, const float *, cudaStream_t);
