@@ -70,6 +70,7 @@ struct Workspace {
   DevBuf binv;                         // n_nodes * nf * nf inverse diagonal blocks (element precision)
   DevBuf binv64;                       // the same blocks in double (FP64 J.w iterations)
   DevBuf red;                          // reduction partials
+  DevBuf seg;                          // batched meshes: first unknown of each instance
   DevBuf hdev;                         // device copy of Gram-Schmidt coefficients
   double *hpinned = nullptr;           // pinned host mirror of reduction results
   // preconditioner kept across steps: valid for `pc_steps_left` more steps

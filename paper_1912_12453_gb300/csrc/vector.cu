@@ -41,15 +41,33 @@ struct alignas(16) V16 {
   T a[L];
 };
 
-// block sums of NV per-thread values (fixed order) -> out[k * gridDim.x + blockIdx.x]
+// block sums of NV per-thread values (fixed order) -> out[k * gridDim.x +
+// blockIdx.x].  Eight values share a warp's tree: each step halves the values a
+// lane carries, 9 additions instead of 40 (in double each is 16 cycles of the
+// narrow pipe).
 template <typename T, int NV>
 __device__ __forceinline__ void block_sum_store(T (&v)[NV], T *out) {
   __shared__ T sh[NV][kB / 32];
   const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
+  if constexpr (NV == 8) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const T s = warp_sum(v[k]);
-    if (ln == 0) sh[k][wid] = s;
+    for (int h = 4; h > 0; h >>= 1) {  // lanes differing in bit 4h keep one half of the values each
+      const bool up = ln & (4 * h);
+#pragma unroll
+      for (int k = 0; k < h; ++k) {
+        const T keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
+        v[k] = keep + __shfl_xor_sync(FULL, send, 4 * h);
+      }
+    }
+    v[0] += __shfl_xor_sync(FULL, v[0], 2);
+    v[0] += __shfl_xor_sync(FULL, v[0], 1);
+    if ((ln & 3) == 0) sh[ln >> 2][wid] = v[0];  // lane bits 4, 3, 2: the value's number
+  } else {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const T s = warp_sum(v[k]);
+      if (ln == 0) sh[k][wid] = s;
+    }
   }
   __syncthreads();
   if (threadIdx.x < NV) {
@@ -103,10 +121,13 @@ __global__ void k_sum_partials(const P *__restrict__ partial, int nblocks, int n
   }
 }
 
-// partial sums of V_k . w for all k < nv, eight vectors at a time (w is
-// re-read per group, from L2); V_i at V + i * ld with ld a multiple of 16
-// bytes / sizeof(T) and V 16-byte aligned; skipped when flag is given and
-// *flag == 0
+// h[k] = V_k . w for all k < nv, eight vectors per blockIdx.y (w is re-read per
+// group, from L2); V_i at V + i * ld with ld a multiple of 16 bytes /
+// sizeof(T) and V 16-byte aligned; skipped when flag is given and *flag == 0.
+// Each group has its own ticket (counter[blockIdx.y]): its last block sums the
+// group's rows.  gridDim.x follows the length: with a fixed 608 blocks and the
+// groups one after another a vector of 5,445 doubles took 19 us, nearly all of
+// it block sums of zeros.
 template <typename T>
 __global__ void __launch_bounds__(kB) k_multidot(const T *__restrict__ V, int64_t ld, int nv,
                                                  const T *__restrict__ w, int64_t n, T *__restrict__ partial,
@@ -116,34 +137,33 @@ __global__ void __launch_bounds__(kB) k_multidot(const T *__restrict__ V, int64_
   constexpr int L = V16<T>::L, NV = 8;
   const int64_t nl = n / L;
   const V16<T> *wv = reinterpret_cast<const V16<T> *>(w);
-  for (int i0 = 0; i0 < nv; i0 += NV) {
-    const int c = nv - i0;
-    T acc[NV];
+  const int i0 = blockIdx.y * NV, c = min(NV, nv - i0);
+  V += int64_t(i0) * ld;
+  T acc[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) acc[k] = T(0);
-    for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < nl; t += int64_t(gridDim.x) * kB) {
-      const V16<T> x = wv[t];
+  for (int k = 0; k < NV; ++k) acc[k] = T(0);
+  for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < nl; t += int64_t(gridDim.x) * kB) {
+    const V16<T> x = wv[t];
 #pragma unroll
-      for (int k = 0; k < NV; ++k)
-        if (k < c) {
-          const V16<T> a = reinterpret_cast<const V16<T> *>(V + (int64_t)(i0 + k) * ld)[t];
+    for (int k = 0; k < NV; ++k)
+      if (k < c) {
+        const V16<T> a = reinterpret_cast<const V16<T> *>(V + (int64_t)k * ld)[t];
 #pragma unroll
-          for (int l = 0; l < L; ++l) acc[k] = fma(a.a[l], x.a[l], acc[k]);
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x < n - nl * L) {
-      const int64_t t = nl * L + threadIdx.x;
-      const T x = w[t];
-#pragma unroll
-      for (int k = 0; k < NV; ++k)
-        if (k < c) acc[k] = fma(V[(int64_t)(i0 + k) * ld + t], x, acc[k]);
-    }
-    block_sum_store<T, NV>(acc, partial + (int64_t)i0 * gridDim.x);
-    __syncthreads();  // the block-sum scratch is reused by the next group
+        for (int l = 0; l < L; ++l) acc[k] = fma(a.a[l], x.a[l], acc[k]);
+      }
   }
-  if (last_block(counter)) {
-    sum_rows<T>(partial, nv, h);
-    if (threadIdx.x == 0) *counter = 0;
+  if (blockIdx.x == 0 && threadIdx.x < n - nl * L) {
+    const int64_t t = nl * L + threadIdx.x;
+    const T x = w[t];
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (k < c) acc[k] = fma(V[(int64_t)k * ld + t], x, acc[k]);
+  }
+  partial += (int64_t)i0 * gridDim.x;
+  block_sum_store<T, NV>(acc, partial);
+  if (last_block(counter + blockIdx.y)) {
+    sum_rows<T>(partial, c, h + i0);
+    if (threadIdx.x == 0) counter[blockIdx.y] = 0;
   }
 }
 
@@ -170,7 +190,7 @@ __global__ void __launch_bounds__(kB) k_update_norm(const T *__restrict__ V, int
   V16<T> *wv = reinterpret_cast<V16<T> *>(w);
   for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < nl; t += int64_t(gridDim.x) * kB) {
     V16<T> s = wv[t];
-#pragma unroll 4
+#pragma unroll 8
     for (int i = 0; i < nv; ++i) {
       const V16<T> a = reinterpret_cast<const V16<T> *>(V + (int64_t)i * ld)[t];
 #pragma unroll
@@ -209,6 +229,16 @@ __global__ void __launch_bounds__(kB) k_dot(const double *__restrict__ x, const 
   for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < n; t += int64_t(gridDim.x) * kB)
     acc[0] = fma(x[t], y[t], acc[0]);
   block_sum_store<double, 1>(acc, partial);
+}
+
+// the same over segments: block (b, q) takes its share of x[start[q]..start[q+1])
+__global__ void __launch_bounds__(kB) k_norm2_segments(const double *__restrict__ x, const int64_t *__restrict__ start,
+                                                       double *__restrict__ partial) {
+  const int64_t e = start[blockIdx.y + 1];
+  double acc[1] = {0.0};
+  for (int64_t t = start[blockIdx.y] + blockIdx.x * int64_t(kB) + threadIdx.x; t < e; t += int64_t(gridDim.x) * kB)
+    acc[0] = fma(x[t], x[t], acc[0]);
+  block_sum_store<double, 1>(acc, partial + int64_t(blockIdx.y) * gridDim.x);
 }
 
 // w *= *scale (a zero scale: |w| = 0, w is left as is)
@@ -324,11 +354,19 @@ __global__ void __launch_bounds__(kB) k_cg_nodes(const int32_t *__restrict__ gpt
   for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
     double sum = 0.0;
     const int e1 = gptr[i + 1];
-    for (int e = gptr[i]; e < e1; ++e) {
-      const uint32_t ent = uint32_t(gent[e]);
-      const double v = E[ent & 0x3fffffffu];
-      const uint32_t code = ent >> 30;
-      sum = code == 0 ? sum + v : fma(code == 1 ? 0.5 : 0.25, v, sum);
+    constexpr int G = 8;  // independent loads, then the sum in list order
+    for (int e = gptr[i]; e < e1; e += G) {
+      uint32_t ent[G];
+      double v[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) ent[g] = e + g < e1 ? uint32_t(gent[e + g]) : 0xffffffffu;
+#pragma unroll
+      for (int g = 0; g < G; ++g) v[g] = ent[g] != 0xffffffffu ? E[ent[g] & 0x3fffffffu] : 0.0;
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const uint32_t code = ent[g] >> 30;  // 3: past the end, v = 0
+        sum = fma(code == 0 ? 1.0 : (code == 1 ? 0.5 : 0.25), v[g], sum);
+      }
     }
     q[i] = sum;
     if (z) {
@@ -393,7 +431,10 @@ __global__ void __launch_bounds__(kB) k_cg_update(int64_t n, const double *__res
     if (blockIdx.x == 0 && threadIdx.x == 0) s->err = s->done = 1;
     return;
   }
-  const double a = s->rz / pq;
+  __shared__ double ash;  // one division a block: it costs ten instructions of the FP64 pipe
+  if (threadIdx.x == 0) ash = s->rz / pq;
+  __syncthreads();
+  const double a = ash;
   double acc[2] = {0.0, 0.0};
   for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
     x[i] = fma(a, p[i], x[i]);
@@ -478,6 +519,12 @@ __global__ void k_invert_blocks(T *__restrict__ B, int64_t n_nodes, int *__restr
 
 // ---------------------------------------------------------------- launchers
 int red_blocks() { return kRedBlocks; }
+// 16 bytes per thread up to the reduction's block count (a function of n: the
+// order of a sum depends on nothing else)
+template <typename T>
+static unsigned red_grid(int64_t n) {
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n / V16<T>::L + kB - 1) / kB, kRedBlocks));
+}
 // one node per thread up to the reduction's block count
 static unsigned cg_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + kB - 1) / kB, kRedBlocks); }
 
@@ -485,7 +532,7 @@ template <typename T>
 void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double *partial, double *h,
                   cudaStream_t st, const int *flag, unsigned *counter) {
   T *pt = reinterpret_cast<T *>(partial);
-  k_multidot<T><<<kRedBlocks, kB, 0, st>>>(V, ld, nv, w, n, pt, flag, counter, h);
+  k_multidot<T><<<dim3(red_grid<T>(n), (unsigned)((nv + 7) / 8)), kB, 0, st>>>(V, ld, nv, w, n, pt, flag, counter, h);
   note_launches(1);
 }
 template void vec_multidot<float>(const float *, int64_t, int, const float *, int64_t, double *, double *,
@@ -496,6 +543,13 @@ template void vec_multidot<double>(const double *, int64_t, int, const double *,
 void vec_dot(const double *x, const double *y, int64_t n, double *partial, double *res, cudaStream_t st) {
   k_dot<<<kRedBlocks, kB, 0, st>>>(x, y, n, partial);
   k_sum_partials<double><<<1, kB, 0, st>>>(partial, kRedBlocks, 1, res);
+  note_launches(2);
+}
+
+void vec_norm2_segments(const double *x, const int64_t *start, int nseg, double *partial, double *res,
+                        cudaStream_t st) {
+  k_norm2_segments<<<dim3(kSegBlocks, (unsigned)nseg), kB, 0, st>>>(x, start, partial);
+  k_sum_partials<double><<<nseg, 32, 0, st>>>(partial, kSegBlocks, nseg, res);
   note_launches(2);
 }
 
@@ -512,11 +566,11 @@ void vec_orthogonalize(T *V, int64_t ld, int nv, int64_t n, double *partial, dou
   T *w = V + (int64_t)nv * ld;
   // pass 1 dots include w itself (stored right after V_{nv-1}): |w|^2 = h1[nv]
   vec_multidot<T>(V, ld, nv + 1, w, n, partial, h1, st, nullptr, counter);
-  k_update_norm<T><<<kRedBlocks, kB, 0, st>>>(V, ld, nv, h1, w, n, nullptr, pt, counter, nrm, scale, h1 + nv,
+  k_update_norm<T><<<red_grid<T>(n), kB, 0, st>>>(V, ld, nv, h1, w, n, nullptr, pt, counter, nrm, scale, h1 + nv,
                                               flag);
   // pass 2, on the device flag
   vec_multidot<T>(V, ld, nv, w, n, partial, h2, st, flag, counter);
-  k_update_norm<T><<<kRedBlocks, kB, 0, st>>>(V, ld, nv, h2, w, n, flag, pt, counter, nrm + 1, scale, nullptr,
+  k_update_norm<T><<<red_grid<T>(n), kB, 0, st>>>(V, ld, nv, h2, w, n, flag, pt, counter, nrm + 1, scale, nullptr,
                                               nullptr);
   note_launches(2);
 }

@@ -26,6 +26,11 @@ void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double 
                   cudaStream_t st, const int *flag, unsigned *counter);
 // x . y (double)
 void vec_dot(const double *x, const double *y, int64_t n, double *partial, double *res, cudaStream_t st);
+// res[q] = |x[start[q]..start[q+1])|^2 for nseg <= 65535 segments (start on the
+// device); partial: kSegBlocks doubles a segment
+constexpr int kSegBlocks = 32;
+void vec_norm2_segments(const double *x, const int64_t *start, int nseg, double *partial, double *res,
+                        cudaStream_t st);
 template <typename T>
 void vec_orthogonalize(T *V, int64_t ld, int nv, int64_t n, double *partial, double *h1, double *h2,
                        double *nrm, int *flag, T *scale, unsigned *counter, cudaStream_t st);
