@@ -30,8 +30,10 @@
 // block-Jacobi, x <- x + omega D^{-1} (b - A x), D the probed nodal diagonal
 // blocks of the level's operator.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <initializer_list>
 #include <vector>
 
 #include "chns_internal.h"
@@ -604,7 +606,22 @@ chns_status mg_build(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
     }
   }
   G.ready[P] = true;
-  ++G.generation;
+  // captured Arnoldi steps hold these pointers (and the number of sweeps); the
+  // values behind them are what a build renews
+  std::vector<const void *> now{reinterpret_cast<const void *>(intptr_t(smooth))};
+  for (MgLevel &L : G.lv) {
+    const chns_mesh *c = L.mesh;
+    const std::initializer_list<const DevBuf *> used{
+        &L.x, &L.b, &L.y, &L.ut[P], &L.dl[P], &L.binv[P], &c->coarse.M, &c->coarse.Minv32, &c->coarse.vec,
+        &c->coarse.rpart, P ? &c->ws.e64 : &c->ws.e32};
+    for (const DevBuf *b : used) now.push_back(b->p);
+    now.push_back(reinterpret_cast<const void *>(intptr_t(c->jv_variant)));
+  }
+  if (now != G.buffers[P]) {
+    static std::atomic<uint64_t> builds{0};  // never repeats, also across hierarchies at the same address
+    G.buffers[P].swap(now);
+    G.generation = ++builds;
+  }
   return check_launch();
 }
 

@@ -30,7 +30,10 @@ struct Multigrid {
   bool ready[2] = {false, false};            // smoothers and bottom inverse built: [float, double]
   double omega = 0.7;
   int smooth = 1;
-  uint64_t generation = 0;                   // bumped at every build (graph keys)
+  // renewed when a build moved a buffer that a V-cycle uses or changed its
+  // sweeps (graph keys): a rebuild in place keeps the captured steps
+  uint64_t generation = 0;
+  std::vector<const void *> buffers[2];      // what the last build saw, [float, double]
   bool autotune = false;                     // tune the J.w schedule of every level
   bool finish64 = false;                     // the FP64 finish needs double V-cycles on this mesh
 };
