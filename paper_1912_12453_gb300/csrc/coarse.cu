@@ -21,6 +21,7 @@
 
 #include "chns_internal.h"
 #include "coarse.h"
+#include "launch.h"
 #include "solver.h"
 
 namespace chns {
@@ -298,24 +299,32 @@ __global__ void k_restrict_sum(int64_t nc, int nf, const int32_t *__restrict__ s
 template <typename T>
 __global__ void k_coarse_matvec(const T *__restrict__ Minv, int64_t ld, int64_t inst_stride, int64_t nc,
                                 int64_t nc0, const T *__restrict__ rc, T *__restrict__ zc) {
-  const int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int64_t r0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int ln = threadIdx.x & 31;
-  if (r >= nc) return;
+  const int64_t r = r0 < nc ? r0 : nc - 1;
   const int64_t inst = r / nc0, lr = r % nc0;
   const T *row = Minv + inst * inst_stride + lr * ld;
+  // the first 24 values of the lane's share of the row (all of it for the
+  // bottom levels) before the vector is there
+  constexpr int G = 24;
+  T a[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) a[g] = ln + 32 * g < nc0 ? row[ln + 32 * g] : T(0);
+  wait_previous(rc, zc);
+  if (r0 != r) return;
   const T *x = rc + inst * nc0;
-  T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);  // four chains for load parallelism
-  int64_t c = ln;
+  T s[4] = {T(0), T(0), T(0), T(0)};  // four chains
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+    if (ln + 32 * g < nc0) s[g & 3] = fma(a[g], x[ln + 32 * g], s[g & 3]);
+  int64_t c = ln + 32 * G;
   for (; c + 96 < nc0; c += 128) {
-    s0 = fma(row[c], x[c], s0);
-    s1 = fma(row[c + 32], x[c + 32], s1);
-    s2 = fma(row[c + 64], x[c + 64], s2);
-    s3 = fma(row[c + 96], x[c + 96], s3);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = fma(row[c + 32 * k], x[c + 32 * k], s[k]);
   }
-  for (; c < nc0; c += 32) s0 = fma(row[c], x[c], s0);
-  T s = (s0 + s1) + (s2 + s3);
-  s = warp_sum_t(s);
-  if (ln == 0) zc[r] = s;
+  for (; c < nc0; c += 32) s[0] = fma(row[c], x[c], s[0]);
+  const T t = warp_sum_t((s[0] + s[1]) + (s[2] + s[3]));
+  if (ln == 0) zc[r] = t;
 }
 
 // z = Binv v + P zc  (nodal block-Jacobi plus the prolonged coarse
@@ -1051,7 +1060,7 @@ void precond_apply(chns_mesh *m, const T *Binv, bool coarse, const T *v, T *z, c
     const T *Mi = sizeof(T) == sizeof(float) ? reinterpret_cast<const T *>(C.Minv32.as<float>())
                                              : reinterpret_cast<const T *>(C.M.as<double>());
     const unsigned gm = (unsigned)((C.nc * 32 + kB - 1) / kB);
-    k_coarse_matvec<T><<<gm, kB, 0, st>>>(Mi, C.nc0, C.nc0 * C.nc0, C.nc, C.nc0, rc, out);
+    launch_next(k_coarse_matvec<T>, gm, kB, st, Mi, C.nc0, C.nc0 * C.nc0, C.nc, C.nc0, rc, out);
     note_launches(1);
     if (out == z) return;
     zc = out;

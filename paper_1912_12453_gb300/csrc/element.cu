@@ -19,6 +19,7 @@
 
 #include "chns_internal.h"
 #include "kernels.h"
+#include "launch.h"
 
 namespace chns {
 
@@ -584,10 +585,6 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     const T *__restrict__ f, O *__restrict__ out, KCoef<T> c0, const KCoef<T> *__restrict__ tab,
     const uint16_t *__restrict__ einst, int64_t wstride, int64_t ostride, const int32_t *__restrict__ eperm) {
   constexpr int NC = 1 << D, NF = D + 3, ND = D + 1;
-  if (MODE == 1) {
-    w += blockIdx.y * wstride;
-    out += blockIdx.y * ostride;
-  }
   constexpr bool UNIT = sizeof(T) == 4, RAW = MODE == 0 || MODE == 2;
   static_assert(!(UNIT && RAW), "the residual is in double");
   const int lc = threadIdx.x & (NC - 1);
@@ -598,6 +595,13 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   const int cn = conn[e * NC + lc];
   // batched meshes: the coefficients of the element's own problem instance
   const KCoef<T> c = tab ? tab[einst[e]] : c0;
+
+  const int l = level[e];
+  wait_previous(ut, dl, w, f, out);
+  if (MODE == 1) {
+    w += blockIdx.y * wstride;
+    out += blockIdx.y * ostride;
+  }
 
   // gather the corner's nodal blocks (MODE 0, 2: the sum of the states, twice
   // the average; the factors of the interpolation carry the half)
@@ -620,7 +624,6 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   if (HASF) gather<NF>(cn, hang, f, fn);
 
   // geometry of this leaf
-  const int l = level[e];
   Stage<D, T> s;
   T nG[D];
   s.v = T((RAW ? 0.5 : 1.0) * CAD<D>);
@@ -940,13 +943,14 @@ __global__ void __launch_bounds__(BS, MINB) k_jv_pair(
     float *__restrict__ out, const __grid_constant__ KCoef<float> c, const __grid_constant__ KPhys<F2> cp,
     int64_t wstride, int64_t ostride) {
   constexpr int NL = 1 << (D - 1), NC = 2 * NL, NF = D + 3, ND = D + 1;
-  w += blockIdx.y * wstride;
-  out += blockIdx.y * ostride;
   const int lc = threadIdx.x & (NL - 1);
   int64_t e = (int64_t(blockIdx.x) * BS + threadIdx.x) >> (D - 1);
   const bool active = e < n_elem;
   if (!active) e = n_elem - 1;
   const int c0 = conn[e * NC + lc], c1 = conn[e * NC + lc + NL], l = level[e];
+  wait_previous(ut, dl, w, out);
+  w += blockIdx.y * wstride;
+  out += blockIdx.y * ostride;
   F2 u[NF], d[ND], wn[NF];
   gather_pair<NF>(c0, c1, hang, ut, u);
   gather_pair<ND>(c0, c1, hang, dl, d);
@@ -982,19 +986,20 @@ __global__ void __launch_bounds__(256) k_mass(const int32_t *__restrict__ conn, 
                                               const int32_t *__restrict__ hang, int64_t n_elem,
                                               const double *__restrict__ z, const double *__restrict__ p,
                                               const double *__restrict__ beta, const int *__restrict__ done, double W0,
-                                              double *__restrict__ E) {
-  if (done && *done) return;
+                                              double *__restrict__ E) {  // W0: of level 0, with the factor
   constexpr int NC = 1 << D;
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   int64_t e = t >> D;
   const bool active = e < n_elem;
   if (!active) e = n_elem - 1;
-  const int cn = conn[e * NC + (threadIdx.x & (NC - 1))];
+  const int cn = conn[e * NC + (threadIdx.x & (NC - 1))], l = level[e];
+  wait_previous(z, p, beta, done, E);
+  if (done && *done) return;
   double u = gather1<1>(cn, hang, z, 0);
   if (p) u = fma(*beta, gather1<1>(cn, hang, p, 0), u);
 #pragma unroll
   for (int a = 0; a < D; ++a) u = fma(0.5, __shfl_xor_sync(FULL, u, 1 << a), u);
-  if (active) E[t] = scale2(W0 * (D == 2 ? 4.0 / 9.0 : 8.0 / 27.0), -D * int(level[e])) * u;
+  if (active) E[t] = scale2(W0, -D * l) * u;
 }
 
 // Element-local part of the chemical-potential row at U_new = U_old = U:
@@ -1058,6 +1063,7 @@ __global__ void __launch_bounds__(256) k_prep(const double *__restrict__ Un, con
                                               T *__restrict__ ut, T *__restrict__ dl) {
   constexpr int NF = D + 3, ND = D + 1;
   const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  wait_previous(Un, Uo, ut, dl);
   if (t >= n * NF) return;
   const unsigned i = unsigned(t / NF);
   const int k = int(t - int64_t(i) * NF);
@@ -1082,11 +1088,7 @@ __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict_
                                                       const T *__restrict__ E, const T *w, const T *bc, T *y,
                                                       uint32_t fmask, int64_t estride) {
   constexpr int NF = D + 3, G = 8, L = NF % 2 == 0 ? 2 : 1, NP = NF / L;
-  E += blockIdx.y * estride;  // gridDim.y directions, one vector after another
-  w += blockIdx.y * n_nodes * NF;
-  y += blockIdx.y * n_nodes * NF;
-  const int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= n_nodes * NP) return;
+  const int64_t t0 = blockIdx.x * int64_t(blockDim.x) + threadIdx.x, t = min(t0, n_nodes * NP - 1);
   const unsigned i = unsigned(t / NP);
   const int k0 = int(t - int64_t(i) * NP) * L;
   T acc[L];
@@ -1094,10 +1096,18 @@ __global__ void __launch_bounds__(256) k_gather_nodes(const int32_t *__restrict_
   for (int k = 0; k < L; ++k) acc[k] = T(0);
   const int p0 = gptr[i], p1 = gptr[i + 1];
   const unsigned fl = nflag[i];
-  for (int pb = p0; pb < p1; pb += G) {
-    uint32_t ent[G];
+  uint32_t ent[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
+  for (int g = 0; g < G; ++g) ent[g] = p0 + g < p1 ? uint32_t(gent[p0 + g]) : 0xffffffffu;
+  wait_previous(E, w, bc, y);
+  if (t0 != t) return;
+  E += blockIdx.y * estride;  // gridDim.y directions, one vector after another
+  w += blockIdx.y * n_nodes * NF;
+  y += blockIdx.y * n_nodes * NF;
+  for (int pb = p0; pb < p1; pb += G) {
+    if (pb != p0)
+#pragma unroll
+      for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
     T v[G][L];
 #pragma unroll
     for (int g = 0; g < G; ++g)
@@ -1142,14 +1152,18 @@ __global__ void __launch_bounds__(256) k_gather_smooth(const int32_t *__restrict
   T row[NF];
 #pragma unroll
   for (int c = 0; c < NF; ++c) row[c] = B[at * NF + c];
-  const T xi = x[at], bi = b[at];
   const unsigned fl = nflag[i];
   const int p0 = gptr[i], p1 = gptr[i + 1], k = int(at - i * NF);
+  uint32_t ent[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) ent[g] = p0 + g < p1 ? uint32_t(gent[p0 + g]) : 0xffffffffu;
+  wait_previous(E, b, x);
+  const T xi = x[at], bi = b[at];
   T acc = T(0);
   for (int pb = p0; pb < p1; pb += G) {
-    uint32_t ent[G];
+    if (pb != p0)
 #pragma unroll
-    for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
+      for (int g = 0; g < G; ++g) ent[g] = pb + g < p1 ? uint32_t(gent[pb + g]) : 0xffffffffu;
     T v[G];
 #pragma unroll
     for (int g = 0; g < G; ++g)
@@ -1209,6 +1223,7 @@ __global__ void __launch_bounds__(256) k_energy(
   const int lc = threadIdx.x & (NC - 1);
   double E = 0.0, M = 0.0, Lt = 0.0;
   const int64_t n = (n_elem + 256 / NC - 1) / (256 / NC);
+  wait_previous(U, partial);
   for (int64_t blk = blockIdx.x; blk < n; blk += gridDim.x) {  // the same trips for all lanes: shuffles below
     int64_t e = blk * (256 / NC) + (threadIdx.x >> D);
     const bool active = e < n_elem;
@@ -1274,6 +1289,7 @@ __global__ void __launch_bounds__(256) k_energy(
 // sum, lanes over the blocks, a fixed shuffle tree
 __global__ void k_energy_sum(const double *__restrict__ partial, int nb, double *__restrict__ out) {
   const int k = threadIdx.x >> 5, ln = threadIdx.x & 31;
+  wait_previous(partial, out);
   double s = 0.0;
   for (int b = ln; b < nb; b += 32) s += partial[b * 3 + k];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(FULL, s, o);
@@ -1333,8 +1349,8 @@ unsigned grid_gather(int64_t n_nodes) { return grid_for(n_nodes * (D == 3 ? 3 : 
 template <typename T>
 void launch_prep(const chns_mesh *m, const double *Un, const double *Uo, T *ut, T *dl, cudaStream_t st) {
   const unsigned g = grid_for(m->n_nodes * m->nf);
-  if (m->dim == 2) k_prep<2, T><<<g, kBlock, 0, st>>>(Un, Uo, m->n_nodes, ut, dl);
-  else k_prep<3, T><<<g, kBlock, 0, st>>>(Un, Uo, m->n_nodes, ut, dl);
+  if (m->dim == 2) launch_next(k_prep<2, T>, g, kBlock, st, Un, Uo, m->n_nodes, ut, dl);
+  else launch_next(k_prep<3, T>, g, kBlock, st, Un, Uo, m->n_nodes, ut, dl);
   note_launches(1);
 }
 template void launch_prep<float>(const chns_mesh *, const double *, const double *, float *, float *, cudaStream_t);
@@ -1350,11 +1366,12 @@ template void launch_prep<double>(const chns_mesh *, const double *, const doubl
 template <int D, bool HASF>
 static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const double *Un, const double *Uo,
                                const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
-  k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks><<<grid_elem(m->n_elem << D), kElemBlock, 0, st>>>(
+  launch_next(
+      k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks>, grid_elem(m->n_elem << D), kElemBlock, st,
       m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
       reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0, nullptr);
-  k_gather_nodes<D, double, kResidual><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E,
-                                                                             Un, bc, F, 0xffu, 0);
+  launch_next(k_gather_nodes<D, double, kResidual>, grid_gather<D>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
+              m->n_nodes, E, Un, bc, F, 0xffu, 0);
   note_launches(2);
 }
 
@@ -1390,9 +1407,8 @@ static void elem_local(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << D;
   const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
-  k_element<D, T, 1, false, T, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
-                                                            nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF,
-                                                            threads * NF, nullptr);
+  launch_next(k_element<D, T, 1, false, T, BS, MINB>, ge, BS, st, m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
+              nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, threads * NF, nullptr);
   note_launches(1);
 }
 
@@ -1418,8 +1434,8 @@ static void elem_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << (D - 1);
   const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
-  k_jv_pair<D, BS, MINB><<<ge, BS, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
-                                            m->n_nodes * NF, (m->n_elem << D) * NF);
+  launch_next(k_jv_pair<D, BS, MINB>, ge, BS, st, m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
+              m->n_nodes * NF, (m->n_elem << D) * NF);
   note_launches(1);
 }
 
@@ -1471,8 +1487,8 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
   }
   elem_dispatch<D, T>(m, variant, c, tab, ut, dl, w, E, st, nv);
   const dim3 gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
-  k_gather_nodes<D, T, kApply><<<gn, kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y, fmask,
-                                                      (m->n_elem << D) * (D + 3));
+  launch_next(k_gather_nodes<D, T, kApply>, gn, kBlock, st, m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y,
+              fmask, (m->n_elem << D) * (D + 3));
   note_launches(1);
 }
 
@@ -1483,11 +1499,11 @@ static void jv_defect(const chns_mesh *m, int variant, const KCoef<T> &c, const 
                       const T *dl, const T *b, const T *B, T *E, T *x, T *r, uint32_t fmask, cudaStream_t st) {
   elem_dispatch<D, T>(m, variant == 4 ? 0 : variant, c, tab, ut, dl, x, E, st, 1);
   if (r)
-    k_gather_nodes<D, T, kDefect><<<grid_gather<D>(m->n_nodes), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag,
-                                                                                m->n_nodes, E, x, b, r, fmask, 0);
+    launch_next(k_gather_nodes<D, T, kDefect>, grid_gather<D>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
+                m->n_nodes, E, x, b, r, fmask, 0);
   else
-    k_gather_smooth<D, T><<<grid_for(m->n_nodes * 8), kBlock, 0, st>>>(m->gptr, m->gent, m->nflag, m->n_nodes, E, b,
-                                                                       B, x, fmask);
+    launch_next(k_gather_smooth<D, T>, grid_for(m->n_nodes * 8), kBlock, st, m->gptr, m->gent, m->nflag, m->n_nodes, E,
+                b, B, x, fmask);
   note_launches(1);
 }
 
@@ -1541,8 +1557,9 @@ void launch_mass(const chns_mesh *m, const PhysCoef &pc, const double *z, const 
                  const int *done, double *E, cudaStream_t st) {
   const KCoef<double> c = kcoef<double>(pc, m->dim);
   const unsigned g = grid_for(m->n_elem << m->dim);
-  if (m->dim == 2) k_mass<2><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, c.W0, E);
-  else k_mass<3><<<g, kBlock, 0, st>>>(m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, c.W0, E);
+  const double W0 = c.W0 * (m->dim == 2 ? 4.0 / 9.0 : 8.0 / 27.0);
+  if (m->dim == 2) launch_next(k_mass<2>, g, kBlock, st, m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, W0, E);
+  else launch_next(k_mass<3>, g, kBlock, st, m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, W0, E);
   note_launches(1);
 }
 
@@ -1614,10 +1631,10 @@ void launch_energy(const chns_mesh *m, const PhysCoef &pc, const double *U, doub
   c.W0 = W;
   const unsigned g = (unsigned)energy_blocks(m);
   if (dim == 2)
-    k_energy<2><<<g, 256, 0, st>>>(m->conn, m->level, m->anchor, m->hang, m->n_elem, m->max_level, U, c, partial);
+    launch_next(k_energy<2>, g, 256, st, m->conn, m->level, m->anchor, m->hang, m->n_elem, m->max_level, U, c, partial);
   else
-    k_energy<3><<<g, 256, 0, st>>>(m->conn, m->level, m->anchor, m->hang, m->n_elem, m->max_level, U, c, partial);
-  k_energy_sum<<<1, 96, 0, st>>>(partial, int(g), out3);
+    launch_next(k_energy<3>, g, 256, st, m->conn, m->level, m->anchor, m->hang, m->n_elem, m->max_level, U, c, partial);
+  launch_next(k_energy_sum, 1, 96, st, partial, int(g), out3);
   note_launches(2);
 }
 

@@ -40,6 +40,7 @@
 #include "coarse.h"
 #include "host_util.h"
 #include "kernels.h"
+#include "launch.h"
 #include "multigrid.h"
 #include "solver.h"
 
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kB) k_smooth(int64_t n, const T *__restrict__ 
   T row[NF];
 #pragma unroll
   for (int c = 0; c < NF; ++c) row[c] = B[at * NF + c];
+  wait_previous(b, x);
   const T s = block_row<T, NF>(row, b[at]);
   if (on) x[at] = s;
 }
@@ -132,10 +134,26 @@ __global__ void __launch_bounds__(kB) k_restrict(int64_t nc, int dim, const int3
   T acc[NF];
 #pragma unroll
   for (int k = 0; k < NF; ++k) acc[k] = T(0);
-  if (on) {
-    const int e1 = rptr[j + 1];
-#pragma unroll 4
-    for (int e = rptr[j] + sub; e < e1; e += kLanes) {
+  const uint8_t fl = cflag[j];
+  const int e0 = rptr[j] + sub, e1 = on ? rptr[j + 1] : 0;
+  // the lane's first entries, before the defect is there
+  constexpr int G = 4;
+  int64_t col[G];
+  T wt[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int e = e0 + g * kLanes;
+    col[g] = e < e1 ? rcol[e] : -1;
+    wt[g] = e < e1 ? T(rw[e]) : T(0);
+  }
+  wait_previous(r, bc, x);
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+    if (col[g] >= 0)
+#pragma unroll
+      for (int k = 0; k < NF; ++k) acc[k] = fma(wt[g], r[col[g] * NF + k], acc[k]);
+  {
+    for (int e = e0 + G * kLanes; e < e1; e += kLanes) {
       const int64_t i = rcol[e];
       const T w = T(rw[e]);
 #pragma unroll
@@ -146,7 +164,6 @@ __global__ void __launch_bounds__(kB) k_restrict(int64_t nc, int dim, const int3
   for (int k = 0; k < NF; ++k)
 #pragma unroll
     for (int o = kLanes / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-  const uint8_t fl = cflag[j];
   T own = T(0), s = T(0);
 #pragma unroll
   for (int k = 0; k < NF; ++k) {
@@ -169,13 +186,27 @@ __global__ void __launch_bounds__(kB) k_prolong_add(int64_t nf_nodes, int dim, c
                                                     T *__restrict__ x) {
   const int64_t i = (blockIdx.x * int64_t(kB) + threadIdx.x) / kLanes;
   const int q = threadIdx.x % kLanes;
-  if (i >= nf_nodes || q >= NF) return;
+  const bool on = i < nf_nodes && q < NF;
+  const int e0 = on ? pptr[i] : 0, e1 = on ? pptr[i + 1] : 0;
+  const uint8_t fl = on ? fflag[i] : 0;
+  constexpr int G = 8;  // a node's list (more behind hanging corners)
+  int64_t col[G];
+  T wt[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    col[g] = e0 + g < e1 ? pcol[e0 + g] : -1;
+    wt[g] = e0 + g < e1 ? T(pw[e0 + g]) : T(0);
+  }
+  wait_previous(xc, x);
+  if (!on) return;
   const T xi = x[i * NF + q];
-  const uint8_t fl = fflag[i];
-  T acc = T(0);
-  const int e1 = pptr[i + 1];
-#pragma unroll 8
-  for (int e = pptr[i]; e < e1; ++e) acc = fma(T(pw[e]), xc[int64_t(pcol[e]) * NF + q], acc);
+  T v[G], acc = T(0);
+#pragma unroll
+  for (int g = 0; g < G; ++g) v[g] = col[g] >= 0 ? xc[col[g] * NF + q] : T(0);
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+    if (col[g] >= 0) acc = fma(wt[g], v[g], acc);
+  for (int e = e0 + G; e < e1; ++e) acc = fma(T(pw[e]), xc[int64_t(pcol[e]) * NF + q], acc);
   if (((fl & 1) && q < dim) || ((fl & 2) && q == dim)) acc = T(0);
   x[i * NF + q] = xi + acc;
 }
@@ -648,8 +679,8 @@ chns_status mg_apply(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
   if (nl > 1) {
     chns_mesh *c = G.lv[0].mesh;
     const T *Bi = G.lv[0].binv[P].as<T>();
-    if (c->nf == 5) k_smooth<T, 5><<<grid_lanes(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(0), X(0));
-    else k_smooth<T, 6><<<grid_lanes(c->n_nodes), kB, 0, st>>>(c->n_nodes, Bi, B(0), X(0));
+    if (c->nf == 5) launch_next(k_smooth<T, 5>, grid_lanes(c->n_nodes), kB, st, c->n_nodes, Bi, B(0), X(0));
+    else launch_next(k_smooth<T, 6>, grid_lanes(c->n_nodes), kB, st, c->n_nodes, Bi, B(0), X(0));
     note_launches(1);
   }
   for (int l = 0; l + 1 < nl; ++l) {
@@ -663,9 +694,9 @@ chns_status mg_apply(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
     T *xc = Bi ? X(l + 1) : nullptr;
     const unsigned gr = grid_lanes(cc->n_nodes);
     if (cc->nf == 5)
-      k_restrict<T, 5><<<gr, kB, 0, st>>>(cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
+      launch_next(k_restrict<T, 5>, gr, kB, st, cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
     else
-      k_restrict<T, 6><<<gr, kB, 0, st>>>(cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
+      launch_next(k_restrict<T, 6>, gr, kB, st, cc->n_nodes, cc->dim, Lc.rptr, Lc.rcol, Lc.rw, y, cc->nflag, bc, Bi, xc);
     note_launches(1);
   }
   // bottom: exact solve
@@ -676,9 +707,9 @@ chns_status mg_apply(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
     const MgLevel &Lc = G.lv[l + 1];
     const unsigned gp = grid_lanes(c->n_nodes);
     if (c->nf == 5)
-      k_prolong_add<T, 5><<<gp, kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
+      launch_next(k_prolong_add<T, 5>, gp, kB, st, c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
     else
-      k_prolong_add<T, 6><<<gp, kB, 0, st>>>(c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
+      launch_next(k_prolong_add<T, 6>, gp, kB, st, c->n_nodes, c->dim, Lc.pptr, Lc.pcol, Lc.pw, X(l + 1), c->nflag, X(l));
     note_launches(1);
     for (int s = 0; s < nu; ++s) sweep(l, nullptr);
   }

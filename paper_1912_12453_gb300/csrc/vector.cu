@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "chns_internal.h"
+#include "launch.h"
 #include "vector.h"
 
 namespace chns {
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(kB) k_multidot(const T *__restrict__ V, int64_
                                                  const T *__restrict__ w, int64_t n, T *__restrict__ partial,
                                                  const int *__restrict__ flag, unsigned *__restrict__ counter,
                                                  double *__restrict__ h) {
+  wait_previous(V, w, partial, flag, counter, h);
   if (flag && *flag == 0) return;
   constexpr int L = V16<T>::L, NV = 8;
   const int64_t nl = n / L;
@@ -180,6 +182,7 @@ __global__ void __launch_bounds__(kB) k_update_norm(const T *__restrict__ V, int
                                                     unsigned *__restrict__ counter, double *__restrict__ nrm,
                                                     T *__restrict__ scale, const double *__restrict__ before,
                                                     int *__restrict__ flag_out) {
+  wait_previous(V, h, w, flag, partial, counter, nrm, scale, before, flag_out);
   if (flag && *flag == 0) return;
   constexpr int L = V16<T>::L;
   __shared__ T hs[kMaxRestart + 1];
@@ -244,6 +247,7 @@ __global__ void __launch_bounds__(kB) k_norm2_segments(const double *__restrict_
 // w *= *scale (a zero scale: |w| = 0, w is left as is)
 template <typename T>
 __global__ void k_normalize(T *__restrict__ w, int64_t n, const T *__restrict__ scale) {
+  wait_previous(w, scale);
   const T s = *scale;
   if (s == T(0)) return;
   constexpr int L = V16<T>::L;
@@ -348,6 +352,7 @@ __global__ void __launch_bounds__(kB) k_cg_nodes(const int32_t *__restrict__ gpt
                                                  int64_t n, const double *__restrict__ E, const double *__restrict__ z,
                                                  double *__restrict__ p, double *__restrict__ q, CgState *s,
                                                  double *__restrict__ partial, unsigned *__restrict__ counter) {
+  wait_previous(E, z, p, q, s, partial, counter);
   if (z && s->done) return;
   const double beta = z ? s->beta : 0.0;
   double acc[1] = {0.0};
@@ -425,6 +430,7 @@ __global__ void __launch_bounds__(kB) k_cg_update(int64_t n, const double *__res
                                                   const double *__restrict__ q, double *__restrict__ x,
                                                   double *__restrict__ r, double *__restrict__ z, CgState *s,
                                                   double *__restrict__ partial, unsigned *__restrict__ counter) {
+  wait_previous(d, p, q, x, r, z, s, partial, counter);
   if (s->done) return;
   const double pq = s->pq;
   if (!(pq > 0.0)) {  // every block returns here: the ticket is not touched
@@ -532,7 +538,8 @@ template <typename T>
 void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double *partial, double *h,
                   cudaStream_t st, const int *flag, unsigned *counter) {
   T *pt = reinterpret_cast<T *>(partial);
-  k_multidot<T><<<dim3(red_grid<T>(n), (unsigned)((nv + 7) / 8)), kB, 0, st>>>(V, ld, nv, w, n, pt, flag, counter, h);
+  launch_next(k_multidot<T>, dim3(red_grid<T>(n), (unsigned)((nv + 7) / 8)), kB, st, V, ld, nv, w, n, pt, flag, counter,
+              h);
   note_launches(1);
 }
 template void vec_multidot<float>(const float *, int64_t, int, const float *, int64_t, double *, double *,
@@ -566,12 +573,12 @@ void vec_orthogonalize(T *V, int64_t ld, int nv, int64_t n, double *partial, dou
   T *w = V + (int64_t)nv * ld;
   // pass 1 dots include w itself (stored right after V_{nv-1}): |w|^2 = h1[nv]
   vec_multidot<T>(V, ld, nv + 1, w, n, partial, h1, st, nullptr, counter);
-  k_update_norm<T><<<red_grid<T>(n), kB, 0, st>>>(V, ld, nv, h1, w, n, nullptr, pt, counter, nrm, scale, h1 + nv,
-                                              flag);
+  launch_next(k_update_norm<T>, red_grid<T>(n), kB, st, V, ld, nv, h1, w, n, nullptr, pt, counter, nrm, scale, h1 + nv,
+              flag);
   // pass 2, on the device flag
   vec_multidot<T>(V, ld, nv, w, n, partial, h2, st, flag, counter);
-  k_update_norm<T><<<red_grid<T>(n), kB, 0, st>>>(V, ld, nv, h2, w, n, flag, pt, counter, nrm + 1, scale, nullptr,
-                                              nullptr);
+  launch_next(k_update_norm<T>, red_grid<T>(n), kB, st, V, ld, nv, h2, w, n, flag, pt, counter, nrm + 1, scale, nullptr,
+              nullptr);
   note_launches(2);
 }
 template void vec_orthogonalize<float>(float *, int64_t, int, int64_t, double *, double *, double *, double *,
@@ -581,7 +588,7 @@ template void vec_orthogonalize<double>(double *, int64_t, int, int64_t, double 
 
 template <typename T>
 void vec_normalize(T *w, int64_t n, const T *scale, cudaStream_t st) {
-  k_normalize<T><<<grid_n(n / V16<T>::L + 1), kB, 0, st>>>(w, n, scale);
+  launch_next(k_normalize<T>, grid_n(n / V16<T>::L + 1), kB, st, w, n, scale);
   note_launches(1);
 }
 template void vec_normalize<float>(float *, int64_t, const float *, cudaStream_t);
@@ -646,7 +653,7 @@ void vec_add_field(double *U, const double *x, int64_t n_nodes, int nf, int k, c
 
 void cg_nodes(const chns_mesh *m, const double *E, const double *z, double *p, double *q, CgState *s, double *partial,
               unsigned *counter, cudaStream_t st) {
-  k_cg_nodes<<<cg_grid(m->n_nodes), kB, 0, st>>>(m->gptr, m->gent, m->n_nodes, E, z, p, q, s, partial, counter);
+  launch_next(k_cg_nodes, cg_grid(m->n_nodes), kB, st, m->gptr, m->gent, m->n_nodes, E, z, p, q, s, partial, counter);
   note_launches(1);
 }
 
@@ -658,7 +665,7 @@ void cg_start(int64_t n, double *d, const double *r, double *z, double *x, doubl
 
 void cg_update(int64_t n, const double *d, const double *p, const double *q, double *x, double *r, double *z,
                CgState *s, double *partial, unsigned *counter, cudaStream_t st) {
-  k_cg_update<<<cg_grid(n), kB, 0, st>>>(n, d, p, q, x, r, z, s, partial, counter);
+  launch_next(k_cg_update, cg_grid(n), kB, st, n, d, p, q, x, r, z, s, partial, counter);
   note_launches(1);
 }
 
