@@ -103,30 +103,25 @@ struct Coarse {
   int64_t ncn_inst = 0, nc0 = 0;    // coarse nodes / unknowns of one instance
   int64_t ncn = 0, nc = 0;          // coarse nodes, coarse unknowns (all instances)
   float *pos = nullptr;             // n_nodes * dim: node positions in coarse units
-  int64_t *rstart = nullptr;        // ncn + 1: restriction lists per coarse node (operator build)
+  // restriction lists (per coarse node: mesh nodes and weights), cut into
+  // pieces of at most kPiece entries
   int32_t *rnode = nullptr;
   float *rw = nullptr;
-  // restriction in the Krylov loop: mesh nodes grouped by coarse cell and cut
-  // into pieces of at most kPiece nodes
-  int64_t ncell_inst = 0, ncell = 0, n_pieces = 0;
-  int32_t *cnodes = nullptr;        // n_nodes: node ids, cell by cell
-  int32_t *piece_cell = nullptr;    // n_pieces
-  int32_t *piece_begin = nullptr;   // n_pieces + 1: ranges in cnodes
-  int32_t *cell_piece = nullptr;    // ncell + 1: pieces of each cell
-  int32_t *sptr = nullptr;          // ncn + 1: restriction-sum entries of each coarse node
-  int32_t *sent = nullptr;          // entries piece * 2^dim + corner
+  int64_t n_pieces = 0;
+  int32_t *piece_node = nullptr;    // n_pieces: the coarse node
+  int64_t *piece_begin = nullptr;   // n_pieces + 1: ranges in the lists
+  int32_t *node_piece = nullptr;    // ncn + 1: pieces of each coarse node
   DevBuf M;                         // per instance A_c -> A_c^{-1} (double), nc0 x nc0
   DevBuf Minv32;                    // per instance A_c^{-1} in float, nc0 x nc0
   DevBuf piv;                       // Gauss-Jordan row interchanges, 3 nc0 indices per instance
   DevBuf gj;                        // Gauss-Jordan working matrices (element precision)
   DevBuf cpart;                     // operator-build partials of a batch of probes
-  int n_chunks = 0;                 // pieces of the longest restriction list
   // the coarse grid is the mesh itself (P = I): the operator and its inverse
   // are in the mesh's node order, cinv[coarse node] is its mesh node
   bool direct = false;
   int32_t *cinv = nullptr;
   DevBuf vec;                       // coarse work vectors
-  DevBuf rpart;                     // restriction partials, n_pieces x 2^dim x nf doubles
+  DevBuf rpart;                     // restriction partials, n_pieces x nf
   bool ready = false;
   ~Coarse();
   void release();

@@ -21,6 +21,7 @@
 
 #include "chns_internal.h"
 #include "coarse.h"
+#include "host_util.h"
 #include "launch.h"
 #include "solver.h"
 
@@ -41,7 +42,6 @@ struct CGeo {
   int64_t n_nodes;
   int64_t ncn_inst;   // coarse nodes per instance
   int64_t nc0;        // coarse unknowns per instance
-  int64_t ncell_inst; // coarse cells per instance, (nc1 - 1)^dim
   int direct;         // the coarse grid is the mesh: unknowns in node order
 };
 
@@ -119,58 +119,63 @@ __device__ __forceinline__ bool slot_owner(const CGeo &g, const int *cpc, const 
   return ok;
 }
 
-constexpr int kChunk = 64;
+constexpr int kPiece = 1024;  // most entries of a restriction list that one block sums
+constexpr int kChunk = 64;    // entries whose slots a block finds together
 
-// Block (c', sl, v) takes the sl-th piece of kChunk entries of the restriction
-// list of coarse row node c' and, for probe v (colour k), sums P[i, c'] y[i, q]
-// per owner slot s (the owner of mesh node i: the nearest coarse node of
-// colour k), in list order: the threads first find the entries' slots
-// together, then thread (s, q) adds up the entries of its slot.  A block of
-// 256 threads with 48 sums each, reduced over the block, spent its time on the
-// reduction: most lists hold 64 to 125 entries.
+// Block (p, v) takes piece p of the restriction list of coarse row node c' and,
+// for probe v (colour k), sums P[i, c'] y[i, q] per owner slot s (the owner of
+// mesh node i: the nearest coarse node of colour k), in list order: the threads
+// first find the slots of kChunk entries together, then thread (s, q) adds up
+// the entries of its slot.  A block of 256 threads with 48 sums each, reduced
+// over the block, spent its time on the reduction: most lists hold 64 to 125
+// entries.
 template <typename T, int NF, int DIM>
-__global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int64_t *__restrict__ rstart,
+__global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t *__restrict__ piece_node,
+                                                          const int64_t *__restrict__ piece_begin,
                                                           const int32_t *__restrict__ rnode,
                                                           const float *__restrict__ rw, const float *__restrict__ pos,
                                                           int v0, const T *__restrict__ y, double *__restrict__ part) {
   constexpr int NS = 1 << DIM;
   static_assert(NS * NF <= kChunk, "one sum per thread");
-  const int cp = blockIdx.x, sl = blockIdx.y, k = (v0 + int(blockIdx.z)) / NF;
+  const int cp = piece_node[blockIdx.x], k = (v0 + int(blockIdx.y)) / NF;
   const int kk[3] = {k % 3, (k / 3) % 3, k / 9};
   __shared__ int32_t node[kChunk], slot[kChunk];
   __shared__ T wgt[kChunk];
-  y += blockIdx.z * g.n_nodes * NF;
-  const int64_t b = rstart[cp] + int64_t(sl) * kChunk;
-  const int cnt = int(min(int64_t(kChunk), rstart[cp + 1] - b));
-  if (int(threadIdx.x) < cnt) {
-    const int64_t i = rnode[b + threadIdx.x];
-    int r = int(cp % g.ncn_inst), s = 0;
-    bool ok = true;
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      const int cpc = r % g.nc1;
-      r /= g.nc1;
-      const float p = pos[i * DIM + a];
-      const int o = kk[a] + 3 * (int)floorf((p - float(kk[a])) / 3.0f + 0.5f);
-      if (o < 0 || o >= g.nc1) ok = false;
-      if (o > cpc) s |= 1 << a;
-    }
-    node[threadIdx.x] = int32_t(i);
-    slot[threadIdx.x] = ok ? s : -1;
-    wgt[threadIdx.x] = T(rw[b + threadIdx.x]);
-  }
-  __syncthreads();
+  y += blockIdx.y * g.n_nodes * NF;
   const int s = threadIdx.x / NF, q = threadIdx.x % NF;
-  if (s >= NS) return;
+  const int64_t end = piece_begin[blockIdx.x + 1];
   T acc = T(0);
-  for (int e = 0; e < cnt; ++e)
-    if (slot[e] == s) acc = fma(wgt[e], y[int64_t(node[e]) * NF + q], acc);
-  part[((blockIdx.z * int64_t(gridDim.x) + cp) * gridDim.y + sl) * NS * NF + threadIdx.x] = double(acc);
+  for (int64_t b = piece_begin[blockIdx.x]; b < end; b += kChunk) {
+    const int cnt = int(min(int64_t(kChunk), end - b));
+    __syncthreads();
+    if (int(threadIdx.x) < cnt) {
+      const int64_t i = rnode[b + threadIdx.x];
+      int r = int(cp % g.ncn_inst), sl = 0;
+      bool ok = true;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) {
+        const int cpc = r % g.nc1;
+        r /= g.nc1;
+        const float p = pos[i * DIM + a];
+        const int o = kk[a] + 3 * (int)floorf((p - float(kk[a])) / 3.0f + 0.5f);
+        if (o < 0 || o >= g.nc1) ok = false;
+        if (o > cpc) sl |= 1 << a;
+      }
+      node[threadIdx.x] = int32_t(i);
+      slot[threadIdx.x] = ok ? sl : -1;
+      wgt[threadIdx.x] = T(rw[b + threadIdx.x]);
+    }
+    __syncthreads();
+    if (s < NS)
+      for (int e = 0; e < cnt; ++e)
+        if (slot[e] == s) acc = fma(wgt[e], y[int64_t(node[e]) * NF + q], acc);
+  }
+  if (s < NS) part[(blockIdx.y * int64_t(gridDim.x) + blockIdx.x) * NS * NF + threadIdx.x] = double(acc);
 }
 
 // A[(c', q), (owner(s), f)] = sum of the pieces, in list order
-__global__ void k_gather_sum(CGeo g, int v0, int n_chunks, const double *__restrict__ part, double *__restrict__ A,
-                             int64_t ldA, int64_t ncn) {
+__global__ void k_gather_sum(CGeo g, int v0, int64_t n_pieces, const int32_t *__restrict__ node_piece,
+                             const double *__restrict__ part, double *__restrict__ A, int64_t ldA, int64_t ncn) {
   const int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x;
   const int nf = g.nf, ns = 1 << g.dim, v = v0 + blockIdx.y, k = v / nf, f = v % nf;
   if (t >= ncn * ns * nf) return;
@@ -184,8 +189,8 @@ __global__ void k_gather_sum(CGeo g, int v0, int n_chunks, const double *__restr
   }
   if (!slot_owner(g, cpc, kk, s, oc)) return;
   double sum = 0.0;
-  for (int sl = 0; sl < n_chunks; ++sl)
-    sum += part[(((blockIdx.y * ncn + cp) * n_chunks + sl) * ns + s) * nf + q];
+  for (int p = node_piece[cp]; p < node_piece[cp + 1]; ++p)
+    sum += part[((blockIdx.y * n_pieces + p) * ns + s) * nf + q];
   double *Ai = A + inst * g.nc0 * ldA;
   Ai[(lcp * nf + q) * ldA + int64_t(lin(g, oc)) * nf + f] = sum;
 }
@@ -215,83 +220,56 @@ __global__ void __launch_bounds__(kB) k_collect_direct(CGeo g, const float *__re
   for (int q = 0; q < NF; ++q) Ai[(li * NF + q) * g.nc0] = double(yi[q]);
 }
 
-constexpr int kPiece = 1024;
+constexpr int kGroups = 32;   // lists are read by 32 groups of eight lanes
 
-// rc = R v = P^T v, node by node.  The mesh nodes of each coarse cell are
-// stored together (cnodes) and cut into pieces; block p sums, for each of
-// its cell's 2^d corners, w_corner(i) v[i, q] over the piece, in T within
-// the block (fixed order; no FP64 instruction on the FP32 path, where the
-// FP64 pipe is the narrow one).  The weights are those of k_block_prolong,
-// so R is exactly P^T.
-template <typename T, int NF, int DIM>
-__global__ void __launch_bounds__(kB) k_restrict_cells(CGeo g, const float *__restrict__ pos,
-                                                       const int32_t *__restrict__ cnodes,
-                                                       const int32_t *__restrict__ piece_cell,
-                                                       const int32_t *__restrict__ piece_begin,
-                                                       const T *__restrict__ v, T *__restrict__ part) {
-  constexpr int NC = 1 << DIM;
-  const int p = blockIdx.x;
-  float base[3] = {0.f, 0.f, 0.f};
-  {
-    int r = int(piece_cell[p] % g.ncell_inst);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) { base[a] = float(r % (g.nc1 - 1)); r /= (g.nc1 - 1); }
+// rc = R v = P^T v: block p sums w v[i, q] over piece p of a coarse node's
+// restriction list, lane q of each group of eight the component q; the groups'
+// sums are added in group order.  part == rc when every list is one piece.
+// (Sums of all corners of a coarse cell, reduced over 256 threads, took a hundred
+// FP64 additions a warp for lists of 49 to 81 nodes.)
+template <typename T, int NF>
+__global__ void __launch_bounds__(kGroups * 8) k_restrict_lists(const int64_t *__restrict__ piece_begin,
+                                                               const int32_t *__restrict__ rnode,
+                                                               const float *__restrict__ rw,
+                                                               const T *__restrict__ v, T *__restrict__ part) {
+  const int grp = threadIdx.x >> 3, q = threadIdx.x & 7;
+  const int64_t b = piece_begin[blockIdx.x];
+  const int cnt = int(piece_begin[blockIdx.x + 1] - b);
+  int32_t i0 = 0;
+  T w0 = T(0);
+  if (grp < cnt) {
+    i0 = rnode[b + grp];
+    w0 = T(rw[b + grp]);
   }
-  T acc[NC][NF];
-#pragma unroll
-  for (int c = 0; c < NC; ++c)
-#pragma unroll
-    for (int q = 0; q < NF; ++q) acc[c][q] = T(0);
-  const int e1 = piece_begin[p + 1];
-  for (int e = piece_begin[p] + threadIdx.x; e < e1; e += kB) {
-    const int64_t i = cnodes[e];
-    T t[DIM], x[NF];
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) t[a] = T(pos[i * DIM + a] - base[a]);
-#pragma unroll
-    for (int q = 0; q < NF; ++q) x[q] = v[i * NF + q];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      T wc = T(1);
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) wc *= ((c >> a) & 1) ? t[a] : T(1) - t[a];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) acc[c][q] = fma(wc, x[q], acc[c][q]);
-    }
+  wait_previous(v, part);
+  T acc = T(0);
+  if (q < NF && grp < cnt) {
+    acc = w0 * v[int64_t(i0) * NF + q];
+#pragma unroll 4
+    for (int e = grp + kGroups; e < cnt; e += kGroups) acc = fma(T(rw[b + e]), v[int64_t(rnode[b + e]) * NF + q], acc);
   }
-  __shared__ T red[kB / 32][NC * NF];
-  const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
-#pragma unroll
-  for (int c = 0; c < NC; ++c)
-#pragma unroll
-    for (int q = 0; q < NF; ++q) {
-      const T sum = warp_sum_t(acc[c][q]);
-      if (ln == 0) red[wid][c * NF + q] = sum;
-    }
+  __shared__ T red[kGroups][8];
+  red[grp][q] = acc;
   __syncthreads();
-  for (int k = threadIdx.x; k < NC * NF; k += kB) {
-    T sum = T(0);
-#pragma unroll
-    for (int w = 0; w < kB / 32; ++w) sum += red[w][k];
-    part[int64_t(p) * NC * NF + k] = sum;
+  if (threadIdx.x < NF) {
+    T s = T(0);
+    const int n = min(kGroups, cnt);
+    for (int g = 0; g < n; ++g) s += red[g][threadIdx.x];
+    part[int64_t(blockIdx.x) * NF + threadIdx.x] = s;
   }
 }
 
-// rc[c', q]: the corner sums of the cells around coarse node c' -- the
-// (piece, corner) entries listed for c' (corner by corner, each cell's
-// pieces in order) -- one warp per coarse unknown, lanes over the entries
+// rc = sum of the pieces, in list order
 template <typename T>
-__global__ void k_restrict_sum(int64_t nc, int nf, const int32_t *__restrict__ sptr,
-                               const int32_t *__restrict__ sent, const T *__restrict__ part, T *__restrict__ rc) {
-  const int64_t t = (blockIdx.x * int64_t(kB) + threadIdx.x) >> 5;
-  const int ln = threadIdx.x & 31;
+__global__ void k_restrict_pieces(int64_t nc, int nf, const int32_t *__restrict__ node_piece,
+                                  const T *__restrict__ part, T *__restrict__ rc) {
+  const int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x;
+  wait_previous(part, rc);
   if (t >= nc) return;
   const int64_t cp = t / nf;
-  const int q = int(t % nf);
-  T sum = T(0);
-  for (int e = sptr[cp] + ln; e < sptr[cp + 1]; e += 32) sum += part[int64_t(sent[e]) * nf + q];
-  sum = warp_sum_t(sum);
-  if (ln == 0) rc[t] = sum;
+  T s = T(0);
+  for (int p = node_piece[cp]; p < node_piece[cp + 1]; ++p) s += part[int64_t(p) * nf + t % nf];
+  rc[t] = s;
 }
 
 // zc = A_c^{-1} rc, one warp per row, in precision T; row r of instance i at
@@ -329,67 +307,62 @@ __global__ void k_coarse_matvec(const T *__restrict__ Minv, int64_t ld, int64_t 
 
 // z = Binv v + P zc  (nodal block-Jacobi plus the prolonged coarse
 // correction; zc == nullptr: block-Jacobi only; Binv == nullptr: the coarse
-// correction only)
+// correction only).  Eight lanes per node, lane q the component q.
 template <typename T, int NF, int DIM>
 __global__ void __launch_bounds__(kB) k_block_prolong(CGeo g, const float *__restrict__ pos,
                                                       const int32_t *__restrict__ node_inst,
                                                       const T *__restrict__ Binv, const T *__restrict__ v,
                                                       const T *__restrict__ zc, T *__restrict__ z) {
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < g.n_nodes; i += int64_t(gridDim.x) * kB) {
-    T x[NF], acc[NF];
+  const int64_t i0 = (blockIdx.x * int64_t(kB) + threadIdx.x) >> 3;
+  const int q = threadIdx.x & 7;
+  const bool on = i0 < g.n_nodes && q < NF;
+  const int64_t i = on ? i0 : 0, at = i * NF + (on ? q : 0);
+  T row[NF];
+  if (Binv)
 #pragma unroll
-    for (int q = 0; q < NF; ++q) { x[q] = v[i * NF + q]; acc[q] = T(0); }
-    if (zc && g.direct) {
+    for (int c = 0; c < NF; ++c) row[c] = Binv[at * NF + c];
+  int64_t idx0 = 0, step[3] = {1, 0, 0};
+  T t[DIM];
+  if (zc && !g.direct) {
+    int b[3];
+    float tf[3];
+    locate(g, pos + i * DIM, b, tf);
+    idx0 = node_inst ? int64_t(node_inst[i]) * g.ncn_inst : 0;
+    step[1] = g.nc1;
+    step[2] = int64_t(g.nc1) * g.nc1;
 #pragma unroll
-      for (int q = 0; q < NF; ++q) acc[q] = zc[i * NF + q];
-    } else if (zc) {
-      int b[3];
-      float tf[3];
-      locate(g, pos + i * DIM, b, tf);
-      const int64_t cbase = node_inst ? int64_t(node_inst[i]) * g.ncn_inst : 0;
-      T t[DIM];
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) t[a] = T(tf[a]);
-#pragma unroll
-      for (int c = 0; c < (1 << DIM); ++c) {
-        T wc = T(1);
-        int64_t idx = 0;
-#pragma unroll
-        for (int a = DIM - 1; a >= 0; --a) idx = idx * g.nc1 + b[a] + ((c >> a) & 1);
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) wc *= ((c >> a) & 1) ? t[a] : T(1) - t[a];
-        const T *zp = zc + (cbase + idx) * NF;
-#pragma unroll
-        for (int q = 0; q < NF; ++q) acc[q] = fma(wc, zp[q], acc[q]);
-      }
-    }
-    if (!Binv) {  // coarse correction only
-#pragma unroll
-      for (int r = 0; r < NF; ++r) z[i * NF + r] = acc[r];
-      continue;
-    }
-    T B[NF * NF];
-    if constexpr ((NF * NF * sizeof(T)) % 16 == 0) {
-      constexpr int L = 16 / sizeof(T);
-      const V16<T> *Bv = reinterpret_cast<const V16<T> *>(Binv + i * NF * NF);
-#pragma unroll
-      for (int k = 0; k < NF * NF / L; ++k) {
-        const V16<T> b = Bv[k];
-#pragma unroll
-        for (int l = 0; l < L; ++l) B[k * L + l] = b.a[l];
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < NF * NF; ++k) B[k] = Binv[i * NF * NF + k];
-    }
-#pragma unroll
-    for (int r = 0; r < NF; ++r) {
-      T s = acc[r];
-#pragma unroll
-      for (int c = 0; c < NF; ++c) s = fma(B[r * NF + c], x[c], s);
-      z[i * NF + r] = s;
+    for (int a = 0; a < DIM; ++a) {
+      idx0 += b[a] * step[a];
+      t[a] = T(tf[a]);
     }
   }
+  wait_previous(v, zc, z);
+  T s = T(0);
+  if (zc && g.direct) {
+    s = zc[at];
+  } else if (zc) {
+    T x[1 << DIM];
+#pragma unroll
+    for (int c = 0; c < (1 << DIM); ++c) {
+      int64_t idx = idx0;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) idx += ((c >> a) & 1) ? step[a] : 0;
+      x[c] = zc[idx * NF + (on ? q : 0)];
+    }
+#pragma unroll
+    for (int c = 0; c < (1 << DIM); ++c) {
+      T wc = T(1);
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) wc *= ((c >> a) & 1) ? t[a] : T(1) - t[a];
+      s = fma(wc, x[c], s);
+    }
+  }
+  if (Binv) {
+    const T r = v[at];
+#pragma unroll
+    for (int c = 0; c < NF; ++c) s = fma(row[c], __shfl_sync(FULL, r, c, 8), s);
+  }
+  if (on) z[at] = s;
 }
 
 // A -> B elementwise with a type change (n values)
@@ -758,22 +731,17 @@ Coarse::~Coarse() { release(); }
 
 void Coarse::release() {
   cudaFree(pos);
-  cudaFree(rstart);
   cudaFree(rnode);
   cudaFree(rw);
-  cudaFree(cnodes);
-  cudaFree(piece_cell);
+  cudaFree(piece_node);
   cudaFree(piece_begin);
-  cudaFree(cell_piece);
-  cudaFree(sptr);
-  cudaFree(sent);
-  sptr = sent = nullptr;
+  cudaFree(node_piece);
   pos = nullptr;
-  rstart = nullptr;
   rnode = nullptr;
   rw = nullptr;
-  cnodes = piece_cell = piece_begin = cell_piece = nullptr;
-  ncell_inst = ncell = n_pieces = 0;
+  piece_node = node_piece = nullptr;
+  piece_begin = nullptr;
+  n_pieces = 0;
   M.release();
   Minv32.release();
   piv.release();
@@ -782,7 +750,6 @@ void Coarse::release() {
   cudaFree(cinv);
   cinv = nullptr;
   direct = false;
-  n_chunks = 0;
   vec.release();
   rpart.release();
   level = -1;
@@ -836,9 +803,6 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   std::vector<int64_t> cnt(ncn_all + 1, 0);
   for (int64_t i = 0; i < m->n_nodes; ++i) corners(i, [&](int64_t idx, double) { cnt[idx + 1]++; });
   for (int64_t c = 0; c < ncn_all; ++c) cnt[c + 1] += cnt[c];
-  int64_t longest = 0;
-  for (int64_t c = 0; c < ncn_all; ++c) longest = std::max(longest, cnt[c + 1] - cnt[c]);
-  C.n_chunks = int((longest + kChunk - 1) / kChunk);
   C.direct = m->uniform && Lc == m->min_level;
   if (C.direct) {
     // node i <-> coarse node (the corners of a node on the coarse grid: itself)
@@ -857,79 +821,28 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
     });
   CHNS_CUDA_TRY(cudaMalloc(&C.pos, sizeof(float) * pos.size()));
   CHNS_CUDA_TRY(cudaMemcpy(C.pos, pos.data(), sizeof(float) * pos.size(), cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.rstart, sizeof(int64_t) * cnt.size()));
-  CHNS_CUDA_TRY(cudaMemcpy(C.rstart, cnt.data(), sizeof(int64_t) * cnt.size(), cudaMemcpyHostToDevice));
   CHNS_CUDA_TRY(cudaMalloc(&C.rnode, sizeof(int32_t) * std::max<size_t>(rnode.size(), 1)));
   CHNS_CUDA_TRY(cudaMemcpy(C.rnode, rnode.data(), sizeof(int32_t) * rnode.size(), cudaMemcpyHostToDevice));
   CHNS_CUDA_TRY(cudaMalloc(&C.rw, sizeof(float) * std::max<size_t>(rw.size(), 1)));
   CHNS_CUDA_TRY(cudaMemcpy(C.rw, rw.data(), sizeof(float) * rw.size(), cudaMemcpyHostToDevice));
-  // nodes grouped by coarse cell (stable: node order within a cell), pieces
-  int64_t ncell_inst = 1;
-  for (int a = 0; a < dim; ++a) ncell_inst *= (nc1 - 1);
-  const int64_t ncell = ncell_inst * ni;
-  std::vector<int64_t> ccnt(ncell + 1, 0);
-  std::vector<int64_t> cell_of(m->n_nodes);
-  for (int64_t i = 0; i < m->n_nodes; ++i) {
-    int64_t c = 0;
-    for (int a = dim - 1; a >= 0; --a) c = c * (nc1 - 1) + base[i * dim + a];
-    cell_of[i] = cbase[i] / ncn * ncell_inst + c;
-    ccnt[cell_of[i] + 1]++;
+  // the lists cut into pieces of at most kPiece entries (an empty list: one)
+  std::vector<int32_t> piece_node, node_piece(ncn_all + 1, 0);
+  std::vector<int64_t> piece_begin;
+  for (int64_t c = 0; c < ncn_all; ++c) {
+    node_piece[c] = (int32_t)piece_node.size();
+    int64_t p = cnt[c];
+    do {
+      piece_node.push_back((int32_t)c);
+      piece_begin.push_back(p);
+      p += kPiece;
+    } while (p < cnt[c + 1]);
   }
-  for (int64_t c = 0; c < ncell; ++c) ccnt[c + 1] += ccnt[c];
-  std::vector<int32_t> cnodes(m->n_nodes);
-  {
-    std::vector<int64_t> f(ccnt.begin(), ccnt.end() - 1);
-    for (int64_t i = 0; i < m->n_nodes; ++i) cnodes[f[cell_of[i]]++] = (int32_t)i;
-  }
-  std::vector<int32_t> piece_cell, piece_begin, cell_piece(ncell + 1, 0);
-  for (int64_t c = 0; c < ncell; ++c) {
-    cell_piece[c] = (int32_t)piece_cell.size();
-    for (int64_t b = ccnt[c]; b < ccnt[c + 1]; b += kPiece) {
-      piece_cell.push_back((int32_t)c);
-      piece_begin.push_back((int32_t)b);
-    }
-  }
-  cell_piece[ncell] = (int32_t)piece_cell.size();
-  piece_begin.push_back((int32_t)m->n_nodes);
-  // restriction-sum lists: for coarse node c', entries piece * 2^dim + corner
-  // of the cells around it (corner of c' in that cell), corner by corner
-  std::vector<int32_t> sptr(ncn_all + 1, 0), sent;
-  for (int64_t cp = 0; cp < ncn_all; ++cp) {
-    const int64_t inst = cp / ncn;
-    int cc[3] = {0, 0, 0};
-    {
-      int64_t r = cp % ncn;
-      for (int a = 0; a < dim; ++a) { cc[a] = int(r % nc1); r /= nc1; }
-    }
-    for (int s = 0; s < (1 << dim); ++s) {
-      int64_t cell = 0;
-      bool ok = true;
-      for (int a = dim - 1; a >= 0; --a) {
-        const int ca = cc[a] - ((s >> a) & 1);
-        if (ca < 0 || ca > nc1 - 2) ok = false;
-        cell = cell * (nc1 - 1) + ca;
-      }
-      if (!ok) continue;
-      const int64_t gc = inst * ncell_inst + cell;
-      for (int32_t p = cell_piece[gc]; p < cell_piece[gc + 1]; ++p) sent.push_back(p * (1 << dim) + s);
-    }
-    sptr[cp + 1] = (int32_t)sent.size();
-  }
-  const int64_t np = (int64_t)piece_cell.size();
-  CHNS_CUDA_TRY(cudaMalloc(&C.cnodes, sizeof(int32_t) * std::max<size_t>(cnodes.size(), 1)));
-  CHNS_CUDA_TRY(cudaMemcpy(C.cnodes, cnodes.data(), sizeof(int32_t) * cnodes.size(), cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.piece_cell, sizeof(int32_t) * std::max<int64_t>(np, 1)));
-  CHNS_CUDA_TRY(cudaMemcpy(C.piece_cell, piece_cell.data(), sizeof(int32_t) * np, cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.piece_begin, sizeof(int32_t) * (np + 1)));
-  CHNS_CUDA_TRY(cudaMemcpy(C.piece_begin, piece_begin.data(), sizeof(int32_t) * (np + 1), cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.sptr, sizeof(int32_t) * sptr.size()));
-  CHNS_CUDA_TRY(cudaMemcpy(C.sptr, sptr.data(), sizeof(int32_t) * sptr.size(), cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.sent, sizeof(int32_t) * std::max<size_t>(sent.size(), 1)));
-  CHNS_CUDA_TRY(cudaMemcpy(C.sent, sent.data(), sizeof(int32_t) * sent.size(), cudaMemcpyHostToDevice));
-  CHNS_CUDA_TRY(cudaMalloc(&C.cell_piece, sizeof(int32_t) * (ncell + 1)));
-  CHNS_CUDA_TRY(cudaMemcpy(C.cell_piece, cell_piece.data(), sizeof(int32_t) * (ncell + 1), cudaMemcpyHostToDevice));
-  C.ncell_inst = ncell_inst;
-  C.ncell = ncell;
+  const int64_t np = (int64_t)piece_node.size();
+  node_piece[ncn_all] = (int32_t)np;
+  piece_begin.push_back(cnt[ncn_all]);
+  TRY_CHNS(upload(&C.piece_node, piece_node));
+  TRY_CHNS(upload(&C.piece_begin, piece_begin));
+  TRY_CHNS(upload(&C.node_piece, node_piece));
   C.n_pieces = np;
   C.level = Lc;
   C.nc1 = nc1;
@@ -942,7 +855,7 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   TRY_CHNS(C.piv.ensure(sizeof(int32_t) * 3 * C.nc0 * ni));
   TRY_CHNS(C.Minv32.ensure(sizeof(float) * C.nc0 * C.nc0 * ni));
   TRY_CHNS(C.vec.ensure(sizeof(double) * (3 * C.nc + 8)));
-  TRY_CHNS(C.rpart.ensure(sizeof(double) * std::max<int64_t>(np, 1) * (1 << dim) * nf));
+  TRY_CHNS(C.rpart.ensure(sizeof(double) * np * nf));
   return CHNS_OK;
 }
 
@@ -951,7 +864,7 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
   Coarse &C = m->coarse;
   Workspace &ws = m->ws;
   const int nf = m->nf, dim = m->dim;
-  CGeo g{dim, nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst, C.direct ? 1 : 0};
+  CGeo g{dim, nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.direct ? 1 : 0};
   double *M = C.M.as<double>();
   const int64_t nc0 = C.nc0, nn = nc0 * nc0 * C.n_inst, n = m->n_nodes * nf;
   CHNS_CUDA_TRY(cudaMemsetAsync(M, 0, sizeof(double) * nn, st));
@@ -961,7 +874,7 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
   // the 2D droplet 18.3 -> 9.1 ms, multigrid of the level-5 3D droplet 22.5 ->
   // 12.6 ms
   const int total = (dim == 2 ? 9 : 27) * nf;
-  const size_t piece = C.direct ? 0 : sizeof(double) * size_t(C.ncn) * C.n_chunks * (size_t(1) << dim) * nf;
+  const size_t piece = C.direct ? 0 : sizeof(double) * size_t(C.n_pieces) * (size_t(1) << dim) * nf;
   const int batch = probe_batch(m, sizeof(T), piece, total);
   TRY_CHNS(ws.wv.ensure(sizeof(T) * n * batch));
   TRY_CHNS(ws.yv.ensure(sizeof(T) * n * batch));
@@ -982,13 +895,15 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
       note_launches(1);
       continue;
     }
-    const dim3 gr((unsigned)C.ncn, (unsigned)C.n_chunks, nv);
+    const dim3 gr((unsigned)C.n_pieces, nv);
     if (dim == 2)
-      k_gather_coarse<T, 5, 2><<<gr, kChunk, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, v0, y, part);
+      k_gather_coarse<T, 5, 2><<<gr, kChunk, 0, st>>>(g, C.piece_node, C.piece_begin, C.rnode, C.rw, C.pos, v0, y,
+                                                  part);
     else
-      k_gather_coarse<T, 6, 3><<<gr, kChunk, 0, st>>>(g, C.rstart, C.rnode, C.rw, C.pos, v0, y, part);
+      k_gather_coarse<T, 6, 3><<<gr, kChunk, 0, st>>>(g, C.piece_node, C.piece_begin, C.rnode, C.rw, C.pos, v0, y,
+                                                  part);
     const dim3 gs((unsigned)((C.ncn * (nf << dim) + kB - 1) / kB), nv);
-    k_gather_sum<<<gs, kB, 0, st>>>(g, v0, C.n_chunks, part, M, nc0, C.ncn);
+    k_gather_sum<<<gs, kB, 0, st>>>(g, v0, C.n_pieces, C.node_piece, part, M, nc0, C.ncn);
     note_launches(2);
   }
   // A_c^{-1} per instance, in the element precision: the FP32 path inverts
@@ -1039,22 +954,25 @@ template <typename T>
 void precond_apply(chns_mesh *m, const T *Binv, bool coarse, const T *v, T *z, cudaStream_t st) {
   Coarse &C = m->coarse;
   const bool use = coarse && C.ready;
-  CGeo g{m->dim, m->nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.ncell_inst, C.direct ? 1 : 0};
+  CGeo g{m->dim, m->nf, C.nc1, m->n_nodes, C.ncn_inst, C.nc0, C.direct ? 1 : 0};
   const T *zc = nullptr;
   if (use) {
     const T *rc = v;
     T *out = C.direct && !Binv ? z : reinterpret_cast<T *>(C.vec.as<double>() + C.nc);
     if (!C.direct) {
       T *r = reinterpret_cast<T *>(C.vec.as<double>());
-      T *part = reinterpret_cast<T *>(C.rpart.as<double>());
+      const bool whole = C.n_pieces == C.ncn;
+      T *part = whole ? r : reinterpret_cast<T *>(C.rpart.as<double>());
       const unsigned np = (unsigned)C.n_pieces;
-      const unsigned gs = (unsigned)((C.nc * 32 + kB - 1) / kB);
       if (m->dim == 2)
-        k_restrict_cells<T, 5, 2><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
+        launch_next(k_restrict_lists<T, 5>, np, kGroups * 8, st, C.piece_begin, C.rnode, C.rw, v, part);
       else
-        k_restrict_cells<T, 6, 3><<<np, kB, 0, st>>>(g, C.pos, C.cnodes, C.piece_cell, C.piece_begin, v, part);
-      k_restrict_sum<T><<<gs, kB, 0, st>>>(C.nc, m->nf, C.sptr, C.sent, part, r);
-      note_launches(2);
+        launch_next(k_restrict_lists<T, 6>, np, kGroups * 8, st, C.piece_begin, C.rnode, C.rw, v, part);
+      note_launches(1);
+      if (!whole) {
+        launch_next(k_restrict_pieces<T>, (unsigned)((C.nc + kB - 1) / kB), kB, st, C.nc, m->nf, C.node_piece, part, r);
+        note_launches(1);
+      }
       rc = r;
     }
     const T *Mi = sizeof(T) == sizeof(float) ? reinterpret_cast<const T *>(C.Minv32.as<float>())
@@ -1066,8 +984,9 @@ void precond_apply(chns_mesh *m, const T *Binv, bool coarse, const T *v, T *z, c
     zc = out;
   }
   const int32_t *ni = (use && m->n_inst > 1) ? m->node_inst : nullptr;
-  if (m->dim == 2) k_block_prolong<T, 5, 2><<<grid_n(m->n_nodes), kB, 0, st>>>(g, C.pos, ni, Binv, v, zc, z);
-  else k_block_prolong<T, 6, 3><<<grid_n(m->n_nodes), kB, 0, st>>>(g, C.pos, ni, Binv, v, zc, z);
+  const unsigned gb = (unsigned)((m->n_nodes * 8 + kB - 1) / kB);
+  if (m->dim == 2) launch_next(k_block_prolong<T, 5, 2>, gb, kB, st, g, C.pos, ni, Binv, v, zc, z);
+  else launch_next(k_block_prolong<T, 6, 3>, gb, kB, st, g, C.pos, ni, Binv, v, zc, z);
   note_launches(1);
 }
 template void precond_apply<float>(chns_mesh *, const float *, bool, const float *, float *, cudaStream_t);
