@@ -402,13 +402,23 @@ __device__ __forceinline__ uint64_t abs_key(double x) {
   const uint64_t b = uint64_t(__double_as_longlong(x)) & 0x7fffffffffffffffull;
   return b > 0x7ff0000000000000ull ? 0 : b;
 }
+// the largest key of the warp and the lowest row that has it, by the warp's
+// integer reductions
+template <typename T>
 __device__ __forceinline__ void warp_arg_max(uint64_t &best, int &arg) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t v = __shfl_xor_sync(FULL, best, o);
-    const int r = __shfl_xor_sync(FULL, arg, o);
-    if (v > best || (v == best && r < arg)) { best = v; arg = r; }
+  bool at = true;
+  if (sizeof(T) == 8) {
+    const uint32_t h = __reduce_max_sync(FULL, uint32_t(best >> 32));
+    at = uint32_t(best >> 32) == h;
+    const uint32_t l = __reduce_max_sync(FULL, at ? uint32_t(best) : 0u);
+    at = at && uint32_t(best) == l;
+    best = (uint64_t(h) << 32) | l;
+  } else {
+    const uint32_t l = __reduce_max_sync(FULL, uint32_t(best));
+    at = uint32_t(best) == l;
+    best = l;
   }
+  arg = int(__reduce_min_sync(FULL, at ? uint32_t(arg) : 0xffffffffu));
 }
 
 template <typename T, int NB, int R>
@@ -448,12 +458,12 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
       const uint64_t v = abs_key(a[i][0]);
       if (r >= k && r < n && (v > best || (v == best && r < arg))) { best = v; arg = r; }
     }
-    warp_arg_max(best, arg);
+    warp_arg_max<T>(best, arg);
     if (ln == 0) { wv[sl][wid] = best; wr[sl][wid] = arg; }
     __syncthreads();
     best = ln < nw ? wv[sl][ln] : 0;
     arg = ln < nw ? wr[sl][ln] : n;
-    warp_arg_max(best, arg);
+    warp_arg_max<T>(best, arg);
     const int p = arg;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
@@ -483,11 +493,15 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
         src[i] = ksrc[sl];
       }
       // row k: prow d; the others: a - (a_k d) prow
-      const bool piv = r == k;
-      if (piv) src[i] = psrc[sl];
-      const T fr = piv ? d : -a[i][0] * d;
+      T fr = -a[i][0] * d;
+      if (r == k) {
+        src[i] = psrc[sl];
+        fr = d;
 #pragma unroll
-      for (int c = 1; c < NB; ++c) a[i][c - 1] = fma(fr, prow[sl][c], piv ? T(0) : a[i][c]);
+        for (int c = 1; c < NB; ++c) a[i][c] = T(0);
+      }
+#pragma unroll
+      for (int c = 1; c < NB; ++c) a[i][c - 1] = fma(fr, prow[sl][c], a[i][c]);
       a[i][NB - 1] = fr;
     }
   }
