@@ -77,10 +77,27 @@ chns_status ensure_ebuf(chns_mesh *m, T **E, int nv) {
   return CHNS_OK;
 }
 
+// The residual's element kernel reads a node's six values (3D) by pairs; states
+// on an 8-byte boundary only (a view that starts at an odd entry) are copied first
+chns_status pair_aligned(chns_mesh *m, const double **Un, const double **Uo, cudaStream_t st) {
+  const size_t n = size_t(m->n_nodes) * m->nf;
+  const double **v[2] = {Un, Uo};
+  if (m->dim == 2) return CHNS_OK;
+  for (int k = 0; k < 2; ++k) {
+    if ((reinterpret_cast<uintptr_t>(*v[k]) & 15) == 0) continue;
+    TRY(m->ws.al.ensure(sizeof(double) * 2 * n));
+    double *c = m->ws.al.as<double>() + k * n;  // n is even
+    CHNS_CUDA_TRY(cudaMemcpyAsync(c, *v[k], sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
+    *v[k] = c;
+  }
+  return CHNS_OK;
+}
+
 chns_status residual_into(chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const double *forcing,
                           const double *bc, double *F, cudaStream_t st) {
   double *E = nullptr;
   TRY(ensure_ebuf<double>(m, &E));
+  TRY(pair_aligned(m, &Un, &Uo, st));
   launch_residual(m, pc, Un, Uo, forcing, bc, E, F, st);
   return check_launch();
 }
@@ -1012,7 +1029,7 @@ void chns_mesh_destroy(chns_mesh *m) {
   m->ws.ut.release(); m->ws.dl.release(); m->ws.ut32.release(); m->ws.dl32.release(); m->ws.f.release();
   m->ws.F.release(); m->ws.dU.release(); m->ws.r.release(); m->ws.V.release(); m->ws.Z.release();
   m->ws.wv.release(); m->ws.yv.release(); m->ws.binv.release(); m->ws.binv64.release(); m->ws.red.release(); m->ws.hdev.release();
-  m->ws.e32.release(); m->ws.e64.release(); m->ws.ctr.release(); m->ws.count.release();
+  m->ws.e32.release(); m->ws.e64.release(); m->ws.ctr.release(); m->ws.count.release(); m->ws.al.release();
   m->ws.seg.release();
   m->ws.Ublk.release(); m->ws.p32a.release(); m->ws.p32b.release();
   delete m;
@@ -1117,6 +1134,7 @@ chns_status chns_tau_floor_count(const chns_mesh *mc, const chns_params *p, cons
   chns_mesh *m = const_cast<chns_mesh *>(mc);
   cudaStream_t st = S(stream);
   Workspace &ws = m->ws;
+  TRY(pair_aligned(m, &U_new, &U_old, st));
   TRY(ws.count.ensure(sizeof(unsigned long long)));
   TRY(ensure_pinned(ws));
   unsigned long long *cnt = ws.count.as<unsigned long long>();

@@ -58,6 +58,7 @@ chns_status check_params(const chns_mesh *m, const chns_params *p);
 // Solver scratch, sized on first use.
 struct Workspace {
   DevBuf ut, dl, ut32, dl32, f;        // prepared nodal fields (time averages / increments)
+  DevBuf al;                           // 2 n_dof: copies of states on 8-byte boundaries
   DevBuf F, dU, r;                     // double n_dof
   DevBuf Ublk;                         // double n_dof: the previous block-iteration state
   DevBuf p32a, p32b;                   // float n_dof: float V-cycle input / output in the FP64 finish
