@@ -1058,7 +1058,10 @@ chns_status chns_jacvec(const chns_mesh *mc, const chns_params *p, const double 
     TRY(prepare<double>(m, U_new, U_old, st, &ut, &dl));
     return jacvec_prepared<double>(m, pc, ut, dl, static_cast<const double *>(w), static_cast<double *>(y), st);
   } else if (prec == CHNS_FP32_BULK) {
-    float *ut = nullptr, *dl = nullptr;
+    float *ut = nullptr, *dl = nullptr, *E = nullptr;
+    TRY(ensure_ebuf<float>(m, &E));
+    if (launch_jacvec_states(m, pc, U_new, U_old, static_cast<const float *>(w), E, static_cast<float *>(y), st))
+      return check_launch();
     TRY(prepare<float>(m, U_new, U_old, st, &ut, &dl));
     return jacvec_prepared<float>(m, pc, ut, dl, static_cast<const float *>(w), static_cast<float *>(y), st);
   }

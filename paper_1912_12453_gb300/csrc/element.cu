@@ -937,10 +937,45 @@ __device__ __forceinline__ void pair_leaf(const KCoef<float> &c, const KPhys<F2>
   }
 }
 
-template <int D, int BS, int MINB>
+// x rounded to T.  To float with integer instructions: the conversion
+// instruction runs on the narrow FP64 pipe.  Round to nearest, ties to even, on
+// the bits: the 29 discarded ones decide whether the kept ones go up by one
+// (a carry moves into the exponent as it should).  Results that are not normal
+// numbers go through the conversion instruction.
+__device__ __forceinline__ float round_to(double x, float) {
+  const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x)), e = (hi >> 20) & 0x7ff;
+  if (e - 897u < 253u) {
+    unsigned b = ((hi << 3) | (lo >> 29)) - (896u << 23);  // exponent bias 1023 -> 127, modulo 2^32
+    const unsigned rest = lo << 3;
+    b += (rest > 0x80000000u || (rest == 0x80000000u && (b & 1u))) ? 1u : 0u;
+    return __uint_as_float((b & 0x7fffffffu) | (hi & 0x80000000u));
+  }
+  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);
+  return float(x);
+}
+__device__ __forceinline__ double round_to(double x, double) { return x; }
+
+// A node's prepared values straight from the states, rounded as k_prep rounds them
+template <int D>
+__device__ __forceinline__ void node_state(int64_t i, const double *__restrict__ Un, const double *__restrict__ Uo,
+                                           float *u, float *d) {
+  constexpr int NF = D + 3;
+  double a[NF], b[NF];
+  load_block<NF>(Un + i * NF, a);
+  load_block<NF>(Uo + i * NF, b);
+#pragma unroll
+  for (int k = 0; k < NF; ++k) u[k] = 0.5f * round_to(a[k] + b[k], 0.0f);
+#pragma unroll
+  for (int k = 0; k < D; ++k) d[k] = round_to(a[k] - b[k], 0.0f);
+  d[D] = round_to(a[D + 1] - b[D + 1], 0.0f);
+}
+
+// RAW: ut, dl are the states U_new, U_old themselves, on a mesh without hanging
+// nodes (see launch_jacvec_states)
+template <int D, int BS, int MINB, bool RAW>
 __global__ void __launch_bounds__(BS, MINB) k_jv_pair(
     const int32_t *__restrict__ conn, const uint8_t *__restrict__ level, const int32_t *__restrict__ hang,
-    int64_t n_elem, const float *__restrict__ ut, const float *__restrict__ dl, const float *__restrict__ w,
+    int64_t n_elem, const void *__restrict__ ut, const void *__restrict__ dl, const float *__restrict__ w,
     float *__restrict__ out, const __grid_constant__ KCoef<float> c, const __grid_constant__ KPhys<F2> cp,
     int64_t wstride, int64_t ostride) {
   constexpr int NL = 1 << (D - 1), NC = 2 * NL, NF = D + 3, ND = D + 1;
@@ -953,8 +988,19 @@ __global__ void __launch_bounds__(BS, MINB) k_jv_pair(
   w += blockIdx.y * wstride;
   out += blockIdx.y * ostride;
   F2 u[NF], d[ND], wn[NF];
-  gather_pair<NF>(c0, c1, hang, ut, u);
-  gather_pair<ND>(c0, c1, hang, dl, d);
+  if constexpr (RAW) {
+    const double *Un = static_cast<const double *>(ut), *Uo = static_cast<const double *>(dl);
+    float u0[NF], d0[ND], u1[NF], d1[ND];
+    node_state<D>(c0, Un, Uo, u0, d0);
+    node_state<D>(c1, Un, Uo, u1, d1);
+#pragma unroll
+    for (int k = 0; k < NF; ++k) u[k] = F2(u0[k], u1[k]);
+#pragma unroll
+    for (int k = 0; k < ND; ++k) d[k] = F2(d0[k], d1[k]);
+  } else {
+    gather_pair<NF>(c0, c1, hang, static_cast<const float *>(ut), u);
+    gather_pair<ND>(c0, c1, hang, static_cast<const float *>(dl), d);
+  }
   gather_pair<NF>(c0, c1, hang, w, wn);
   float r0[NF], r1[NF];
   pair_leaf<D>(c, cp, lc, l, u, d, wn, r0, r1);
@@ -1036,24 +1082,6 @@ __global__ void __launch_bounds__(256) k_mu_row(const int32_t *__restrict__ conn
 }
 
 // ---------------------------------------------------------------- node kernels
-// x rounded to T.  To float with integer instructions: the conversion
-// instruction runs on the narrow FP64 pipe.  Round to nearest, ties to even, on
-// the bits: the 29 discarded ones decide whether the kept ones go up by one
-// (a carry moves into the exponent as it should).  Results that are not normal
-// numbers go through the conversion instruction.
-__device__ __forceinline__ float round_to(double x, float) {
-  const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x)), e = (hi >> 20) & 0x7ff;
-  if (e - 897u < 253u) {
-    unsigned b = ((hi << 3) | (lo >> 29)) - (896u << 23);  // exponent bias 1023 -> 127, modulo 2^32
-    const unsigned rest = lo << 3;
-    b += (rest > 0x80000000u || (rest == 0x80000000u && (b & 1u))) ? 1u : 0u;
-    return __uint_as_float((b & 0x7fffffffu) | (hi & 0x80000000u));
-  }
-  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);
-  return float(x);
-}
-__device__ __forceinline__ double round_to(double x, double) { return x; }
-
 // v~ = (U_new + U_old)/2 for all fields; increments of v and phi, formed in
 // double and rounded once (the half is taken after the rounding, exactly).  A
 // thread per value.  FP64 pipe: two sums a value; with a thread per node (loads
@@ -1448,7 +1476,7 @@ static void elem_pair(const chns_mesh *m, const KCoef<float> &c, const float *ut
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << (D - 1);
   const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
-  launch_next(k_jv_pair<D, BS, MINB>, ge, BS, st, m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
+  launch_next(k_jv_pair<D, BS, MINB, false>, ge, BS, st, m->conn, m->level, m->hang, m->n_elem, ut, dl, w, E, c, pair_coef(c),
               m->n_nodes * NF, (m->n_elem << D) * NF);
   note_launches(1);
 }
@@ -1534,6 +1562,39 @@ template void launch_jacvec<float>(const chns_mesh *, const PhysCoef &, const fl
                                    const float *, float *, float *, cudaStream_t, int, int);
 template void launch_jacvec<double>(const chns_mesh *, const PhysCoef &, const double *, const double *,
                                     const double *, double *, double *, cudaStream_t, int, int);
+
+// J.w straight from the states, without the preparation before it: two launches
+// for a single apply.  On small meshes the host's launches are what an apply
+// costs, back to back: 13.9..15.0 -> 11.7..12.7 us on uniform meshes of 64 to
+// 16,384 leaves in 2D and 64 to 4,096 in 3D (a call waited for by itself: the
+// same, 23..26 us).  Every corner of a leaf averages its node again, in double, so
+// a large mesh loses: 32,768 leaves in 3D 15.6 -> 18.1 us, 65,536 in 2D
+// 14.4 -> 13.8 but 31.1 -> 31.6 by itself.  With hanging nodes one corner
+// averages up to four, one lane after another: 21,960 leaves 17.9 -> 31.8 us.
+// false: the mesh, its schedule or the states' alignment is not for this path.
+bool launch_jacvec_states(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const float *w,
+                          float *E, float *y, cudaStream_t st) {
+  constexpr int64_t kStateCorners = 65536;
+  if (m->n_hang || (m->n_elem << m->dim) > kStateCorners || m->jv_variant >= 4 || m->coef32) return false;
+  // node blocks of six doubles are read by pairs; the preparation reads single values
+  if (m->dim == 3 && ((reinterpret_cast<uintptr_t>(Un) | reinterpret_cast<uintptr_t>(Uo)) & 15)) return false;
+  const KCoef<float> c = kcoef<float>(pc, m->dim);
+  const KPhys<F2> cp = pair_coef(c);
+  const int64_t z = 0;
+  if (m->dim == 2) {
+    launch_next(k_jv_pair<2, 64, 8, true>, (unsigned)((m->n_elem * 2 + 63) / 64), 64, st, m->conn, m->level, m->hang,
+                m->n_elem, Un, Uo, w, E, c, cp, z, z);
+    launch_next(k_gather_nodes<2, float, kApply>, grid_gather<2>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
+                m->n_nodes, E, w, nullptr, y, pc.fmask, z);
+  } else {
+    launch_next(k_jv_pair<3, 64, 6, true>, (unsigned)((m->n_elem * 4 + 63) / 64), 64, st, m->conn, m->level, m->hang,
+                m->n_elem, Un, Uo, w, E, c, cp, z, z);
+    launch_next(k_gather_nodes<3, float, kApply>, grid_gather<3>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
+                m->n_nodes, E, w, nullptr, y, pc.fmask, z);
+  }
+  note_launches(2);
+  return true;
+}
 
 template <typename T>
 void launch_jacvec_defect(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *b, const T *B,

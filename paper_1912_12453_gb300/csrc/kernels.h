@@ -22,6 +22,10 @@ constexpr int kJacvecVariants = 7;
 template <typename T>
 void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, const T *w, T *E, T *y,
                    cudaStream_t st, int variant = -1, int nv = 1);
+// y = J w (float) at (U_new, U_old) without a preparation; false: not for this
+// mesh, nothing launched
+bool launch_jacvec_states(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const float *w,
+                          float *E, float *y, cudaStream_t st);
 // r = b - J x (r given), or one block-Jacobi sweep x += B (b - J x) with the
 // nodal blocks B; E: the element-local buffer
 template <typename T>
