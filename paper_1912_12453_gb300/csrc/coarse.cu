@@ -377,8 +377,8 @@ __global__ void k_copy_cast(const A *__restrict__ x, int64_t n, B *__restrict__ 
 // diagonal and eliminates column k from the other rows, whose column k becomes
 // -a_rk d.  NB steps change the other columns by one matrix product:
 //   A' = [r not in panel] S A + G (S A)[panel rows],
-// S the row interchanges of the panel, G (n x NB) what the steps leave in the
-// panel's own columns.  So k_gj_panel runs the NB steps on the panel alone, in
+// S the row interchanges of the panel, G (n x NB, stored column by column) what
+// the steps leave in the panel's own columns.  So k_gj_panel runs the NB steps on the panel alone, in
 // the registers of one block (a row per thread, two barriers a step), and
 // k_gj_update applies (S, G) to the whole matrix, from one buffer into the
 // other (in place, a row could be overwritten before another one reads it).
@@ -386,12 +386,14 @@ __global__ void k_copy_cast(const A *__restrict__ x, int64_t n, B *__restrict__ 
 // back by it at the end (A^-1 = G_all S_all).
 //
 // Bound: the chain of n pivot searches and two barriers each in one block,
-// about 1 us a column in float, more in double (the panel's products run on one
-// SM's FP64 pipe).  A launch pair per column (pivot, rank-1 elimination of all
-// rows) cost 12 to 24 us per column.  Preconditioner build of a step around
-// this inverse, before -> after: n = 405 float 9.2 -> 2.1 ms, n = 750 float
-// 21.2 -> 7.9 ms, n = 4374 float 172 -> 62 ms, n = 405 double 19.7 -> 10.1 ms
-// (what is left is the probing of the matrix).
+// about 0.85 us a column in float (n = 750: 177 instructions a warp and column,
+// the schedulers 54 % busy), more in double (the panel's products run on one
+// SM's FP64 pipe).  A panel is read in pieces of 32 bytes of a row and G is
+// stored column by column: with each thread reading and writing its own row a
+// word at a time an access touched 32 lines, and a panel of 32 columns of 750
+// rows took 41.6 instead of 31.2 us (8 columns of 405 rows in double: 16.5, 16.0).
+// A launch pair per column (pivot, rank-1 elimination of all rows) cost 12 to
+// 24 us per column, 9 to 18 ms for n = 405 and 750.
 // (abs_key: |x| as an integer of the same order, NaN below everything; the
 // search then needs no FP64 comparisons, which run on the narrow FP64 pipe)
 __device__ __forceinline__ uint64_t abs_key(float x) {
@@ -430,35 +432,57 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
   T *G = Gall + int64_t(blockIdx.x) * n * NB;
   const int nb = min(NB, n - k0);
   const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+  constexpr int L = 16 / sizeof(T);
+  using Row = V16<T>;
   __shared__ uint64_t wv[2][32];
   __shared__ int wr[2][32];
-  __shared__ T prow[2][NB], krow[2][NB], dinv[2];
+  __shared__ Row prow[2][NB / L], krow[2][NB / L];
+  __shared__ T dinv[2];
   __shared__ int psrc[2], ksrc[2];
+  // A row's NB values go to one thread by way of shared memory, C columns at a
+  // time: a warp reads 32 / C rows at once
+  constexpr int C = 32 / sizeof(T);
+  __shared__ T tile[32][32][C + 1];
   T a[R][NB];
   int src[R];
+  wait_previous(M, G, permall, origin_in, origin_out, bad);
 #pragma unroll
   for (int i = 0; i < R; ++i) {
-    const int r = threadIdx.x + i * blockDim.x;
-    src[i] = r;
+    src[i] = threadIdx.x + i * blockDim.x;
+    const int w0 = src[i] - ln;
 #pragma unroll
-    for (int c = 0; c < NB; ++c) a[i][c] = r < n && c < nb ? M[int64_t(r) * n + k0 + c] : T(0);
+    for (int c = 0; c < NB; c += C) {
+      T v[C];
+#pragma unroll
+      for (int j = 0; j < C; ++j) {
+        const int r = w0 + ln / C + j * (32 / C), q = c + ln % C;
+        v[j] = r < n && q < nb ? M[int64_t(r) * n + k0 + q] : T(0);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < C; ++j) tile[wid][ln / C + j * (32 / C)][ln % C] = v[j];
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < C; ++j) a[i][c + j] = tile[wid][ln][j];
+    }
   }
+  // the warp's row of the largest |a_rk|, r >= k, the lowest of equals
+  uint64_t best = 0;
+  int arg = k0;
+  auto candidate = [&](int i, int k, T x) {
+    const int r = threadIdx.x + i * blockDim.x;
+    const uint64_t v = abs_key(x);
+    if (r >= k && r < n && (v > best || (v == best && r < arg))) { best = v; arg = r; }
+  };
+#pragma unroll
+  for (int i = 0; i < R; ++i) candidate(i, k0, a[i][0]);
+  warp_arg_max<T>(best, arg);
   // The loop stays rolled (unrolled it is 80 KB of code that runs once): the
   // current column is always a[.][0], each step writes its results one place
   // down and the finished column to the end.
 #pragma unroll 1
   for (int kk = 0; kk < nb; ++kk) {
     const int k = k0 + kk, sl = kk & 1;
-    // row of the largest |a_rk|, r >= k, the lowest of equals
-    uint64_t best = 0;
-    int arg = k;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int r = threadIdx.x + i * blockDim.x;
-      const uint64_t v = abs_key(a[i][0]);
-      if (r >= k && r < n && (v > best || (v == best && r < arg))) { best = v; arg = r; }
-    }
-    warp_arg_max<T>(best, arg);
     if (ln == 0) { wv[sl][wid] = best; wr[sl][wid] = arg; }
     __syncthreads();
     best = ln < nw ? wv[sl][ln] : 0;
@@ -470,7 +494,12 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
       const int r = threadIdx.x + i * blockDim.x;
       if (r == p) {
 #pragma unroll
-        for (int c = 0; c < NB; ++c) prow[sl][c] = a[i][c];
+        for (int c = 0; c < NB; c += L) {
+          Row v;
+#pragma unroll
+          for (int j = 0; j < L; ++j) v.a[j] = a[i][c + j];
+          prow[sl][c / L] = v;
+        }
         psrc[sl] = src[i];
         const bool ok = fabs(a[i][0]) > T(0);  // false for NaN too
         if (!ok) *bad = 1;
@@ -478,32 +507,56 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
       }
       if (r == k) {
 #pragma unroll
-        for (int c = 0; c < NB; ++c) krow[sl][c] = a[i][c];
+        for (int c = 0; c < NB; c += L) {
+          Row v;
+#pragma unroll
+          for (int j = 0; j < L; ++j) v.a[j] = a[i][c + j];
+          krow[sl][c / L] = v;
+        }
         ksrc[sl] = src[i];
       }
     }
     __syncthreads();
     const T d = dinv[sl];
+    T fr[R];
+    best = 0;
+    arg = k + 1;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       const int r = threadIdx.x + i * blockDim.x;
       if (r == p && p != k) {
 #pragma unroll
-        for (int c = 0; c < NB; ++c) a[i][c] = krow[sl][c];
+        for (int c = 0; c < NB; c += L) {
+          const Row v = krow[sl][c / L];
+#pragma unroll
+          for (int j = 0; j < L; ++j) a[i][c + j] = v.a[j];
+        }
         src[i] = ksrc[sl];
       }
       // row k: prow d; the others: a - (a_k d) prow
-      T fr = -a[i][0] * d;
+      fr[i] = -a[i][0] * d;
       if (r == k) {
         src[i] = psrc[sl];
-        fr = d;
+        fr[i] = d;
 #pragma unroll
         for (int c = 1; c < NB; ++c) a[i][c] = T(0);
       }
-#pragma unroll
-      for (int c = 1; c < NB; ++c) a[i][c - 1] = fma(fr, prow[sl][c], a[i][c]);
-      a[i][NB - 1] = fr;
+      // the next column first: its pivot search overlaps the other products
+      a[i][0] = fma(fr[i], prow[sl][0].a[1], a[i][1]);
+      candidate(i, k + 1, a[i][0]);
     }
+    warp_arg_max<T>(best, arg);
+#pragma unroll
+    for (int c = 0; c < NB; c += L) {
+      const Row v = prow[sl][c / L];
+#pragma unroll
+      for (int j = 0; j < L; ++j)
+        if (c + j > 1)
+#pragma unroll
+          for (int i = 0; i < R; ++i) a[i][c + j - 1] = fma(fr[i], v.a[j], a[i][c + j]);
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) a[i][NB - 1] = fr[i];
   }
 #pragma unroll
   for (int i = 0; i < R; ++i) {
@@ -512,7 +565,7 @@ __global__ void __launch_bounds__(1024) k_gj_panel(const T *__restrict__ Mall, i
     // a narrow last panel: its nb columns have moved to the end
 #pragma unroll
     for (int c = 0; c < NB; ++c)
-      if (c >= NB - nb) G[int64_t(r) * NB + c - (NB - nb)] = a[i][c];
+      if (c >= NB - nb) G[int64_t(c - (NB - nb)) * n + r] = a[i][c];  // column by column
     const int64_t o = int64_t(blockIdx.x) * n;
     permall[o + r] = src[i];
     origin_out[o + r] = origin_in[o + src[i]];
@@ -533,9 +586,10 @@ __global__ void __launch_bounds__(256) k_gj_update(const T *__restrict__ inall, 
   const int nb = min(NB, n - k0);
   const int r0 = blockIdx.y * TS, j0 = blockIdx.x * TS;
   __shared__ T g[TS][NB + 1], u[NB][TS];
+  wait_previous(in, out, G, perm);
   for (int t = threadIdx.x; t < TS * NB; t += 256) {
-    const int r = t / NB, c = t % NB;
-    g[r][c] = r0 + r < n && c < nb ? G[int64_t(r0 + r) * NB + c] : T(0);
+    const int r = t % TS, c = t / TS;
+    g[r][c] = r0 + r < n && c < nb ? G[int64_t(c) * n + r0 + r] : T(0);
   }
   for (int t = threadIdx.x; t < NB * TS; t += 256) {
     const int c = t / TS, j = t % TS;
@@ -714,8 +768,9 @@ T *gj_panels(T *buf0, T *buf1, int64_t n, int n_inst, T *G, int32_t *idx, int32_
   int32_t *perm = idx, *o0 = idx + n * n_inst, *o1 = idx + 2 * n * n_inst;
   k_gj_init<<<grid_n(n * n_inst), kB, 0, st>>>(o0, n, n_inst);
   for (int64_t k = 0; k < n; k += NB) {
-    k_gj_panel<T, NB, R><<<n_inst, threads, 0, st>>>(buf0, int(n), int(k), G, perm, o0, o1, bad);
-    k_gj_update<T, NB, TS><<<dim3(tiles, tiles, (unsigned)n_inst), 256, 0, st>>>(buf0, buf1, int(n), int(k), G, perm);
+    launch_next(k_gj_panel<T, NB, R>, (unsigned)n_inst, threads, st, buf0, int(n), int(k), G, perm, o0, o1, bad);
+    launch_next(k_gj_update<T, NB, TS>, dim3(tiles, tiles, (unsigned)n_inst), 256, st, buf0, buf1, int(n), int(k), G,
+                perm);
     std::swap(buf0, buf1);
     std::swap(o0, o1);
     note_launches(2);
