@@ -129,7 +129,8 @@ template <typename T> __device__ __forceinline__ Dl<T> nrsqrt_(Dl<T> a) {
   return Dl<T>(r, (a.d * T(-0.5f)) * (r * r) * r);
 }
 
-// x 2^k, exact.  In double on the exponent bits: the FP64 pipe issues one
+// x 2^k, exact, for constants (an infinity or NaN would come out as some number).
+// In double on the exponent bits: the FP64 pipe issues one
 // warp instruction every 16 cycles on this part, the integer pipe is idle (x
 // is zero or normal, and so is the result for box extents between 1e-60 and
 // 1e60 and levels up to 20: |k| <= 80).
@@ -1283,8 +1284,7 @@ __global__ void __launch_bounds__(256) k_energy(
     double phi, g[D], t = 0.0;
     ip_vg<D>(u[D + 1], s, phi, g);
 #pragma unroll
-    for (int a = 0; a < D; ++a) t = fma(g[a] * g[a], c.kg[a], t);
-    t = scale2(t, 2 * l);
+    for (int a = 0; a < D; ++a) t = fma(g[a] * g[a], scale2(c.kg[a], 2 * l), t);
     // phi*: bits of |phi| compare like the numbers; NaN stays NaN
     const int sg = __double2hiint(phi), hi = sg & 0x7fffffff;
     const double phis = hi < 0x3ff00000 || hi > 0x7ff00000 ? phi : flip_if(1.0, sg < 0);
