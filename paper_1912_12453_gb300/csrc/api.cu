@@ -1080,45 +1080,27 @@ chns_status chns_init_mu(const chns_mesh *mc, const chns_params *p, double *U, v
   // M mu_new = M mu + F_mu(U; U): conjugate gradients on scalar node vectors,
   // preconditioned by the lumped mass (the row sums of M), which keeps the
   // iteration count bounded however much the leaf sizes differ.  M is applied
-  // on its own, not through the J.w of all fields, and the loop runs on the
-  // device: the host queues kAhead iterations at a time and reads the flags of
-  // the previous ones meanwhile.  77,932 leaves, 72 iterations: 99.8 -> 4.4 ms.
+  // on its own, not through the J.w of all fields, and the iteration runs on the
+  // device (launch_cg).
   TRY(ws.V.ensure(sizeof(double) * 6 * n));
   TRY(ws.e64.ensure(sizeof(double) * (m->n_elem << m->dim)));
-  TRY(ws.red.ensure(sizeof(double) * (kMaxRestart + 16) * red_blocks()));
+  TRY(ws.red.ensure(sizeof(double) * std::max<int64_t>((kMaxRestart + 16) * red_blocks(), cg_partials())));
   TRY(ws.hdev.ensure(sizeof(double) * 8 * kHessSlot));
   TRY(ws.ctr.ensure(64));
   TRY(ensure_pinned(ws));
-  TRY(ensure_events(ws, 2));
-  double *r = ws.V.as<double>(), *x = r + n, *pv = r + 2 * n, *q = r + 3 * n, *d = r + 4 * n, *z = r + 5 * n;
-  double *E = ws.e64.as<double>(), *part = ws.red.as<double>();
+  double *E = ws.e64.as<double>(), *v = ws.V.as<double>(), *x = v + n;
   CgState *s = ws.hdev.as<CgState>(), *hs = reinterpret_cast<CgState *>(ws.hpinned);
   unsigned *ctr = ws.ctr.as<unsigned>();
   CHNS_CUDA_TRY(cudaMemsetAsync(ctr, 0, 64, st));
   launch_mu_row(m, pc, U, E, st);
-  cg_nodes(m, E, nullptr, nullptr, r, s, part, ctr, st);
-  vec_fill(z, n, 1.0, st);
-  launch_mass(m, pc, z, nullptr, nullptr, nullptr, E, st);
-  cg_nodes(m, E, nullptr, nullptr, d, s, part, ctr, st);
-  cg_start(n, d, r, z, x, pv, s, part, ctr, st);
-  constexpr int kAhead = 4, kMaxIt = 10000;
-  int queued = 0;
-  for (int slot = 0;; slot ^= 1) {
-    for (int k = 0; k < kAhead && queued < kMaxIt; ++k, ++queued) {
-      launch_mass(m, pc, z, pv, &s->beta, &s->done, E, st);
-      cg_nodes(m, E, z, pv, q, s, part, ctr, st);
-      cg_update(n, d, pv, q, x, r, z, s, part, ctr, st);
-    }
-    CHNS_CUDA_TRY(cudaMemcpyAsync(&hs[slot], s, sizeof(CgState), cudaMemcpyDeviceToHost, st));
-    CHNS_CUDA_TRY(cudaEventRecord(ws.ev[slot], st));
-    if (queued > kAhead) {
-      CHNS_CUDA_TRY(cudaEventSynchronize(ws.ev[slot ^ 1]));
-      if (hs[slot ^ 1].done) break;
-      if (queued >= kMaxIt) break;
-    }
-  }
+  CHNS_CUDA_TRY(launch_cg(m, pc, E, v, ws.red.as<double>(), ctr, s, 10000, st));
+  CHNS_CUDA_TRY(cudaMemcpyAsync(hs, s, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+  CHNS_CUDA_TRY(cudaMemsetAsync(ctr, 0, 64, st));  // the other users' counters start at zero
   CHNS_CUDA_TRY(cudaStreamSynchronize(st));
-  if (hs[0].err || hs[1].err) { set_error("mass matrix not positive in CG"); return CHNS_ERR_KRYLOV; }
+  if (hs->err) {
+    set_error(hs->err == 1 ? "mass matrix not positive in CG" : "grid barrier given up in CG");
+    return CHNS_ERR_KRYLOV;
+  }
   vec_add_field(U, x, n, m->nf, m->dim + 2, st);
   return check_launch();
 }

@@ -1024,30 +1024,211 @@ __device__ __forceinline__ double gather1(int cn, const int32_t *__restrict__ ha
   return 0.25 * (a + (__ldg(u + int64_t(p.z) * S + k) + __ldg(u + int64_t(p.w) * S + k)));
 }
 
-// Element-local part of the Q1 mass matrix times p' = z + *beta p (a scalar
-// per node) into the slots E.  With the 2-point Gauss rule the element matrix
-// is the product over the axes of (h/6) [2 1; 1 2]: u + o/2 per axis and one
-// factor W (2/3)^D, nine FP64 instructions a lane.  The J.w of all fields took
-// 72 times a full apply (1.27 ms on 77,932 leaves) for the same product.
-template <int D>
-__global__ void __launch_bounds__(256) k_mass(const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
-                                              const int32_t *__restrict__ hang, int64_t n_elem,
-                                              const double *__restrict__ z, const double *__restrict__ p,
-                                              const double *__restrict__ beta, const int *__restrict__ done, double W0,
-                                              double *__restrict__ E) {  // W0: of level 0, with the factor
-  constexpr int NC = 1 << D;
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  int64_t e = t >> D;
-  const bool active = e < n_elem;
-  if (!active) e = n_elem - 1;
-  const int cn = conn[e * NC + (threadIdx.x & (NC - 1))], l = level[e];
-  wait_previous(z, p, beta, done, E);
-  if (done && *done) return;
-  double u = gather1<1>(cn, hang, z, 0);
-  if (p) u = fma(*beta, gather1<1>(cn, hang, p, 0), u);
+// Conjugate gradients on the Q1 mass matrix (a scalar per node), preconditioned
+// by its row sums, the whole iteration in one cooperative kernel.  With the
+// 2-point Gauss rule the element matrix is the product over the axes of
+// (h/6) [2 1; 1 2]: u + o/2 per axis and one factor W (2/3)^D, nine FP64
+// instructions a lane.
+//
+// An iteration is three phases with a grid barrier after each: element products
+// into the slots E, node sums with p.q, vector update with r.z and r.r.  Bound:
+// the barriers, the sums and the first loads of each phase, about 12 us an
+// iteration even on a mesh of 4,096 leaves; the FP64 pipe is worth about 8 of
+// the 34 us on 77,932 leaves.  Three launches an iteration -> one kernel, whole
+// call: 77,932 leaves 3.48 -> 2.47 ms, 4,096 uniform 1.28 -> 1.13, 262,144 3.44
+// -> 2.57, 1,375,648 25.6 -> 22.3, 6,976,432 110 -> 114 (there half the threads
+// an SM could hold cost more than the launches did).
+// Block shape, 77,932 / 4,096 leaves: 1,024 threads with two products in flight
+// 2.48 / 1.13 ms, with four 2.52 / 1.31, 512 x 2 2.55 / 1.09, 512 x 3 2.95 /
+// 1.03, 256 x 6 3.54 / 0.97: more blocks, more partial sums to add.
+// Sums go through shared memory to one warp a scheduler: a shuffle sum in every
+// warp is five FP64 instructions a warp of 64 cycles each.  Every block adds the
+// blocks' partial sums itself, in the same order, so all of them take the same
+// decisions.  What other blocks wrote is read past L1 (__ldcg).  Warps, not
+// blocks, are dealt out over the nodes: the last round is spread over all SMs.
+constexpr int kCgBlock = 1024, kCgPerSm = 1, kCgMaxGrid = 512, kCgUnroll = 2;
+constexpr int kCgPolls = 1 << 25;  // about 20 s: a barrier that never fills ends as an error
+
+struct CgArgs {
+  const int32_t *conn, *hang, *gptr, *gent;
+  const uint8_t *level;
+  int64_t n_elem, n;
+  double W0;  // of level 0, with the factor (2/3)^D
+  double *E, *r, *x, *p, *q, *d, *z, *partial;
+  unsigned *bar;
+  CgState *s;
+  int max_it;
+};
+
+__device__ __forceinline__ double gather1_l2(int cn, const int32_t *__restrict__ hang, const double *u) {
+  if (cn >= 0) return __ldcg(u + cn);
+  const int4 p = reinterpret_cast<const int4 *>(hang)[-cn - 1];
+  const double a = __ldcg(u + p.x) + __ldcg(u + p.y);
+  if (p.z < 0) return 0.5 * a;
+  return 0.25 * (a + (__ldcg(u + p.z) + __ldcg(u + p.w)));
+}
+
+// all blocks have arrived for the epoch-th time; false: given up
+__device__ __forceinline__ bool cg_barrier(unsigned *bar, unsigned &epoch, int *given_up) {
+  ++epoch;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    const unsigned want = epoch * gridDim.x;
+    unsigned have;
+    int polls = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(have) : "l"(bar) : "memory");
+    } while (have < want && ++polls < kCgPolls);
+    *given_up = have < want;
+    __threadfence();
+  }
+  __syncthreads();
+  return !*given_up;
+}
+
+// tot[v] = sum over all threads of the grid of acc[v], with a grid barrier
+template <int N>
+__device__ __forceinline__ bool cg_sum(const double (&acc)[N], double *tot, double *partial, unsigned *bar,
+                                       unsigned &epoch, int *given_up) {
+  __shared__ double all[N][kCgBlock], four[N][4];
+  const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
 #pragma unroll
-  for (int a = 0; a < D; ++a) u = fma(0.5, __shfl_xor_sync(FULL, u, 1 << a), u);
-  if (active) E[t] = scale2(W0, -D * l) * u;
+  for (int v = 0; v < N; ++v) all[v][threadIdx.x] = acc[v];
+  __syncthreads();
+  if (wid < 4 * N) {
+    const double *a = all[wid >> 2] + (wid & 3) * (kCgBlock / 4);
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < kCgBlock / 128; ++k) t += a[k * 32 + ln];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL, t, o);
+    if (ln == 0) four[wid >> 2][wid & 3] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x < N) {
+    const double *f = four[threadIdx.x];
+    __stcg(partial + threadIdx.x * gridDim.x + blockIdx.x, (f[0] + f[1]) + (f[2] + f[3]));
+  }
+  if (!cg_barrier(bar, epoch, given_up)) return false;
+  if (wid < N) {
+    double t = 0.0;
+    for (unsigned b = ln; b < gridDim.x; b += 32) t += __ldcg(partial + wid * gridDim.x + b);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL, t, o);
+    if (ln == 0) tot[wid] = t;
+  }
+  __syncthreads();
+  return true;
+}
+
+__device__ __forceinline__ double cg_node_sum(const CgArgs &g, int64_t i) {
+  double sum = 0.0;
+  const int e1 = g.gptr[i + 1];
+  constexpr int G = 8;  // independent loads, then the sum in list order
+  for (int e = g.gptr[i]; e < e1; e += G) {
+    uint32_t ent[G];
+    double v[G];
+#pragma unroll
+    for (int k = 0; k < G; ++k) ent[k] = e + k < e1 ? uint32_t(g.gent[e + k]) : 0xffffffffu;
+#pragma unroll
+    for (int k = 0; k < G; ++k) v[k] = ent[k] != 0xffffffffu ? __ldcg(g.E + (ent[k] & 0x3fffffffu)) : 0.0;
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const uint32_t code = ent[k] >> 30;  // 3: past the end, v = 0
+      sum = fma(code == 0 ? 1.0 : (code == 1 ? 0.5 : 0.25), v[k], sum);
+    }
+  }
+  return sum;
+}
+
+// E: the right-hand side's element parts; x = M^-1 (their node sums)
+template <int D>
+__global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant__ CgArgs g) {
+  constexpr int NC = 1 << D, U = kCgUnroll;
+  const int lc = threadIdx.x & (NC - 1);
+  const int64_t step = int64_t(gridDim.x) * kCgBlock;
+  const int64_t t0 = (int64_t(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+  const int64_t slots = g.n_elem << D;
+  __shared__ int given_up;
+  __shared__ double tot[2], tpq[1], ash;
+  unsigned epoch = 0;
+  int err = 0, it = 0;
+  for (int64_t i = t0; i < g.n; i += step) g.r[i] = cg_node_sum(g, i);
+  if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; goto end; }
+  for (int64_t t = t0; t < slots; t += step)
+    g.E[t] = scale2(g.W0, -D * int(g.level[t >> D])) * (D == 2 ? 2.25 : 3.375);  // the product with ones
+  if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; goto end; }
+  {
+    double acc[2] = {0.0, 0.0};
+    for (int64_t i = t0; i < g.n; i += step) {
+      const double m = cg_node_sum(g, i), di = m > 0.0 ? 1.0 / m : 0.0, ri = g.r[i], zi = di * ri;
+      g.d[i] = di;
+      g.z[i] = zi;
+      g.x[i] = 0.0;
+      g.p[i] = 0.0;
+      acc[0] = fma(ri, zi, acc[0]);
+      acc[1] = fma(ri, ri, acc[1]);
+    }
+    if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, &given_up)) { err = 2; goto end; }
+  }
+  {
+    double rz = tot[0], rr = tot[1], beta = 0.0;
+    const double stop = 1e-26 * fmax(rr, 1e-300);
+    for (; it < g.max_it && rr > stop && rz > 0.0; ++it) {
+      for (int64_t b = t0; b - (threadIdx.x & 31) < slots; b += U * step) {  // whole warps: shuffles
+        int cn[U], l[U];
+        double u[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+          const int64_t t = b + k * step, e = (t < slots ? t : slots - NC + lc) >> D;
+          cn[k] = g.conn[e * NC + lc];
+          l[k] = g.level[e];
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) u[k] = fma(beta, gather1_l2(cn[k], g.hang, g.p), gather1_l2(cn[k], g.hang, g.z));
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+#pragma unroll
+          for (int a = 0; a < D; ++a) u[k] = fma(0.5, __shfl_xor_sync(FULL, u[k], 1 << a), u[k]);
+          const int64_t t = b + k * step;
+          if (t < slots) g.E[t] = scale2(g.W0, -D * l[k]) * u[k];
+        }
+      }
+      if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; break; }
+      double pq[1] = {0.0}, acc[2] = {0.0, 0.0};
+      for (int64_t i = t0; i < g.n; i += step) {
+        const double sum = cg_node_sum(g, i), pi = fma(beta, g.p[i], g.z[i]);
+        g.q[i] = sum;
+        g.p[i] = pi;
+        pq[0] = fma(pi, sum, pq[0]);
+      }
+      if (!cg_sum<1>(pq, tpq, g.partial + 2 * gridDim.x, g.bar, epoch, &given_up)) { err = 2; break; }
+      if (!(tpq[0] > 0.0)) { err = 1; break; }
+      if (threadIdx.x == 0) ash = rz / tpq[0];  // one division a block: ten instructions of the FP64 pipe
+      __syncthreads();
+      const double a = ash;
+      for (int64_t i = t0; i < g.n; i += step) {
+        g.x[i] = fma(a, g.p[i], g.x[i]);
+        const double ri = fma(-a, g.q[i], g.r[i]), zi = g.d[i] * ri;
+        g.r[i] = ri;
+        g.z[i] = zi;
+        acc[0] = fma(ri, zi, acc[0]);
+        acc[1] = fma(ri, ri, acc[1]);
+      }
+      if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, &given_up)) { err = 2; break; }
+      if (threadIdx.x == 0) ash = tot[0] / rz;
+      __syncthreads();
+      beta = ash;
+      rz = tot[0];
+      rr = tot[1];
+      __syncthreads();  // tot and ash are read before the next sums
+    }
+  }
+end:
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    g.s->err = err;
+    g.s->its = it;
+  }
 }
 
 // Element-local part of the chemical-potential row at U_new = U_old = U:
@@ -1628,14 +1809,32 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
   note_launches(1);
 }
 
-void launch_mass(const chns_mesh *m, const PhysCoef &pc, const double *z, const double *p, const double *beta,
-                 const int *done, double *E, cudaStream_t st) {
-  const KCoef<double> c = kcoef<double>(pc, m->dim);
-  const unsigned g = grid_for(m->n_elem << m->dim);
-  const double W0 = c.W0 * (m->dim == 2 ? 4.0 / 9.0 : 8.0 / 27.0);
-  if (m->dim == 2) launch_next(k_mass<2>, g, kBlock, st, m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, W0, E);
-  else launch_next(k_mass<3>, g, kBlock, st, m->conn, m->level, m->hang, m->n_elem, z, p, beta, done, W0, E);
+// x = M^-1 (node sums of E); v: six vectors of n_nodes; part: at least
+// cg_partials() doubles; ctr: zero.  Status in *s (err 1: M not positive, 2: a
+// barrier was given up).
+int cg_partials() { return 3 * kCgMaxGrid; }
+cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double *v, double *part, unsigned *ctr,
+                      CgState *s, int max_it, cudaStream_t st) {
+  CgArgs g{};
+  const int64_t n = m->n_nodes;
+  g.conn = m->conn; g.hang = m->hang; g.gptr = m->gptr; g.gent = m->gent; g.level = m->level;
+  g.n_elem = m->n_elem; g.n = n;
+  g.W0 = kcoef<double>(pc, m->dim).W0 * (m->dim == 2 ? 4.0 / 9.0 : 8.0 / 27.0);
+  g.E = E; g.r = v; g.x = v + n; g.p = v + 2 * n; g.q = v + 3 * n; g.d = v + 4 * n; g.z = v + 5 * n;
+  g.partial = part; g.bar = ctr; g.s = s; g.max_it = max_it;
+  int dev = 0, sms = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const void *k = m->dim == 2 ? reinterpret_cast<const void *>(k_cg<2>) : reinterpret_cast<const void *>(k_cg<3>);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kCgBlock, 0);
+  if (e != cudaSuccess) return e;
+  // a warp of slots each is enough for a small mesh: fewer blocks, cheaper barriers
+  const int64_t want = ((m->n_elem << m->dim) + kCgBlock - 1) / kCgBlock;
+  const int grid = int(std::max<int64_t>(1, std::min<int64_t>({want, int64_t(sms) * per, kCgMaxGrid})));
+  void *args[] = {&g};
+  e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kCgBlock), args, 0, st);
   note_launches(1);
+  return e;
 }
 
 void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st) {

@@ -33,11 +33,17 @@ void launch_jacvec_defect(const chns_mesh *m, const PhysCoef &pc, const T *ut, c
                           T *E, T *x, T *r, cudaStream_t st);
 void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo,
                             unsigned long long *count, cudaStream_t st);
-// scalar Q1 mass matrix times z + *beta p (p nullable: z), and the
-// chemical-potential row of U, into element-local slots (n_elem * 2^dim
-// doubles); launch_mass does nothing once *done (nullable) is set
-void launch_mass(const chns_mesh *m, const PhysCoef &pc, const double *z, const double *p, const double *beta,
-                 const int *done, double *E, cudaStream_t st);
+// x (the second of the six vectors of n_nodes doubles at v) = M^-1 (node sums of
+// the element-local slots E), M the scalar Q1 mass matrix, by conjugate gradients
+// in one cooperative kernel; part: cg_partials() doubles, ctr: zero.  Status in
+// *s on the device: err 1: M not positive, 2: a grid barrier was given up
+struct CgState {
+  int err, its;
+};
+int cg_partials();
+cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double *v, double *part, unsigned *ctr,
+                      CgState *s, int max_it, cudaStream_t st);
+// the chemical-potential row of U into element-local slots (n_elem * 2^dim doubles)
 void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st);
 int64_t energy_blocks(const chns_mesh *m);
 // per-instance element coefficients of a batched (union) mesh

@@ -341,122 +341,6 @@ __global__ void k_max_partials(const double *__restrict__ partial, int nb, doubl
   }
 }
 
-// ---------------------------------------------------------------- conjugate gradients on the mass matrix
-// Scalars (rz, rr, p.q, stop, beta) and flags stay on the device: three
-// launches an iteration (k_mass, k_cg_nodes, k_cg_update), nothing waits for
-// the host, and once `done` is set the launches still queued return at once.
-
-// q[i] = sum over the slots of node i of weight * E[slot]; with z: also p[i] =
-// z[i] + beta p[i] and s->pq = p . q
-__global__ void __launch_bounds__(kB) k_cg_nodes(const int32_t *__restrict__ gptr, const int32_t *__restrict__ gent,
-                                                 int64_t n, const double *__restrict__ E, const double *__restrict__ z,
-                                                 double *__restrict__ p, double *__restrict__ q, CgState *s,
-                                                 double *__restrict__ partial, unsigned *__restrict__ counter) {
-  wait_previous(E, z, p, q, s, partial, counter);
-  if (z && s->done) return;
-  const double beta = z ? s->beta : 0.0;
-  double acc[1] = {0.0};
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
-    double sum = 0.0;
-    const int e1 = gptr[i + 1];
-    constexpr int G = 8;  // independent loads, then the sum in list order
-    for (int e = gptr[i]; e < e1; e += G) {
-      uint32_t ent[G];
-      double v[G];
-#pragma unroll
-      for (int g = 0; g < G; ++g) ent[g] = e + g < e1 ? uint32_t(gent[e + g]) : 0xffffffffu;
-#pragma unroll
-      for (int g = 0; g < G; ++g) v[g] = ent[g] != 0xffffffffu ? E[ent[g] & 0x3fffffffu] : 0.0;
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const uint32_t code = ent[g] >> 30;  // 3: past the end, v = 0
-        sum = fma(code == 0 ? 1.0 : (code == 1 ? 0.5 : 0.25), v[g], sum);
-      }
-    }
-    q[i] = sum;
-    if (z) {
-      const double pi = fma(beta, p[i], z[i]);
-      p[i] = pi;
-      acc[0] = fma(pi, sum, acc[0]);
-    }
-  }
-  if (!z) return;
-  block_sum_store<double, 1>(acc, partial);
-  if (last_block(counter)) {
-    sum_rows<double>(partial, 1, &s->pq);
-    if (threadIdx.x == 0) *counter = 0;
-  }
-}
-
-// the two sums of k_cg_start / k_cg_update, by the last block: rr, rz and what
-// follows from them
-__device__ __forceinline__ void cg_sums(double (&acc)[2], CgState *s, double *partial, unsigned *counter, bool start) {
-  block_sum_store<double, 2>(acc, partial);
-  if (!last_block(counter)) return;
-  __shared__ double tot[2];
-  sum_rows<double>(partial, 2, tot);
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double rz = tot[0], rr = tot[1];
-  if (start) s->stop = 1e-26 * fmax(rr, 1e-300);
-  s->beta = start ? 0.0 : rz / s->rz;
-  s->rz = rz;
-  s->rr = rr;
-  s->done = !(rr > s->stop && rz > 0.0);
-  s->err = 0;
-  *counter = 0;
-}
-
-// d <- 1/d (0 where d <= 0), z = d r, x = p = 0
-__global__ void __launch_bounds__(kB) k_cg_start(int64_t n, double *__restrict__ d, const double *__restrict__ r,
-                                                 double *__restrict__ z, double *__restrict__ x,
-                                                 double *__restrict__ p, CgState *s, double *__restrict__ partial,
-                                                 unsigned *__restrict__ counter) {
-  double acc[2] = {0.0, 0.0};
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
-    const double di = d[i] > 0.0 ? 1.0 / d[i] : 0.0, ri = r[i], zi = di * ri;
-    d[i] = di;
-    z[i] = zi;
-    x[i] = 0.0;
-    p[i] = 0.0;
-    acc[0] = fma(ri, zi, acc[0]);
-    acc[1] = fma(ri, ri, acc[1]);
-  }
-  cg_sums(acc, s, partial, counter, true);
-}
-
-// x += a p, r -= a q (a = rz / p.q), z = d r
-__global__ void __launch_bounds__(kB) k_cg_update(int64_t n, const double *__restrict__ d, const double *__restrict__ p,
-                                                  const double *__restrict__ q, double *__restrict__ x,
-                                                  double *__restrict__ r, double *__restrict__ z, CgState *s,
-                                                  double *__restrict__ partial, unsigned *__restrict__ counter) {
-  wait_previous(d, p, q, x, r, z, s, partial, counter);
-  if (s->done) return;
-  const double pq = s->pq;
-  if (!(pq > 0.0)) {  // every block returns here: the ticket is not touched
-    if (blockIdx.x == 0 && threadIdx.x == 0) s->err = s->done = 1;
-    return;
-  }
-  __shared__ double ash;  // one division a block: it costs ten instructions of the FP64 pipe
-  if (threadIdx.x == 0) ash = s->rz / pq;
-  __syncthreads();
-  const double a = ash;
-  double acc[2] = {0.0, 0.0};
-  for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n; i += int64_t(gridDim.x) * kB) {
-    x[i] = fma(a, p[i], x[i]);
-    const double ri = fma(-a, q[i], r[i]), zi = d[i] * ri;
-    r[i] = ri;
-    z[i] = zi;
-    acc[0] = fma(ri, zi, acc[0]);
-    acc[1] = fma(ri, ri, acc[1]);
-  }
-  cg_sums(acc, s, partial, counter, false);
-}
-
-__global__ void k_fill(double *__restrict__ y, int64_t n, double v) {
-  for (int64_t t = blockIdx.x * int64_t(kB) + threadIdx.x; t < n; t += int64_t(gridDim.x) * kB) y[t] = v;
-}
-
 // field k of each node block += x
 __global__ void k_add_field(double *__restrict__ U, const double *__restrict__ x, int64_t n_nodes, int nf, int k) {
   for (int64_t i = blockIdx.x * int64_t(kB) + threadIdx.x; i < n_nodes; i += int64_t(gridDim.x) * kB)
@@ -532,7 +416,6 @@ static unsigned red_grid(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n / V16<T>::L + kB - 1) / kB, kRedBlocks));
 }
 // one node per thread up to the reduction's block count
-static unsigned cg_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + kB - 1) / kB, kRedBlocks); }
 
 template <typename T>
 void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double *partial, double *h,
@@ -641,31 +524,8 @@ void vec_maxabs_diff(const double *x, const double *y, int64_t n, double *partia
   note_launches(2);
 }
 
-void vec_fill(double *y, int64_t n, double v, cudaStream_t st) {
-  k_fill<<<grid_n(n), kB, 0, st>>>(y, n, v);
-  note_launches(1);
-}
-
 void vec_add_field(double *U, const double *x, int64_t n_nodes, int nf, int k, cudaStream_t st) {
   k_add_field<<<grid_n(n_nodes), kB, 0, st>>>(U, x, n_nodes, nf, k);
-  note_launches(1);
-}
-
-void cg_nodes(const chns_mesh *m, const double *E, const double *z, double *p, double *q, CgState *s, double *partial,
-              unsigned *counter, cudaStream_t st) {
-  launch_next(k_cg_nodes, cg_grid(m->n_nodes), kB, st, m->gptr, m->gent, m->n_nodes, E, z, p, q, s, partial, counter);
-  note_launches(1);
-}
-
-void cg_start(int64_t n, double *d, const double *r, double *z, double *x, double *p, CgState *s, double *partial,
-              unsigned *counter, cudaStream_t st) {
-  k_cg_start<<<cg_grid(n), kB, 0, st>>>(n, d, r, z, x, p, s, partial, counter);
-  note_launches(1);
-}
-
-void cg_update(int64_t n, const double *d, const double *p, const double *q, double *x, double *r, double *z,
-               CgState *s, double *partial, unsigned *counter, cudaStream_t st) {
-  launch_next(k_cg_update, cg_grid(n), kB, st, n, d, p, q, x, r, z, s, partial, counter);
   note_launches(1);
 }
 

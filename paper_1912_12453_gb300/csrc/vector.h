@@ -49,21 +49,8 @@ void vec_lincomb(double a, const double *x, double b, const double *y, double *z
 void vec_mask_fields(double *y, int64_t n_nodes, int nf, uint32_t fmask, cudaStream_t st);
 // *res = max_i |x_i - y_i| (partial: red_blocks() doubles)
 void vec_maxabs_diff(const double *x, const double *y, int64_t n, double *partial, double *res, cudaStream_t st);
-// Conjugate gradients on the mass matrix (device state of one solve)
-struct CgState {
-  double rz, rr, pq, stop, beta;
-  int done, err;
-};
-void vec_fill(double *y, int64_t n, double v, cudaStream_t st);
 // field k of each node block of U += x
 void vec_add_field(double *U, const double *x, int64_t n_nodes, int nf, int k, cudaStream_t st);
-// q = node sums of the slots E; with z: p = z + beta p and s->pq = p . q
-void cg_nodes(const chns_mesh *m, const double *E, const double *z, double *p, double *q, CgState *s, double *partial,
-              unsigned *counter, cudaStream_t st);
-void cg_start(int64_t n, double *d, const double *r, double *z, double *x, double *p, CgState *s, double *partial,
-              unsigned *counter, cudaStream_t st);
-void cg_update(int64_t n, const double *d, const double *p, const double *q, double *x, double *r, double *z,
-               CgState *s, double *partial, unsigned *counter, cudaStream_t st);
 // nv probing vectors from number v0 on (number c nf + f: 1 in field f of the
 // nodes of colour c), and the columns of the nodal blocks they read off
 template <typename T>
