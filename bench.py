@@ -58,14 +58,15 @@ DESCRIPTION = {
                      "ratios 1e-3 / 1e-2, dt 1e-4",
 }
 # FP32 operations per leaf of one J.w apply of the element kernel, counted by
-# ncu on k_element<3, float, J.w> (thread-level FADD + FMUL + 2 x FFMA).  The
+# ncu on k_jv_pair<3> (thread-level FADD + FMUL + 2 x FFMA, and twice these for
+# the packed FADD2, FMUL2, FFMA2).  The
 # kernel does the same arithmetic for every leaf of every 3D mesh (hanging
 # corners only add gather loads), so the count holds for any 3D mesh while the
 # kernel is unchanged.
-JV_FLOP_PER_LEAF = {3: 10825}
+JV_FLOP_PER_LEAF = {3: 7020}
 # DRAM bytes (read + write) of one J.w apply, element kernel + node gather,
 # from one ncu capture of the named workload; valid for that mesh only.
-JV_TRAFFIC_PER_APPLY = {"droplet3d_l6": 45_309_312 + 90_735_360}
+JV_TRAFFIC_PER_APPLY = {"droplet3d_l6": 36_147_968 + 81_940_224}
 # Algorithmic bytes of one FP32 J.w apply per node (read U~, dU and w, write y)
 JV_ALG_BYTES_PER_NODE = {3: 4 * (6 + 4 + 6 + 6), 2: 4 * (5 + 3 + 5 + 5)}
 
@@ -684,7 +685,7 @@ def main():
                 "traffic": traffic,
                 "per": f"one J.w apply inside the timed CN steps (element kernel over {mesh.n_elem} leaves + node "
                        f"gather), {fpl} FP32 flop per leaf (ncu count of the element kernel)",
-                "kernel": "k_element<3,float,J.w> + k_gather_nodes<3,float>",
+                "kernel": "k_jv_pair<3> + k_gather_nodes<3,float>",
                 "peak_source": "FP32 FMA pipe measured in this run (libchns_peak.so), of measured",
                 "algorithmic_bytes_per_apply": alg_bytes,
                 "hbm_gbs_algorithmic": alg_bytes / (jv_apply_ms / 1e3) / 1e9,

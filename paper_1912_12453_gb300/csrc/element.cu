@@ -427,8 +427,9 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 // of two times a constant of the box.  Bound by the FP64 pipe (residual, J.w)
 // and by the FP32 issue slots (J.w in float).  Measured on GB300, before ->
 // after: residual of the level-6 octree (262,144 leaves) 2.34 -> 1.41 ms, FP64
-// J.w of 77,932 adaptive leaves 1.27 -> 0.79 ms, FP32 J.w of the level-6 octree
-// 132 -> 116 us (element kernel alone 88 -> 69 us).
+// J.w of 77,932 adaptive leaves 1.27 -> 0.79 ms (0.75 with the later element
+// order and node gather), FP32 J.w of the level-6 octree with one Gauss point a
+// lane 132 -> 116 us (element kernel alone 88 -> 69 us).
 //
 // nG, CI_GG, inv_trG, CnWeH come per leaf; T is the number type (a pair: two
 // Gauss points), S is T or its dual.
@@ -746,8 +747,12 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
 // All arithmetic of the pair is packed, the last axis' stage stays in the lane.
 // Bound by issue slots with one point a lane (896 instructions per Gauss point:
 // 586 of arithmetic, 125 shuffles): packing halves the arithmetic's slots, the
-// in-lane axis half of the shuffles.  One apply, before -> after: level-6 octree
-// 117 -> 98 us, 1,375,648 adaptive leaves 631 -> 585 us.
+// in-lane axis half of the shuffles: 83.9 -> 37.1 M warp instructions on the
+// level-6 octree, 7,020 flop a leaf.  What bounds it now is the latency of the
+// gathers (54 % of the issue slots used, 128 registers, 14.6 warps an SM).  The
+// element kernel 69 -> 58 us; the whole apply when this came, 117 -> 98 us and
+// 631 -> 585 us (1,375,648 adaptive leaves), with the later element order and
+// node gather 81 and 455 us.
 template <int D>
 struct Stage2 {
   F2 sg[D - 1];  // derivative factors of the lane axes, both halves
@@ -1583,7 +1588,8 @@ template void launch_prep<double>(const chns_mesh *, const double *, const doubl
 // the node gather with the constrained rows, as J.w.  One launch per element
 // colour with in-place adds read and wrote every node once per colour, needed
 // the output zeroed first and left eight partly filled last waves; E costs 96
-// B per corner of L2 / HBM traffic instead, 6 % of the FP64 time.
+// B per corner of L2 / HBM traffic instead: the gather takes 35 of 1,382 us on
+// 262,144 leaves.
 // U_new and U_old are averaged in the element kernel (10 FP64 instructions a
 // lane) rather than by a node pass before it: a state is evaluated once.
 template <int D, bool HASF>
@@ -1615,9 +1621,10 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 //   0-3: two Gauss points per lane (k_jv_pair), all elements at once into the
 //      element-local buffer E (n_elem * 2^dim * nf values), then the node
 //      gather with the constrained rows; (threads, blocks per SM) = (64, 8),
-//      (128, 3), (64, 6), (128, 4).  0 is the default: 14 warps an SM hide the
-//      scattered loads of an adaptive mesh better than 12 (585 against 661 us
-//      on 1,375,648 leaves) and cost 4 % on a uniform one (97.7 against 93.8)
+//      (128, 3), (64, 6), (128, 4).  0 is the default: 16 warps an SM hide the
+//      scattered loads of an adaptive mesh better than 12 (455 against 491 us on
+//      1,375,648 leaves, in spite of 76 bytes of spills) and cost 1 % on a
+//      uniform one (81.0 against 80.4 us, 262,144 leaves)
 //   4: element colours one launch after another, each element adding its
 //      contributions into y (disjoint nodes within a colour; no E buffer),
 //      then the constrained rows
