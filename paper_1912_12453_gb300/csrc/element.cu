@@ -136,7 +136,7 @@ template <typename T> __device__ __forceinline__ Dl<T> nrsqrt_(Dl<T> a) {
 // 1e60 and levels up to 20: |k| <= 80).
 __device__ __forceinline__ double scale2(double x, int k) {
   const int hi = __double2hiint(x);
-  return __hiloint2double(hi == 0 ? 0 : hi + k * (1 << 20), __double2loint(x));
+  return __hiloint2double((hi << 1) == 0 ? hi : hi + k * (1 << 20), __double2loint(x));
 }
 __device__ __forceinline__ float scale2(float x, int k) { return x * __int_as_float((127 + k) << 23); }
 __device__ __forceinline__ double flip_if(double x, bool f) {
@@ -144,6 +144,9 @@ __device__ __forceinline__ double flip_if(double x, bool f) {
 }
 __device__ __forceinline__ float flip_if(float x, bool f) {
   return __int_as_float(__float_as_int(x) ^ (f ? int(0x80000000u) : 0));
+}
+template <typename T> __device__ __forceinline__ Dl<T> flip_if(Dl<T> x, bool f) {
+  return Dl<T>(flip_if(x.v, f), flip_if(x.d, f));
 }
 
 // ---------------------------------------------------------------- butterflies
@@ -393,8 +396,13 @@ struct KPhys {
   T inv_We, ninv_We, CnWe, nCnWe, inv_PeCn, Cn2;
   T ngFr[3];               // - gravity / Fr
 };
+template <typename T> struct KBox {};
+template <> struct KBox<double> {
+  double f0, rf0, nk;  // see kcube
+  double ext, C_I;     // side of the box along the first axis; C_I
+};
 template <typename T>
-struct KCoef : KPhys<T> {
+struct KCoef : KPhys<T>, KBox<T> {
   // geometry of a leaf of level 0; a leaf of level l has these times a power of 2^l
   T nG0[3];                // - G = - 4 / ext^2
   T CIGG0, inv_trG0;       // C_I G:G and 1 / tr G
@@ -433,7 +441,21 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 //
 // nG, CI_GG, inv_trG, CnWeH come per leaf; T is the number type (a pair: two
 // Gauss points), S is T or its dual.
-template <int D, bool HASF, typename T, typename S, typename C>
+//
+// CUBE: a 3D box with equal sides (FP64; c: KCube).  Gradients come as plain
+// differences of the corner data along the lane's own axes (own minus other
+// corner: axis a is reversed where c.neg[a]), so d_a = f sign_a x difference with
+// one f per leaf, and the factors sit in the constants: vt is f sign_i v~_i, cm is
+// f sign_j c_j, V comes out for plain differences of the test functions, the
+// continuity row over f.  Signs of the vector components that are not summed over
+// are flipped back on the bits.  That saves the products of 21 gradients, three
+// mixed derivatives and 18 contraction weights of 352 FP64 instructions a lane:
+// residual of the level-6 octree 1.41 -> 1.26 ms, J.w of 77,932 leaves 0.75 ->
+// 0.68 ms.  Error against plain double code, general form -> this: residual
+// 2.7e-16 -> 2.5e-16 (uniform), 7.3e-16 -> 7.3e-16 (hanging nodes), J.w 2.6e-16 ->
+// 2.6e-16.  In 2D it was 1.5e-16 -> 1.7e-16 (J.w), so 2D keeps the general form;
+// so do other boxes, and union meshes, whose constants come from a table.
+template <int D, bool HASF, bool CUBE, typename T, typename S, typename C>
 __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T inv_trG, T CnWeH,
                                            const GpIn<D, S> &q, const T *f, S *Sq, S (*Vq)[D],
                                            typename Cond<T>::type &floored) {
@@ -461,20 +483,31 @@ __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T i
   const S ntau = nrsqrt_(rad);
   // strong residuals
   S A[D], nt[D];  // nt = - tau_m R_m
-  S divv = q.dvt[0][0];
+  S divv;
+  if constexpr (CUBE) {
+    divv = flip_if(q.dvt[0][0], c.neg[0]);
 #pragma unroll
-  for (int i = 1; i < D; ++i) divv = divv + q.dvt[i][i];
-  if (HASF) divv = subc(divv, f[D]);  // R_c
+    for (int i = 1; i < D; ++i) divv = divv + flip_if(q.dvt[i][i], c.neg[i]);
+  } else {
+    divv = q.dvt[0][0];
+#pragma unroll
+    for (int i = 1; i < D; ++i) divv = divv + q.dvt[i][i];
+  }
+  if constexpr (HASF && CUBE) divv = subc(divv, f[D] * c.rf);
+  else if (HASF) divv = subc(divv, f[D]);  // R_c
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     A[i] = rho * madc(q.dv[i], c.inv_dt, c.ngFr[i]);
     if (HASF) A[i] = subc(A[i], f[i]);
-    S R = mad(q.dpt[i], c.inv_We, A[i]);
+    S R;
+    if constexpr (CUBE) R = mad(flip_if(q.dpt[i], c.neg[i]), c.inv_We, A[i]);
+    else R = mad(q.dpt[i], c.inv_We, A[i]);
     S cap = D == 2 ? q.hphit[0] * q.dphit[1 - i] : S(T(0.0f));
     if (D == 3) {
       const int j0 = i == 0 ? 1 : 0, j1 = i == 2 ? 1 : 2;
       cap = mad(q.hphit[hidx<D>(i, j0)], q.dphit[j0], q.hphit[hidx<D>(i, j1)] * q.dphit[j1 < D ? j1 : 0]);
     }
+    if constexpr (CUBE) cap = flip_if(cap, c.neg[i]);
     R = mad(cap, CnWeH, R);
 #pragma unroll
     for (int j = 0; j < D; ++j) R = mad(q.dvt[i][j], cR[j], R);
@@ -484,7 +517,10 @@ __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T i
   const S ntau_c = (rad * ntau) * inv_trG;
   const S diag = mad(rho * ntau_c, divv, q.pt) * c.ninv_We;
 #pragma unroll
-  for (int j = 0; j < D; ++j) cm[j] = cm[j] + nt[j];
+  for (int j = 0; j < D; ++j) {
+    if constexpr (CUBE) cm[j] = mad(nt[j], c.fs[j], cm[j]);
+    else cm[j] = cm[j] + nt[j];
+  }
   S cphi[D];
 #pragma unroll
   for (int i = 0; i < D; ++i) cphi[i] = q.dphit[i] * c.nCnWe;
@@ -494,7 +530,8 @@ __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T i
 #pragma unroll
     for (int j = 0; j < D; ++j) Si = mad(q.dvt[i][j], cm[j], Si);
     Sq[i] = Si;
-    Vq[D][i] = nt[i] * ninv_rho;  // PSPG; tau_m R_m / rho
+    if constexpr (CUBE) Vq[D][i] = nt[i] * (ninv_rho * c.nk);
+    else Vq[D][i] = nt[i] * ninv_rho;  // PSPG; tau_m R_m / rho
   }
 #pragma unroll
   for (int i = 0; i < D; ++i)
@@ -502,14 +539,24 @@ __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T i
     for (int j = i; j < D; ++j) {
       S cc = cphi[i] * q.dphit[j];
       if (i == j) cc = cc + diag;
-      Vq[i][j] = mad(Vq[D][i], cm[j], mad(etaRe, q.dvt[i][j], cc));
-      if (i != j) Vq[j][i] = mad(Vq[D][j], cm[i], mad(etaRe, q.dvt[j][i], cc));
+      if constexpr (CUBE) {
+        Vq[i][j] = mad(Vq[D][i], cm[j], mad(etaRe, q.dvt[i][j], flip_if(cc, c.neg[i])));
+        if (i != j) Vq[j][i] = mad(Vq[D][j], cm[i], mad(etaRe, q.dvt[j][i], flip_if(cc, c.neg[j])));
+      } else {
+        Vq[i][j] = mad(Vq[D][i], cm[j], mad(etaRe, q.dvt[i][j], cc));
+        if (i != j) Vq[j][i] = mad(Vq[D][j], cm[i], mad(etaRe, q.dvt[j][i], cc));
+      }
     }
+  if constexpr (CUBE)
+#pragma unroll
+    for (int i = 0; i < D; ++i) Vq[D][i] = flip_if(Vq[D][i], c.neg[i]);
   // continuity row
   Sq[D] = divv;
   // Cahn-Hilliard row
   Sq[D + 1] = q.dphi * c.inv_dt;
-  const S nphi = q.phit * T(-1.0f);
+  S nphi;
+  if constexpr (CUBE) nphi = q.phit * -c.nk;
+  else nphi = q.phit * T(-1.0f);
 #pragma unroll
   for (int i = 0; i < D; ++i) Vq[D + 1][i] = mad(q.vt[i], nphi, q.dmut[i] * c.inv_PeCn);
   // chemical-potential row, psi'(phi~) = phi~^3 - phi~
@@ -527,15 +574,62 @@ struct Interp {  // one state interpolated at the lane's Gauss point
   T vt[D], dvt[D][D], pt, dpt[D], phit, dphit[D], hphit[3], mut, dmut[D];
 };
 
-template <int D, bool UNIT, typename T>
-__device__ __forceinline__ void interp_state(const T *u, const Stage<D, T> &s, Interp<D, T> &I) {
+// vs: factors of the velocity components (CUBE; others: the stage's)
+template <int D, bool UNIT, bool CUBE = false, typename T>
+__device__ __forceinline__ void interp_state(const T *u, const Stage<D, T> &s, Interp<D, T> &I,
+                                             const T *vs = nullptr) {
 #pragma unroll
-  for (int i = 0; i < D; ++i) ip_vg<D>(u[i], s, I.vt[i], I.dvt[i]);
+  for (int i = 0; i < D; ++i) {
+    Stage<D, T> si = s;
+    if (CUBE) si.v = vs[i];
+    ip_vg<D>(u[i], si, I.vt[i], I.dvt[i]);
+  }
   ip_vg<D>(u[D], s, I.pt, I.dpt);
   I.hphit[1] = I.hphit[2] = T(0);
   ip_full<D, UNIT>(u[D + 1], s, I.phit, I.dphit, I.hphit);
   ip_vg<D>(u[D + 2], s, I.mut, I.dmut);
 }
+
+// The constants of the CUBE form, per leaf: those of kcube with the powers of two
+// of the level
+template <int D>
+struct KCube : KPhys<double> {
+  double f, rf, nk, fs[D];  // f, 1 / f, factor of V, f with the signs
+  bool neg[D];
+};
+
+// Constants of a box with equal sides, gradients as plain differences (see
+// gp_physics).  f = CA^(D-1) / h of level 0 is the factor of a gradient (half of
+// it for the residual, which sums two states), ft that of the test functions'
+// gradients; the contraction applies CA^D W to a row, so V is over CA^D.  Formed
+// from the side in extended precision and rounded once: a constant's error is the
+// same at every Gauss point, and of f it would enter to the third power.
+KCoef<double> kcube(const KCoef<double> &g, bool raw) {
+  KCoef<double> c = g;
+  typedef long double R;
+  const R ca = R(0.5) + R(0.28867513459481288225457439025L), cad = ca * ca * ca;
+  const R ft = ca * ca / g.ext, f = raw ? ft / 2 : ft, v = ft / cad;
+  c.jcP = double(g.jcP * f * f);
+  c.ngRe = double(g.ngRe * f * f);
+  c.gRe = double(g.gRe * v * f);
+  c.xRe = double(g.xRe * v * f);
+  const R G = 4 / (R(g.ext) * g.ext);
+  for (int a = 0; a < 3; ++a) c.nG0[a] = double(-G / (f * f));
+  c.CIGG0 = double(g.C_I * 3 * G * G / (v * f * v * f));
+  c.inv_trG0 = double(f / (3 * G));
+  c.CnWe = double(g.CnWe * (raw ? 2 : 1) / cad * f * f * f);
+  c.nCnWe = double(g.nCnWe * v * f * f);
+  c.inv_We = double(g.inv_We * f);
+  c.ninv_We = double(g.ninv_We * v);
+  c.inv_PeCn = double(g.inv_PeCn * v * f);
+  c.Cn2 = double(g.Cn2 * v * f);
+  c.f0 = double(f);
+  c.rf0 = double(1 / f);
+  c.nk = double(v / f);
+  return c;
+}
+template <typename T>
+bool is_cube(const KCoef<T> &c) { return c.sg0[0] == c.sg0[1] && c.sg0[0] == c.sg0[2]; }
 
 template <typename T>
 KCoef<T> kcoef(const PhysCoef &p, int dim) {
@@ -556,6 +650,11 @@ KCoef<T> kcoef(const PhysCoef &p, int dim) {
       GG += G * G;
       W *= 0.5 * p.ext[a];
     }
+  }
+  if constexpr (sizeof(T) == 8) {
+    c.f0 = c.rf0 = c.nk = 0.0;
+    c.ext = p.ext[0];
+    c.C_I = p.C_I;
   }
   c.CIGG0 = T(p.C_I * GG);
   c.inv_trG0 = T(1.0 / trG);
@@ -580,7 +679,7 @@ KCoef<T> kcoef(const PhysCoef &p, int dim) {
 // state), the J.w modes the prepared averages and increments.  MODE 1 takes
 // gridDim.y directions at a time (w and out at strides).  BS, MINB: block size
 // and minimum resident blocks per SM (the register budget).
-template <int D, typename T, int MODE, bool HASF, typename O, int BS = 128, int MINB = 6>
+template <int D, typename T, int MODE, bool HASF, typename O, int BS = 128, int MINB = 6, bool CUBE = false>
 __global__ void __launch_bounds__(BS, MINB) k_element(
     const int32_t *__restrict__ conn, const uint8_t *__restrict__ level,
     const int32_t *__restrict__ hang, int64_t e_begin, int64_t e_end,
@@ -590,6 +689,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   constexpr int NC = 1 << D, NF = D + 3, ND = D + 1;
   constexpr bool UNIT = sizeof(T) == 4, RAW = MODE == 0 || MODE == 2;
   static_assert(!(UNIT && RAW), "the residual is in double");
+  static_assert(!CUBE || (!UNIT && D == 3 && (MODE == 0 || MODE == 1)), "FP64, one coefficient set");
   const int lc = threadIdx.x & (NC - 1);
   int64_t e = e_begin + ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> D);
   const bool active = e < e_end;
@@ -628,24 +728,58 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
 
   // geometry of this leaf
   Stage<D, T> s;
-  T nG[D];
+  T nG[D], vs[D], row = T(0), rowp = T(0);
+  KCube<D> kc;
   s.v = T((RAW ? 0.5 : 1.0) * CAD<D>);
-  s.cS = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     const bool neg = !((lc >> a) & 1);
-    s.sg[a] = flip_if(scale2(c.sg0[a], l - (RAW ? 1 : 0)), neg);
-    s.sh[a] = UNIT ? flip_if(scale2(c.sh0[a], l), neg) : T(0);
-    s.cV[a] = flip_if(scale2(c.cV0[a], (1 - D) * l - (RAW ? 0 : 1)), neg);
-    nG[a] = scale2(c.nG0[a], 2 * l);
+    if constexpr (CUBE) {
+      kc.neg[a] = neg;
+      kc.fs[a] = flip_if(scale2(c.f0, l), neg);
+      vs[a] = kc.fs[a] * s.v;
+      s.sg[a] = s.sh[a] = s.cV[a] = T(1);  // folded away
+      nG[a] = c.nG0[a];
+    } else {
+      s.sg[a] = flip_if(scale2(c.sg0[a], l - (RAW ? 1 : 0)), neg);
+      s.sh[a] = UNIT ? flip_if(scale2(c.sh0[a], l), neg) : T(0);
+      s.cV[a] = flip_if(scale2(c.cV0[a], (1 - D) * l - (RAW ? 0 : 1)), neg);
+      nG[a] = scale2(c.nG0[a], 2 * l);
+    }
   }
-  const T CI_GG = scale2(c.CIGG0, 4 * l), inv_trG = scale2(c.inv_trG0, -2 * l);
-  // d_a d_b = sg_a sg_b / CA^D (half of it with the halved factors)
-  const T CnWeH = UNIT ? c.CnWe : c.CnWe * T((RAW ? 2.0 : 1.0) / CAD<D>);
+  T CI_GG, inv_trG, CnWeH;
+  if constexpr (CUBE) {
+    kc.inv_dt = c.inv_dt; kc.four_dt2 = c.four_dt2; kc.alpha = c.alpha; kc.beta = c.beta;
+    for (int a = 0; a < 3; ++a) kc.ngFr[a] = c.ngFr[a];
+    kc.jcP = scale2(c.jcP, 2 * l);
+    kc.ngRe = scale2(c.ngRe, 2 * l);
+    kc.gRe = scale2(c.gRe, 2 * l);
+    kc.xRe = scale2(c.xRe, 2 * l);
+    kc.nCnWe = scale2(c.nCnWe, 3 * l);
+    kc.inv_We = scale2(c.inv_We, l);
+    kc.ninv_We = scale2(c.ninv_We, l);
+    kc.inv_PeCn = scale2(c.inv_PeCn, 2 * l);
+    kc.Cn2 = scale2(c.Cn2, 2 * l);
+    kc.f = scale2(c.f0, l);
+    kc.rf = scale2(c.rf0, -l);
+    kc.nk = c.nk;
+    s.cS = T(1);
+    row = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
+    rowp = row * kc.f;
+    CI_GG = c.CIGG0;
+    inv_trG = scale2(c.inv_trG0, -l);
+    CnWeH = scale2(c.CnWe, 3 * l);
+  } else {
+    s.cS = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
+    CI_GG = scale2(c.CIGG0, 4 * l);
+    inv_trG = scale2(c.inv_trG0, -2 * l);
+    // d_a d_b = sg_a sg_b / CA^D (half of it with the halved factors)
+    CnWeH = UNIT ? c.CnWe : c.CnWe * T((RAW ? 2.0 : 1.0) / CAD<D>);
+  }
 
   // interpolate to the lane's Gauss point
   Interp<D, T> A;
-  interp_state<D, UNIT>(u, s, A);
+  interp_state<D, UNIT, CUBE>(u, s, A, vs);
   T dvq[D], dphiq, dphig[D];
 #pragma unroll
   for (int i = 0; i < D; ++i) dvq[i] = ip_v<D>(d[i]) * T(CAD<D>);
@@ -678,25 +812,37 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     q.dphi = T(2) * dphiq;
     q.phin = A.phit + dphiq;
     T Sq[NF], Vq[NF][D];
-    gp_physics<D, HASF, T, T>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    if constexpr (CUBE) gp_physics<D, HASF, true, T, T>(kc, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    else gp_physics<D, HASF, false, T, T>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
     if constexpr (MODE == 2) {
       const unsigned b = __ballot_sync(FULL, floored && active);
       if ((threadIdx.x & 31) == 0 && b) atomicAdd(reinterpret_cast<unsigned long long *>(out), (unsigned long long)__popc(b));
     } else {
 #pragma unroll
-      for (int k = 0; k < NF; ++k) r[k] = contract<D>(Sq[k], Vq[k], s);
+      for (int k = 0; k < NF; ++k) {
+        r[k] = contract<D>(Sq[k], Vq[k], s);
+        if (CUBE) r[k] *= k == D ? rowp : row;
+      }
     }
   } else {
     // perturbation U_new + 2 e w (the weights of the contraction carry the
     // half): the averages move by w, the increments and phi^{k+1} by 2 w
     Interp<D, T> B;
-    interp_state<D, UNIT>(wn, s, B);
+    T one[D], w2[D];  // CUBE: plain values of the velocities' perturbation first
+#pragma unroll
+    for (int i = 0; i < D; ++i) one[i] = T(1);
+    interp_state<D, UNIT, CUBE>(wn, s, B, one);
     GpIn<D, Dl<T>> q;
     const T two = T(2), hf = T(0.5);
 #pragma unroll
     for (int i = 0; i < D; ++i) {
+      w2[i] = (CUBE ? two * s.v : two) * B.vt[i];
+      if (CUBE) B.vt[i] *= vs[i];
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
       q.vt[i] = Dl<T>(A.vt[i], B.vt[i]);
-      q.dv[i] = Dl<T>(dvq[i], two * B.vt[i]);
+      q.dv[i] = Dl<T>(dvq[i], w2[i]);
       q.dpt[i] = Dl<T>(A.dpt[i], B.dpt[i]);
       q.dphit[i] = Dl<T>(A.dphit[i], B.dphit[i]);
       q.dmut[i] = Dl<T>(A.dmut[i], B.dmut[i]);
@@ -712,13 +858,15 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     q.dphi = Dl<T>(dphiq, two * B.phit);
     q.phin = Dl<T>(mad(hf, dphiq, A.phit), two * B.phit);
     Dl<T> Sq[NF], Vq[NF][D];
-    gp_physics<D, HASF, T, Dl<T>>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    if constexpr (CUBE) gp_physics<D, HASF, true, T, Dl<T>>(kc, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
+    else gp_physics<D, HASF, false, T, Dl<T>>(c, nG, CI_GG, inv_trG, CnWeH, q, fq, Sq, Vq, floored);
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
       T Vk[D];
 #pragma unroll
       for (int j = 0; j < D; ++j) Vk[j] = Vq[k][j].d;
       r[k] = contract<D>(Sq[k].d, Vk, s);
+      if (CUBE) r[k] *= k == D ? rowp : row;
     }
   }
   if constexpr (MODE == 0 || MODE == 1) {
@@ -924,7 +1072,7 @@ __device__ __forceinline__ void pair_leaf(const KCoef<float> &c, const KPhys<F2>
   const F2 CI_GG(scale2(c.CIGG0, 4 * l)), inv_trG(scale2(c.inv_trG0, -2 * l));
   Dl<F2> Sq[NF], Vq[NF][D];
   B2 floored;
-  gp_physics<D, false, F2, Dl<F2>>(cp, nG, CI_GG, inv_trG, cp.CnWe, q, static_cast<const F2 *>(nullptr), Sq, Vq,
+  gp_physics<D, false, false, F2, Dl<F2>>(cp, nG, CI_GG, inv_trG, cp.CnWe, q, static_cast<const F2 *>(nullptr), Sq, Vq,
                                    floored);
   asm volatile("" : "+r"(l));
 #pragma unroll
@@ -1595,10 +1743,14 @@ template void launch_prep<double>(const chns_mesh *, const double *, const doubl
 template <int D, bool HASF>
 static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const double *Un, const double *Uo,
                                const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
-  launch_next(
-      k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks>, grid_elem(m->n_elem << D), kElemBlock, st,
-      m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
-      reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0, nullptr);
+  if (D == 3 && !m->coef64 && is_cube(c))
+    launch_next(k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks, D == 3>, grid_elem(m->n_elem << D),
+                kElemBlock, st, m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, kcube(c, true),
+                nullptr, m->elem_inst, 0, 0, nullptr);
+  else
+    launch_next(k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks>, grid_elem(m->n_elem << D),
+                kElemBlock, st, m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, c,
+                reinterpret_cast<const KCoef<double> *>(m->coef64), m->elem_inst, 0, 0, nullptr);
   launch_next(k_gather_nodes<D, double, kResidual>, grid_gather<D>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
               m->n_nodes, E, Un, bc, F, 0xffu, 0);
   note_launches(2);
@@ -1623,7 +1775,7 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 //      gather with the constrained rows; (threads, blocks per SM) = (64, 8),
 //      (128, 3), (64, 6), (128, 4).  0 is the default: 16 warps an SM hide the
 //      scattered loads of an adaptive mesh better than 12 (455 against 491 us on
-//      1,375,648 leaves, in spite of 76 bytes of spills) and cost 1 % on a
+//      1,375,648 leaves, in spite of 124 bytes of spills) and cost 1 % on a
 //      uniform one (81.0 against 80.4 us, 262,144 leaves)
 //   4: element colours one launch after another, each element adding its
 //      contributions into y (disjoint nodes within a colour; no E buffer),
@@ -1637,9 +1789,15 @@ static void elem_local(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << D;
   const dim3 ge((unsigned)((threads + BS - 1) / BS), (unsigned)nv);
+  note_launches(1);
+  if constexpr (sizeof(T) == 8 && D == 3)
+    if (!tab && is_cube(c)) {
+      launch_next(k_element<D, T, 1, false, T, BS, MINB, true>, ge, BS, st, m->conn, m->level, m->hang, 0, m->n_elem, ut,
+                  dl, w, nullptr, E, kcube(c, false), tab, m->elem_inst, m->n_nodes * NF, threads * NF, nullptr);
+      return;
+    }
   launch_next(k_element<D, T, 1, false, T, BS, MINB>, ge, BS, st, m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
               nullptr, E, c, tab, m->elem_inst, m->n_nodes * NF, threads * NF, nullptr);
-  note_launches(1);
 }
 
 static F2 host_pair(float a) {
