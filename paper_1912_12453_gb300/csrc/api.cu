@@ -664,14 +664,8 @@ chns_status newton_step(chns_mesh *m, const chns_params *p, const chns_solver_op
     // all instances in one launch pair (two launches each otherwise)
     TRY(ws.red.ensure(sizeof(double) * std::max<int64_t>((kMaxRestart + 16) * red_blocks(), int64_t(kSegBlocks) * ni)));
     TRY(ws.hdev.ensure(sizeof(double) * std::max<int64_t>(8 * kHessSlot, ni + 8)));
-    if (!ws.seg.p) {
-      std::vector<int64_t> start(m->inst_node_start);
-      for (int64_t &v : start) v *= nf;
-      TRY(ws.seg.ensure(sizeof(int64_t) * start.size()));
-      CHNS_CUDA_TRY(cudaMemcpy(ws.seg.p, start.data(), sizeof(int64_t) * start.size(), cudaMemcpyHostToDevice));
-    }
     double *hd = ws.hdev.as<double>();
-    vec_norm2_segments(F, ws.seg.as<int64_t>(), ni, ws.red.as<double>(), hd, st);
+    vec_norm2_segments(F, m->inst_dof, ni, ws.red.as<double>(), hd, st);
     std::vector<double> h(ni);
     CHNS_CUDA_TRY(cudaMemcpyAsync(h.data(), hd, sizeof(double) * ni, cudaMemcpyDeviceToHost, st));
     CHNS_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1021,6 +1015,7 @@ void chns_mesh_destroy(chns_mesh *m) {
   cudaFree(m->pins);
   cudaFree(m->elem_inst);
   cudaFree(m->node_inst);
+  cudaFree(m->inst_dof);
   cudaFree(m->coef32);
   cudaFree(m->coef64);
   chns::mg_release(m->mg);
@@ -1030,7 +1025,6 @@ void chns_mesh_destroy(chns_mesh *m) {
   m->ws.F.release(); m->ws.dU.release(); m->ws.r.release(); m->ws.V.release(); m->ws.Z.release();
   m->ws.wv.release(); m->ws.yv.release(); m->ws.binv.release(); m->ws.binv64.release(); m->ws.red.release(); m->ws.hdev.release();
   m->ws.e32.release(); m->ws.e64.release(); m->ws.ctr.release(); m->ws.count.release(); m->ws.al.release();
-  m->ws.seg.release();
   m->ws.Ublk.release(); m->ws.p32a.release(); m->ws.p32b.release();
   delete m;
   cudaSetDevice(prev);

@@ -71,7 +71,6 @@ struct Workspace {
   DevBuf binv;                         // n_nodes * nf * nf inverse diagonal blocks (element precision)
   DevBuf binv64;                       // the same blocks in double (FP64 J.w iterations)
   DevBuf red;                          // reduction partials
-  DevBuf seg;                          // batched meshes: first unknown of each instance
   DevBuf hdev;                         // device copy of Gram-Schmidt coefficients
   double *hpinned = nullptr;           // pinned host mirror of reduction results
   // preconditioner kept across steps: valid for `pc_steps_left` more steps
@@ -147,6 +146,7 @@ struct chns_mesh {
   int n_inst = 1;
   uint16_t *elem_inst = nullptr;       // n_elem instance of each element (device)
   int32_t *node_inst = nullptr;        // n_nodes instance of each node (device)
+  int64_t *inst_dof = nullptr;         // n_inst + 1: first unknown of each instance (device; union meshes)
   void *coef32 = nullptr, *coef64 = nullptr;  // per-instance element coefficients (device)
   std::vector<int64_t> inst_node_start;      // n_inst + 1 (host)
   std::vector<int> inst_max_level;           // n_inst (host)

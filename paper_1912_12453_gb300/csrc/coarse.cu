@@ -925,7 +925,7 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   TRY_CHNS(C.Minv32.ensure(sizeof(float) * C.nc0 * C.nc0 * ni));
   TRY_CHNS(C.vec.ensure(sizeof(double) * (3 * C.nc + 8)));
   TRY_CHNS(C.rpart.ensure(sizeof(double) * np * nf));
-  return CHNS_OK;
+  return uploads_done(C.node_piece, ncn_all + 1);
 }
 
 template <typename T>

@@ -152,6 +152,16 @@ inline chns_status upload(T **dst, const std::vector<T> &src) {
   return CHNS_OK;
 }
 
+// After the last upload() of a set-up: a copy from pageable memory may still be
+// on its way to the device when the call returns, and a caller's non-blocking
+// stream is not ordered after the legacy stream it runs in.  A copy back into
+// pageable memory returns when it is done, and with it all copies before it.
+template <class T>
+inline chns_status uploads_done(const T *last, int64_t n) {
+  T x;
+  if (n > 0) CHNS_CUDA_TRY(cudaMemcpy(&x, last + (n - 1), sizeof(T), cudaMemcpyDeviceToHost));
+  return CHNS_OK;
+}
 
 template <class T>
 inline std::vector<T> download(const T *d, size_t n) {

@@ -518,7 +518,7 @@ chns_status build_gather(chns_mesh *m) {
   if ((st = upload(&m->gptr, gptr)) != CHNS_OK) return st;
   if ((st = upload(&m->gent, gent)) != CHNS_OK) return st;
   if ((st = upload(&m->nflag, nflag)) != CHNS_OK) return st;
-  return CHNS_OK;
+  return uploads_done(m->nflag, m->n_nodes);
 }
 
 // Host-side validation of a built mesh (single or union) against its device
@@ -734,6 +734,9 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   if ((st = upload(&u->node_colour, ncol8)) != CHNS_OK) return st;
   if ((st = upload(&u->elem_inst, einst)) != CHNS_OK) return st;
   if ((st = upload(&u->node_inst, ninst)) != CHNS_OK) return st;
+  std::vector<int64_t> dof(u->inst_node_start);
+  for (int64_t &v : dof) v *= u->nf;
+  if ((st = upload(&u->inst_dof, dof)) != CHNS_OK) return st;
   return CHNS_OK;
 }
 

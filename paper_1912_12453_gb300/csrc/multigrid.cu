@@ -408,7 +408,7 @@ chns_status upload_transfer(const std::vector<TransferLists> &parts, const std::
   TRY_MG(upload(&L.rw, rw));
   TRY_MG(upload(&L.inj, inj));
   L.nnz = (int64_t)pcol.size();
-  return CHNS_OK;
+  return uploads_done(L.inj, ncoarse);  // also the coefficient tables that a union level copied before
 }
 
 // one level coarser: every family of leaves at the mesh's finest leaf level
