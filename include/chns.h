@@ -181,7 +181,8 @@ chns_status chns_mesh_check(const chns_mesh *mesh);
  * (block size, blocks per SM) = (64, 8), (128, 3), (64, 6), (128, 4) (as 5 on a
  * batch's union mesh); 5, 6 the same with one Gauss point per lane, (128, 5)
  * and (128, 6); 4 element colours with in-place adds.  variant = -1 only
- * reads. */
+ * reads.  On a small uniform mesh without a fixed schedule chns_jacvec reads
+ * the states in the element kernel, with a launch shape of its own. */
 chns_status chns_mesh_jacvec_schedule(chns_mesh *mesh, int variant, int *current, double *times_ms);
 
 void chns_mesh_destroy(chns_mesh *mesh);

@@ -1133,7 +1133,7 @@ chns_status chns_mesh_jacvec_schedule(chns_mesh *m, int variant, int *current, d
   if (variant < -1 || variant >= kJacvecVariants) { set_error("schedule %d out of range", variant); return CHNS_ERR_ARG; }
   if (variant >= 0) {
     m->jv_variant = variant;
-    m->jv_tuned = true;
+    m->jv_tuned = m->jv_fixed = true;
   }
   if (current) *current = m->jv_variant;
   if (times_ms)

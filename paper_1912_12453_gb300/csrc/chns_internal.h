@@ -177,6 +177,7 @@ struct chns_mesh {
   // times per schedule (ms; negative: not measured)
   int jv_variant = 0;
   bool jv_tuned = false;
+  bool jv_fixed = false;               // chosen by the caller: every FP32 apply runs it
   double jv_times[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
   chns::Workspace ws;
   chns::Coarse coarse;

@@ -1918,11 +1918,12 @@ template void launch_jacvec<double>(const chns_mesh *, const PhysCoef &, const d
 // a large mesh loses: 32,768 leaves in 3D 15.6 -> 18.1 us, 65,536 in 2D
 // 14.4 -> 13.8 but 31.1 -> 31.6 by itself.  With hanging nodes one corner
 // averages up to four, one lane after another: 21,960 leaves 17.9 -> 31.8 us.
-// false: the mesh, its schedule or the states' alignment is not for this path.
+// false: the mesh, its schedule (one that the caller fixed runs as it is) or the
+// states' alignment is not for this path.
 bool launch_jacvec_states(const chns_mesh *m, const PhysCoef &pc, const double *Un, const double *Uo, const float *w,
                           float *E, float *y, cudaStream_t st) {
   constexpr int64_t kStateCorners = 65536;
-  if (m->n_hang || (m->n_elem << m->dim) > kStateCorners || m->jv_variant >= 4 || m->coef32) return false;
+  if (m->n_hang || (m->n_elem << m->dim) > kStateCorners || m->jv_variant >= 4 || m->jv_fixed || m->coef32) return false;
   // node blocks of six doubles are read by pairs; the preparation reads single values
   if (m->dim == 3 && ((reinterpret_cast<uintptr_t>(Un) | reinterpret_cast<uintptr_t>(Uo)) & 15)) return false;
   const KCoef<float> c = kcoef<float>(pc, m->dim);
