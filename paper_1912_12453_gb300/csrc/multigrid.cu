@@ -569,6 +569,12 @@ template <typename T>
 static chns_status jv_level(void *ctx, const T *w, T *y, int nv);
 
 namespace {
+// never repeats, across precisions and across hierarchies at the same address
+uint64_t next_generation() {
+  static std::atomic<uint64_t> builds{0};
+  return ++builds;
+}
+
 template <typename T>
 struct LevelCtx {
   chns_mesh *m;
@@ -649,9 +655,8 @@ chns_status mg_build(chns_mesh *m, const PhysCoef &pc, const T *ut0, const T *dl
     now.push_back(reinterpret_cast<const void *>(intptr_t(c->jv_variant)));
   }
   if (now != G.buffers[P]) {
-    static std::atomic<uint64_t> builds{0};  // never repeats, also across hierarchies at the same address
     G.buffers[P].swap(now);
-    G.generation = ++builds;
+    G.generation = next_generation();
   }
   return check_launch();
 }
