@@ -302,7 +302,7 @@ struct Timer {
 // What an Arnoldi-step graph bakes in: buffers, sizes, coarse-space state and
 // the element coefficients (kernel arguments by value)
 struct StepKey {
-  const void *p[16];
+  const void *p[15];
   int64_t i[8];
   PhysCoef pc;
 };
@@ -415,9 +415,9 @@ chns_status fgmres(chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, c
     key.p[0] = V; key.p[1] = Z; key.p[2] = ut; key.p[3] = dl; key.p[4] = Binv; key.p[5] = part;
     key.p[6] = hd; key.p[7] = ws.hpinned; key.p[8] = m->coarse.vec.as<void>();
     key.p[9] = m->coarse.rpart.as<void>(); key.p[10] = m->coarse.M.as<void>();
-    key.p[11] = m->coarse.Minv32.as<void>(); key.p[12] = m->coarse.piece_begin; key.p[13] = Ebuf;
-    key.p[14] = ctr; key.p[15] = mg ? m->mg : nullptr;
-    key.i[0] = ld; key.i[1] = n; key.i[2] = coarse; key.i[3] = m->coarse.ready; key.i[4] = m->coarse.level;
+    key.p[11] = m->coarse.Minv32.as<void>(); key.p[12] = Ebuf;
+    key.p[13] = ctr; key.p[14] = mg ? m->mg : nullptr;
+    key.i[0] = ld; key.i[1] = n; key.i[2] = coarse; key.i[3] = m->coarse.ready; key.i[4] = m->coarse.serial;
     key.i[5] = mg ? (int64_t)m->mg->generation : -1; key.i[6] = o.use_graph + 2 * (mg32 != nullptr);
     key.i[7] = m->jv_variant;
     key.pc = pc;

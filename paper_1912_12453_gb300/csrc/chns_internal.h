@@ -123,6 +123,7 @@ struct Coarse {
   DevBuf vec;                       // coarse work vectors
   DevBuf rpart;                     // restriction partials, n_pieces x nf
   bool ready = false;
+  int64_t serial = 0;               // of the set-up; never repeats (captured steps hold the lists above)
   ~Coarse();
   void release();
 };

@@ -15,6 +15,7 @@
 // leaf at least one level finer than L_c.  All reductions run in a fixed
 // order (one block per coarse node); nothing is atomic.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <vector>
@@ -913,6 +914,8 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   TRY_CHNS(upload(&C.piece_begin, piece_begin));
   TRY_CHNS(upload(&C.node_piece, node_piece));
   C.n_pieces = np;
+  static std::atomic<int64_t> setups{0};
+  C.serial = ++setups;
   C.level = Lc;
   C.nc1 = nc1;
   C.n_inst = ni;

@@ -1,6 +1,6 @@
 """Captured Arnoldi steps are not kept past a rebuild that changes the V-cycle,
-in whatever order builds in the two precisions come.  Own process: the numbers
-that tell the builds apart count from its start."""
+in whatever order builds in the two precisions come (own process: the numbers
+that tell the builds apart count from its start), nor past another coarse space."""
 import os
 import subprocess
 import sys
@@ -56,3 +56,30 @@ def test_a_step_does_not_depend_on_the_builds_before_it(order):
     assert r.returncode == 0, r.stderr[-2000:]
     got, want, same = (int(x) for x in r.stdout.split()[-3:])
     assert got == want and same == 1
+
+
+def test_coarse_level_there_and_back():
+    """The coarse space of a captured step is released and set up again in between
+    by steps that capture nothing."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1912_12453_gb300 import build, chns, workloads as W
+    build.build()
+    wl = W.workload("droplet2d_l5")
+    meshes = [chns.Mesh(wl.leaves) for _ in range(2)]
+    U0 = torch.from_numpy(W.initial_state(meshes[0].coords, wl).reshape(-1)).cuda()
+    chns.init_mu(meshes[0], wl.params, U0)
+
+    def step(m, level, graph):
+        out = torch.empty_like(U0)
+        st = chns.step(m, wl.params, U0, out, chns.SolverOpts.make(newton_rtol=1e-6, coarse_level=level,
+                                                                   use_graph=graph))
+        return out, st["krylov_its_total"]
+
+    for level, graph in ((2, True), (3, False), (2, True)):
+        got = step(meshes[0], level, graph)
+    want = step(meshes[1], 2, True)
+    assert got[1] == want[1] and torch.equal(got[0], want[0])
+    for m in meshes:
+        m.close()
