@@ -107,6 +107,7 @@ struct Coarse {
   // pieces of at most kPiece entries
   int32_t *rnode = nullptr;
   float *rw = nullptr;
+  double *rw64 = nullptr;           // the weights where some are not floats (FP64 restriction); else nullptr
   int64_t n_pieces = 0;
   int32_t *piece_node = nullptr;    // n_pieces: the coarse node
   int64_t *piece_begin = nullptr;   // n_pieces + 1: ranges in the lists

@@ -18,6 +18,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 #include <vector>
 
 #include "chns_internal.h"
@@ -225,13 +226,16 @@ constexpr int kGroups = 32;   // lists are read by 32 groups of eight lanes
 
 // rc = R v = P^T v: block p sums w v[i, q] over piece p of a coarse node's
 // restriction list, lane q of each group of eight the component q; the groups'
-// sums are added in group order.  part == rc when every list is one piece.
+// sums are added in group order.  part == rc when every list is one piece.  The
+// weights are exact (W), so in double R is P^T: a product of the three fractions of
+// a node k levels below the coarse grid has up to 3 k bits, more than a float from
+// k = 9 on (2D: 13).
 // (Sums of all corners of a coarse cell, reduced over 256 threads, took a hundred
 // FP64 additions a warp for lists of 49 to 81 nodes.)
-template <typename T, int NF>
+template <typename T, int NF, typename W>
 __global__ void __launch_bounds__(kGroups * 8) k_restrict_lists(const int64_t *__restrict__ piece_begin,
                                                                const int32_t *__restrict__ rnode,
-                                                               const float *__restrict__ rw,
+                                                               const W *__restrict__ rw,
                                                                const T *__restrict__ v, T *__restrict__ part) {
   const int grp = threadIdx.x >> 3, q = threadIdx.x & 7;
   const int64_t b = piece_begin[blockIdx.x];
@@ -803,12 +807,14 @@ void Coarse::release() {
   cudaFree(pos);
   cudaFree(rnode);
   cudaFree(rw);
+  cudaFree(rw64);
   cudaFree(piece_node);
   cudaFree(piece_begin);
   cudaFree(node_piece);
   pos = nullptr;
   rnode = nullptr;
   rw = nullptr;
+  rw64 = nullptr;
   piece_node = node_piece = nullptr;
   piece_begin = nullptr;
   n_pieces = 0;
@@ -883,12 +889,17 @@ chns_status coarse_setup(chns_mesh *m, int Lc) {
   }
   std::vector<int32_t> rnode(cnt[ncn_all]);
   std::vector<float> rw(cnt[ncn_all]);
+  std::vector<double> rw64(cnt[ncn_all]);
+  bool floats = true;
   std::vector<int64_t> fill(cnt.begin(), cnt.end() - 1);
   for (int64_t i = 0; i < m->n_nodes; ++i)
     corners(i, [&](int64_t idx, double w) {
       rnode[fill[idx]] = (int32_t)i;
+      floats = floats && double(float(w)) == w;
+      rw64[fill[idx]] = w;
       rw[fill[idx]++] = (float)w;
     });
+  if (!floats) TRY_CHNS(upload(&C.rw64, rw64));
   CHNS_CUDA_TRY(cudaMalloc(&C.pos, sizeof(float) * pos.size()));
   CHNS_CUDA_TRY(cudaMemcpy(C.pos, pos.data(), sizeof(float) * pos.size(), cudaMemcpyHostToDevice));
   CHNS_CUDA_TRY(cudaMalloc(&C.rnode, sizeof(int32_t) * std::max<size_t>(rnode.size(), 1)));
@@ -1036,10 +1047,19 @@ void precond_apply(chns_mesh *m, const T *Binv, bool coarse, const T *v, T *z, c
       const bool whole = C.n_pieces == C.ncn;
       T *part = whole ? r : reinterpret_cast<T *>(C.rpart.as<double>());
       const unsigned np = (unsigned)C.n_pieces;
-      if (m->dim == 2)
-        launch_next(k_restrict_lists<T, 5>, np, kGroups * 8, st, C.piece_begin, C.rnode, C.rw, v, part);
-      else
-        launch_next(k_restrict_lists<T, 6>, np, kGroups * 8, st, C.piece_begin, C.rnode, C.rw, v, part);
+      auto restrict_with = [&](auto *rw) {
+        using W = std::remove_cv_t<std::remove_reference_t<decltype(*rw)>>;
+        if (m->dim == 2)
+          launch_next(k_restrict_lists<T, 5, W>, np, kGroups * 8, st, C.piece_begin, C.rnode, rw, v, part);
+        else
+          launch_next(k_restrict_lists<T, 6, W>, np, kGroups * 8, st, C.piece_begin, C.rnode, rw, v, part);
+      };
+      if constexpr (sizeof(T) == sizeof(double)) {
+        if (C.rw64) restrict_with(C.rw64);
+        else restrict_with(C.rw);
+      } else {
+        restrict_with(C.rw);
+      }
       note_launches(1);
       if (!whole) {
         launch_next(k_restrict_pieces<T>, (unsigned)((C.nc + kB - 1) / kB), kB, st, C.nc, m->nf, C.node_piece, part, r);
