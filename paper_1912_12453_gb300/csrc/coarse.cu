@@ -126,9 +126,10 @@ constexpr int kChunk = 64;    // entries whose slots a block finds together
 
 // Block (p, v) takes piece p of the restriction list of coarse row node c' and,
 // for probe v (colour k), sums P[i, c'] y[i, q] per owner slot s (the owner of
-// mesh node i: the nearest coarse node of colour k), in list order: the threads
-// first find the slots of kChunk entries together, then thread (s, q) adds up
-// the entries of its slot.  A block of 256 threads with 48 sums each, reduced
+// mesh node i: the nearest coarse node of colour k): the threads first find the
+// slots of kChunk entries together, then thread (s, q) adds up the entries of its
+// slot, in T in eight chains of at most eight terms, and the chunks in double:
+// 11 roundings of T on the longest way, as many as a tree over the block has.  A block of 256 threads with 48 sums each, reduced
 // over the block, spent its time on the reduction: most lists hold 64 to 125
 // entries.
 template <typename T, int NF, int DIM>
@@ -146,10 +147,12 @@ __global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t 
   y += blockIdx.y * g.n_nodes * NF;
   const int s = threadIdx.x / NF, q = threadIdx.x % NF;
   const int64_t end = piece_begin[blockIdx.x + 1];
-  T acc = T(0);
+  constexpr int G = 8;
+  double acc = 0.0;
   for (int64_t b = piece_begin[blockIdx.x]; b < end; b += kChunk) {
     const int cnt = int(min(int64_t(kChunk), end - b));
     __syncthreads();
+    slot[threadIdx.x] = -1;
     if (int(threadIdx.x) < cnt) {
       const int64_t i = rnode[b + threadIdx.x];
       int r = int(cp % g.ncn_inst), sl = 0;
@@ -168,11 +171,18 @@ __global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t 
       wgt[threadIdx.x] = T(rw[b + threadIdx.x]);
     }
     __syncthreads();
-    if (s < NS)
-      for (int e = 0; e < cnt; ++e)
-        if (slot[e] == s) acc = fma(wgt[e], y[int64_t(node[e]) * NF + q], acc);
+    if (s < NS) {
+      T a[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) a[g] = T(0);
+      for (int e = 0; e < cnt; e += G)
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+          if (slot[e + g] == s) a[g] = fma(wgt[e + g], y[int64_t(node[e + g]) * NF + q], a[g]);
+      acc += double(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
+    }
   }
-  if (s < NS) part[(blockIdx.y * int64_t(gridDim.x) + blockIdx.x) * NS * NF + threadIdx.x] = double(acc);
+  if (s < NS) part[(blockIdx.y * int64_t(gridDim.x) + blockIdx.x) * NS * NF + threadIdx.x] = acc;
 }
 
 // A[(c', q), (owner(s), f)] = sum of the pieces, in list order

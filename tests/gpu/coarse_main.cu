@@ -1,6 +1,7 @@
 // Checks of the coarse space's kernels on their own, compared with the same sums
 // in long double on the host.  Test infrastructure only.
 //   coarse_main weights <leaves.bin> <level>   R against P^T in FP64
+//   coarse_main gather <entries>               sums of the operator build in float
 // Prints one number: the largest error over its bound.
 #include "coarse.cu"
 
@@ -81,11 +82,52 @@ double weights(const char *path, int level) {
   chns_mesh_destroy(m);
   return worst;
 }
+
+// A list of n entries of weight 1 around one coarse node, all in one slot: a one,
+// then terms of just under half its last place, each of which is lost when it is
+// added to a sum that holds the one.  Of the most roundings on the way of a term,
+// 11, each is off by at most 2^-24 of the sum.
+double gather_sums(int n) {
+  constexpr int NF = 6, DIM = 3;
+  // level 1: three coarse nodes an axis, the middle one (1, 1, 1) has number 13;
+  // probe 13 NF: colour (1, 1, 1), whose node is the owner of the mesh nodes
+  std::vector<int32_t> node(n), piece{13};
+  std::vector<int64_t> begin{0, n};
+  std::vector<float> w(n, 1.0f), pos(size_t(n) * DIM, 1.0f), y(size_t(n) * NF);
+  long double ref[NF] = {0};
+  for (int e = 0; e < n; ++e) {
+    node[e] = e;
+    for (int q = 0; q < NF; ++q) {
+      y[size_t(e) * NF + q] = e == 0 ? 1.0f : 0x1.fffffep-25f * float(q + 1) / NF;
+      ref[q] += (long double)y[size_t(e) * NF + q];
+    }
+  }
+  int32_t *dpiece = nullptr, *dnode = nullptr;
+  int64_t *dbegin = nullptr;
+  float *dw = nullptr, *dpos = nullptr, *dy = nullptr;
+  if (upload(&dpiece, piece) || upload(&dnode, node) || upload(&dbegin, begin) || upload(&dw, w) ||
+      upload(&dpos, pos) || upload(&dy, y))
+    std::exit(3);
+  DevBuf part;
+  if (part.ensure(sizeof(double) * 8 * NF) != CHNS_OK) std::exit(3);
+  must(cudaDeviceSynchronize());
+  CGeo g{DIM, NF, 3, n, 27, 27 * NF, 0};
+  k_gather_coarse<float, NF, DIM><<<1, kChunk>>>(g, dpiece, dbegin, dnode, dw, dpos, 13 * NF, dy, part.as<double>());
+  double out[8 * NF], worst = 0.0;
+  must(cudaMemcpy(out, part.p, sizeof(out), cudaMemcpyDeviceToHost));
+  for (int s = 0; s < 8; ++s)
+    for (int q = 0; q < NF; ++q) {
+      const long double want = s == 0 ? ref[q] : 0.0L;
+      worst = std::max(worst, double(std::fabs((long double)out[s * NF + q] - want) / (11 * 0x1p-24L * ref[q])));
+    }
+  return worst;
+}
 }  // namespace
 
 int main(int argc, char **argv) {
   double r = -1.0;
   if (argc == 4 && !std::strcmp(argv[1], "weights")) r = weights(argv[2], std::atoi(argv[3]));
+  if (argc == 3 && !std::strcmp(argv[1], "gather")) r = gather_sums(std::atoi(argv[2]));
   if (r < 0.0) return 2;
   std::printf("%.6g\n", r);
   return 0;

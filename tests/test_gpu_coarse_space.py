@@ -46,6 +46,11 @@ def _corner_leaves(dim, top):
     return np.array(lev, np.uint8), np.array(anc, np.uint32)
 
 
+@pytest.mark.parametrize("entries", [1, 7, 63, 64, 65, 127, 1000, 1024])
+def test_sums_of_the_operator_build(exe, entries):
+    assert _run(exe, "gather", entries) <= 1.0
+
+
 # 2D products are floats down to 12 levels below the coarse grid, 3D ones to 8
 @pytest.mark.parametrize("dim,top", [(2, 8), (2, 13), (2, 15), (2, 20), (3, 6), (3, 9), (3, 11), (3, 20)])
 def test_restriction_is_the_transpose_of_the_prolongation(exe, tmp_path, dim, top):
