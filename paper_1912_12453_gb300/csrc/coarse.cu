@@ -235,8 +235,9 @@ __global__ void __launch_bounds__(kB) k_collect_direct(CGeo g, const float *__re
 constexpr int kGroups = 32;   // lists are read by 32 groups of eight lanes
 
 // rc = R v = P^T v: block p sums w v[i, q] over piece p of a coarse node's
-// restriction list, lane q of each group of eight the component q; the groups'
-// sums are added in group order.  part == rc when every list is one piece.  The
+// restriction list, lane q of each group of eight the component q: four chains of
+// at most eight terms a group, then a tree over the chains and the groups (15
+// roundings on the longest way).  part == rc when every list is one piece.  The
 // weights are exact (W), so in double R is P^T: a product of the three fractions of
 // a node k levels below the coarse grid has up to 3 k bits, more than a float from
 // k = 9 on (2D: 13).
@@ -257,24 +258,35 @@ __global__ void __launch_bounds__(kGroups * 8) k_restrict_lists(const int64_t *_
     w0 = T(rw[b + grp]);
   }
   wait_previous(v, part);
-  T acc = T(0);
+  T a[4] = {T(0), T(0), T(0), T(0)};
   if (q < NF && grp < cnt) {
-    acc = w0 * v[int64_t(i0) * NF + q];
-#pragma unroll 4
-    for (int e = grp + kGroups; e < cnt; e += kGroups) acc = fma(T(rw[b + e]), v[int64_t(rnode[b + e]) * NF + q], acc);
+    a[0] = w0 * v[int64_t(i0) * NF + q];
+    for (int e = grp + kGroups; e < cnt; e += 4 * kGroups)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (e + k * kGroups < cnt)
+          a[k] = fma(T(rw[b + e + k * kGroups]), v[int64_t(rnode[b + e + k * kGroups]) * NF + q], a[k]);
   }
-  __shared__ T red[kGroups][8];
-  red[grp][q] = acc;
+  T acc = (a[0] + a[1]) + (a[2] + a[3]);
+  acc += __shfl_xor_sync(FULL, acc, 8);
+  acc += __shfl_xor_sync(FULL, acc, 16);
+  constexpr int NW = kGroups / 4;
+  __shared__ T red[NW][8];
+  if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][q] = acc;
   __syncthreads();
   if (threadIdx.x < NF) {
-    T s = T(0);
-    const int n = min(kGroups, cnt);
-    for (int g = 0; g < n; ++g) s += red[g][threadIdx.x];
-    part[int64_t(blockIdx.x) * NF + threadIdx.x] = s;
+    T s[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) s[w] = red[w][threadIdx.x];
+#pragma unroll
+    for (int h = NW / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int w = 0; w < h; ++w) s[w] += s[w + h];
+    part[int64_t(blockIdx.x) * NF + threadIdx.x] = s[0];
   }
 }
 
-// rc = sum of the pieces, in list order
+// rc = sum of the pieces, every eighth in one chain
 template <typename T>
 __global__ void k_restrict_pieces(int64_t nc, int nf, const int32_t *__restrict__ node_piece,
                                   const T *__restrict__ part, T *__restrict__ rc) {
@@ -282,9 +294,16 @@ __global__ void k_restrict_pieces(int64_t nc, int nf, const int32_t *__restrict_
   wait_previous(part, rc);
   if (t >= nc) return;
   const int64_t cp = t / nf;
-  T s = T(0);
-  for (int p = node_piece[cp]; p < node_piece[cp + 1]; ++p) s += part[int64_t(p) * nf + t % nf];
-  rc[t] = s;
+  constexpr int G = 8;
+  T s[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) s[g] = T(0);
+  const int e = node_piece[cp + 1];
+  for (int p = node_piece[cp]; p < e; p += G)
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (p + g < e) s[g] += part[int64_t(p + g) * nf + t % nf];
+  rc[t] = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 }
 
 // zc = A_c^{-1} rc, one warp per row, in precision T; row r of instance i at

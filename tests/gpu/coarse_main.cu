@@ -2,6 +2,8 @@
 // in long double on the host.  Test infrastructure only.
 //   coarse_main weights <leaves.bin> <level>   R against P^T in FP64
 //   coarse_main gather <entries>               sums of the operator build in float
+//   coarse_main restrict <entries>             sums of the restriction in float
+//   coarse_main pieces <pieces>                the restriction's sum over a list's pieces
 // Prints one number: the largest error over its bound.
 #include "coarse.cu"
 
@@ -83,44 +85,78 @@ double weights(const char *path, int level) {
   return worst;
 }
 
-// A list of n entries of weight 1 around one coarse node, all in one slot: a one,
-// then terms of just under half its last place, each of which is lost when it is
-// added to a sum that holds the one.  Of the most roundings on the way of a term,
-// 11, each is off by at most 2^-24 of the sum.
+// n terms a component: a one, then terms of just under half its last place, each
+// of which is lost when it is added to a sum that holds the one.  Of the `most`
+// roundings on the way of a term each is off by at most 2^-24 of the sum.
+constexpr int NF = 6;
+struct Terms {
+  std::vector<float> y;
+  long double ref[NF] = {0};
+  explicit Terms(int n) : y(size_t(n) * NF) {
+    for (int e = 0; e < n; ++e)
+      for (int q = 0; q < NF; ++q) {
+        y[size_t(e) * NF + q] = e == 0 ? 1.0f : 0x1.fffffep-25f * float(q + 1) / NF;
+        ref[q] += (long double)y[size_t(e) * NF + q];
+      }
+  }
+  double error(const double *out, int most) const {
+    double worst = 0.0;
+    for (int q = 0; q < NF; ++q)
+      worst = std::max(worst, double(std::fabs((long double)out[q] - ref[q]) / (most * 0x1p-24L * ref[q])));
+    return worst;
+  }
+};
+
+template <class T>
+T *on_device(const std::vector<T> &x) {
+  T *d = nullptr;
+  if (upload(&d, x) != CHNS_OK || uploads_done(d, int64_t(x.size())) != CHNS_OK) std::exit(3);
+  return d;
+}
+
+// a list of n entries of weight 1 around one coarse node, all in one slot
 double gather_sums(int n) {
-  constexpr int NF = 6, DIM = 3;
+  constexpr int DIM = 3;
   // level 1: three coarse nodes an axis, the middle one (1, 1, 1) has number 13;
   // probe 13 NF: colour (1, 1, 1), whose node is the owner of the mesh nodes
   std::vector<int32_t> node(n), piece{13};
-  std::vector<int64_t> begin{0, n};
-  std::vector<float> w(n, 1.0f), pos(size_t(n) * DIM, 1.0f), y(size_t(n) * NF);
-  long double ref[NF] = {0};
-  for (int e = 0; e < n; ++e) {
-    node[e] = e;
-    for (int q = 0; q < NF; ++q) {
-      y[size_t(e) * NF + q] = e == 0 ? 1.0f : 0x1.fffffep-25f * float(q + 1) / NF;
-      ref[q] += (long double)y[size_t(e) * NF + q];
-    }
-  }
-  int32_t *dpiece = nullptr, *dnode = nullptr;
-  int64_t *dbegin = nullptr;
-  float *dw = nullptr, *dpos = nullptr, *dy = nullptr;
-  if (upload(&dpiece, piece) || upload(&dnode, node) || upload(&dbegin, begin) || upload(&dw, w) ||
-      upload(&dpos, pos) || upload(&dy, y))
-    std::exit(3);
+  for (int e = 0; e < n; ++e) node[e] = e;
+  const std::vector<int64_t> begin{0, n};
+  const std::vector<float> w(n, 1.0f), pos(size_t(n) * DIM, 1.0f);
+  const Terms t(n);
   DevBuf part;
   if (part.ensure(sizeof(double) * 8 * NF) != CHNS_OK) std::exit(3);
-  must(cudaDeviceSynchronize());
   CGeo g{DIM, NF, 3, n, 27, 27 * NF, 0};
-  k_gather_coarse<float, NF, DIM><<<1, kChunk>>>(g, dpiece, dbegin, dnode, dw, dpos, 13 * NF, dy, part.as<double>());
-  double out[8 * NF], worst = 0.0;
+  k_gather_coarse<float, NF, DIM><<<1, kChunk>>>(g, on_device(piece), on_device(begin), on_device(node), on_device(w),
+                                                 on_device(pos), 13 * NF, on_device(t.y), part.as<double>());
+  double out[8 * NF];
   must(cudaMemcpy(out, part.p, sizeof(out), cudaMemcpyDeviceToHost));
-  for (int s = 0; s < 8; ++s)
-    for (int q = 0; q < NF; ++q) {
-      const long double want = s == 0 ? ref[q] : 0.0L;
-      worst = std::max(worst, double(std::fabs((long double)out[s * NF + q] - want) / (11 * 0x1p-24L * ref[q])));
-    }
-  return worst;
+  for (int k = NF; k < 8 * NF; ++k)
+    if (out[k] != 0.0) return 1e30;
+  return t.error(out, 11);
+}
+
+// the restriction of one piece of n entries of weight 1, or of n pieces
+double restrict_sums(int n, bool pieces) {
+  const Terms t(n);
+  DevBuf rc;
+  if (rc.ensure(sizeof(float) * NF) != CHNS_OK) std::exit(3);
+  if (pieces) {
+    const std::vector<int32_t> node_piece{0, n};
+    k_restrict_pieces<float><<<1, kB>>>(NF, NF, on_device(node_piece), on_device(t.y), rc.as<float>());
+  } else {
+    std::vector<int32_t> node(n);
+    for (int e = 0; e < n; ++e) node[e] = e;
+    const std::vector<int64_t> begin{0, n};
+    const std::vector<float> w(n, 1.0f);
+    k_restrict_lists<float, NF><<<1, kGroups * 8>>>(on_device(begin), on_device(node), on_device(w), on_device(t.y),
+                                                    rc.as<float>());
+  }
+  float f[NF];
+  must(cudaMemcpy(f, rc.p, sizeof(f), cudaMemcpyDeviceToHost));
+  double out[NF];
+  for (int q = 0; q < NF; ++q) out[q] = f[q];
+  return t.error(out, pieces ? (n + 7) / 8 + 3 : 15);
 }
 }  // namespace
 
@@ -128,6 +164,8 @@ int main(int argc, char **argv) {
   double r = -1.0;
   if (argc == 4 && !std::strcmp(argv[1], "weights")) r = weights(argv[2], std::atoi(argv[3]));
   if (argc == 3 && !std::strcmp(argv[1], "gather")) r = gather_sums(std::atoi(argv[2]));
+  if (argc == 3 && !std::strcmp(argv[1], "restrict")) r = restrict_sums(std::atoi(argv[2]), false);
+  if (argc == 3 && !std::strcmp(argv[1], "pieces")) r = restrict_sums(std::atoi(argv[2]), true);
   if (r < 0.0) return 2;
   std::printf("%.6g\n", r);
   return 0;

@@ -51,6 +51,16 @@ def test_sums_of_the_operator_build(exe, entries):
     assert _run(exe, "gather", entries) <= 1.0
 
 
+@pytest.mark.parametrize("entries", [1, 8, 31, 32, 33, 125, 1000, 1024])
+def test_sums_of_the_restriction(exe, entries):
+    assert _run(exe, "restrict", entries) <= 1.0
+
+
+@pytest.mark.parametrize("pieces", [1, 7, 8, 9, 100])
+def test_sum_of_the_pieces(exe, pieces):
+    assert _run(exe, "pieces", pieces) <= 1.0
+
+
 # 2D products are floats down to 12 levels below the coarse grid, 3D ones to 8
 @pytest.mark.parametrize("dim,top", [(2, 8), (2, 13), (2, 15), (2, 20), (3, 6), (3, 9), (3, 11), (3, 20)])
 def test_restriction_is_the_transpose_of_the_prolongation(exe, tmp_path, dim, top):
