@@ -212,7 +212,10 @@ chns_status chns_jacvec(const chns_mesh *mesh, const chns_params *params,
 
 /* Replace the chemical potential of U (in place) by the L2 projection of
  * psi'(phi) - Cn^2 lap(phi), i.e. solve M mu = (N, psi'(phi)) + Cn^2 (grad N,
- * grad phi) (the chemical-potential row with U_new = U_old). */
+ * grad phi) (the chemical-potential row with U_new = U_old).  CHNS_ERR_KRYLOV,
+ * with U as it was, when a grid barrier of the solver is given up (about 20 s;
+ * CHNS_INJECT=barrier makes the next call meet one after milliseconds, for tests
+ * of the caller's error handling). */
 chns_status chns_init_mu(const chns_mesh *mesh, const chns_params *params, double *U,
                          void *stream);
 

@@ -307,11 +307,13 @@ struct StepKey {
   PhysCoef pc;
 };
 
-// CHNS_INJECT=krylov: the next FGMRES reports a breakdown (host-side fault
-// injection; read at every solve so a test can set and clear it)
-bool inject_krylov_fault() {
+// CHNS_INJECT=krylov: the next FGMRES reports a breakdown; =barrier: the grid
+// barriers of the mu projection start one arrival short, so the first one never
+// fills and is given up after milliseconds (read at every solve so a test can set
+// and clear it)
+bool inject_fault(const char *what) {
   const char *e = std::getenv("CHNS_INJECT");
-  return e && std::strcmp(e, "krylov") == 0;
+  return e && std::strcmp(e, what) == 0;
 }
 
 // ---------------------------------------------------------------- FGMRES
@@ -509,7 +511,7 @@ chns_status fgmres(chns_mesh *m, const PhysCoef &pc, const T *ut, const T *dl, c
       }
       double a = H[j * mr + j], c = H[(j + 1) * mr + j];
       double rr = std::hypot(a, c);
-      if (rr == 0.0 || inject_krylov_fault()) {
+      if (rr == 0.0 || inject_fault("krylov")) {
         CHNS_CUDA_TRY(cudaStreamSynchronize(st));  // the queued step j + 1 has finished
         set_error("FGMRES breakdown at iteration %d", total + 1);
         return CHNS_ERR_KRYLOV;
@@ -1085,9 +1087,10 @@ chns_status chns_init_mu(const chns_mesh *mc, const chns_params *p, double *U, v
   double *E = ws.e64.as<double>(), *v = ws.V.as<double>(), *x = v + n;
   CgState *s = ws.hdev.as<CgState>(), *hs = reinterpret_cast<CgState *>(ws.hpinned);
   unsigned *ctr = ws.ctr.as<unsigned>();
-  CHNS_CUDA_TRY(cudaMemsetAsync(ctr, 0, 64, st));
+  const bool never = inject_fault("barrier");
+  CHNS_CUDA_TRY(cudaMemsetAsync(ctr, never ? 0xff : 0, 64, st));  // arrivals: -1, or none
   launch_mu_row(m, pc, U, E, st);
-  CHNS_CUDA_TRY(launch_cg(m, pc, E, v, ws.red.as<double>(), ctr, s, 10000, st));
+  CHNS_CUDA_TRY(launch_cg(m, pc, E, v, ws.red.as<double>(), ctr, s, 10000, never ? 4096 : 0, st));
   CHNS_CUDA_TRY(cudaMemcpyAsync(hs, s, sizeof(CgState), cudaMemcpyDeviceToHost, st));
   CHNS_CUDA_TRY(cudaMemsetAsync(ctr, 0, 64, st));  // the other users' counters start at zero
   CHNS_CUDA_TRY(cudaStreamSynchronize(st));

@@ -1212,6 +1212,7 @@ struct CgArgs {
   unsigned *bar;
   CgState *s;
   int max_it;
+  int polls;  // of a barrier, until it is given up
 };
 
 __device__ __forceinline__ double gather1_l2(int cn, const int32_t *__restrict__ hang, const double *u) {
@@ -1223,7 +1224,7 @@ __device__ __forceinline__ double gather1_l2(int cn, const int32_t *__restrict__
 }
 
 // all blocks have arrived for the epoch-th time; false: given up
-__device__ __forceinline__ bool cg_barrier(unsigned *bar, unsigned &epoch, int *given_up) {
+__device__ __forceinline__ bool cg_barrier(unsigned *bar, unsigned &epoch, int limit, int *given_up) {
   ++epoch;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1231,10 +1232,9 @@ __device__ __forceinline__ bool cg_barrier(unsigned *bar, unsigned &epoch, int *
     atomicAdd(bar, 1u);
     const unsigned want = epoch * gridDim.x;
     unsigned have;
-    int polls = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(have) : "l"(bar) : "memory");
-    } while (have < want && ++polls < kCgPolls);
+    } while (have < want && --limit > 0);
     *given_up = have < want;
     __threadfence();
   }
@@ -1245,7 +1245,7 @@ __device__ __forceinline__ bool cg_barrier(unsigned *bar, unsigned &epoch, int *
 // tot[v] = sum over all threads of the grid of acc[v], with a grid barrier
 template <int N>
 __device__ __forceinline__ bool cg_sum(const double (&acc)[N], double *tot, double *partial, unsigned *bar,
-                                       unsigned &epoch, int *given_up) {
+                                       unsigned &epoch, int limit, int *given_up) {
   __shared__ double all[N][kCgBlock], four[N][4];
   const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31;
 #pragma unroll
@@ -1264,7 +1264,7 @@ __device__ __forceinline__ bool cg_sum(const double (&acc)[N], double *tot, doub
     const double *f = four[threadIdx.x];
     __stcg(partial + threadIdx.x * gridDim.x + blockIdx.x, (f[0] + f[1]) + (f[2] + f[3]));
   }
-  if (!cg_barrier(bar, epoch, given_up)) return false;
+  if (!cg_barrier(bar, epoch, limit, given_up)) return false;
   if (wid < N) {
     double t = 0.0;
     for (unsigned b = ln; b < gridDim.x; b += 32) t += __ldcg(partial + wid * gridDim.x + b);
@@ -1308,10 +1308,10 @@ __global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant
   unsigned epoch = 0;
   int err = 0, it = 0;
   for (int64_t i = t0; i < g.n; i += step) g.r[i] = cg_node_sum(g, i);
-  if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; goto end; }
+  if (!cg_barrier(g.bar, epoch, g.polls, &given_up)) { err = 2; goto end; }
   for (int64_t t = t0; t < slots; t += step)
     g.E[t] = scale2(g.W0, -D * int(g.level[t >> D])) * (D == 2 ? 2.25 : 3.375);  // the product with ones
-  if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; goto end; }
+  if (!cg_barrier(g.bar, epoch, g.polls, &given_up)) { err = 2; goto end; }
   {
     double acc[2] = {0.0, 0.0};
     for (int64_t i = t0; i < g.n; i += step) {
@@ -1323,7 +1323,7 @@ __global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant
       acc[0] = fma(ri, zi, acc[0]);
       acc[1] = fma(ri, ri, acc[1]);
     }
-    if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, &given_up)) { err = 2; goto end; }
+    if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, g.polls, &given_up)) { err = 2; goto end; }
   }
   {
     double rz = tot[0], rr = tot[1], beta = 0.0;
@@ -1348,7 +1348,7 @@ __global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant
           if (t < slots) g.E[t] = scale2(g.W0, -D * l[k]) * u[k];
         }
       }
-      if (!cg_barrier(g.bar, epoch, &given_up)) { err = 2; break; }
+      if (!cg_barrier(g.bar, epoch, g.polls, &given_up)) { err = 2; break; }
       double pq[1] = {0.0}, acc[2] = {0.0, 0.0};
       for (int64_t i = t0; i < g.n; i += step) {
         const double sum = cg_node_sum(g, i), pi = fma(beta, g.p[i], g.z[i]);
@@ -1356,7 +1356,7 @@ __global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant
         g.p[i] = pi;
         pq[0] = fma(pi, sum, pq[0]);
       }
-      if (!cg_sum<1>(pq, tpq, g.partial + 2 * gridDim.x, g.bar, epoch, &given_up)) { err = 2; break; }
+      if (!cg_sum<1>(pq, tpq, g.partial + 2 * gridDim.x, g.bar, epoch, g.polls, &given_up)) { err = 2; break; }
       if (!(tpq[0] > 0.0)) { err = 1; break; }
       if (threadIdx.x == 0) ash = rz / tpq[0];  // one division a block: ten instructions of the FP64 pipe
       __syncthreads();
@@ -1369,7 +1369,7 @@ __global__ void __launch_bounds__(kCgBlock, kCgPerSm) k_cg(const __grid_constant
         acc[0] = fma(ri, zi, acc[0]);
         acc[1] = fma(ri, ri, acc[1]);
       }
-      if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, &given_up)) { err = 2; break; }
+      if (!cg_sum<2>(acc, tot, g.partial, g.bar, epoch, g.polls, &given_up)) { err = 2; break; }
       if (threadIdx.x == 0) ash = tot[0] / rz;
       __syncthreads();
       beta = ash;
@@ -1978,10 +1978,10 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
 
 // x = M^-1 (node sums of E); v: six vectors of n_nodes; part: at least
 // cg_partials() doubles; ctr: zero.  Status in *s (err 1: M not positive, 2: a
-// barrier was given up).
+// barrier was given up).  polls: of a barrier, 0 for the default.
 int cg_partials() { return 3 * kCgMaxGrid; }
 cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double *v, double *part, unsigned *ctr,
-                      CgState *s, int max_it, cudaStream_t st) {
+                      CgState *s, int max_it, int polls, cudaStream_t st) {
   CgArgs g{};
   const int64_t n = m->n_nodes;
   g.conn = m->conn; g.hang = m->hang; g.gptr = m->gptr; g.gent = m->gent; g.level = m->level;
@@ -1989,6 +1989,7 @@ cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double 
   g.W0 = kcoef<double>(pc, m->dim).W0 * (m->dim == 2 ? 4.0 / 9.0 : 8.0 / 27.0);
   g.E = E; g.r = v; g.x = v + n; g.p = v + 2 * n; g.q = v + 3 * n; g.d = v + 4 * n; g.z = v + 5 * n;
   g.partial = part; g.bar = ctr; g.s = s; g.max_it = max_it;
+  g.polls = polls > 0 ? polls : kCgPolls;
   int dev = 0, sms = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -36,13 +36,14 @@ void launch_tau_floor_count(const chns_mesh *m, const PhysCoef &pc, const double
 // x (the second of the six vectors of n_nodes doubles at v) = M^-1 (node sums of
 // the element-local slots E), M the scalar Q1 mass matrix, by conjugate gradients
 // in one cooperative kernel; part: cg_partials() doubles, ctr: zero.  Status in
-// *s on the device: err 1: M not positive, 2: a grid barrier was given up
+// *s on the device: err 1: M not positive, 2: a grid barrier was given up, after `polls` polls (0: the
+// default, about 20 s)
 struct CgState {
   int err, its;
 };
 int cg_partials();
 cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double *v, double *part, unsigned *ctr,
-                      CgState *s, int max_it, cudaStream_t st);
+                      CgState *s, int max_it, int polls, cudaStream_t st);
 // the chemical-potential row of U into element-local slots (n_elem * 2^dim doubles)
 void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st);
 int64_t energy_blocks(const chns_mesh *m);
