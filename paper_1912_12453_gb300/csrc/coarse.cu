@@ -826,6 +826,10 @@ T *gauss_jordan_panels(T *buf0, T *buf1, int64_t n, int n_inst, T *G, int32_t *i
   return gj_panels<T, F ? 8 : 4, 5>(buf0, buf1, n, n_inst, G, idx, origin, bad, st);
 }
 constexpr int kPanelMax = 32;  // widest panel
+// Working matrices of the inverse are kept for the next build up to this size
+// (all instances; one matrix of 2,800 rows in double), beyond it an allocation is a
+// small part of the build and they would be the larger part of the coarse space
+constexpr size_t kKeepGj = size_t(128) << 20;
 
 }  // namespace
 
@@ -1050,6 +1054,7 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
   int hbad = 0;
   CHNS_CUDA_TRY(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CHNS_CUDA_TRY(cudaStreamSynchronize(st));
+  if (C.gj.bytes > kKeepGj) C.gj.release();  // the stream has drained
   if (hbad) { set_error("singular coarse operator"); return CHNS_ERR_KRYLOV; }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error("coarse build: %s", cudaGetErrorString(e)); return CHNS_ERR_CUDA; }
