@@ -1008,13 +1008,10 @@ void chns_mesh_destroy(chns_mesh *m) {
   cudaFree(m->level);
   cudaFree(m->anchor);
   cudaFree(m->hang);
-  cudaFree(m->wall);
-  cudaFree(m->node_perm);
   cudaFree(m->node_colour);
   cudaFree(m->gptr);
   cudaFree(m->gent);
   cudaFree(m->nflag);
-  cudaFree(m->pins);
   cudaFree(m->elem_inst);
   cudaFree(m->node_inst);
   cudaFree(m->inst_dof);

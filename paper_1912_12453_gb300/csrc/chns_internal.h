@@ -139,11 +139,10 @@ struct chns_mesh {
   int n_colours = 0;
   std::vector<int64_t> colour_start;   // n_colours + 1: ranges of the colours in elem_perm
   int n_node_colours = 0;
-  std::vector<int64_t> node_colour_start;  // nodes of each node colour (for probing)
   int64_t origin = -1;                 // node at the box origin (pressure pin)
-  // pinned pressure nodes (one per problem instance)
-  int32_t *pins = nullptr;
-  int64_t n_pins = 0;
+  // host: nodes on the box boundary and pinned pressure nodes (one per problem
+  // instance); the kernels read nflag
+  std::vector<int32_t> wall, pins;
   // batched (union) meshes: several independent problems in one mesh
   int n_inst = 1;
   uint16_t *elem_inst = nullptr;       // n_elem instance of each element (device)
@@ -164,8 +163,6 @@ struct chns_mesh {
   uint8_t *level = nullptr;            // n_elem
   uint32_t *anchor = nullptr;          // n_elem * dim
   int32_t *hang = nullptr;             // n_hang * 4 parent nodes (-1 padded for edge midpoints)
-  int32_t *wall = nullptr;             // n_wall node indices on the box boundary
-  int32_t *node_perm = nullptr;        // n_nodes node indices grouped by node colour
   uint8_t *node_colour = nullptr;      // n_nodes: the node's colour (at most 256)
   // node gather of element-local J.w contributions: the (element, corner)
   // slots feeding node i are gent[gptr[i] .. gptr[i+1]), each slot e*nc+c

@@ -438,19 +438,12 @@ chns_status build_mesh(int dim, int64_t n, const uint8_t *level, const uint32_t 
     }
   }
   m->n_node_colours = n_ncol;
-  m->node_colour_start.assign(n_ncol + 1, 0);
-  for (int64_t i = 0; i < n_nodes; ++i) m->node_colour_start[ncol[i] + 1]++;
-  for (int c = 0; c < n_ncol; ++c) m->node_colour_start[c + 1] += m->node_colour_start[c];
-  // nodes grouped by colour, increasing index within a colour (counting sort)
-  std::vector<int32_t> nperm(n_nodes);
-  {
-    std::vector<int64_t> at(m->node_colour_start.begin(), m->node_colour_start.end() - 1);
-    for (int64_t i = 0; i < n_nodes; ++i) nperm[at[ncol[i]]++] = (int32_t)i;
-  }
 
   m->n_nodes = n_nodes;
   m->n_hang = n_hang;
   m->n_wall = (int64_t)wall.size();
+  m->wall = std::move(wall);
+  if (m->origin >= 0) m->pins.push_back((int32_t)m->origin);
   m->node_xyz = std::move(node_xyz);
   m->leaf_level.assign(level, level + n);
   m->leaf_anchor.assign(anchor, anchor + n * dim);
@@ -462,17 +455,9 @@ chns_status build_mesh(int dim, int64_t n, const uint8_t *level, const uint32_t 
   if ((st = upload(&m->anchor, m->leaf_anchor)) != CHNS_OK) return st;
   if ((st = upload(&m->elem_perm, eperm)) != CHNS_OK) return st;
   if ((st = upload(&m->hang, hang_dev)) != CHNS_OK) return st;
-  if ((st = upload(&m->wall, wall)) != CHNS_OK) return st;
-  {
-    std::vector<int32_t> pins;
-    if (m->origin >= 0) pins.push_back((int32_t)m->origin);
-    m->n_pins = (int64_t)pins.size();
-    if ((st = upload(&m->pins, pins)) != CHNS_OK) return st;
-  }
   m->n_inst = 1;
   m->inst_node_start = {0, n_nodes};
   m->inst_max_level = {max_level};
-  if ((st = upload(&m->node_perm, nperm)) != CHNS_OK) return st;
   const std::vector<uint8_t> ncol8(ncol.begin(), ncol.end());
   if ((st = upload(&m->node_colour, ncol8)) != CHNS_OK) return st;
   return CHNS_OK;
@@ -490,8 +475,6 @@ chns_status build_gather(chns_mesh *m) {
   if (ns >= (int64_t(1) << 30)) { set_error("mesh too large for the node gather"); return CHNS_ERR_ARG; }
   const std::vector<int32_t> conn = download(m->conn, size_t(ns));
   const std::vector<int32_t> hang = download(m->hang, size_t(m->n_hang) * 4);
-  const std::vector<int32_t> wall = download(m->wall, size_t(m->n_wall));
-  const std::vector<int32_t> pins = download(m->pins, size_t(m->n_pins));
   std::vector<int64_t> cnt(size_t(m->n_nodes) + 1, 0);
   auto each = [&](auto &&fn) {
     for (int64_t s = 0; s < ns; ++s) {
@@ -512,8 +495,8 @@ chns_status build_gather(chns_mesh *m) {
   std::vector<int64_t> fill(cnt.begin(), cnt.end() - 1);
   each([&](int32_t i, int64_t s, int code) { gent[fill[i]++] = int32_t(uint32_t(s) | (uint32_t(code) << 30)); });
   std::vector<uint8_t> nflag(size_t(m->n_nodes), 0);
-  for (int32_t i : wall) nflag[i] |= 1;
-  for (int32_t i : pins) nflag[i] |= 2;
+  for (int32_t i : m->wall) nflag[i] |= 1;
+  for (int32_t i : m->pins) nflag[i] |= 2;
   chns_status st;
   if ((st = upload(&m->gptr, gptr)) != CHNS_OK) return st;
   if ((st = upload(&m->gent, gent)) != CHNS_OK) return st;
@@ -690,36 +673,22 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
     }
     u->colour_start[c + 1] = (int64_t)eperm.size();
   }
-  std::vector<int32_t> hang, wall, pins, nperm, ninst(n_nodes);
+  std::vector<int32_t> hang, ninst(n_nodes);
   for (size_t i = 0; i < ms.size(); ++i) {
     auto h = download(ms[i]->hang, size_t(ms[i]->n_hang) * 4);
     for (int32_t v : h) hang.push_back(v >= 0 ? int32_t(v + node_off[i]) : v);
-    auto w = download(ms[i]->wall, size_t(ms[i]->n_wall));
-    for (int32_t v : w) wall.push_back(int32_t(v + node_off[i]));
-    if (ms[i]->origin >= 0) pins.push_back(int32_t(ms[i]->origin + node_off[i]));
+    for (int32_t v : ms[i]->wall) u->wall.push_back(int32_t(v + node_off[i]));
+    for (int32_t v : ms[i]->pins) u->pins.push_back(int32_t(v + node_off[i]));
     for (int64_t k = node_off[i]; k < node_off[i + 1]; ++k) ninst[k] = (int32_t)i;
     for (int64_t k = 0; k < ms[i]->n_nodes * dim; ++k) u->node_xyz.push_back(ms[i]->node_xyz[k]);
   }
   // node colours: colour c of the union = colour c of every instance
-  u->node_colour_start.assign(n_ncol + 1, 0);
-  std::vector<std::vector<int32_t>> hperm(ms.size());
   std::vector<uint8_t> ncol8;
   ncol8.reserve(size_t(n_nodes));
   for (size_t i = 0; i < ms.size(); ++i) {
-    hperm[i] = download(ms[i]->node_perm, size_t(ms[i]->n_nodes));
     const std::vector<uint8_t> c8 = download(ms[i]->node_colour, size_t(ms[i]->n_nodes));
     ncol8.insert(ncol8.end(), c8.begin(), c8.end());
   }
-  for (int c = 0; c < n_ncol; ++c) {
-    for (size_t i = 0; i < ms.size(); ++i) {
-      const chns_mesh *m = ms[i];
-      if (c >= m->n_node_colours) continue;
-      for (int64_t k = m->node_colour_start[c]; k < m->node_colour_start[c + 1]; ++k)
-        nperm.push_back(int32_t(hperm[i][k] + node_off[i]));
-    }
-    u->node_colour_start[c + 1] = (int64_t)nperm.size();
-  }
-  u->n_pins = (int64_t)pins.size();
   u->origin = -1;
   chns_status st;
   CHNS_CUDA_TRY(cudaGetDevice(&u->device));
@@ -728,9 +697,6 @@ chns_status build_union(const std::vector<const chns_mesh *> &ms, chns_mesh *u) 
   if ((st = upload(&u->anchor, anc)) != CHNS_OK) return st;
   if ((st = upload(&u->elem_perm, eperm)) != CHNS_OK) return st;
   if ((st = upload(&u->hang, hang)) != CHNS_OK) return st;
-  if ((st = upload(&u->wall, wall)) != CHNS_OK) return st;
-  if ((st = upload(&u->pins, pins)) != CHNS_OK) return st;
-  if ((st = upload(&u->node_perm, nperm)) != CHNS_OK) return st;
   if ((st = upload(&u->node_colour, ncol8)) != CHNS_OK) return st;
   if ((st = upload(&u->elem_inst, einst)) != CHNS_OK) return st;
   if ((st = upload(&u->node_inst, ninst)) != CHNS_OK) return st;

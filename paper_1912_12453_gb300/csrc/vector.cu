@@ -415,7 +415,6 @@ template <typename T>
 static unsigned red_grid(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n / V16<T>::L + kB - 1) / kB, kRedBlocks));
 }
-// one node per thread up to the reduction's block count
 
 template <typename T>
 void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double *partial, double *h,

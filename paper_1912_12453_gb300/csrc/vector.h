@@ -19,8 +19,9 @@ constexpr int64_t kVecAlign = 64;
 inline int64_t vec_ld(int64_t n) { return (n + kVecAlign - 1) / kVecAlign * kVecAlign; }
 
 // h[i] = V_i . w for i < nv; partial: (nv + 8) * red_blocks() doubles;
-// counter: a device word that is zero between launches (grid reduction
-// ticket); skipped (h unchanged) when flag is given and *flag == 0
+// counter: ceil(nv / 8) device words that are zero between launches (the tickets
+// of the grid reduction, one per eight vectors); skipped (h unchanged) when flag
+// is given and *flag == 0
 template <typename T>
 void vec_multidot(const T *V, int64_t ld, int nv, const T *w, int64_t n, double *partial, double *h,
                   cudaStream_t st, const int *flag, unsigned *counter);
