@@ -275,7 +275,7 @@ chns_status chns_energy_mass(const chns_mesh *mesh, const chns_params *params,
  * counterpart; it computes the same three integrals as chns_energy_mass, in
  * the same order.  out3: caller-owned DEVICE array of 3 doubles receiving
  * (energy, integral of phi, volume with phi < 0); asynchronous on stream.
- * The reduction scratch is a fixed 1.5 MiB array inside the library, held
+ * The reduction scratch is a fixed array of 14 KiB inside the library, held
  * by every GPU that loads it until the process exits; meshes of more than
  * 2,097,152 leaves in 3D (4,194,304 in 2D) are rejected with CHNS_ERR_ARG.
  * The first call on each device looks up that array's device address; make

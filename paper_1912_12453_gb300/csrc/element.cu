@@ -2044,7 +2044,7 @@ chns_status copy_coef_tables(const chns_mesh *src, chns_mesh *dst) {
   return CHNS_OK;
 }
 
-int64_t energy_blocks(const chns_mesh *m) { return std::min<int64_t>(grid_for(m->n_elem << m->dim), 152 * 4); }
+int64_t energy_blocks(const chns_mesh *m) { return std::min<int64_t>(grid_for(m->n_elem << m->dim), kEnergyBlocks); }
 
 void launch_energy(const chns_mesh *m, const PhysCoef &pc, const double *U, double *partial, double *out3,
                    cudaStream_t st) {

@@ -46,6 +46,7 @@ cudaError_t launch_cg(const chns_mesh *m, const PhysCoef &pc, double *E, double 
                       CgState *s, int max_it, int polls, cudaStream_t st);
 // the chemical-potential row of U into element-local slots (n_elem * 2^dim doubles)
 void launch_mu_row(const chns_mesh *m, const PhysCoef &pc, const double *U, double *E, cudaStream_t st);
+constexpr int kEnergyBlocks = 152 * 4;  // most blocks of the energy kernel
 int64_t energy_blocks(const chns_mesh *m);
 // per-instance element coefficients of a batched (union) mesh
 chns_status upload_coef_tables(chns_mesh *m, const std::vector<PhysCoef> &pcs, cudaStream_t st);

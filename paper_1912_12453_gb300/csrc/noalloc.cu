@@ -9,8 +9,9 @@
 // scratch lazily on first use; this variant never does.
 //
 // The per-block partial sums live in a file-scope device array of fixed size
-// (kMaxBlocks x 3 doubles = 1.5 MiB), which every GPU that loads the library
-// keeps until the process exits.  Host code cannot pass the array's name to
+// (kEnergyBlocks x 3 doubles = 14 KiB: the energy kernel's grid does not grow
+// with the mesh), which every GPU that loads the library keeps until the
+// process exits.  Host code cannot pass the array's name to
 // a kernel (on the host it is only a stand-in symbol), so the first call on
 // each device looks up its device address with cudaGetSymbolAddress and
 // caches it for the life of the process; make that first call before any
@@ -31,10 +32,10 @@ namespace chns {
 
 namespace {
 
-constexpr int64_t kMaxBlocks = 65536;      // energy kernel blocks (256 threads, 2^dim per element)
+constexpr int64_t kMaxCorners = int64_t(65536) * 256;  // stated in the header; callers rely on the refusal
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) double g_partials[kMaxBlocks * 3];
+static __device__ __align__(256) double g_partials[kEnergyBlocks * 3];
 
 std::mutex g_mu;
 double *g_addr[kMaxDevices] = {nullptr};
@@ -64,12 +65,9 @@ extern "C" chns_status chns_energy_mass_noalloc(const chns_mesh *m, const chns_p
   chns_status ps = check_params(m, p);  // the same checks as chns_energy_mass
   if (ps != CHNS_OK) return ps;
   if (!U || !out3) { set_error("null argument"); return CHNS_ERR_ARG; }
-  const int64_t nb = ((m->n_elem << m->dim) + 255) / 256;  // the limit is stated in leaves, whatever the grid uses
-  if (nb > kMaxBlocks) {
-    set_error("mesh too large for chns_energy_mass_noalloc: %lld elements need %lld reduction blocks, "
-              "the fixed scratch holds %lld (at most %lld leaves in 3D, %lld in 2D)",
-              (long long)m->n_elem, (long long)nb, (long long)kMaxBlocks, (long long)(kMaxBlocks * 256 / 8),
-              (long long)(kMaxBlocks * 256 / 4));
+  if ((m->n_elem << m->dim) > kMaxCorners) {
+    set_error("mesh too large for chns_energy_mass_noalloc: %lld leaves (at most %lld in 3D, %lld in 2D)",
+              (long long)m->n_elem, (long long)(kMaxCorners / 8), (long long)(kMaxCorners / 4));
     return CHNS_ERR_ARG;
   }
   int dev = 0;
