@@ -64,6 +64,14 @@ DESCRIPTION = {
 # corners only add gather loads), so the count holds for any 3D mesh while the
 # kernel is unchanged.
 JV_FLOP_PER_LEAF = {3: 7020}
+
+
+def jv_flop_per_leaf(dim, schedule):
+    """The count for the schedule that ran: 0 to 3 are k_jv_pair; 4 to 6 run
+    k_element, which is not counted (None: no roofline)."""
+    return JV_FLOP_PER_LEAF.get(dim) if 0 <= schedule < 4 else None
+
+
 # DRAM bytes (read + write) of one J.w apply, element kernel + node gather,
 # from one ncu capture of the named workload; valid for that mesh only.
 JV_TRAFFIC_PER_APPLY = {"droplet3d_l6": 36_147_968 + 81_940_224}
@@ -676,7 +684,7 @@ def main():
     peaks = _measured_peaks()
     jv_apply_ms = jv_ms / max(jv_calls, 1)
     roof = None
-    fpl = JV_FLOP_PER_LEAF.get(mesh.dim)
+    fpl = jv_flop_per_leaf(mesh.dim, stats32[-1]["jacvec_variant"])
     if fpl:
         ach = fpl * mesh.n_elem / (jv_apply_ms / 1e3) / 1e12
         traffic = JV_TRAFFIC_PER_APPLY.get(args.workload)
