@@ -129,7 +129,10 @@ constexpr int kChunk = 64;    // entries whose slots a block finds together
 // mesh node i: the nearest coarse node of colour k): the threads first find the
 // slots of kChunk entries together, then thread (s, q) adds up the entries of its
 // slot, in T in eight chains of at most eight terms, and the chunks in double:
-// 11 roundings of T on the longest way, as many as a tree over the block has.  A block of 256 threads with 48 sums each, reduced
+// 11 roundings of T on the longest way, as many as a tree over the block has.  In
+// double two chains of at most 32, since each further chain costs additions on the
+// FP64 pipe that binds there, for which entries of other warps' slots are skipped
+// too (eight chains: 4.6 ms more of 252 for the build on 29,016 adaptive leaves).  A block of 256 threads with 48 sums each, reduced
 // over the block, spent its time on the reduction: most lists hold 64 to 125
 // entries.
 template <typename T, int NF, int DIM>
@@ -147,7 +150,8 @@ __global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t 
   y += blockIdx.y * g.n_nodes * NF;
   const int s = threadIdx.x / NF, q = threadIdx.x % NF;
   const int64_t end = piece_begin[blockIdx.x + 1];
-  constexpr int G = 8;
+  constexpr int G = sizeof(T) == 8 ? 2 : 8;
+  const int s0 = (threadIdx.x & ~31) / NF, s1 = (threadIdx.x | 31) / NF;  // slots of the warp
   double acc = 0.0;
   for (int64_t b = piece_begin[blockIdx.x]; b < end; b += kChunk) {
     const int cnt = int(min(int64_t(kChunk), end - b));
@@ -177,9 +181,16 @@ __global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t 
       for (int g = 0; g < G; ++g) a[g] = T(0);
       for (int e = 0; e < cnt; e += G)
 #pragma unroll
-        for (int g = 0; g < G; ++g)
-          if (slot[e + g] == s) a[g] = fma(wgt[e + g], y[int64_t(node[e + g]) * NF + q], a[g]);
-      acc += double(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
+        for (int g = 0; g < G; ++g) {
+          const int se = slot[e + g];
+          const bool mine = sizeof(T) == 8 ? se >= s0 && se <= s1 && se == s : se == s;
+          if (mine) a[g] = fma(wgt[e + g], y[int64_t(node[e + g]) * NF + q], a[g]);
+        }
+#pragma unroll
+      for (int h = G / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int g = 0; g < h; ++g) a[g] += a[g + h];
+      acc += double(a[0]);
     }
   }
   if (s < NS) part[(blockIdx.y * int64_t(gridDim.x) + blockIdx.x) * NS * NF + threadIdx.x] = acc;
@@ -237,7 +248,7 @@ constexpr int kGroups = 32;   // lists are read by 32 groups of eight lanes
 // rc = R v = P^T v: block p sums w v[i, q] over piece p of a coarse node's
 // restriction list, lane q of each group of eight the component q: four chains of
 // at most eight terms a group, then a tree over the chains and the groups (15
-// roundings on the longest way).  part == rc when every list is one piece.  The
+// roundings on the longest way; in double two chains, fewer additions, 22).  part == rc when every list is one piece.  The
 // weights are exact (W), so in double R is P^T: a product of the three fractions of
 // a node k levels below the coarse grid has up to 3 k bits, more than a float from
 // k = 9 on (2D: 13).
@@ -258,35 +269,52 @@ __global__ void __launch_bounds__(kGroups * 8) k_restrict_lists(const int64_t *_
     w0 = T(rw[b + grp]);
   }
   wait_previous(v, part);
-  T a[4] = {T(0), T(0), T(0), T(0)};
+  constexpr int K = sizeof(T) == 8 ? 2 : 4;
+  T a[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) a[k] = T(0);
   if (q < NF && grp < cnt) {
     a[0] = w0 * v[int64_t(i0) * NF + q];
-    for (int e = grp + kGroups; e < cnt; e += 4 * kGroups)
+    constexpr int G = 8;  // independent loads, then the products
+    for (int e = grp + kGroups; e < cnt; e += G * kGroups) {
+      int32_t i[G];
+      T w[G], x[G];
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (e + k * kGroups < cnt)
-          a[k] = fma(T(rw[b + e + k * kGroups]), v[int64_t(rnode[b + e + k * kGroups]) * NF + q], a[k]);
+      for (int g = 0; g < G; ++g) {
+        const bool on = e + g * kGroups < cnt;
+        i[g] = on ? rnode[b + e + g * kGroups] : -1;
+        w[g] = on ? T(rw[b + e + g * kGroups]) : T(0);
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) x[g] = i[g] >= 0 ? v[int64_t(i[g]) * NF + q] : T(0);
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (i[g] >= 0) a[g % K] = fma(w[g], x[g], a[g % K]);
+    }
   }
-  T acc = (a[0] + a[1]) + (a[2] + a[3]);
-  acc += __shfl_xor_sync(FULL, acc, 8);
-  acc += __shfl_xor_sync(FULL, acc, 16);
-  constexpr int NW = kGroups / 4;
-  __shared__ T red[NW][8];
-  if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][q] = acc;
+#pragma unroll
+  for (int h = K / 2; h > 0; h >>= 1)
+#pragma unroll
+    for (int k = 0; k < h; ++k) a[k] += a[k + h];
+  __shared__ T red[kGroups][8];
+  red[grp][q] = a[0];
   __syncthreads();
-  if (threadIdx.x < NF) {
-    T s[NW];
+  if (threadIdx.x < 32) {  // a quarter of the groups a lane, then the quarters
+    constexpr int G = kGroups / 4;
+    T t[G];
 #pragma unroll
-    for (int w = 0; w < NW; ++w) s[w] = red[w][threadIdx.x];
+    for (int g = 0; g < G; ++g) t[g] = red[4 * g + grp][q];
 #pragma unroll
-    for (int h = NW / 2; h > 0; h >>= 1)
+    for (int h = G / 2; h > 0; h >>= 1)
 #pragma unroll
-      for (int w = 0; w < h; ++w) s[w] += s[w + h];
-    part[int64_t(blockIdx.x) * NF + threadIdx.x] = s[0];
+      for (int g = 0; g < h; ++g) t[g] += t[g + h];
+    t[0] += __shfl_xor_sync(FULL, t[0], 8);
+    t[0] += __shfl_xor_sync(FULL, t[0], 16);
+    if (threadIdx.x < NF) part[int64_t(blockIdx.x) * NF + threadIdx.x] = t[0];
   }
 }
 
-// rc = sum of the pieces, every eighth in one chain
+// rc = sum of the pieces, every eighth in one chain (double: every second)
 template <typename T>
 __global__ void k_restrict_pieces(int64_t nc, int nf, const int32_t *__restrict__ node_piece,
                                   const T *__restrict__ part, T *__restrict__ rc) {
@@ -294,16 +322,21 @@ __global__ void k_restrict_pieces(int64_t nc, int nf, const int32_t *__restrict_
   wait_previous(part, rc);
   if (t >= nc) return;
   const int64_t cp = t / nf;
-  constexpr int G = 8;
+  constexpr int G = sizeof(T) == 8 ? 2 : 8;
   T s[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) s[g] = T(0);
   const int e = node_piece[cp + 1];
+#pragma unroll 4
   for (int p = node_piece[cp]; p < e; p += G)
 #pragma unroll
     for (int g = 0; g < G; ++g)
       if (p + g < e) s[g] += part[int64_t(p + g) * nf + t % nf];
-  rc[t] = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+#pragma unroll
+  for (int h = G / 2; h > 0; h >>= 1)
+#pragma unroll
+    for (int g = 0; g < h; ++g) s[g] += s[g + h];
+  rc[t] = s[0];
 }
 
 // zc = A_c^{-1} rc, one warp per row, in precision T; row r of instance i at
