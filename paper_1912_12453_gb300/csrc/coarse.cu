@@ -132,9 +132,9 @@ constexpr int kChunk = 64;    // entries whose slots a block finds together
 // 11 roundings of T on the longest way, as many as a tree over the block has.  In
 // double two chains of at most 32, since each further chain costs additions on the
 // FP64 pipe that binds there, for which entries of other warps' slots are skipped
-// too (eight chains: 4.6 ms more of 252 for the build on 29,016 adaptive leaves).  A block of 256 threads with 48 sums each, reduced
-// over the block, spent its time on the reduction: most lists hold 64 to 125
-// entries.
+// too (eight chains: 4.6 ms more of 252 for the build on 29,016 adaptive leaves).
+// A block of 256 threads with 48 sums each, reduced over the block, spends its time
+// on the reduction: most lists hold 64 to 125 entries.
 template <typename T, int NF, int DIM>
 __global__ void __launch_bounds__(kChunk) k_gather_coarse(CGeo g, const int32_t *__restrict__ piece_node,
                                                           const int64_t *__restrict__ piece_begin,
@@ -1019,9 +1019,8 @@ chns_status coarse_build(chns_mesh *m, JvFn<T> jv, void *ctx, cudaStream_t st) {
   CHNS_CUDA_TRY(cudaMemsetAsync(M, 0, sizeof(double) * nn, st));
   // the probes (9 colours in 2D, 27 in 3D, times the fields) go through J.w in
   // batches: 45 or 162 times five launches otherwise, most of them too small to
-  // fill the GPU.  With the batches of the nodal blocks, one CN step: FP64 of
-  // the 2D droplet 18.3 -> 9.1 ms, multigrid of the level-5 3D droplet 22.5 ->
-  // 12.6 ms
+  // fill the GPU (9 of 18 ms of an FP64 CN step of the 2D droplet, 10 of 22 of a
+  // multigrid step of the level-5 3D droplet, with the probes of the nodal blocks)
   const int total = (dim == 2 ? 9 : 27) * nf;
   const size_t piece = C.direct ? 0 : sizeof(double) * size_t(C.n_pieces) * (size_t(1) << dim) * nf;
   const int batch = probe_batch(m, sizeof(T), piece, total);

@@ -432,12 +432,10 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 // That takes two matrix-vector products instead of four, one outer product
 // instead of three, and the two quotients 1/rho and rad^(-1/2) only (tau_c =
 // sqrt(rad)/tr G = rad tau_m/tr G).  Every quotient of the geometry is a power
-// of two times a constant of the box.  Bound by the FP64 pipe (residual, J.w)
-// and by the FP32 issue slots (J.w in float).  Measured on GB300, before ->
-// after: residual of the level-6 octree (262,144 leaves) 2.34 -> 1.41 ms, FP64
-// J.w of 77,932 adaptive leaves 1.27 -> 0.79 ms (0.75 with the later element
-// order and node gather), FP32 J.w of the level-6 octree with one Gauss point a
-// lane 132 -> 116 us (element kernel alone 88 -> 69 us).
+// of two times a constant of the box.  In double bound by the FP64 pipe (86 % busy):
+// residual of the level-6 octree (262,144 leaves) 1.41 ms, J.w of 77,932 adaptive
+// leaves 0.75 ms, each with its node gather (CUBE: 1.26 and 0.68); term by term as
+// in Sec. 3.4 and with a division per quotient of the geometry, 2.34 and 1.27 ms.
 //
 // nG, CI_GG, inv_trG, CnWeH come per leaf; T is the number type (a pair: two
 // Gauss points), S is T or its dual.
@@ -449,13 +447,11 @@ template <int D> __device__ __forceinline__ int hidx(int i, int j) {
 // f sign_j c_j, V comes out for plain differences of the test functions, the
 // continuity row over f.  Signs of the vector components that are not summed over
 // are flipped back on the bits.  That saves the products of 21 gradients, three
-// mixed derivatives and 18 contraction weights, FP64 instructions a lane: residual
-// 352 -> 315, J.w 616 -> 557;
-// residual of the level-6 octree 1.41 -> 1.26 ms, J.w of 77,932 leaves 0.75 ->
-// 0.68 ms.  Error against plain double code, general form -> this: residual
-// 2.7e-16 -> 2.5e-16 (uniform), 7.3e-16 -> 7.3e-16 (hanging nodes), J.w 2.6e-16 ->
-// 2.6e-16.  In 2D it was 1.5e-16 -> 1.7e-16 (J.w), so 2D keeps the general form;
-// so do other boxes, and union meshes, whose constants come from a table.
+// mixed derivatives and 18 contraction weights: 315 FP64 instructions a lane in the
+// residual (general form 352), 557 in J.w (616).  Error against plain double code:
+// residual 2.5e-16 (general form 2.7e-16; 7.3e-16 both with hanging nodes), J.w
+// 2.6e-16 both.  In 2D J.w would go from 1.5e-16 to 1.7e-16, so 2D keeps the general
+// form; so do other boxes, and union meshes, whose constants come from a table.
 template <int D, bool HASF, bool CUBE, typename T, typename S, typename C>
 __device__ __forceinline__ void gp_physics(const C &c, const T *nG, T CI_GG, T inv_trG, T CnWeH,
                                            const GpIn<D, S> &q, const T *f, S *Sq, S (*Vq)[D],
@@ -894,14 +890,12 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
 // As k_element MODE 1, with 2^(D-1) lanes per leaf: lane c holds the corners c
 // and c + 2^(D-1) (the last axis' bit) and the two Gauss points of that pair.
 // All arithmetic of the pair is packed, the last axis' stage stays in the lane.
-// Bound by issue slots with one point a lane (896 instructions per Gauss point:
-// 586 of arithmetic, 125 shuffles): packing halves the arithmetic's slots, the
-// in-lane axis half of the shuffles: 83.9 -> 37.1 M warp instructions on the
-// level-6 octree, 7,020 flop a leaf.  What bounds it now is the latency of the
-// gathers (54 % of the issue slots used, 128 registers, 14.6 warps an SM).  The
-// element kernel 69 -> 58 us; the whole apply when this came, 117 -> 98 us and
-// 631 -> 585 us (1,375,648 adaptive leaves), with the later element order and
-// node gather 81 and 455 us.
+// With one point a lane the issue slots bind (125 shuffles among the instructions
+// of a Gauss point); packing halves the arithmetic's slots, the in-lane axis half of
+// the shuffles: 37.1 M warp instructions on the level-6 octree, 7,020 flop a leaf.
+// Bound by the latency of the gathers (54 % of the issue slots used, 128 registers,
+// 14.6 warps an SM): 58 us, the whole apply with preparation and node gather 81 us
+// and 455 us on 1,375,648 adaptive leaves; with one point a lane (schedule 5) 93 us.
 template <int D>
 struct Stage2 {
   F2 sg[D - 1];  // derivative factors of the lane axes, both halves
@@ -1188,10 +1182,10 @@ __device__ __forceinline__ double gather1(int cn, const int32_t *__restrict__ ha
 // into the slots E, node sums with p.q, vector update with r.z and r.r.  Bound:
 // the barriers, the sums and the first loads of each phase, about 12 us an
 // iteration even on a mesh of 4,096 leaves; the FP64 pipe is worth about 8 of
-// the 34 us on 77,932 leaves.  Three launches an iteration -> one kernel, whole
-// call: 77,932 leaves 3.48 -> 2.47 ms, 4,096 uniform 1.28 -> 1.13, 262,144 3.44
-// -> 2.57, 1,375,648 25.6 -> 22.3, 6,976,432 110 -> 114 (there half the threads
-// an SM could hold cost more than the launches did).
+// the 34 us on 77,932 leaves.  Whole call, in brackets with three launches an
+// iteration: 77,932 leaves 2.45 ms (3.48), 4,096 uniform 1.13 (1.28), 262,144 2.57
+// (3.44), 1,375,648 22.3 (25.6), 6,976,432 114 (110: there half the threads an SM
+// could hold cost more than the launches do).
 // Block shape, 77,932 / 4,096 leaves: 1,024 threads with two products in flight
 // 2.48 / 1.13 ms, with four 2.52 / 1.31, 512 x 2 2.55 / 1.09, 512 x 3 2.95 /
 // 1.03, 256 x 6 3.54 / 0.97: more blocks, more partial sums to add.
@@ -1573,7 +1567,7 @@ __global__ void k_fix_rows(const uint8_t *__restrict__ nflag, int64_t n_nodes, c
 // constants; comparisons and conversions of integers are done on the bits, and
 // the volume is counted in cells of the finest level.  FP64 instructions a
 // leaf's lane: 58 with the comparisons in double, 39 now.  381,256 leaves, the
-// whole call: 0.84 (six divisions a lane, sums on the host) -> 0.38 -> 0.34 ms.
+// whole call: 0.33 ms; 0.84 with six divisions a lane and the sums on the host.
 struct EnergyCoef {
   double kv;                 // CA^(2D) / 2: kinetic energy from unscaled velocities
   double kpsi, kg[3];        // Cn/(We 4 Cn^2) and Cn/(2 We) times the squared derivative factors
