@@ -322,6 +322,51 @@ __device__ __forceinline__ void gather(int cn, const int32_t *__restrict__ hang,
   }
 }
 
+// Sum and increments (v and phi) of two states at a corner.  A hanging corner takes
+// the mean of its parents' increments: the difference of two means would carry the
+// rounding of the states, over dt, however small the step.
+template <int D, typename T>
+__device__ __forceinline__ void state_pair(const T *__restrict__ a, const T *__restrict__ b, T *u, T *d) {
+  constexpr int NF = D + 3;
+  T x[NF], y[NF];
+  load_block<NF>(a, x);
+  load_block<NF>(b, y);
+#pragma unroll
+  for (int k = 0; k < NF; ++k) u[k] = x[k] + y[k];
+#pragma unroll
+  for (int k = 0; k < D; ++k) d[k] = x[k] - y[k];
+  d[D] = x[D + 1] - y[D + 1];
+}
+template <int D, typename T>
+__device__ __forceinline__ void gather_states(int cn, const int32_t *__restrict__ hang, const T *__restrict__ Un,
+                                              const T *__restrict__ Uo, T *u, T *d) {
+  constexpr int NF = D + 3, ND = D + 1;
+  auto add = [&](int p) {
+    T v[NF], e[ND];
+    state_pair<D>(Un + (int64_t)p * NF, Uo + (int64_t)p * NF, v, e);
+#pragma unroll
+    for (int k = 0; k < NF; ++k) u[k] += v[k];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) d[k] += e[k];
+  };
+  const bool hangs = cn < 0;
+  const int4 p = hangs ? reinterpret_cast<const int4 *>(hang)[-cn - 1] : make_int4(cn, -1, -1, -1);
+  state_pair<D>(Un + (int64_t)p.x * NF, Uo + (int64_t)p.x * NF, u, d);
+  if (hangs) {
+    add(p.y);
+    T f = T(0.5);
+    if (p.z >= 0) {
+      add(p.z);
+      add(p.w);
+      f = T(0.25);
+    }
+#pragma unroll
+    for (int k = 0; k < NF; ++k) u[k] *= f;
+#pragma unroll
+    for (int k = 0; k < ND; ++k) d[k] *= f;
+  }
+}
+
 template <int N, typename T, typename O>
 __device__ __forceinline__ void add_block(O *__restrict__ p, const T *r, T wgt) {
   if constexpr (N % 2 == 0) {
@@ -757,16 +802,10 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
   // gather the corner's nodal blocks (MODE 0, 2: the sum of the states, twice
   // the average; the factors of the interpolation carry the half)
   T u[NF], d[ND];
-  gather<NF>(cn, hang, ut, u);
-  if (RAW) {
-    T b[NF];
-    gather<NF>(cn, hang, dl, b);
-#pragma unroll
-    for (int k = 0; k < D; ++k) d[k] = u[k] - b[k];
-    d[D] = u[D + 1] - b[D + 1];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) u[k] += b[k];
+  if constexpr (RAW) {
+    gather_states<D>(cn, hang, ut, dl, u, d);
   } else {
+    gather<NF>(cn, hang, ut, u);
     gather<ND>(cn, hang, dl, d);
   }
   T wn[NF];
