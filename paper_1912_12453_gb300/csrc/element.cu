@@ -451,8 +451,7 @@ struct KPhys : KEnd<T> {
 };
 template <typename T> struct KBox {};
 template <> struct KBox<double> {
-  double f0, rf0, nk;  // see kcube
-  double ext, C_I;     // side of the box along the first axis; C_I
+  double f0, rf0, nk, rowp0;  // see kcube
 };
 template <typename T>
 struct KCoef : KPhys<T>, KBox<T> {
@@ -656,109 +655,125 @@ struct KCube : KPhys<double> {
 // it for the residual, which sums two states), ft that of the test functions'
 // gradients; the contraction applies CA^D W to a row, so V is over CA^D.  Formed
 // from the side in extended precision and rounded once: a constant's error is the
-// same at every Gauss point, and of f it would enter to the third power.
-KCoef<double> kcube(const KCoef<double> &g, bool raw) {
-  KCoef<double> c = g;
+// same at every Gauss point, and of f it would enter to the third power.  Errors of
+// the factors on the way are taken out as in kcoef.
+KCoef<double> kcube(const PhysCoef &p, KCoef<double> c, bool raw) {
   typedef long double R;
   const R ca = R(0.5) + R(0.28867513459481288225457439025L), cad = ca * ca * ca;
-  const R ft = ca * ca / g.ext, f = raw ? ft / 2 : ft, v = ft / cad;
-  c.jcP = double(g.jcP * f * f);
-  c.ngRe = double(g.ngRe * f * f);
-  c.gRe = double(g.gRe * v * f);
-  c.xRe = double(g.xRe * v * f);
-  const R G = 4 / (R(g.ext) * g.ext);
-  for (int a = 0; a < 3; ++a) c.nG0[a] = double(-G / (f * f));
-  c.CIGG0 = double(g.C_I * 3 * G * G / (v * f * v * f));
+  const R ext = p.ext[0], ft = ca * ca / ext, f = raw ? ft / 2 : ft, v = ft / cad;
+  const R bv = R(CAD<3>) / cad;  // of values, as in kcoef
+  const R W = ext * ext * ext / 8;
+  c.cS0 = double(W * cad);
+  const R bS = R(c.cS0) / (W * cad), G = 4 / (ext * ext);
+  c.inv_dt = double(1 / (R(p.dt) * bv));
+  c.jcP = double(R(p.jc) * p.inv_Pe * f * f);
+  c.ngRe = double(-R(p.gamma) * p.inv_Re * f * f);
+  c.gRe = double(R(p.gamma) * p.inv_Re * v * f / bS);
+  c.xRe = double(R(p.xi) * p.inv_Re * v * f / bS);
+  for (int a = 0; a < 3; ++a) {
+    c.nG0[a] = double(-G / (f * f));
+    c.ngFr[a] = double(-R(p.g[a]) * p.inv_Fr / bS);
+  }
+  c.CIGG0 = double(R(p.C_I) * 3 * G * G / (v * f * v * f) * bS * bS);
   c.inv_trG0 = double(f / (3 * G));
-  c.CnWe = double(g.CnWe * (raw ? 2 : 1) / cad * f * f * f);
-  c.nCnWe = double(g.nCnWe * v * f * f);
-  c.inv_We = double(g.inv_We * f);
-  c.ninv_We = double(g.ninv_We * v);
-  c.inv_PeCn = double(g.inv_PeCn * v * f);
-  c.Cn2 = double(g.Cn2 * v * f);
+  c.CnWe = double(R(p.CnWe) * (raw ? 2 : 1) / cad * f * f * f);
+  c.nCnWe = double(-R(p.CnWe) * v * f * f / bS);
+  c.inv_We = double(R(p.inv_We) * f);
+  c.ninv_We = double(-R(p.inv_We) * v / (bv * bS));
+  c.inv_PeCn = double(R(p.inv_PeCn) * v * f / bS);
+  c.Cn2 = double(R(p.Cn2) * v * f / bS);
   c.f0 = double(f);
   c.rf0 = double(1 / f);
   c.nk = double(v / f);
+  c.rowp0 = double(W * cad * f);
   return c;
 }
 template <typename T>
 bool is_cube(const KCoef<T> &c) { return c.sg0[0] == c.sg0[1] && c.sg0[0] == c.sg0[2]; }
 
-// The constants in float.  A constant's rounding is the same at every Gauss point:
-// it shifts a whole row of J.w, where the roundings of the values average out (CA^2
-// as a float is off by 4e-8, once in a gradient and once in the test function's).
+// A constant's rounding is the same at every Gauss point: it shifts a whole row,
+// where the roundings of the values average out (CA^2 as a float is off by 4e-8, once
+// in a gradient and once in the test function's; CA^3 as a double by 4.7e-17).
 //  - Each product's constant is over the errors of the rounded factors that its
 //    terms meet on their way (values, gradients, test functions; the mean over the
 //    axes), so that a term is off by the last rounding only.
-//  - rho and eta are straight lines over phi* + end, from the lighter phase's end of
-//    the range: alpha phi* + beta leaves the light phase with the errors of two
-//    numbers that nearly cancel (2e-7 of rho at a ratio of 0.1).
-// Error of J.w against double over meshes and parameters of the tests' kind, without
-// -> with both: 2D 14 % smaller (geometric mean; the worst 44 %), 3D 5 %, momentum
-// rows of a light phase by half.  Time -0.8 % (2D) to +0.7 % (3D with hanging nodes).
-void float_constants(const PhysCoef &p, int dim, double W, double cad1, double GG, KCoef<float> &c) {
-  const double cad = cad1 * CA, bv = double(float(cad)) / cad;
-  c.cS0 = float(W * cad * (1.5 - 0.5 * bv));  // values meet both factors, phi's increment this one
-  const double bS = double(c.cS0) / (W * cad);
-  double bg = 0.0, bh = 0.0, bV = 0.0;
+//  - In float rho and eta are straight lines over phi* + end, from the lighter
+//    phase's end of the range: alpha phi* + beta leaves the light phase with the
+//    errors of two numbers that nearly cancel (2e-7 of rho at a ratio of 0.1).
+// Error without -> with, geometric means over meshes and parameters of the tests'
+// kind.  Float J.w against double: 2D -14 % (up to -44 %), 3D -5 %, momentum rows of
+// a light phase by half; time -0.8 % (2D) to +0.7 % (3D with hanging nodes).  Double
+// against 80 bits: J.w 2D -3 %, cubes (kcube) -7 %, residual of cubes -4 %.
+// Errors are held as such, in double: long double is software on Arm, 2 us a call.
+template <typename T>
+void fit_constants(const PhysCoef &p, int dim, double W, double GG, KCoef<T> &c) {
+  constexpr bool F = sizeof(T) == 4;
+  constexpr long double ca = 0.5L + 0.28867513459481288225457439025L, ca2 = ca * ca, ca3 = ca2 * ca;
+  constexpr double hi[3] = {double(ca), double(ca2), double(ca3)};
+  constexpr double lo[3] = {double(ca - hi[0]), double(ca2 - hi[1]), double(ca3 - hi[2])};
+  // error of x k as CA^n; of no use where x is beyond the range of T
+  auto error = [&](double x, double k, int n) {
+    const double e = (std::fma(x, k, -hi[n - 1]) - lo[n - 1]) / hi[n - 1];
+    return std::fabs(e) < 1e-6 ? e : 0.0;
+  };
+  auto fit = [](double x, double e) { return T(std::fma(-e, x, x)); };  // x over 1 + e
+  const double ev = error(T(dim == 2 ? CAD<2> : CAD<3>), 1.0, dim);  // of values
+  double eg = 0.0, eh = 0.0, eV = 0.0;  // of gradients (in float phi's has 1/h alone), of test gradients
   for (int a = 0; a < dim; ++a) {
-    bg += double(c.sg0[a]) * p.ext[a] / cad1 / dim;
-    bh += double(c.sh0[a]) * p.ext[a] / dim;
-    bV += double(c.cV0[a]) * p.ext[a] / (W * cad1) / dim;
+    const double x = p.ext[a], g = error(c.sg0[a], x, dim - 1), h = std::fma(double(c.sh0[a]), x, -1.0);
+    c.cV0[a] = fit(W * hi[dim - 2] / x, F ? 0.0 : g);
+    eg += g / dim;
+    eh += (F ? (std::fabs(h) < 1e-6 ? h : 0.0) : g) / dim;
+    eV += error(c.cV0[a], x / W, dim - 1) / dim;
   }
-  c.inv_dt = float(p.inv_dt / (bv * bS));
-  c.inv_dtp = float(p.inv_dt / bS);
-  c.jcP = float(p.jc * p.inv_Pe / bg);
-  c.inv_We = float(p.inv_We / bg);
-  c.ninv_We = float(-p.inv_We / (bv * bV));
-  c.CnWe = float(p.CnWe / (bh * bh * bh));
-  c.nCnWe = float(-p.CnWe / (bh * bh * bV));
-  c.inv_PeCn = float(p.inv_PeCn / (bg * bV));
-  c.Cn2 = float(p.Cn2 / (bh * bV));
-  c.ngRe = float(-p.gamma * p.inv_Re / (bg * bh));
-  c.CIGG0 = float(p.C_I * GG * (bg * bV) * (bg * bV));
-  c.end = p.alpha >= 0.0 ? 1.0f : -1.0f;
-  c.beta = float(p.beta - double(c.end) * p.alpha);
-  c.gRe = float(p.gamma * p.inv_Re / (bg * bV));
-  c.xRe = float((p.xi - double(c.end) * p.gamma) * p.inv_Re / (bg * bV));
+  // a value meets ev and eS; in float phi and its increment eS only.  In double 1/dt
+  // leaves eS: the strong residual in the continuity row then matches div v
+  c.cS0 = fit(W * hi[dim - 1], F ? 0.5 * ev : 0.0);
+  const double eS = error(c.cS0, 1.0 / W, dim), et = std::fma(p.inv_dt, p.dt, -1.0);
+  c.inv_dt = fit(p.inv_dt, et + ev + (F ? eS : 0.0));
+  if constexpr (F) c.inv_dtp = fit(p.inv_dt, et + eS);
+  for (int a = 0; a < 3; ++a) c.ngFr[a] = fit(-p.g[a] * p.inv_Fr, eS);
+  c.jcP = fit(p.jc * p.inv_Pe, eg);
+  c.inv_We = fit(p.inv_We, eg);
+  c.ninv_We = fit(-p.inv_We, ev + eV);
+  c.CnWe = fit(p.CnWe, F ? 3 * eh : 3 * eh - ev);  // in double 1 / CA^D follows
+  c.nCnWe = fit(-p.CnWe, 2 * eh + eV);
+  c.inv_PeCn = fit(p.inv_PeCn, eg + eV);
+  c.Cn2 = fit(p.Cn2, eh + eV);
+  c.ngRe = fit(-p.gamma * p.inv_Re, eg + eh);
+  c.CIGG0 = fit(p.C_I * GG, -2.0 * (eg + eV));
+  c.gRe = fit(p.gamma * p.inv_Re, eg + eV);
+  double xi = p.xi;
+  if constexpr (F) {
+    c.end = p.alpha >= 0.0 ? 1.0f : -1.0f;
+    c.beta = T(p.beta - c.end * p.alpha);
+    xi -= c.end * p.gamma;
+  }
+  c.xRe = fit(xi * p.inv_Re, eg + eV);
 }
 
 template <typename T>
 KCoef<T> kcoef(const PhysCoef &p, int dim) {
-  KCoef<T> c;
-  c.inv_dt = T(p.inv_dt); c.four_dt2 = T(p.four_dt2);
-  c.alpha = T(p.alpha); c.beta = T(p.beta);
-  c.gRe = T(p.gamma * p.inv_Re); c.ngRe = -c.gRe; c.xRe = T(p.xi * p.inv_Re);
-  c.jcP = T(p.jc * p.inv_Pe);
-  c.inv_We = T(p.inv_We); c.ninv_We = -c.inv_We; c.CnWe = T(p.CnWe); c.nCnWe = -c.CnWe;
-  c.inv_PeCn = T(p.inv_PeCn); c.Cn2 = T(p.Cn2);
+  KCoef<T> c{};
+  c.four_dt2 = T(p.four_dt2);
+  c.alpha = T(p.alpha);
+  c.beta = T(p.beta);
+  const double cad1 = dim == 2 ? CA : CA * CA;  // CA^(D-1)
   double trG = 0.0, GG = 0.0, W = 1.0;
   for (int a = 0; a < 3; ++a) {
-    c.ngFr[a] = T(-p.g[a] * p.inv_Fr);
     const double G = 4.0 / (p.ext[a] * p.ext[a]);
     c.nG0[a] = T(-G);
+    c.sg0[a] = T(cad1 / p.ext[a]);
+    c.sh0[a] = T(1.0 / p.ext[a]);
     if (a < dim) {
       trG += G;
       GG += G * G;
       W *= 0.5 * p.ext[a];
     }
   }
-  if constexpr (sizeof(T) == 8) {
-    c.f0 = c.rf0 = c.nk = 0.0;
-    c.ext = p.ext[0];
-    c.C_I = p.C_I;
-  }
-  c.CIGG0 = T(p.C_I * GG);
   c.inv_trG0 = T(1.0 / trG);
   c.W0 = T(W);
-  const double cad1 = dim == 2 ? CA : CA * CA;  // CA^(D-1)
-  c.cS0 = T(W * cad1 * CA);
-  for (int a = 0; a < 3; ++a) {
-    c.sg0[a] = T(cad1 / p.ext[a]);
-    c.sh0[a] = T(1.0 / p.ext[a]);
-    c.cV0[a] = T(W * cad1 / p.ext[a]);
-  }
-  if constexpr (sizeof(T) == 4) float_constants(p, dim, W, cad1, GG, c);
+  fit_constants<T>(p, dim, W, GG, c);
   return c;
 }
 
@@ -852,7 +867,7 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
     kc.nk = c.nk;
     s.cS = T(1);
     row = scale2(c.cS0, -D * l - (RAW ? 0 : 1));
-    rowp = row * kc.f;
+    rowp = scale2(c.rowp0, (1 - D) * l - (RAW ? 0 : 1));
     CI_GG = c.CIGG0;
     inv_trG = scale2(c.inv_trG0, -l);
     CnWeH = scale2(c.CnWe, 3 * l);
@@ -1826,11 +1841,11 @@ template void launch_prep<double>(const chns_mesh *, const double *, const doubl
 // U_new and U_old are averaged in the element kernel (10 FP64 instructions a
 // lane) rather than by a node pass before it: a state is evaluated once.
 template <int D, bool HASF>
-static void residual_elemlocal(const chns_mesh *m, const KCoef<double> &c, const double *Un, const double *Uo,
+static void residual_elemlocal(const chns_mesh *m, const PhysCoef &pc, const KCoef<double> &c, const double *Un, const double *Uo,
                                const double *f, const double *bc, double *E, double *F, cudaStream_t st) {
   if (D == 3 && !m->coef64 && is_cube(c))
     launch_next(k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks, D == 3>, grid_elem(m->n_elem << D),
-                kElemBlock, st, m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, kcube(c, true),
+                kElemBlock, st, m->conn, m->level, m->hang, 0, m->n_elem, Un, Uo, nullptr, f, E, kcube(pc, c, true),
                 nullptr, m->elem_inst, 0, 0, nullptr);
   else
     launch_next(k_element<D, double, 0, HASF, double, kElemBlock, kFp64MinBlocks>, grid_elem(m->n_elem << D),
@@ -1845,11 +1860,11 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
                      const double *bc, double *E, double *F, cudaStream_t st) {
   const KCoef<double> c = kcoef<double>(pc, m->dim);
   if (m->dim == 2) {
-    if (f) residual_elemlocal<2, true>(m, c, Un, Uo, f, bc, E, F, st);
-    else residual_elemlocal<2, false>(m, c, Un, Uo, f, bc, E, F, st);
+    if (f) residual_elemlocal<2, true>(m, pc, c, Un, Uo, f, bc, E, F, st);
+    else residual_elemlocal<2, false>(m, pc, c, Un, Uo, f, bc, E, F, st);
   } else {
-    if (f) residual_elemlocal<3, true>(m, c, Un, Uo, f, bc, E, F, st);
-    else residual_elemlocal<3, false>(m, c, Un, Uo, f, bc, E, F, st);
+    if (f) residual_elemlocal<3, true>(m, pc, c, Un, Uo, f, bc, E, F, st);
+    else residual_elemlocal<3, false>(m, pc, c, Un, Uo, f, bc, E, F, st);
   }
 }
 
@@ -1869,7 +1884,7 @@ void launch_residual(const chns_mesh *m, const PhysCoef &pc, const double *Un, c
 //      what a batch's union mesh uses (each element has its own coefficients,
 //      which as pairs would take twice the registers)
 template <int D, typename T, int BS, int MINB>
-static void elem_local(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
+static void elem_local(const chns_mesh *m, const PhysCoef &pc, const KCoef<T> &c, const KCoef<T> *tab, const T *ut, const T *dl,
                        const T *w, T *E, cudaStream_t st, int nv) {
   constexpr int NF = D + 3;
   const int64_t threads = m->n_elem << D;
@@ -1878,7 +1893,7 @@ static void elem_local(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
   if constexpr (sizeof(T) == 8 && D == 3)
     if (!tab && is_cube(c)) {
       launch_next(k_element<D, T, 1, false, T, BS, MINB, true>, ge, BS, st, m->conn, m->level, m->hang, 0, m->n_elem, ut,
-                  dl, w, nullptr, E, kcube(c, false), tab, m->elem_inst, m->n_nodes * NF, threads * NF, nullptr);
+                  dl, w, nullptr, E, kcube(pc, c, false), tab, m->elem_inst, m->n_nodes * NF, threads * NF, nullptr);
       return;
     }
   launch_next(k_element<D, T, 1, false, T, BS, MINB>, ge, BS, st, m->conn, m->level, m->hang, 0, m->n_elem, ut, dl, w,
@@ -1929,12 +1944,12 @@ static void jv_colours(const chns_mesh *m, const KCoef<T> &c, const KCoef<T> *ta
 
 // element part of J.w into E (any schedule but the colours)
 template <int D, typename T>
-static void elem_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+static void elem_dispatch(const chns_mesh *m, const PhysCoef &pc, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
                           const T *dl, const T *w, T *E, cudaStream_t st, int nv) {
   if constexpr (sizeof(T) == 8) {
     // FP64: bound by the narrow FP64 pipe, so occupancy matters less than
     // the register spills a 6-blocks-per-SM budget causes
-    elem_local<D, T, 128, kFp64MinBlocks>(m, c, tab, ut, dl, w, E, st, nv);
+    elem_local<D, T, 128, kFp64MinBlocks>(m, pc, c, tab, ut, dl, w, E, st, nv);
   } else {
     if (!tab) switch (variant) {
         case 0: elem_pair<D, 64, 8>(m, c, ut, dl, w, E, st, nv); return;
@@ -1943,13 +1958,13 @@ static void elem_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, co
         case 3: elem_pair<D, 128, 4>(m, c, ut, dl, w, E, st, nv); return;
         default: break;
       }
-    if (variant == 6) elem_local<D, T, 128, 6>(m, c, tab, ut, dl, w, E, st, nv);
-    else elem_local<D, T, 128, 5>(m, c, tab, ut, dl, w, E, st, nv);  // 5, and the pair schedules on a union mesh
+    if (variant == 6) elem_local<D, T, 128, 6>(m, pc, c, tab, ut, dl, w, E, st, nv);
+    else elem_local<D, T, 128, 5>(m, pc, c, tab, ut, dl, w, E, st, nv);  // 5, and the pair schedules on a union mesh
   }
 }
 
 template <int D, typename T>
-static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+static void jv_dispatch(const chns_mesh *m, const PhysCoef &pc, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
                         const T *dl, const T *w, T *E, T *y, uint32_t fmask, cudaStream_t st, int nv) {
   if constexpr (sizeof(T) == 4) {
     if (variant == 4 && nv == 1) {
@@ -1958,7 +1973,7 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
     }
     if (variant == 4) variant = 0;  // the colour schedule takes one direction at a time
   }
-  elem_dispatch<D, T>(m, variant, c, tab, ut, dl, w, E, st, nv);
+  elem_dispatch<D, T>(m, pc, variant, c, tab, ut, dl, w, E, st, nv);
   const dim3 gn(grid_gather<D>(m->n_nodes), (unsigned)nv);
   launch_next(k_gather_nodes<D, T, kApply>, gn, kBlock, st, m->gptr, m->gent, m->nflag, m->n_nodes, E, w, nullptr, y,
               fmask, (m->n_elem << D) * (D + 3));
@@ -1968,9 +1983,9 @@ static void jv_dispatch(const chns_mesh *m, int variant, const KCoef<T> &c, cons
 // r = b - J x, and x += B (b - J x): the element part, then one node kernel.
 // The colour schedule, which has no element-local buffer, is not used here.
 template <int D, typename T>
-static void jv_defect(const chns_mesh *m, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
+static void jv_defect(const chns_mesh *m, const PhysCoef &pc, int variant, const KCoef<T> &c, const KCoef<T> *tab, const T *ut,
                       const T *dl, const T *b, const T *B, T *E, T *x, T *r, uint32_t fmask, cudaStream_t st) {
-  elem_dispatch<D, T>(m, variant == 4 ? 0 : variant, c, tab, ut, dl, x, E, st, 1);
+  elem_dispatch<D, T>(m, pc, variant == 4 ? 0 : variant, c, tab, ut, dl, x, E, st, 1);
   if (r)
     launch_next(k_gather_nodes<D, T, kDefect>, grid_gather<D>(m->n_nodes), kBlock, st, m->gptr, m->gent, m->nflag,
                 m->n_nodes, E, x, b, r, fmask, 0);
@@ -1986,8 +2001,8 @@ void launch_jacvec(const chns_mesh *m, const PhysCoef &pc, const T *ut, const T 
   KCoef<T> c = kcoef<T>(pc, m->dim);
   const KCoef<T> *tab = reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32);
   if (variant < 0) variant = sizeof(T) == 4 ? m->jv_variant : 0;
-  if (m->dim == 2) jv_dispatch<2, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
-  else jv_dispatch<3, T>(m, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
+  if (m->dim == 2) jv_dispatch<2, T>(m, pc, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
+  else jv_dispatch<3, T>(m, pc, variant, c, tab, ut, dl, w, E, y, pc.fmask, st, nv);
 }
 template void launch_jacvec<float>(const chns_mesh *, const PhysCoef &, const float *, const float *,
                                    const float *, float *, float *, cudaStream_t, int, int);
@@ -2034,8 +2049,8 @@ void launch_jacvec_defect(const chns_mesh *m, const PhysCoef &pc, const T *ut, c
   const KCoef<T> c = kcoef<T>(pc, m->dim);
   const KCoef<T> *tab = reinterpret_cast<const KCoef<T> *>(sizeof(T) == 8 ? m->coef64 : m->coef32);
   const int variant = sizeof(T) == 4 ? m->jv_variant : 0;
-  if (m->dim == 2) jv_defect<2, T>(m, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
-  else jv_defect<3, T>(m, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
+  if (m->dim == 2) jv_defect<2, T>(m, pc, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
+  else jv_defect<3, T>(m, pc, variant, c, tab, ut, dl, b, B, E, x, r, pc.fmask, st);
 }
 template void launch_jacvec_defect<float>(const chns_mesh *, const PhysCoef &, const float *, const float *,
                                           const float *, const float *, float *, float *, float *, cudaStream_t);
