@@ -997,10 +997,10 @@ __global__ void __launch_bounds__(BS, MINB) k_element(
 // All arithmetic of the pair is packed, the last axis' stage stays in the lane.
 // With one point a lane the issue slots bind (125 shuffles among the instructions
 // of a Gauss point); packing halves the arithmetic's slots, the in-lane axis half of
-// the shuffles: 37.1 M warp instructions on the level-6 octree, 7,020 flop a leaf.
+// the shuffles: 37.5 M warp instructions on the level-6 octree, 7,028 flop a leaf.
 // Bound by the latency of the gathers (54 % of the issue slots used, 128 registers,
 // 14.6 warps an SM): 58 us, the whole apply with preparation and node gather 81 us
-// and 455 us on 1,375,648 adaptive leaves; with one point a lane (schedule 5) 93 us.
+// and 457 us on 1,375,648 adaptive leaves; with one point a lane (schedule 5) 93 us.
 template <int D>
 struct Stage2 {
   F2 sg[D - 1];  // derivative factors of the lane axes, both halves
